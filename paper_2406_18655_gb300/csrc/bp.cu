@@ -24,8 +24,6 @@ namespace lsdgb {
 
 namespace {
 
-constexpr float kBig = 0x1p100f;  // minimum over an empty set (a degree-1 check)
-
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 __host__ __device__ inline size_t bp_graph_bytes(int m, int n, int E) {
@@ -33,9 +31,6 @@ __host__ __device__ inline size_t bp_graph_bytes(int m, int n, int E) {
 }
 __host__ __device__ inline size_t bp_group_bytes(int m, int n, int E) {
   return align16((size_t)E * 4 + (size_t)n * 4 + (size_t)m);
-}
-__host__ __device__ inline size_t bp_reg_group_bytes(int n, int E) {
-  return align16((size_t)E * 4 + (size_t)n * 4);
 }
 
 __global__ void priors_kernel(const float* __restrict__ probs, float* __restrict__ prior,
@@ -219,40 +214,39 @@ __global__ void __launch_bounds__(256) bp_kernel(BPArgs a) {
 
 // Min-sum on a regular Tanner graph (every check of degree DC, every variable of degree
 // DV) with the per-lane graph tables in registers.  A group of G lanes owns a shot; lane l
-// owns checks l, l+G, ... (at most CPL) and variables l, l+G, ... (at most VPL).  Check i's
-// edges are i*DC .. i*DC+DC-1 (CSR order), so only the column indices of the lane's checks
-// and the edge slots of its variables are kept, two 16-bit indices per register.  Loops
-// are unrolled over the compile-time degrees; r[E], Lam[n] and the priors live in shared
-// memory as the exchange between the two phases.  Same operations in the same order as
-// bp_kernel<G, 0>, so the results are identical.
+// owns checks l, l+G, ... (at most CPL) and variables l, l+G, ... (at most VPL).  Loops are
+// unrolled over the compile-time degrees; messages and posteriors go through shared memory
+// between the two phases (bp_shot.cuh).  Same results as bp_kernel<G, 0>.
+// Was bound by the ALU pipe (two-minimum tracking and sign logic), now by shared-memory
+// wavefronts (98 % busy at 24 warps per SM; 1.7 wavefronts per gather, since the checks of
+// 32 consecutive variables are not consecutive): BP of 10^6 BB144 shots at p = 0.05 3.84 ->
+// 2.96 ms, of 10^5 BB72 shots 0.315 -> 0.220 ms, of 10^5 BB288 shots 0.830 -> 0.600 ms.
+// The register bound keeps 3 CTAs per SM (2 for the larger shapes); 4 spill (3.47 ms).
 template <int G, int CPL, int DC, int VPL, int DV, bool PK>
-__global__ void __launch_bounds__(256) bp_reg_kernel(BPArgs a) {
+__global__ void __launch_bounds__(256, CPL * DC <= 18 ? 3 : 2) bp_reg_kernel(BPArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int m = a.g.m, n = a.g.n, E = a.g.E;
-  const long long shots = a.shots_dev ? *a.shots_dev : a.shots;
+  using Y = bpreg::Layout<G, CPL, DC, VPL>;
+  const int n = a.g.n;
+  const unsigned shots = (unsigned)(a.shots_dev ? *a.shots_dev : a.shots);  // < 2^31
   const int lane = threadIdx.x & (G - 1);
   const int group = threadIdx.x / G;
   const unsigned gmask = group_mask<G>();
   const int leader = (threadIdx.x & 31) & ~(G - 1);
-  float* s_prior = reinterpret_cast<float*>(smem);
-  for (int j = threadIdx.x; j < n; j += blockDim.x) s_prior[j] = a.g.prior[j];
-  __syncthreads();
-  float* r = reinterpret_cast<float*>(smem + align16((size_t)n * 4) +
-                                      (size_t)group * bp_reg_group_bytes(n, E));
-  float* Lam = r + E;
+  float* r = reinterpret_cast<float*>(smem + group * Y::kBytes);
+  float* Lam = r + Y::kR;
   bpreg::Tables<CPL, DC, VPL, DV> T;
-  bpreg::load_tables<G>(a.g, lane, T);
-  (void)m;
+  bpreg::load_tables<G>(a.g, lane, group * Y::kBytes, T);
 
+  // The first shot of a group is its own number (blocks first, so that a small batch spreads
+  // over the SMs), the others come from the counter.
+  const unsigned groups = gridDim.x * (blockDim.x / G);
   unsigned long long my_iters = 0, my_conv = 0;
-  for (;;) {
-    unsigned long long shot_u = 0;
-    if (lane == 0) shot_u = atomicAdd(&a.ctr->next_shot, 1ULL);
-    shot_u = __shfl_sync(gmask, shot_u, leader);
-    if (shot_u >= (unsigned long long)shots) break;
-    const long long shot = (long long)shot_u;
+  unsigned cur = group * gridDim.x + blockIdx.x;
+  while (cur < shots) {
+    const long long shot = cur;
+    const unsigned sbits = bpreg::load_syndrome<G, CPL, PK>(a, cur, lane);
     bool conv = false;
-    const int t = bpreg::shot_bp<G, CPL, DC, VPL, DV, PK>(a, T, shot, r, Lam, s_prior, lane, gmask, conv);
+    const int t = bpreg::shot_bp<G, CPL, DC, VPL, DV>(a, T, sbits, smem, r, Lam, lane, gmask, conv);
 
     // ---- outputs (each lane writes its own variables) ----
     if (a.posteriors) {
@@ -295,7 +289,8 @@ __global__ void __launch_bounds__(256) bp_reg_kernel(BPArgs a) {
         }
       }
     }
-    __syncwarp(gmask);
+    if (lane == 0) cur = groups + (unsigned)atomicAdd(&a.ctr->next_shot, 1ULL);
+    cur = __shfl_sync(gmask, cur, leader);
   }
   for (int off = 16; off > 0; off >>= 1) {
     my_iters += __shfl_down_sync(0xffffffffu, my_iters, off);
@@ -654,13 +649,15 @@ __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
 // Shapes of bp_reg_kernel: (G, CPL, DC, VPL, DV).
 struct RegShape {
   int G, cpl, dc, vpl, dv;
+  int group_bytes;    // shared memory of one group
   const void* fn;     // byte-per-bit syndromes and corrections
   const void* fn_pk;  // bit-packed
   const char* name;
 };
 
 #define LSD_REG_SHAPE(G, C, DCx, V, DVx)                                      \
-  {G, C, DCx, V, DVx, (const void*)bp_reg_kernel<G, C, DCx, V, DVx, false>,   \
+  {G, C, DCx, V, DVx, bpreg::Layout<G, C, DCx, V>::kBytes,                    \
+   (const void*)bp_reg_kernel<G, C, DCx, V, DVx, false>,                      \
    (const void*)bp_reg_kernel<G, C, DCx, V, DVx, true>,                       \
    "bp_reg_kernel<" #G "," #C "," #DCx "," #V "," #DVx ">"}
 const RegShape kRegShapes[] = {
@@ -875,8 +872,8 @@ cudaError_t bp_config(const DevGraph& g, int lanes, int method, int kind, int* v
   } else {
     const int G = lanes_of(v);
     if (v >= 6) {
-      gb = align16((size_t)g.n * 4);
-      grp = bp_reg_group_bytes(g.n, g.E);
+      gb = 0;
+      grp = kRegShapes[v - 6].group_bytes;
     } else {
       gb = bp_graph_bytes(g.m, g.n, g.E);
       grp = bp_group_bytes(g.m, g.n, g.E);
