@@ -441,157 +441,201 @@ __global__ void __launch_bounds__(512) bp_cta_kernel(BPArgs a) {
 }
 
 // BP for large graphs with register-resident tables: one CTA of NT threads owns one shot;
-// like bp_reg_kernel, thread t keeps the column indices of checks t, t + NT, ... and the
-// message slots of variables t, t + NT, ... in registers (two 16-bit indices per register),
-// so no graph table is read while iterating.  Messages r live in shared memory row-major
-// with DC slots per check (slot i * DC + k for the k-th edge of check i) plus a slot Z = m DC
-// that stays zero; columns of degree < DV are padded with Z, added last, which leaves Lambda
-// unchanged.  PAD: checks of degree < DC are padded with a dummy column n whose Lambda stays
-// 2^100 (kBig) and whose slots are read as zero and never written.  kBig is also where the
-// two running minima of a check start, so a padded edge changes neither minimum, sign nor
-// hard-decision parity: the update equals the unpadded one bit for bit.  Same operations in
-// the same order as bp_kernel<G, 0>.
-template <int NT, int CPL, int DC, int VPL, int DV, bool PAD, int MINB, bool PK>
+// like bp_reg_kernel, thread t keeps the shared-memory words of the posteriors of checks
+// t, t + NT, ... and of the messages of variables t, t + NT, ... in registers (two 16-bit
+// word indices per register), so no graph table is read while iterating.  Message k of check
+// slot c of thread t is word (c DC + k) NT + t: the threads of a store, and of a gather over
+// consecutive checks, hit consecutive banks.  Columns of degree < DV are padded with a word
+// that stays zero, added last, which leaves Lambda unchanged.  Checks of degree < DC (and
+// check slots past m) are padded with a dummy posterior +inf: q = inf - r = inf changes no
+// minimum (they start at kBig) and no sign or parity, and the message written for it is read
+// by nobody but its own q: the update equals the unpadded one bit for bit, without a
+// predicate.  Same results as bp_kernel<G, 0>.
+// Bound by shared-memory wavefronts: with DC words per row the row stride of 8 words made
+// every store, reload and gather of a message an 8-way bank conflict.  BP of 100 003 shots of
+// the BB144 d = 12 space-time matrix 3.30 -> 1.21 ms, 20 000 of BB288 d = 18 2.62 -> 1.20 ms,
+// 99 991 of the BB144 d = 6 hooks matrix 3.19 -> 2.10 ms, 50 000 of HGP at p = 0.02 8.89 ->
+// 5.86 ms.  Testing the parities before the messages are computed (MSG) costs a barrier and
+// saves a converged shot's last update: 1.34 -> 1.21 ms of the first of these.
+//   PAD  rows may be shorter than DC (else chk_ptr[i] = i DC)
+//   MSG  the thread's messages stay in registers too (else they are read back from its words)
+//   PRI  the priors of its variables as well (else shared memory)
+template <int NT, int CPL, int DC, int VPL, int DV, bool PAD, int MINB, bool PK, bool MSG, bool PRI>
 __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned long long s_shot;
+  __shared__ unsigned s_shot[2];
   __shared__ unsigned long long s_slot;
+  constexpr int kLam = CPL * DC * NT;       // posteriors start here (words)
+  constexpr int kInf = kLam + VPL * NT;     // the dummy posterior, then the zero message
   const int m = a.g.m, n = a.g.n;
-  const int Z = m * DC;
-  const long long shots = a.shots_dev ? *a.shots_dev : a.shots;
+  const unsigned shots = (unsigned)(a.shots_dev ? *a.shots_dev : a.shots);  // < 2^31
   const int tid = threadIdx.x;
-  float* r = reinterpret_cast<float*>(smem);           // [m DC + 1], r[Z] == 0
-  float* Lam = r + align16((size_t)(Z + 1) * 4) / 4;   // [n + 1], Lam[n] == kBig
-  float* s_prior = Lam + align16((size_t)(n + 1) * 4) / 4;  // [n]
-  const float alpha = a.alpha;
+  float* const w = reinterpret_cast<float*>(smem);
+  float* const Lam = w + kLam;
+  float* const s_prior = w + kInf + 4;      // [VPL NT] when !PRI
   uint32_t cv[CPL][(DC + 1) / 2];
 #pragma unroll
   for (int c = 0; c < CPL; ++c) {
     const int i = tid + NT * c;
+    const int p0 = PAD && i < m ? a.g.chk_ptr[i] : i * DC;
+    const int deg = i >= m ? 0 : PAD ? a.g.chk_ptr[i + 1] - p0 : DC;
 #pragma unroll
     for (int k = 0; k < (DC + 1) / 2; ++k) cv[c][k] = 0;
-    if (i < m) {
-      // row-regular graphs (PAD false): chk_ptr[i] = i DC
-      const int p0 = PAD ? a.g.chk_ptr[i] : i * DC;
-      const int deg = PAD ? a.g.chk_ptr[i + 1] - p0 : DC;
 #pragma unroll
-      for (int k = 0; k < DC; ++k) {
-        const uint32_t j = k < deg ? (uint32_t)a.g.chk_var[p0 + k] : (uint32_t)n;
-        cv[c][k >> 1] |= j << (16 * (k & 1));
-      }
+    for (int k = 0; k < DC; ++k) {
+      const uint32_t j = k < deg ? (uint32_t)(kLam + a.g.chk_var[p0 + k]) : (uint32_t)kInf;
+      cv[c][k >> 1] |= j << (16 * (k & 1));
     }
   }
   uint32_t ve[VPL][(DV + 1) / 2];
+  float prior[PRI ? VPL : 1];
 #pragma unroll
   for (int v = 0; v < VPL; ++v) {
     const int j = tid + NT * v;
+    const int q0 = j < n ? a.g.var_ptr[j] : 0, deg = j < n ? a.g.var_ptr[j + 1] - q0 : 0;
 #pragma unroll
     for (int k = 0; k < (DV + 1) / 2; ++k) ve[v][k] = 0;
-    if (j < n) {
-      const int q0 = a.g.var_ptr[j], deg = a.g.var_ptr[j + 1] - q0;
 #pragma unroll
-      for (int k = 0; k < DV; ++k) {
-        uint32_t e = (uint32_t)Z;
-        if (k < deg) {
-          if constexpr (PAD) {
-            const int i = a.g.var_chk[q0 + k];
-            e = (uint32_t)(i * DC + (a.g.var_edge[q0 + k] - a.g.chk_ptr[i]));
-          } else {
-            e = (uint32_t)a.g.var_edge[q0 + k];  // = i DC + k when every row has DC edges
-          }
-        }
-        ve[v][k >> 1] |= e << (16 * (k & 1));
+    for (int k = 0; k < DV; ++k) {
+      uint32_t e = (uint32_t)(kInf + 1);
+      if (k < deg) {
+        const int i = a.g.var_chk[q0 + k];
+        const int pos = a.g.var_edge[q0 + k] - (PAD ? a.g.chk_ptr[i] : i * DC);
+        e = (uint32_t)(((i / NT) * DC + pos) * NT + i % NT);
       }
-      s_prior[j] = a.g.prior[j];
+      ve[v][k >> 1] |= e << (16 * (k & 1));
     }
+    const float lam = j < n ? a.g.prior[j] : 0.f;
+    if constexpr (PRI) prior[v] = lam;
+    else s_prior[j] = lam;
   }
-  if (tid == 0) {
-    r[Z] = 0.f;
-    Lam[n] = kBig;
-  }
-  unsigned long long my_iters = 0, my_conv = 0;
-  for (;;) {
-    if (tid == 0) s_shot = atomicAdd(&a.ctr->next_shot, 1ULL);
-    __syncthreads();
-    const unsigned long long shot_u = s_shot;
-    if (shot_u >= (unsigned long long)shots) break;
-    const long long shot = (long long)shot_u;
-    const uint8_t* sp = a.syndromes + shot * m;
-    unsigned sbits = 0;
+  auto word = [&](uint32_t pair, int half) { return w[half ? pair >> 16 : pair & 0xffffu]; };
+  // the syndrome bits of a shot's checks of this thread
+  auto load_syndrome = [&](long long shot) {
+    unsigned bits = 0;
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
       const int i = tid + NT * c;
       if (i < m) {
         if constexpr (PK) {
           const uint32_t* spw = reinterpret_cast<const uint32_t*>(a.syndromes) + shot * packed_words(m);
-          if ((spw[i >> 5] >> (i & 31)) & 1u) sbits |= 1u << c;
+          if ((spw[i >> 5] >> (i & 31)) & 1u) bits |= 1u << c;
         } else {
-          if (sp[i]) sbits |= 1u << c;
+          if (a.syndromes[shot * m + i]) bits |= 1u << c;
         }
-#pragma unroll
-        for (int k = 0; k < DC; ++k) r[i * DC + k] = 0.f;
       }
     }
+    return bits;
+  };
+  // The first shot of a CTA is its block index, the others come from the counter.  With one
+  // CTA per SM nothing hides the counter's reply and the syndrome load, so while many shots
+  // are left a CTA takes its next two ahead (50 000 HGP shots 6.03 -> 5.86 ms); near the end it
+  // takes one at a time, so that none waits behind a long shot (taken ahead to the very end,
+  // 1000 HGP shots take 0.45 ms instead of 0.42).
+  constexpr bool kAhead = MINB == 1;
+  constexpr unsigned kNone = 0xffffffffu;
+  const unsigned ahead_end = shots > 4 * gridDim.x ? shots - 4 * gridDim.x : 0u;
+  auto take = [&] { return gridDim.x + (unsigned)atomicAdd(&a.ctr->next_shot, 1ULL); };
+  if (tid == 0) {
+    w[kInf] = __uint_as_float(0x7f800000u);
+    w[kInf + 1] = 0.f;
+    if constexpr (kAhead) s_shot[1] = blockIdx.x < ahead_end ? take() : kNone;
+  }
+  unsigned long long my_iters = 0, my_conv = 0;
+  unsigned cur = blockIdx.x;
+  unsigned next_bits = cur < shots ? load_syndrome(cur) : 0u;
+  for (int ph = 1; cur < shots; ph ^= 1) {
+    const long long shot = cur;
+    const unsigned sbits = next_bits;
+    unsigned pending = kNone;
+    if (kAhead && tid == 0 && cur < ahead_end) pending = take();
+    float msg[MSG ? CPL : 1][DC];
+    if constexpr (MSG) {
 #pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int j = tid + NT * v;
-      if (j < n) Lam[j] = s_prior[j];
+      for (int c = 0; c < CPL; ++c)
+#pragma unroll
+        for (int k = 0; k < DC; ++k) msg[c][k] = 0.f;
+    } else {
+#pragma unroll
+      for (int c = 0; c < CPL * DC; ++c) w[c * NT + tid] = 0.f;
     }
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) Lam[tid + NT * v] = PRI ? prior[PRI ? v : 0] : s_prior[tid + NT * v];
     __syncthreads();
+    if constexpr (kAhead) {
+      cur = s_shot[ph];
+      if (cur < shots) next_bits = load_syndrome(cur);
+    }
     int t = 0;
     bool conv = false;
     for (;;) {
       const bool msgs = t < a.iters;
-      unsigned unsat = 0;
-      // ---- check phase (the update of bp_reg_kernel) ----
+      uint32_t unsat = 0;
+      if constexpr (MSG) {
+        // ---- check phase: parities and q (in the messages' place), then the new messages ----
 #pragma unroll
-      for (int c = 0; c < CPL; ++c) {
-        const int i = tid + NT * c;
-        if (i >= m) continue;
-        uint32_t hp = (sbits >> c) << 31;
-        uint32_t sx = hp;
-        float min1 = kBig, min2 = kBig;
-        float aq[DC];
-        uint32_t qb[DC];
-        float* rc = r + i * DC;
-#pragma unroll
-        for (int k = 0; k < DC; ++k) {
-          const int j = (cv[c][k >> 1] >> (16 * (k & 1))) & 0xffff;
-          const float L = Lam[j];
-          hp ^= __float_as_uint(L);
-          const float q = __fsub_rn(L, rc[k]);
-          qb[k] = __float_as_uint(q);
-          sx ^= qb[k];
-          aq[k] = fabsf(q);
-          min2 = fminf(min2, fmaxf(min1, aq[k]));
-          min1 = fminf(min1, aq[k]);
-        }
-        unsat |= hp >> 31;
-        if (msgs) {
-          const float m1 = __fmul_rn(alpha, min1), m2 = __fmul_rn(alpha, min2);
+        for (int c = 0; c < CPL; ++c) {
+          uint32_t hp = (sbits >> c) << 31;
 #pragma unroll
           for (int k = 0; k < DC; ++k) {
-            const float mag = (aq[k] == min1) ? m2 : m1;
-            if (!PAD || ((cv[c][k >> 1] >> (16 * (k & 1))) & 0xffff) != (uint32_t)n)
-              rc[k] = __uint_as_float(__float_as_uint(mag) | ((sx ^ qb[k]) & 0x80000000u));
+            const float L = word(cv[c][k >> 1], k & 1);
+            hp ^= __float_as_uint(L);
+            msg[c][k] = __fsub_rn(L, msg[c][k]);
+          }
+          unsat |= hp;
+        }
+        if (t > 0) {
+          conv = !__syncthreads_or((int)(unsat >> 31));
+          if (conv && a.early_exit) break;
+        }
+        if (!msgs) break;
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+          float x[DC];
+          excluded_min<DC>(msg[c], x);
+          const float salpha = __uint_as_float(__float_as_uint(a.alpha) ^ ((sbits >> c) << 31));
+#pragma unroll
+          for (int k = 0; k < DC; ++k) {
+            msg[c][k] = __fmul_rn(x[k], salpha);
+            w[(c * DC + k) * NT + tid] = msg[c][k];
           }
         }
+        __syncthreads();
+      } else {
+        // ---- check phase (the update of bp_reg_kernel) ----
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+          const uint32_t sbit = (sbits >> c) << 31;
+          uint32_t hp = sbit;
+          float q[DC], x[DC];
+#pragma unroll
+          for (int k = 0; k < DC; ++k) {
+            const float L = word(cv[c][k >> 1], k & 1);
+            hp ^= __float_as_uint(L);
+            q[k] = __fsub_rn(L, w[(c * DC + k) * NT + tid]);
+          }
+          unsat |= hp;
+          if (msgs) {
+            excluded_min<DC>(q, x);
+            const float salpha = __uint_as_float(__float_as_uint(a.alpha) ^ sbit);
+#pragma unroll
+            for (int k = 0; k < DC; ++k) w[(c * DC + k) * NT + tid] = __fmul_rn(x[k], salpha);
+          }
+        }
+        const int any_unsat = __syncthreads_or((int)(unsat >> 31));
+        if (t > 0) {
+          conv = !any_unsat;
+          if (conv && a.early_exit) break;
+        }
+        if (!msgs) break;
       }
-      const int any_unsat = __syncthreads_or((int)unsat);
-      if (t > 0) {
-        conv = !any_unsat;
-        if (conv && a.early_exit) break;
-      }
-      if (!msgs) break;
       // ---- variable phase ----
 #pragma unroll
       for (int v = 0; v < VPL; ++v) {
-        const int j = tid + NT * v;
-        if (j >= n) continue;
-        float L = s_prior[j];
+        float L = PRI ? prior[PRI ? v : 0] : s_prior[tid + NT * v];
 #pragma unroll
-        for (int k = 0; k < DV; ++k) L = __fadd_rn(L, r[(ve[v][k >> 1] >> (16 * (k & 1))) & 0xffff]);
-        Lam[j] = L;
+        for (int k = 0; k < DV; ++k) L = __fadd_rn(L, word(ve[v][k >> 1], k & 1));
+        Lam[tid + NT * v] = L;
       }
       __syncthreads();
       ++t;
@@ -638,7 +682,21 @@ __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
         }
       }
     }
+    if (kAhead && tid == 0) s_shot[ph ^ 1] = pending;  // read after the next shot's first barrier
+    if (!kAhead && shots <= gridDim.x) break;
+    if (!kAhead && tid == 0) s_shot[ph] = take();
     __syncthreads();
+    if constexpr (kAhead) {
+      if (cur == kNone && shots > gridDim.x) {
+        if (tid == 0) s_shot[ph] = take();
+        __syncthreads();
+        cur = s_shot[ph];
+        if (cur < shots) next_bits = load_syndrome(cur);
+      }
+    } else {
+      cur = s_shot[ph];
+      if (cur < shots) next_bits = load_syndrome(cur);
+    }
   }
   if (tid == 0) {
     if (my_iters) atomicAdd(&a.ctr->bp_iterations, my_iters);
@@ -697,48 +755,51 @@ const void* generic_fn(int v) {
     default: return (const void*)bp_kernel<32, 1>;
   }
 }
-// Shapes of bp_regcta_kernel: (NT, CPL, DC, VPL, DV, PAD, MINB); rows of degree exactly DC
-// (PAD false) or at most DC (PAD true), columns of degree at most DV; MINB CTAs per SM bound
-// the registers a thread may take.
+// Shapes of bp_regcta_kernel: (NT, CPL, DC, VPL, DV, PAD, MINB), then MSG and PRI; rows of
+// degree exactly DC (PAD false) or at most DC (PAD true), columns of degree at most DV; MINB
+// CTAs per SM bound the registers a thread may take.  MSG and PRI are set where the bound
+// leaves room for them (spilled messages cost more than reading them back from shared memory).
 struct RegCtaShape {
   int nt, cpl, dc, vpl, dv;
-  bool pad;
+  bool pad, pri;
   const void* fn;
   const void* fn_pk;
   const char* name;
 };
-#define LSD_REGCTA_SHAPE(NT, C, DCx, V, DVx, P, MB)                                       \
-  {NT, C, DCx, V, DVx, P, (const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, false>, \
-   (const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, true>,                         \
+#define LSD_REGCTA_SHAPE(NT, C, DCx, V, DVx, P, MB, MS, PR)                                        \
+  {NT, C, DCx, V, DVx, P, PR, (const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, false, MS, PR>, \
+   (const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, true, MS, PR>,                          \
    "bp_regcta_kernel<" #NT "," #C "," #DCx "," #V "," #DVx "," #P "," #MB ">"}
 const RegCtaShape kRegCtaShapes[] = {
-    LSD_REGCTA_SHAPE(768, 4, 7, 9, 4, false, 1),   // m <= 3072, n <= 6912 (HGP of a 48 x 64 (3,4) code)
-    LSD_REGCTA_SHAPE(512, 6, 7, 13, 4, false, 1),  // same graphs, fewer threads
+    LSD_REGCTA_SHAPE(512, 6, 7, 13, 4, false, 1, false, false),  // m <= 3072, n <= 6656 (HGP of a 48 x 64 (3,4) code)
     // space-time matrices of BB codes: rows of degree w + 2 (and 1 in the last block),
     // columns of degree <= 3
-    LSD_REGCTA_SHAPE(128, 3, 8, 6, 3, true, 6),  // m <= 384, n <= 768 (BB144 (3,1) windows)
-    LSD_REGCTA_SHAPE(256, 4, 8, 11, 3, true, 2),  // m <= 1024, n <= 2816 (BB144, d = 12)
-    LSD_REGCTA_SHAPE(512, 2, 8, 6, 3, true, 1),  // m <= 1024, n <= 3072
-    LSD_REGCTA_SHAPE(512, 6, 8, 16, 3, true, 1),  // m <= 3072, n <= 8192 (BB288, d = 18)
+    LSD_REGCTA_SHAPE(128, 2, 8, 6, 3, true, 6, true, true),   // m <= 256, n <= 768 (BB72, d = 6)
+    LSD_REGCTA_SHAPE(128, 3, 8, 6, 3, true, 6, true, false),  // m <= 384, n <= 768 (BB144 (3,1) windows)
+    LSD_REGCTA_SHAPE(256, 4, 8, 11, 3, true, 2, true, false),  // m <= 1024, n <= 2816 (BB144, d = 12)
+    LSD_REGCTA_SHAPE(512, 2, 8, 6, 3, true, 1, true, true),   // m <= 1024, n <= 3072
+    LSD_REGCTA_SHAPE(512, 6, 8, 16, 3, true, 1, false, false),  // m <= 3072, n <= 8192 (BB288, d = 18)
     // ... with mid-round hook faults: rows of degree up to 17
-    LSD_REGCTA_SHAPE(256, 2, 17, 9, 3, true, 2),  // m <= 512, n <= 2304 (BB144, d = 6)
-    LSD_REGCTA_SHAPE(512, 1, 17, 5, 3, true, 1),  // m <= 512, n <= 2560
+    // (the smallest took the generic kernel, having fewer checks than 256: 100 003 shots of
+    // BB72 d = 6 4.48 -> 0.80 ms)
+    LSD_REGCTA_SHAPE(128, 2, 17, 9, 3, true, 4, true, false),  // m <= 256, n <= 1152 (BB72, d = 6)
+    LSD_REGCTA_SHAPE(256, 2, 17, 9, 3, true, 2, true, false),  // m <= 512, n <= 2304 (BB144, d = 6)
+    LSD_REGCTA_SHAPE(512, 1, 17, 5, 3, true, 1, true, true),  // m <= 512, n <= 2560
     // latency shapes (bp_kernel = 3, small batches): as many threads per shot as a CTA holds
-    LSD_REGCTA_SHAPE(1024, 3, 8, 8, 3, true, 1),  // m <= 3072, n <= 8192 (BB288, d = 18)
-    LSD_REGCTA_SHAPE(1024, 1, 8, 3, 3, true, 1),  // m <= 1024, n <= 3072 (BB144, d = 12)
-    LSD_REGCTA_SHAPE(512, 1, 8, 2, 3, true, 1),   // m <= 512, n <= 1024 (BB72, d = 6)
+    LSD_REGCTA_SHAPE(1024, 3, 7, 7, 4, false, 1, false, false),  // m <= 3072, n <= 7168 (HGP)
+    LSD_REGCTA_SHAPE(1024, 3, 8, 8, 3, true, 1, false, false),  // m <= 3072, n <= 8192 (BB288, d = 18)
+    LSD_REGCTA_SHAPE(1024, 1, 8, 3, 3, true, 1, true, true),  // m <= 1024, n <= 3072 (BB144, d = 12)
+    LSD_REGCTA_SHAPE(512, 1, 8, 2, 3, true, 1, true, true),   // m <= 512, n <= 1024 (BB72, d = 6)
 };
 #undef LSD_REGCTA_SHAPE
 constexpr int kNumRegCtaShapes = sizeof(kRegCtaShapes) / sizeof(kRegCtaShapes[0]);
 
-size_t regcta_smem(const RegCtaShape& s, const DevGraph& g) {
-  return align16(((size_t)g.m * s.dc + 1) * 4) + align16(((size_t)g.n + 1) * 4) +
-         align16((size_t)g.n * 4);
+size_t regcta_smem(const RegCtaShape& s, const DevGraph&) {
+  return ((size_t)s.nt * (s.cpl * s.dc + s.vpl * (s.pri ? 1 : 2)) + 4) * 4;
 }
 bool regcta_fits(const RegCtaShape& s, const DevGraph& g) {
   const bool rows = s.pad ? g.max_row_deg <= s.dc : (g.min_row_deg == s.dc && g.max_row_deg == s.dc);
-  return rows && g.m <= s.nt * s.cpl && g.n <= s.nt * s.vpl && g.max_col_deg <= s.dv &&
-         (long)g.m * s.dc < 65535 && g.n < 65535;
+  return rows && g.m <= s.nt * s.cpl && g.n <= s.nt * s.vpl && g.max_col_deg <= s.dv;
 }
 
 constexpr int kCtaBase = 6 + kNumRegShapes;     // + method: one CTA per shot
