@@ -50,6 +50,7 @@ struct lsd_decoder {
   int bp_variant = -1, bp_grid = 0, bp_block = 0;
   size_t bp_smem = 0;
   bool lsd_ok = false;
+  bool dense = false;        // the dense LSD kernel takes this matrix
   int lsd_warps = 0, lsd_grid = 0, lsd_W = 0;
   size_t lsd_smem = 0;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
@@ -60,8 +61,8 @@ struct lsd_decoder {
   // sparse LSD (large matrices)
   bool sparse = false;
   int sp_grid_small = 0, sp_grid_big = 0;
-  int* d_sp_small = nullptr;
-  int* d_sp_big = nullptr;
+  unsigned char* d_sp_small = nullptr;
+  unsigned char* d_sp_big = nullptr;
   int* d_spill = nullptr;
   size_t sp_stride_small = 0, sp_stride_big = 0, spill_cap = 0;
 };
@@ -241,13 +242,12 @@ int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
     return e == cudaSuccess ? LSD_OK : cuda_fail(e);
   }
   int rc;
-  if (!d->d_sp_small) {
-    const size_t warps = (size_t)d->sp_grid_small * sparse_warps_small();
+  if (!d->d_sp_big) {
     if ((rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_small),
-                        warps * d->sp_stride_small * sizeof(int))))
+                        (size_t)d->sp_grid_small * d->sp_stride_small)))
       return rc;
     if ((rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_big),
-                        (size_t)d->sp_grid_big * d->sp_stride_big * sizeof(int))))
+                        (size_t)d->sp_grid_big * d->sp_stride_big)))
       return rc;
   }
   if ((size_t)max_items > d->spill_cap) {
@@ -261,13 +261,11 @@ int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
     d->spill_cap = (size_t)max_items;
   }
   cudaError_t e = launch_sparse(l, false, d->sp_grid_small, d->d_sp_small, d->sp_stride_small,
-                                d->d_spill, &d->d_ctr->spill_count, nullptr, nullptr, d->st);
+                                d->d_spill, nullptr, d->st);
   d->launches++;
   if (e == cudaSuccess)
-    e = cudaMemsetAsync(&d->d_ctr->lsd_next, 0, sizeof(unsigned long long), d->st);
-  if (e == cudaSuccess)
-    e = launch_sparse(l, true, d->sp_grid_big, d->d_sp_big, d->sp_stride_big, nullptr, nullptr,
-                      d->d_spill, &d->d_ctr->spill_count, d->st);
+    e = launch_sparse(l, true, d->sp_grid_big, d->d_sp_big, d->sp_stride_big, nullptr, d->d_spill,
+                      d->st);
   d->launches++;
   return e == cudaSuccess ? LSD_OK : cuda_fail(e);
 }
@@ -445,18 +443,39 @@ int lsd_create(lsd_decoder** out, int32_t m, int32_t n, int64_t nnz, const int32
   ce = o.lsd_kernel == 2 ? cudaErrorInvalidValue
                          : lsd_config(g, lsd_order, o.lsd_warps, &d->lsd_warps, &d->lsd_grid,
                                       &d->lsd_smem, &d->lsd_W);
-  if (ce == cudaSuccess) {
-    d->lsd_ok = true;
-  } else {
+  if (ce == cudaSuccess)
+    d->dense = d->lsd_ok = true;
+  else
     cudaGetLastError();
-    // large matrices: the sparse LSD (not for the single-cluster mode, whose one cluster holds
-    // every detector from the start)
-    if (o.lsd_kernel != 1 && !o.single_cluster &&
-        sparse_config(g, lsd_order, &d->sp_grid_small, &d->sp_grid_big) == cudaSuccess) {
+  // The sparse LSD takes the matrices that the dense kernel does not, and those whose dense
+  // ranking is a sort in shared memory (more than 144 detectors or 288 faults).  Not for the
+  // single-cluster mode, whose one cluster holds every detector from the start.
+  const bool prefer_sparse = !d->dense || (o.lsd_kernel == 0 && (m > 144 || n > 288));
+  if (prefer_sparse && o.lsd_kernel != 1 && !o.single_cluster) {
+    const int D = std::max(max_row, 1);
+    std::vector<uint16_t> chk_pad((size_t)m * D, 0xffff), var_pad((size_t)n * 4, 0xffff);
+    for (int i = 0; i < m; ++i)
+      for (int q = chk_ptr[i]; q < chk_ptr[i + 1]; ++q) chk_pad[(size_t)i * D + q - chk_ptr[i]] = chk_var[q];
+    for (int j = 0; j < n; ++j)
+      for (int q = var_ptr[j]; q < std::min(var_ptr[j + 1], var_ptr[j] + 4); ++q)
+        var_pad[(size_t)j * 4 + q - var_ptr[j]] = var_chk[q];
+    uint16_t *d_chk_pad = nullptr, *d_var_pad = nullptr;
+    if ((rc = upload(d, &d_chk_pad, chk_pad)) || (rc = upload(d, &d_var_pad, var_pad))) {
+      lsd_destroy(d);
+      return rc;
+    }
+    ce = cudaStreamSynchronize(d->st);
+    if (ce != cudaSuccess) {
+      lsd_destroy(d);
+      return cuda_fail(ce);
+    }
+    g.chk_pad = d_chk_pad;
+    g.var_pad = d_var_pad;
+    if (sparse_config(g, lsd_order, &d->sp_grid_small, &d->sp_grid_big) == cudaSuccess) {
       d->sparse = true;
       d->lsd_ok = true;
-      d->sp_stride_small = sparse_scratch_ints(m, n, false, lsd_order > 0);
-      d->sp_stride_big = sparse_scratch_ints(m, n, true, lsd_order > 0);
+      d->sp_stride_small = sparse_scratch_bytes(m, n, false, lsd_order > 0);
+      d->sp_stride_big = sparse_scratch_bytes(m, n, true, lsd_order > 0);
     } else {
       cudaGetLastError();  // BP still works; LSD entry points report LSD_ERR_UNSUPPORTED
     }
@@ -767,7 +786,7 @@ extern "C" int lsd_decode_batch_static(lsd_decoder* d, int64_t shots, const uint
   if (!d || shots < 0 || shots > INT32_MAX) return LSD_ERR_INVALID_ARG;
   if (shots == 0) return LSD_OK;
   if (!syndromes || !corrections) return LSD_ERR_INVALID_ARG;
-  if (!d->lsd_ok || d->sparse) return LSD_ERR_UNSUPPORTED;
+  if (!d->dense) return LSD_ERR_UNSUPPORTED;
   const size_t ctr_bytes = round256(sizeof(DevCounters));
   const size_t queue_bytes = round256((size_t)shots * sizeof(int32_t));
   const size_t llr_bytes = (size_t)shots * (size_t)d->n * sizeof(float);
@@ -1236,7 +1255,7 @@ int lsdgb::bp_batch_counted(lsd_decoder* d, int64_t max_shots, const long long* 
   if (!d || max_shots <= 0 || !shots_dev || !syndromes || !corrections) return LSD_ERR_INVALID_ARG;
   if (!d->lsd_ok) return LSD_ERR_UNSUPPORTED;
   if ((size_t)max_shots > d->cap_shots) return LSD_ERR_ADMISSION;
-  if (d->sparse && (!d->d_sp_small || (size_t)max_shots > d->spill_cap)) return LSD_ERR_ADMISSION;
+  if (d->sparse && (!d->d_sp_big || (size_t)max_shots > d->spill_cap)) return LSD_ERR_ADMISSION;
   int rc = reset_counters(d);
   if (rc) return rc;
   BPArgs a = bp_args(d, max_shots, syndromes);

@@ -24,6 +24,8 @@ struct DevGraph {
   const int32_t* var_ptr;   // [n+1]
   const uint16_t* var_edge; // [E]  edges of column j (ascending row)
   const uint16_t* var_chk;  // [E]  rows of column j (ascending)
+  const uint16_t* chk_pad;  // [m][max_row_deg] columns of row i, 0xffff past its end (sparse LSD)
+  const uint16_t* var_pad;  // [n][4] the first four rows of column j, 0xffff past its end
   const float* prior;       // [n]  lambda_j (float32)
   const long long* wfix;    // [n]  2^-32 fixed point of lambda_j, LSD-mu costs
 };
@@ -42,6 +44,7 @@ struct DevCounters {
   int timeout_flag;
   int pad;
   unsigned long long spill_count;   // shots the small sparse LSD instance handed on
+  unsigned long long spill_next;    // work queue head of its large instance
 };
 
 struct BPArgs {
@@ -244,12 +247,10 @@ int window_decoder(lsd_decoder** out, int m, int n, const std::vector<std::pair<
 int window_final_round(int d, int w, int c);
 
 // LSD for large matrices (lsd_sparse.cu).
-size_t sparse_scratch_ints(int m, int n, bool big, bool mu);
+size_t sparse_scratch_bytes(int m, int n, bool big, bool mu);
 cudaError_t sparse_config(const DevGraph& g, int order, int* grid_small, int* grid_big);
-int sparse_warps_small();
-cudaError_t launch_sparse(const LSDArgs& a, bool big, int grid, int* scratch, size_t stride,
-                          int* spill, unsigned long long* spill_count, const int* items,
-                          const unsigned long long* item_count, cudaStream_t st);
+cudaError_t launch_sparse(const LSDArgs& a, bool big, int grid, unsigned char* scratch, size_t stride,
+                          int* spill, const int* items, cudaStream_t st);
 
 // Limits of this build's kernels.
 constexpr int kMaxLsdWords = 16;    // LSD: m <= 32 * kMaxLsdWords detectors per shot

@@ -1,22 +1,45 @@
-// LSD for large check matrices (space-time and hypergraph-product codes): the same
-// algorithm and results as lsd.cu (Alg. 1 of Sec. 4.1, on-the-fly elimination of Sec. 4.2,
-// LSD-mu of App. D), with state sized by what a shot touches instead of by m and n.
+// LSD for check matrices beyond the dense kernel (space-time, hook-fault and hypergraph-product
+// codes): the same algorithm and results as lsd.cu (Alg. 1 of Sec. 4.1, on-the-fly elimination
+// of Sec. 4.2, LSD-mu of App. D), with state sized by what a shot touches.
 //
-// One warp owns one shot.
-//   * Per-detector and per-fault arrays live in a per-warp global scratch (L1/L2 resident):
-//       dlab[m]  cluster of a claimed detector (seed ordinal, flattened to the root; -1 none)
-//       slot[m]  elimination row of a claimed detector (claim order; -1 none)
-//       fst[n]   fault state: -2 untouched, -1 candidate (next to a claimed detector),
-//                >= 0 the seed ordinal of the cluster it joined
-//       front[n] the candidate list (Def. 4.3's Lambda over all clusters), compacted per step
-//   * Clusters are indexed by seed ordinal (flipped detectors in ascending order, so a root
-//     -- the smallest seed of a cluster -- is the same as in lsd.cu), elimination rows by
-//     slot: R[slot][W], T[slot][W] over CAP slots, in shared memory, or in global scratch
-//     for the spill instance.
-//   * A pick is the minimum 64-bit key (order-preserving LLR bits, index) over the candidate
-//     list of each growing cluster (atomicMin), so no per-shot sort is needed.
-// A shot that needs more than CAP slots (or SC seeds, or CAP dependent columns) stops with
-// status LSD_SHOT_SPILL_ and is queued for the global-memory instance.
+// One CTA owns one shot.  A shot needs few growth steps on a handful of clusters, or a thousand
+// columns when its clusters percolate, and a batch has from one such shot to a few per cent of
+// it; so what bounds the kernel is the latency of its longest shot (the SMs are busy for a
+// tenth to a fifth of it), and a step is spread over the CTA with the state in shared memory
+// and few barriers.  One warp per shot with its state in global scratch took, for
+//   50 000 HGP shots, p = 0.02, LSD-0 / LSD-10   5.3 / 13.0 ms, now 0.82 / 2.3 ms
+//   5000 HGP shots, p = 0.05 (percolating)       80-84 ms, now 7.8 ms
+//   100 003 BB144 d = 12, 20 000 BB288 d = 18    1.0, 0.58 ms, now 0.16, 0.09 ms
+//   99 991 BB144 hooks d = 6                     2.8 ms, now 0.38 ms
+// and the dense kernel, which ranks every fault first, 1.9 ms for 100 003 BB72 hooks d = 6
+// (now 0.12) and 0.69 ms for 50 001 BB144 windows (now 0.12).  Threads per shot, small / large
+// instance: 128 / 256 1.46 and 17.5 ms (HGP p = 0.02, 0.05), 256 / 512 0.98 and 11.1, 512 /
+// 1024 0.82 and 7.8.
+//   lab[m]     of a claimed detector: label << 16 | slot, else kFree.  A label is the number
+//              of a seed (flipped detector), flattened to the cluster's root after a merge; a
+//              slot is the detector's elimination row, in the order of claiming.
+//   cand, joined  bitmaps over the faults: next to a claimed detector (Def. 4.3's Lambda over
+//              all clusters); in a cluster.  lk, lf, ld list the candidates: LLR bits, fault,
+//              its first four detectors.
+//   best, bidx of a growing cluster's root: least LLR bits over its candidates, then the least
+//              fault index among the equal ones (the order of lsd.cu's ranks, without a sort).
+//   M          elimination rows, bits over slots, word w of row i at M[w CAP + i].  M is the
+//              product of the row operations done so far: M h has its only bit at the pivot
+//              row for a column h already added, so a new column's image h' = M h is one bit
+//              per row, the parity of the row's bits at the column's detectors; a bit on a
+//              row without pivot makes that row the pivot, and the pivot row is added to the
+//              other rows with a bit.  Row i belongs to thread i mod NT, which alone reads
+//              (but for a pivot row) and writes it: one barrier per column, no atomics and no
+//              search for the rows to update.
+//   flags[i]   bit 0: (M s)_i, bit 1: row i has a pivot, column pcol[i].  A cluster is valid
+//              (Def. 4.2) iff no row without pivot has (M s)_i; its solution is the columns of
+//              the pivot rows that have it.
+// Pivot columns, representations and solutions are unique, so neither the choice of the pivot
+// row nor the numbering of seeds and slots shows in the results.
+//
+// Two instances: the small one keeps everything in shared memory; a shot that outgrows it (CAP
+// rows, SC seeds, its candidate list) is queued for the large one, whose rows lie in global
+// scratch (read through the SM's L1).
 #include <climits>
 
 #include "lsd_internal.cuh"
@@ -26,97 +49,141 @@ namespace lsdgb {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr unsigned long long kNoKey = ~0ull;
-constexpr int kSpill = 4;  // internal status: retry with the large-capacity instance
-constexpr int kMaskSeeds = 1024;  // spill instance: shots with at most this many seeds use masks
+constexpr uint32_t kFree = 0xffffffffu;
+constexpr uint16_t kNone16 = 0xffffu;
+constexpr unsigned kNoKey = 0xffffffffu;
+constexpr int kSpill = 4;         // internal status: retry with the large instance
+// Dynamic shared memory of a CTA; a graph too large for it takes the LG instances, whose lab
+// and (large instance) candidate list lie in global scratch.
+constexpr size_t kSmemLimit = 225 << 10;
 
 __host__ __device__ constexpr size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-// Per-warp layout of the parts kept in shared memory (or global for GLOBAL_RT).
-template <int CAP, int SC, bool MU>
-struct SLay {
-  static constexpr int W = CAP / 32;
-  static constexpr size_t R = 0;
-  static constexpr size_t T = R + (size_t)CAP * W * 4;
-  static constexpr size_t pcol = T + (size_t)CAP * W * 4;
-  static constexpr size_t dslot = pcol + (size_t)CAP * 4;         // detector of a slot
-  static constexpr size_t npN = dslot + (size_t)CAP * 4;          // dependent columns
-  static constexpr size_t npk = npN + (MU ? (size_t)CAP * W * 4 : 0);
-  static constexpr size_t ext = npk + (MU ? (size_t)CAP * 8 : 0);
-  static constexpr size_t rt_total = al16(ext + (MU ? (size_t)CAP * 4 : 0));
-  // always in shared memory
-  static constexpr size_t best = 0;                               // [SC] u64
-  static constexpr size_t newk = best + (size_t)SC * 8;           // [SC] u64
-  static constexpr size_t srt = newk + (size_t)SC * 8;            // [SC] u64
-  static constexpr size_t seed = srt + (size_t)SC * 8;            // [SC] detector of a seed
-  static constexpr size_t parent = seed + (size_t)SC * 4;
-  static constexpr size_t mark = parent + (size_t)SC * 4;
-  static constexpr size_t inv = mark + (size_t)SC * 4;
-  static constexpr size_t mlist = inv + (size_t)SC * 4;
-  static constexpr size_t dnew = mlist + (size_t)SC * 4;          // [CAP]
-  static constexpr size_t words = dnew + (size_t)CAP * 4;         // syn sred xsol cm [W]
-  static constexpr size_t scal = words + (size_t)4 * W * 4;
-  static constexpr size_t gflag = scal + 16 * 4;                  // [SC] growing flags
-  static constexpr size_t sm_total = al16(gflag + (size_t)SC);
+// Sizes and offsets of an instance.  Arrays with atomics are in shared memory (but lab for LG);
+// the others ("lists") follow there (small) or in the CTA's global scratch (big).
+template <int NT_, int CAP_, int SC_, bool MU_, bool BIG_, bool LG_>
+struct Inst {
+  static constexpr int NT = NT_, CAP = CAP_, SC = SC_, W = CAP_ / 32, RPT = CAP_ / NT_, NW = NT_ / 32;
+  static constexpr bool MU = MU_, BIG = BIG_, LG = LG_;
+  // shared
+  static constexpr size_t best = 0;
+  static constexpr size_t bidx = best + (size_t)SC * 4;
+  static constexpr size_t growb = bidx + (size_t)SC * 4;          // growing labels, one bit each
+  static constexpr size_t parent = growb + (size_t)SC / 8;
+  static constexpr size_t inv = parent + (size_t)SC * 2;          // growing labels
+  static constexpr size_t pcol = inv + (size_t)SC * 2;
+  static constexpr size_t sdet = pcol + (size_t)CAP * 2;          // detector of a slot
+  static constexpr size_t slab = sdet + (size_t)CAP * 2;          // label of a slot
+  static constexpr size_t rows = slab + (size_t)CAP * 2;          // per warp: a cluster's rows
+  static constexpr size_t flags = rows + (size_t)NW * 32 * 2;
+  static constexpr size_t osd = al16(flags + (size_t)CAP);        // per warp: cluster's x, U words
+  static constexpr size_t fixed = al16(osd + (MU ? (size_t)NW * 2 * W * 4 : 0));
+  // lists
+  static constexpr size_t newk = 0;                               // new columns of a step
+  static constexpr size_t M = newk + (size_t)SC * 8;
+  static constexpr size_t npN = M + (size_t)CAP * W * 4;          // dependent columns' images
+  static constexpr size_t ssl = npN + (MU ? (size_t)CAP * W * 4 : 0);  // slots of new columns
+  static constexpr size_t sg = ssl + (size_t)SC * 8;              // their faults, in key order
+  static constexpr size_t sroot = sg + (size_t)SC * 2;            // their clusters
+  static constexpr size_t dpf = sroot + (size_t)SC * 2;           // faults of dependent columns
+  static constexpr size_t ext = dpf + (MU ? (size_t)CAP * 2 : 0);
+  static constexpr size_t dpr = ext + (MU ? (size_t)CAP * 2 : 0);      // their clusters
+  static constexpr size_t dpk = dpr + (MU ? (size_t)CAP * 2 : 0);      // their LLR bits
+  static constexpr size_t lists = al16(dpk + (MU ? (size_t)CAP * 4 : 0));
+  // Candidate list entries.  A shot that lists half of a large code's faults has percolated
+  // and goes to the large instance.
+  static __host__ __device__ int lcap(int n) {
+    if (BIG) return n;
+    const int half = n / 2 > 1024 ? n / 2 : 1024;
+    return half < 2816 ? half : 2816;
+  }
 };
+
+// Candidate list of `cap` entries: detectors, LLR bits, faults.
+__host__ __device__ inline size_t cand_bytes(size_t cap) {
+  return al16(cap * 8) + al16(cap * 4) + al16(cap * 2);
+}
+
+template <class I>
+size_t smem_bytes(int m, int n) {
+  return I::fixed + (I::LG ? 0 : al16((size_t)m * 4)) + 2 * al16((size_t)(n + 31) / 32 * 4) +
+         (I::BIG ? 0 : I::lists) + (I::BIG && I::LG ? 0 : cand_bytes((size_t)I::lcap(n)));
+}
+// Global scratch bytes of a CTA.
+template <class I>
+size_t scratch_bytes(int m, int n) {
+  return (I::LG ? al16((size_t)m * 4) : 0) + (I::BIG ? I::lists : 0) +
+         (I::BIG && I::LG ? cand_bytes((size_t)n) : 0);
+}
 
 struct SGraph {
   const int32_t* chk_ptr;
-  const uint16_t* chk_var;
   const int32_t* var_ptr;
   const uint16_t* var_chk;
-  int max_col_deg;
+  const uint16_t* chk_pad;  // [m][max_row_deg], 0xffff past the row's end
+  const uint2* var_pad;     // [n] the first four detectors, 0xffff past the column's end
+  int max_col_deg, max_row_deg;
 };
 
-template <class L>
-struct SShot {
-  unsigned char* sm;    // shared part
-  unsigned char* rt;    // elimination part (shared or global)
-  int* dlab;            // [m]  global scratch
-  int* slot;            // [m]
-  int* fst;             // [n]
-  int* front;           // [n]
-  uint32_t* cmask;      // spill instance: per seed, its clusters' candidate faults [SC][wn]
-  int wn;               // words of a candidate mask (ceil(n / 32)); 0 = no masks
+struct Scal {        // shared scalars
+  int ns, nsl, nf;   // seeds, slots, candidates so far
+  int n_new, merged; // columns and merges of the step
+  int ng, ncr;       // growing clusters; clusters with new columns
+  int np, ext;       // dependent columns kept for LSD-mu; those in the solution
+  int ovf;
+  int piv[3];
+  unsigned item;
+  uint2 ssl;         // the single cluster's new column: slots of its detectors,
+  uint2 mlab;        // labels of the clusters it absorbs there,
+  unsigned fresh;    // and which of them are newly claimed
+  unsigned red[2][32];
+};
+
+template <class I>
+struct Shot {
+  unsigned char* sm;
+  unsigned char* li;
+  uint32_t* lab;
+  uint32_t* cand;
+  uint32_t* joined;
+  uint2* ld;
+  uint32_t* lk;
+  uint16_t* lf;
+  int lcap;
+  Scal* sc;
   template <class T>
   __device__ __forceinline__ T* s(size_t off) const { return reinterpret_cast<T*>(sm + off); }
   template <class T>
-  __device__ __forceinline__ T* r(size_t off) const { return reinterpret_cast<T*>(rt + off); }
-  __device__ __forceinline__ uint32_t* R() const { return r<uint32_t>(L::R); }
-  __device__ __forceinline__ uint32_t* T() const { return r<uint32_t>(L::T); }
-  __device__ __forceinline__ int* pcol() const { return r<int>(L::pcol); }
-  __device__ __forceinline__ int* dslot() const { return r<int>(L::dslot); }
-  __device__ __forceinline__ uint32_t* npN() const { return r<uint32_t>(L::npN); }
-  __device__ __forceinline__ unsigned long long* npk() const { return r<unsigned long long>(L::npk); }
-  __device__ __forceinline__ int* ext() const { return r<int>(L::ext); }
-  __device__ __forceinline__ unsigned long long* best() const { return s<unsigned long long>(L::best); }
-  __device__ __forceinline__ unsigned long long* newk() const { return s<unsigned long long>(L::newk); }
-  __device__ __forceinline__ unsigned long long* srt() const { return s<unsigned long long>(L::srt); }
-  __device__ __forceinline__ int* seed() const { return s<int>(L::seed); }
-  __device__ __forceinline__ int* parent() const { return s<int>(L::parent); }
-  __device__ __forceinline__ unsigned* mark() const { return s<unsigned>(L::mark); }
-  __device__ __forceinline__ int* inv() const { return s<int>(L::inv); }
-  __device__ __forceinline__ int* mlist() const { return s<int>(L::mlist); }
-  __device__ __forceinline__ int* dnew() const { return s<int>(L::dnew); }
-  __device__ __forceinline__ uint32_t* syn() const { return s<uint32_t>(L::words); }
-  __device__ __forceinline__ uint32_t* sred() const { return s<uint32_t>(L::words + L::W * 4); }
-  __device__ __forceinline__ uint32_t* xsol() const { return s<uint32_t>(L::words + 2 * L::W * 4); }
-  __device__ __forceinline__ uint32_t* cm() const { return s<uint32_t>(L::words + 3 * L::W * 4); }
-  __device__ __forceinline__ int* scal() const { return s<int>(L::scal); }
-  __device__ __forceinline__ unsigned char* gflag() const { return s<unsigned char>(L::gflag); }
+  __device__ __forceinline__ T* l(size_t off) const { return reinterpret_cast<T*>(li + off); }
+  __device__ __forceinline__ uint32_t* best() const { return s<uint32_t>(I::best); }
+  __device__ __forceinline__ uint32_t* bidx() const { return s<uint32_t>(I::bidx); }
+  __device__ __forceinline__ uint32_t* growb() const { return s<uint32_t>(I::growb); }
+  __device__ __forceinline__ uint16_t* parent() const { return s<uint16_t>(I::parent); }
+  __device__ __forceinline__ uint16_t* inv() const { return s<uint16_t>(I::inv); }
+  __device__ __forceinline__ uint16_t* pcol() const { return s<uint16_t>(I::pcol); }
+  __device__ __forceinline__ uint16_t* sdet() const { return s<uint16_t>(I::sdet); }
+  __device__ __forceinline__ uint16_t* slab() const { return s<uint16_t>(I::slab); }
+  __device__ __forceinline__ unsigned char* flags() const { return s<unsigned char>(I::flags); }
+  __device__ __forceinline__ unsigned long long* newk() const { return l<unsigned long long>(I::newk); }
+  __device__ __forceinline__ uint32_t* M() const { return l<uint32_t>(I::M); }
+  __device__ __forceinline__ uint32_t* npN() const { return l<uint32_t>(I::npN); }
+  __device__ __forceinline__ uint16_t* ssl() const { return l<uint16_t>(I::ssl); }
+  __device__ __forceinline__ uint16_t* sg() const { return l<uint16_t>(I::sg); }
+  __device__ __forceinline__ uint16_t* sroot() const { return l<uint16_t>(I::sroot); }
+  __device__ __forceinline__ uint16_t* dpf() const { return l<uint16_t>(I::dpf); }
+  __device__ __forceinline__ uint16_t* ext() const { return l<uint16_t>(I::ext); }
+  __device__ __forceinline__ uint16_t* dpr() const { return l<uint16_t>(I::dpr); }
+  __device__ __forceinline__ uint32_t* dpk() const { return l<uint32_t>(I::dpk); }
 };
 
-// scal slots
-enum { S_NEW = 0, S_NP, S_EXT, S_MERGED, S_DNEW, S_INV, S_SLOTS, S_NSEED, S_NFRONT, S_OVF };
-
-__device__ __forceinline__ unsigned long long llr_key(float x, int j) {
+// Order-preserving bits of an LLR (-0.0 folded into +0.0).
+__device__ __forceinline__ unsigned llr_bits(float x) {
   x = __fadd_rn(x, 0.0f);
-  unsigned u = __float_as_uint(x);
-  u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-  return ((unsigned long long)u << 32) | (unsigned)j;
+  const unsigned u = __float_as_uint(x);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-__device__ __forceinline__ int uf_find(const volatile int* parent, int x) {
+__device__ __forceinline__ int uf_find(const volatile uint16_t* parent, int x) {
   int p = parent[x];
   while (p != x) {
     x = p;
@@ -125,10 +192,9 @@ __device__ __forceinline__ int uf_find(const volatile int* parent, int x) {
   return x;
 }
 
-template <class L>
-__device__ __forceinline__ void uf_unite(const SShot<L>& S, int a, int b) {
-  int* parent = S.parent();
-  const volatile int* vp = parent;
+template <class I>
+__device__ __forceinline__ void uf_unite(const Shot<I>& S, int a, int b) {
+  const volatile uint16_t* vp = S.parent();
   for (;;) {
     a = uf_find(vp, a);
     b = uf_find(vp, b);
@@ -138,854 +204,1055 @@ __device__ __forceinline__ void uf_unite(const SShot<L>& S, int a, int b) {
       a = b;
       b = t;
     }
-    if (atomicCAS(parent + a, a, b) == a) {
-      const int k = atomicAdd(&S.scal()[S_MERGED], 1);
-      S.mlist()[k] = a;
+    if (atomicCAS(reinterpret_cast<unsigned short*>(S.parent()) + a, (unsigned short)a,
+                  (unsigned short)b) == (unsigned short)a) {
+      S.sc->merged = 1;
       return;
     }
   }
 }
 
-__device__ __forceinline__ bool bit_of(const uint32_t* v, int i) {
-  return (v[i >> 5] >> (i & 31)) & 1u;
-}
-
-// Claims detector d for cluster r (lane-local).  Returns false on slot overflow.
-template <class L, int CAP>
-__device__ __forceinline__ void claim(const SShot<L>& S, int d, int r) {
-  const int o = atomicCAS(&S.dlab[d], -1, r);
-  if (o == -1) {
-    const int sl = atomicAdd(&S.scal()[S_SLOTS], 1);
-    if (sl >= CAP) {
-      S.scal()[S_OVF] = 1;
+// Claims detector d for the cluster of label r.
+template <class I>
+__device__ __forceinline__ void claim(const Shot<I>& S, int d, int r) {
+  const uint32_t o = atomicCAS(&S.lab[d], kFree, ((uint32_t)r << 16) | 0xffffu);
+  if (o == kFree) {
+    const int sl = atomicAdd(&S.sc->nsl, 1);
+    if (sl >= I::CAP) {
+      S.sc->ovf = 1;
       return;
     }
-    S.slot[d] = sl;
-    S.dslot()[sl] = d;
-    const int k = atomicAdd(&S.scal()[S_DNEW], 1);
-    S.dnew()[k] = d;
-  } else if (o != r) {
-    uf_unite(S, r, o);
+    S.lab[d] = ((uint32_t)r << 16) | (uint32_t)sl;
+    S.sdet()[sl] = (uint16_t)d;
+    S.slab()[sl] = (uint16_t)r;
+    S.flags()[sl] = 0;
+  } else if ((int)(o >> 16) != r) {
+    uf_unite(S, r, (int)(o >> 16));
   }
 }
 
-template <class L>
-__device__ int collect_invalid(const SShot<L>& S, int lane) {
-  if (lane == 0) S.scal()[S_INV] = 0;
-  __syncwarp();
-  for (int w = lane; w < L::W; w += 32) {
-    uint32_t bits = S.sred()[w];
-    while (bits) {
-      const int sl = w * 32 + __ffs(bits) - 1;
-      bits &= bits - 1;
-      const int root = S.dlab[S.dslot()[sl]];
-      if (root >= 0 && atomicCAS(&S.mark()[root], 0u, 1u) == 0u) {
-        const int k = atomicAdd(&S.scal()[S_INV], 1);
-        S.inv()[k] = root;
+// The i-th of the four packed 16-bit values.
+__device__ __forceinline__ uint32_t half4(uint2 v, int i) {
+  return ((i & 2 ? v.y : v.x) >> (16 * (i & 1))) & 0xffffu;
+}
+
+// Calls fn(d) for every detector of fault f, the first four of which are v.
+template <class F>
+__device__ __forceinline__ void each_det(const SGraph& G, uint2 v, int f, F&& fn) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t d = half4(v, i);
+    if (d != kNone16) fn((int)d);
+  }
+  if (G.max_col_deg > 4) {
+    const int v1 = G.var_ptr[f + 1];
+    for (int q = G.var_ptr[f] + 4; q < v1; ++q) fn((int)G.var_chk[q]);
+  }
+}
+
+// The thread's rows among the slots from..to become unit rows; its older rows get zeros in the
+// words that the new slots opened.
+template <class I>
+__device__ __forceinline__ void open_rows(const Shot<I>& S, int from, int to, int tid) {
+  const int w0 = (from + 31) >> 5, w1 = (to + 31) >> 5;
+  for (int i = tid; i < to; i += I::NT)
+    for (int w = i < from ? w0 : 0; w < w1; ++w)
+      S.M()[(size_t)w * I::CAP + i] = (i >> 5) == w && i >= from ? 1u << (i & 31) : 0u;
+}
+
+// Fault f is next to a newly claimed detector: lists it if it is not listed; returns its entry
+// (key and detectors in k, v) or -1.
+template <class I>
+__device__ __forceinline__ int list_candidate(const SGraph& G, const Shot<I>& S, const float* llr,
+                                              int f, unsigned& k, uint2& v) {
+  const uint32_t b = 1u << (f & 31);
+  if ((atomicOr(&S.cand[f >> 5], b) & b) != 0) return -1;
+  const int q = atomicAdd(&S.sc->nf, 1);
+  if (q >= S.lcap) {
+    S.sc->ovf = 1;
+    return -1;
+  }
+  v = G.var_pad[f];
+  k = llr_bits(llr[f]);
+  S.lf[q] = (uint16_t)f;
+  S.ld[q] = v;
+  S.lk[q] = k;
+  return q;
+}
+
+// Rows and candidates of the slots from..to.
+template <class I>
+__device__ __forceinline__ void open_slots(const SGraph& G, const Shot<I>& S, const float* llr,
+                                           int from, int to, int tid) {
+  open_rows(S, from, to, tid);
+  const int D = G.max_row_deg;
+  for (int x = tid; x < (to - from) * D; x += I::NT) {
+    const int f = G.chk_pad[(size_t)S.sdet()[from + x / D] * D + x % D];
+    unsigned k;
+    uint2 v;
+    if (f != kNone16) list_candidate(G, S, llr, f, k, v);
+  }
+}
+
+// Image of a column under M on the thread's rows i = tid + NT j < nsl: bit j of the result; pc
+// = one of those with a bit and no pivot (or unchanged).  sl: slots of its first four detectors.
+template <class I>
+__device__ __forceinline__ uint32_t column_image(const SGraph& G, const Shot<I>& S, uint2 sl, int g,
+                                                 int nsl, int tid, int& pc) {
+  constexpr int NT = I::NT, CAP = I::CAP;
+  uint32_t hit = 0;
+#pragma unroll
+  for (int j = 0; j < I::RPT; ++j) {
+    const int i = tid + NT * j;
+    if (i < nsl) {
+      uint32_t x = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t s = half4(sl, q);
+        if (s != kNone16) x ^= S.M()[(size_t)(s >> 5) * CAP + i] >> (s & 31);
       }
+      hit |= (x & 1u) << j;
     }
   }
-  __syncwarp();
-  const int count = S.scal()[S_INV];
-  for (int t = lane; t < count; t += 32) S.mark()[S.inv()[t]] = 0u;
-  __syncwarp();
-  return count;
-}
-
-template <class L>
-__device__ int collect_all(const SShot<L>& S, int lane) {
-  const int ns = S.scal()[S_NSEED];
-  int count = 0;
-  for (int b = 0; b < ns; b += 32) {
-    const int k = b + lane;
-    const bool pred = k < ns && S.parent()[k] == k;
-    const unsigned bal = __ballot_sync(kFull, pred);
-    if (pred) S.inv()[count + __popc(bal & ((1u << lane) - 1u))] = k;
-    count += __popc(bal);
+  if (G.max_col_deg > 4) {
+    const int v1 = G.var_ptr[g + 1];
+    for (int q = G.var_ptr[g] + 4; q < v1; ++q) {
+      const uint32_t s = S.lab[G.var_chk[q]] & 0xffffu;
+      for (int j = 0; tid + NT * j < nsl; ++j)
+        hit ^= ((S.M()[(size_t)(s >> 5) * CAP + tid + NT * j] >> (s & 31)) & 1u) << j;
+    }
   }
-  __syncwarp();
-  return count;
+  for (uint32_t h = hit; h; h &= h - 1) {
+    const int i = tid + NT * (__ffs(h) - 1);
+    if (!(S.flags()[i] & 2)) pc = i;
+  }
+  return hit;
 }
 
-// Adds fault g (order key `key`) to its cluster's factorization, rows in slot space.  Lane l
-// holds words l, l+32, ... of the column being reduced.
-// Only the first wc = ceil(slots / 32) words of a row can be nonzero: rows are written in
-// full (zeros past the slots in use) when they become pivots, and every later update XORs
-// rows that are zero there too.
-template <class L, bool MU, int CAP>
-__device__ void add_column(const SGraph& G, const SShot<L>& S, int g, unsigned long long key,
-                           int lane) {
-  constexpr int W = L::W;
-  constexpr int WC = (W + 31) / 32;
-  const int nsl = min(S.scal()[S_SLOTS], CAP);
-  const int wc = (nsl + 31) >> 5;
-  uint32_t bw[WC], tw[WC];
+// Makes p the pivot row of column g (hit: the column's image on the thread's rows) and adds it
+// to the other rows with a bit.
+template <class I>
+__device__ __forceinline__ void pivot_update(const Shot<I>& S, int p, int g, uint32_t hit, int nsl,
+                                             int tid) {
+  constexpr int NT = I::NT, CAP = I::CAP;
+  const int lane = tid & 31, wc = (nsl + 31) >> 5;
+  if (p % NT == tid) {
+    hit &= ~(1u << (p / NT));
+    S.flags()[p] |= 2;
+    S.pcol()[p] = (uint16_t)g;
+  }
+  const bool sp = S.flags()[p] & 1;
+  if (!__any_sync(kFull, hit != 0)) return;
+  for (int c0 = 0; c0 < wc; c0 += 32) {
+    const uint32_t v = c0 + lane < wc ? S.M()[(size_t)(c0 + lane) * CAP + p] : 0u;
+    unsigned nz = __ballot_sync(kFull, v != 0);
+    while (nz) {
+      const int w = __ffs(nz) - 1;
+      nz &= nz - 1;
+      const uint32_t pv = __shfl_sync(kFull, v, w);
+      uint32_t* const row = S.M() + (size_t)(c0 + w) * CAP + tid;
 #pragma unroll
-  for (int c = 0; c < WC; ++c) bw[c] = tw[c] = 0;
-  const int v0 = G.var_ptr[g], v1 = G.var_ptr[g + 1];
-  for (int q = v0; q < v1; ++q) {
-    const int sl = S.slot[G.var_chk[q]];
-    const bool piv = S.pcol()[sl] >= 0;
+      for (int j = 0; j < I::RPT; ++j)
+        if ((hit >> j) & 1u) row[NT * j] ^= pv;
+    }
+  }
+  if (sp)
+    for (uint32_t h = hit; h; h &= h - 1) S.flags()[tid + NT * (__ffs(h) - 1)] ^= 1;
+}
+
+// Keeps a dependent column for LSD-mu: its image is its combination of pivot rows.
+template <class I>
+__device__ __forceinline__ void keep_dependent(const Shot<I>& S, int& np, int g, uint32_t hit, int tid) {
+  if constexpr (I::MU) {
+    if (np >= I::CAP) {
+      S.sc->ovf = 1;
+      return;
+    }
 #pragma unroll
-    for (int c = 0; c < WC; ++c) {
-      const int w = c * 32 + lane;
-      if (w < wc) {
-        if ((sl >> 5) == w) bw[c] ^= 1u << (sl & 31);
-        if (piv) {
-          bw[c] ^= S.R()[sl * W + w];
-          tw[c] ^= S.T()[sl * W + w];
+    for (int j = 0; j < I::RPT; ++j) {
+      const unsigned b = __ballot_sync(kFull, (hit >> j) & 1u);
+      if ((tid & 31) == 0) S.npN()[(size_t)np * I::W + I::NW * j + (tid >> 5)] = b;
+    }
+    if (tid == 0) S.dpf()[np] = (uint16_t)g;
+    ++np;
+  }
+}
+
+// Columns of the clusters with at most 32 rows, a warp per cluster.  Larger clusters keep
+// their bit in growb.
+template <class I>
+__device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int tid) {
+  constexpr int CAP = I::CAP;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int ncr = S.sc->ncr, wc = (nsl + 31) >> 5;
+  uint16_t* const rows = S.template s<uint16_t>(I::rows) + warp * 32;
+  uint32_t* const M = S.M();
+  for (int c = warp; c < ncr; c += I::NW) {
+    const int r = S.inv()[c];
+    int cnt = 0;
+    for (int b0 = 0; b0 < nsl; b0 += 32) {
+      const bool in = b0 + lane < nsl && S.slab()[b0 + lane] == r;
+      const unsigned b = __ballot_sync(kFull, in);
+      const int at = cnt + __popc(b & ((1u << lane) - 1u));
+      if (in && at < 32) rows[at] = (uint16_t)(b0 + lane);
+      cnt += __popc(b);
+    }
+    if (cnt > 32) continue;
+    __syncwarp();
+    const bool mine = lane < cnt;
+    const int i = mine ? rows[lane] : 0;
+    for (int t0 = 0; t0 < n_new; t0 += 32) {
+      unsigned todo = __ballot_sync(kFull, t0 + lane < n_new && S.sroot()[t0 + lane] == r);
+      while (todo) {
+        const int t = t0 + __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint2 sl = reinterpret_cast<const uint2*>(S.ssl())[t];
+        const int g = S.sg()[t];
+        uint32_t x = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t s = half4(sl, q);
+          if (mine && s != kNone16) x ^= M[(size_t)(s >> 5) * CAP + i] >> (s & 31);
         }
-      }
-    }
-  }
-  int p = -1;
-#pragma unroll
-  for (int c = 0; c < WC; ++c) {
-    const unsigned nz = __ballot_sync(kFull, bw[c] != 0);
-    if (p < 0 && nz) {
-      const int wl = __ffs(nz) - 1;
-      const uint32_t word = __shfl_sync(kFull, bw[c], wl);
-      p = (c * 32 + wl) * 32 + __ffs(word) - 1;
-    }
-  }
-  if (p < 0) {
-    if constexpr (MU) {
-      const int k = __shfl_sync(kFull, S.scal()[S_NP], 0);
-      if (k >= CAP) {
-        if (lane == 0) S.scal()[S_OVF] = 1;
-      } else {
-#pragma unroll
-        for (int c = 0; c < WC; ++c) {
-          const int w = c * 32 + lane;
-          if (w < W) S.npN()[k * W + w] = tw[c];
+        bool hit = (x & 1u) != 0;
+        const unsigned nb = __ballot_sync(kFull, hit && !(S.flags()[i] & 2));
+        if (nb == 0) {
+          if constexpr (I::MU) {
+            int k = 0;
+            if (lane == 0) k = atomicAdd(&S.sc->np, 1);
+            k = __shfl_sync(kFull, k, 0);
+            if (k >= CAP) {
+              S.sc->ovf = 1;
+              continue;
+            }
+            uint32_t* const row = S.npN() + (size_t)k * I::W;
+            for (int w = lane; w < I::W; w += 32) row[w] = 0u;
+            __syncwarp();
+            if (hit) atomicOr(row + (i >> 5), 1u << (i & 31));
+            if (lane == 0) S.dpf()[k] = (uint16_t)g;
+          }
+          continue;
+        }
+        const int pl = __ffs(nb) - 1;
+        const int p = __shfl_sync(kFull, i, pl);
+        const bool sp = S.flags()[p] & 1;
+        __syncwarp();
+        if (lane == pl) {
+          hit = false;
+          S.flags()[p] |= 2;
+          S.pcol()[p] = (uint16_t)g;
+        }
+        if (__any_sync(kFull, hit)) {
+          for (int c0 = 0; c0 < wc; c0 += 32) {
+            const uint32_t v = c0 + lane < wc ? M[(size_t)(c0 + lane) * CAP + p] : 0u;
+            unsigned nz = __ballot_sync(kFull, v != 0);
+            while (nz) {
+              const int w = __ffs(nz) - 1;
+              nz &= nz - 1;
+              const uint32_t pv = __shfl_sync(kFull, v, w);
+              if (hit) M[(size_t)(c0 + w) * CAP + i] ^= pv;
+            }
+          }
+          if (sp && hit) S.flags()[i] ^= 1;
         }
         __syncwarp();
-        if (lane == 0) {
-          S.npk()[k] = key;
-          S.scal()[S_NP] = k + 1;
-        }
-      }
-      __syncwarp();
-    }
-    return;
-  }
-  const int pw = p >> 5;
-  const uint32_t pb = 1u << (p & 31);
-#pragma unroll
-  for (int c = 0; c < WC; ++c)
-    if (c * 32 + lane == pw) tw[c] ^= pb;
-  const bool sflag = (S.sred()[pw] & pb) != 0;
-#pragma unroll
-  for (int c = 0; c < WC; ++c) {
-    const int w = c * 32 + lane;
-    if (w < W) {
-      S.R()[p * W + w] = bw[c];
-      S.T()[p * W + w] = tw[c];
-    }
-  }
-  if (lane == 0) S.pcol()[p] = g;
-  __syncwarp();
-  // back-elimination: rows holding bit p found by ballot, each XORed by the whole warp
-  // (lane = word) with the new pivot row, which the lanes still hold in registers
-  for (int d0 = 0; d0 < nsl; d0 += 32) {
-    const int d = d0 + lane;
-    const bool hit = d < nsl && d != p && S.pcol()[d] >= 0 && (S.R()[d * W + pw] & pb) != 0;
-    unsigned bal = __ballot_sync(kFull, hit);
-    while (bal) {
-      const int dd = d0 + __ffs(bal) - 1;
-      bal &= bal - 1;
-#pragma unroll
-      for (int c = 0; c < WC; ++c) {
-        const int w = c * 32 + lane;
-        if (w < wc) {
-          S.R()[dd * W + w] ^= bw[c];
-          S.T()[dd * W + w] ^= tw[c];
-        }
       }
     }
+    if (lane == 0) atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
+    __syncwarp();
   }
-  if (sflag) {
-#pragma unroll
-    for (int c = 0; c < WC; ++c) {
-      const int w = c * 32 + lane;
-      if (w < W) {
-        S.sred()[w] ^= bw[c];
-        S.xsol()[w] ^= tw[c];
-      }
-    }
-  }
-  __syncwarp();
 }
 
-// One synchronous growth step of the k clusters in inv[] (same contract as lsd.cu).
-template <class L, bool MU, int CAP>
-__device__ int sparse_step(const SGraph& G, const SShot<L>& S, const float* llr, int k,
-                           bool strict, int lane) {
-  for (int t = lane; t < k; t += 32) {
+// Adds the n_new columns of a step, in key order within each cluster, to the eliminations.
+template <class I>
+__device__ __forceinline__ void add_columns(const SGraph& G, const Shot<I>& S, int n_new, int nsl,
+                                            int tid) {
+  const bool by_warp = n_new > 1 && G.max_col_deg <= 4;
+  if (by_warp) {
+    add_columns_by_warp(S, n_new, nsl, tid);
+    __syncthreads();
+  }
+  int np = S.sc->np, done = 0;
+  for (int t = 0; t < n_new; ++t) {
+    if (by_warp) {
+      const int r = S.sroot()[t];
+      if (!((S.growb()[r >> 5] >> (r & 31)) & 1u)) continue;
+    }
+    const int g = S.sg()[t];
+    int pc = -1;
+    const uint32_t hit = column_image(G, S, reinterpret_cast<const uint2*>(S.ssl())[t], g, nsl, tid, pc);
+    // any row with a bit and no pivot will do: one of the stores stands
+    if (pc >= 0) S.sc->piv[done % 3] = pc;
+    if (tid == 0) S.sc->piv[(done + 1) % 3] = -1;
+    __syncthreads();
+    const int p = S.sc->piv[done % 3];
+    ++done;
+    if (p < 0) keep_dependent(S, np, g, hit, tid);
+    else pivot_update(S, p, g, hit, nsl, tid);
+  }
+  __syncthreads();
+  if (by_warp)
+    for (int c = tid; c < S.sc->ncr; c += I::NT) {
+      const int r = S.inv()[c];
+      atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
+    }
+  if (tid == 0) S.sc->np = np;
+  __syncthreads();
+}
+
+// Lists the labels of the invalid clusters (only_invalid) or of all clusters in inv.
+template <class I>
+__device__ __forceinline__ int collect(const Shot<I>& S, int nsl, bool only_invalid, int tid) {
+  if (only_invalid) {
+    for (int i = tid; i < nsl; i += I::NT) {
+      if ((S.flags()[i] & 3) != 1) continue;
+      const int r = S.slab()[i];
+      const uint32_t b = 1u << (r & 31);
+      if (!(atomicOr(&S.growb()[r >> 5], b) & b)) S.inv()[atomicAdd(&S.sc->ng, 1)] = (uint16_t)r;
+    }
+  } else {
+    const int ns = S.sc->ns;
+    for (int r = tid; r < ns; r += I::NT) {
+      if (S.parent()[r] != r) continue;
+      atomicOr(&S.growb()[r >> 5], 1u << (r & 31));
+      S.inv()[atomicAdd(&S.sc->ng, 1)] = (uint16_t)r;
+    }
+  }
+  __syncthreads();
+  return S.sc->ng;
+}
+
+// One synchronous growth step of the k clusters listed in inv (marked in growb).  On return the
+// list is empty.  0: grown, 1: strict and a cluster had no candidate, 2: none grew, 3: no room.
+template <class I>
+__device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, int k, bool strict,
+                           int tid) {
+  constexpr int NT = I::NT;
+  Scal& sc = *S.sc;
+  const int nf = sc.nf, nsl0 = sc.nsl;
+  // ---- find_candidate: the least LLR bits of every growing cluster, then the least fault
+  // that has them ----
+  for (int t = tid; t < k; t += NT) {
     const int r = S.inv()[t];
     S.best()[r] = kNoKey;
-    S.gflag()[r] = 1;
+    S.bidx()[r] = kNoKey;
   }
-  __syncwarp();
-  // find_candidate.  With few growing clusters (the spill instance's late steps, one huge
-  // cluster growing alone), each scans its own candidate mask: the set bits are the free
-  // faults next to it, so only their LLRs are read.  Otherwise one pass over the compacted
-  // candidate list, 4 entries per lane at a time: the dependent loads (entry, state,
-  // column, labels) of the four are issued together.
-  if (S.wn > 0 && (long long)k * S.wn < 2LL * S.scal()[S_NFRONT]) {
-    for (int t = 0; t < k; ++t) {
-      const int r = S.inv()[t];
-      const uint32_t* cm = S.cmask + (size_t)r * S.wn;
-      unsigned long long best = kNoKey;
-      for (int w = lane; w < S.wn; w += 32) {
-        uint32_t bits = cm[w];
-        while (bits) {
-          const int f = w * 32 + __ffs(bits) - 1;
-          bits &= bits - 1;
-          if (S.fst[f] != -1) continue;  // already in a cluster
-          const unsigned long long key = llr_key(llr[f], f);
-          if (key < best) best = key;
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int x = tid; x < nf; x += NT) {
+      const int f = S.lf[x];
+      if ((S.joined[f >> 5] >> (f & 31)) & 1u) continue;
+      const unsigned key = S.lk[x];
+      each_det(G, S.ld[x], f, [&](int d) {
+        const uint32_t y = S.lab[d];
+        if (y == kFree) return;
+        const int r = (int)(y >> 16);
+        if (!((S.growb()[r >> 5] >> (r & 31)) & 1u)) return;
+        if (pass == 0) {
+          if (key < S.best()[r]) atomicMin(&S.best()[r], key);
+        } else if (key == S.best()[r]) {
+          atomicMin(&S.bidx()[r], (unsigned)f);
         }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(kFull, best, off);
-        if (o < best) best = o;
-      }
-      if (lane == 0) S.best()[r] = best;
+      });
     }
-    __syncwarp();
-  } else {
-    const int nf = S.scal()[S_NFRONT];
-    const unsigned below = (1u << lane) - 1u;
-    int kept = 0;
-    for (int b = 0; b < nf; b += 128) {
-      int f[4], q0[4], q1[4];
-      unsigned long long key[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = b + 32 * u + lane;
-        f[u] = i < nf ? S.front[i] : -1;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (f[u] >= 0 && S.fst[f[u]] != -1) f[u] = -1;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        key[u] = kNoKey;
-        q0[u] = q1[u] = 0;
-        if (f[u] >= 0) {
-          key[u] = llr_key(llr[f[u]], f[u]);
-          q0[u] = G.var_ptr[f[u]];
-          q1[u] = G.var_ptr[f[u] + 1];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const unsigned bal = __ballot_sync(kFull, f[u] >= 0);
-        if (f[u] >= 0) S.front[kept + __popc(bal & below)] = f[u];
-        kept += __popc(bal);
-      }
-      for (int qq = 0; qq < G.max_col_deg; ++qq) {
-        int r[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q = q0[u] + qq;
-          r[u] = q < q1[u] ? S.dlab[G.var_chk[q]] : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (r[u] >= 0 && S.gflag()[r[u]]) atomicMin(&S.best()[r[u]], key[u]);
-      }
-      __syncwarp();
-    }
-    if (lane == 0) S.scal()[S_NFRONT] = kept;
+    __syncthreads();
   }
-  __syncwarp();
-  bool none = false, some = false;
-  for (int t = lane; t < k; t += 32) {
+  bool some = false, none = false;
+  for (int t = tid; t < k; t += NT) {
+    const bool has = S.bidx()[S.inv()[t]] != kNoKey;
+    some |= has;
+    none |= !has;
+  }
+  none = __syncthreads_or(none);
+  some = __syncthreads_or(some);
+  const bool stop = (strict && none) || !some;
+  // ---- every pick joins its cluster and claims its detectors; clusters that meet merge ----
+  for (int t = tid; t < k; t += NT) {
     const int r = S.inv()[t];
-    S.gflag()[r] = 0;
-    if (S.best()[r] == kNoKey) none = true;
-    else some = true;
+    atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
+    const unsigned f = S.bidx()[r];
+    if (stop || f == kNoKey) continue;
+    const uint32_t b = 1u << (f & 31);
+    // (a fault picked twice joins once; its pickers meet at its detectors)
+    if (!(atomicOr(&S.joined[f >> 5], b) & b))
+      S.newk()[atomicAdd(&sc.n_new, 1)] = ((unsigned long long)S.best()[r] << 32) | f;
+    each_det(G, G.var_pad[f], (int)f, [&](int d) { claim(S, d, r); });
   }
-  none = __any_sync(kFull, none);
-  some = __any_sync(kFull, some);
-  if ((strict && none) || !some) {
-    __syncwarp();
-    return (strict && none) ? 1 : 2;
+  if (tid == 0) {
+    sc.ng = sc.ncr = 0;
+    sc.piv[0] = -1;
   }
-  if (lane == 0) {
-    S.scal()[S_NEW] = 0;
-    S.scal()[S_MERGED] = 0;
-    S.scal()[S_DNEW] = 0;
-  }
-  __syncwarp();
-  // parallel_union
-  for (int t = lane; t < k; t += 32) {
-    const int r = S.inv()[t];
-    const unsigned long long key = S.best()[r];
-    if (key == kNoKey) continue;
-    const int g = (int)(key & 0xffffffffu);
-    const int old = atomicCAS(&S.fst[g], -1, r);
-    if (old == -1) {
-      const int q = atomicAdd(&S.scal()[S_NEW], 1);
-      S.newk()[q] = key;
-    } else {
-      uf_unite(S, r, old);
+  __syncthreads();
+  if (stop) return strict && none ? 1 : 2;
+  if (sc.ovf) return 3;
+  const int nsl = sc.nsl, n_new = sc.n_new;
+  // ---- labels to roots after a merge ----
+  if (sc.merged) {
+    const int ns = sc.ns;
+    for (int x = tid; x < ns; x += NT) S.parent()[x] = (uint16_t)uf_find(S.parent(), x);
+    __syncthreads();
+    for (int i = tid; i < nsl; i += NT) {
+      const int r = S.parent()[S.slab()[i]];
+      S.slab()[i] = (uint16_t)r;
+      S.lab[S.sdet()[i]] = ((uint32_t)r << 16) | (uint32_t)i;
     }
-    const int v1 = G.var_ptr[g + 1];
-    for (int q = G.var_ptr[g]; q < v1; ++q) claim<L, CAP>(S, G.var_chk[q], r);
+    __syncthreads();
   }
-  __syncwarp();
-  if (S.scal()[S_OVF]) return 3;
-  // flatten after merges
-  if (S.scal()[S_MERGED]) {
-    const int ns = S.scal()[S_NSEED];
-    for (int x = lane; x < ns; x += 32) S.parent()[x] = uf_find(S.parent(), x);
-    __syncwarp();
-    const int nsl = S.scal()[S_SLOTS];
-    for (int sl = lane; sl < nsl; sl += 32) {
-      const int d = S.dslot()[sl];
-      S.dlab[d] = S.parent()[S.dlab[d]];
-    }
-    __syncwarp();
-  }
-  // candidate masks: the absorbed clusters' masks fold into their roots
-  if (S.wn > 0 && S.scal()[S_MERGED]) {
-    const int nm = S.scal()[S_MERGED];
-    for (int i = 0; i < nm; ++i) {
-      const int x = S.mlist()[i];
-      const uint32_t* src = S.cmask + (size_t)x * S.wn;
-      uint32_t* dst = S.cmask + (size_t)S.parent()[x] * S.wn;
-      for (int w = lane; w < S.wn; w += 32) {
-        const uint32_t v = src[w];
-        if (v) atomicOr(&dst[w], v);
-      }
-    }
-    __syncwarp();
-  }
-  // candidates next to the newly claimed detectors (and, with masks, in their cluster's mask)
-  {
-    const int nd = S.scal()[S_DNEW];
-    for (int t = lane; t < nd; t += 32) {
-      const int d = S.dnew()[t];
-      uint32_t* cm = S.wn > 0 ? S.cmask + (size_t)S.dlab[d] * S.wn : nullptr;
-      const int c1 = G.chk_ptr[d + 1];
-      for (int e = G.chk_ptr[d]; e < c1; ++e) {
-        const int f = G.chk_var[e];
-        if (atomicCAS(&S.fst[f], -2, -1) == -2) {
-          const int q = atomicAdd(&S.scal()[S_NFRONT], 1);
-          S.front[q] = f;
-        }
-        if (cm && S.fst[f] < 0) atomicOr(&cm[f >> 5], 1u << (f & 31));
-      }
-    }
-  }
-  __syncwarp();
-  // new columns in key order
-  const int n_new = S.scal()[S_NEW];
-  for (int t = lane; t < n_new; t += 32) {
+  open_slots(G, S, llr, nsl0, nsl, tid);
+  // ---- the new columns in key order, with their clusters and the slots of their detectors ----
+  for (int t = tid; t < n_new; t += NT) {
     const unsigned long long kt = S.newk()[t];
     int pos = 0;
-    for (int u = 0; u < n_new; ++u) pos += (S.newk()[u] < kt) ? 1 : 0;
-    S.srt()[pos] = kt;
+    for (int u = 0; u < n_new; ++u) pos += S.newk()[u] < kt ? 1 : 0;
+    const int g = (int)(kt & 0xffffffffu);
+    S.sg()[pos] = (uint16_t)g;
+    const uint2 v = G.var_pad[g];
+    uint32_t sl[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t d = half4(v, q);
+      sl[q] = d != kNone16 ? S.lab[d] & 0xffffu : kNone16;
+    }
+    reinterpret_cast<uint2*>(S.ssl())[pos] = make_uint2(sl[0] | sl[1] << 16, sl[2] | sl[3] << 16);
+    if (n_new > 1) {
+      const int r = S.slab()[sl[0]];
+      const uint32_t b = 1u << (r & 31);
+      S.sroot()[pos] = (uint16_t)r;
+      if (!(atomicOr(&S.growb()[r >> 5], b) & b)) S.inv()[atomicAdd(&sc.ncr, 1)] = (uint16_t)r;
+    }
   }
-  __syncwarp();
-  for (int t = 0; t < n_new; ++t) {
-    const unsigned long long key = S.srt()[t];
-    add_column<L, MU, CAP>(G, S, (int)(key & 0xffffffffu), key, lane);
+  __syncthreads();
+  if (sc.ovf) return 3;
+  if (tid == 0) sc.n_new = sc.merged = 0;
+  add_columns(G, S, n_new, nsl, tid);
+  if (I::MU && sc.ovf) return 3;
+  if (n_new > 1 && G.max_col_deg > 4) {  // (the marks of the clusters with columns, unused there)
+    for (int c = tid; c < sc.ncr; c += NT) {
+      const int r = S.inv()[c];
+      atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
+    }
+    __syncthreads();
   }
-  return S.scal()[S_OVF] ? 3 : 0;
+  return 0;
 }
 
-template <class L>
-__device__ void sparse_osd_e(const LSDArgs& a, const SShot<L>& S, int lane) {
-  constexpr int W = L::W;
-  const long long* wfix = a.g.wfix;
-  const int order = a.order;
-  const int nroots = collect_all(S, lane);
-  const int n_np = S.scal()[S_NP];
-  const int nsl = S.scal()[S_SLOTS];
-  for (int ci = 0; ci < nroots; ++ci) {
-    const int r = S.inv()[ci];
-    for (int c = 0; c < W; ++c) {
-      const int sl = c * 32 + lane;
-      const bool in = sl < nsl && S.dlab[S.dslot()[sl]] == r;
-      const unsigned bal = __ballot_sync(kFull, in);
-      if (lane == 0) S.cm()[c] = bal;
+// Growth of the only invalid cluster (label r) until it is valid: the step of sparse_step with
+// three barriers.  While the new column is eliminated the candidates of the next step are
+// searched, so the next pick is known when the validity is.  No other cluster grows, so the
+// absorbed clusters are relabelled at once and r stays the root.  Steps taken are added to
+// `steps`; returns as sparse_step (0: valid).  Needs columns of at most four detectors.
+template <class I>
+__device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, uint32_t r, int n,
+                           int& steps, int tid) {
+  constexpr int NT = I::NT;
+  Scal& sc = *S.sc;
+  const int lane = tid & 31, warp = tid >> 5;
+  int nf = sc.nf, nsl = sc.nsl, np = sc.np;
+  const int D = G.max_row_deg;
+  unsigned bk, bx;  // the thread's best entry: LLR bits, then fault << 16 | entry
+  auto scan = [&] {
+    for (int x = tid; x < nf; x += NT) {
+      const unsigned key = S.lk[x];
+      if (key > bk) continue;
+      const unsigned fx = ((unsigned)S.lf[x] << 16) | (unsigned)x;
+      if (key == bk && fx > bx) continue;
+      const int f = (int)(fx >> 16);
+      if ((S.joined[f >> 5] >> (f & 31)) & 1u) continue;
+      const uint2 v = S.ld[x];
+      bool mine = false;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t d = half4(v, i);
+        if (d != kNone16) mine |= (S.lab[d] >> 16) == r;
+      }
+      if (mine) {
+        bk = key;
+        bx = fx;
+      }
     }
-    __syncwarp();
-    int sel[kMaxOrder];
-    int nt = 0;
-    unsigned long long last = 0;
-    for (int it = 0; it < order; ++it) {
-      unsigned long long bk = kNoKey;
-      int bi = -1;
-      for (int u = lane; u < n_np; u += 32) {
-        const unsigned long long ku = S.npk()[u];
-        if (it > 0 && ku <= last) continue;
-        if (S.parent()[S.fst[(int)(ku & 0xffffffffu)]] != r) continue;
-        if (ku < bk) {
-          bk = ku;
-          bi = u;
-        }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long ok = __shfl_xor_sync(kFull, bk, off);
-        const int oi = __shfl_xor_sync(kFull, bi, off);
-        if (ok < bk) {
-          bk = ok;
-          bi = oi;
-        }
-      }
-      if (bk == kNoKey) break;
-      sel[nt++] = bi;
-      last = bk;
+  };
+  auto publish = [&] {
+    const unsigned wk = __reduce_min_sync(kFull, bk);
+    const unsigned wx = __reduce_min_sync(kFull, bk == wk ? bx : kNoKey);
+    if (lane == 0) {
+      sc.red[0][warp] = wk;
+      sc.red[1][warp] = wx;
     }
-    if (nt == 0) continue;
-    long long bcost = LLONG_MAX;
-    int bt = 0;
-    for (int t = lane; t < (1 << nt); t += 32) {
-      long long cost = 0;
-      for (int w = 0; w < W; ++w) {
-        uint32_t mw = S.xsol()[w] & S.cm()[w];
-        for (int k2 = 0; k2 < nt; ++k2)
-          if ((t >> k2) & 1) mw ^= S.npN()[sel[k2] * W + w];
-        while (mw) {
-          const int b = __ffs(mw) - 1;
-          mw &= mw - 1;
-          cost += wfix[S.pcol()[w * 32 + b]];
+  };
+  auto fetch = [&] {
+    const unsigned k0 = lane < I::NW ? sc.red[0][lane] : kNoKey;
+    const unsigned x0 = lane < I::NW ? sc.red[1][lane] : kNoKey;
+    bk = __reduce_min_sync(kFull, k0);
+    bx = __reduce_min_sync(kFull, k0 == bk ? x0 : kNoKey);
+  };
+  bk = bx = kNoKey;
+  scan();
+  publish();
+  if (tid == 0) {
+    S.growb()[r >> 5] = 0u;
+    sc.ng = 0;
+    sc.merged = 0;
+    sc.piv[0] = -1;
+  }
+  __syncthreads();
+  fetch();
+  for (int it = 0;; ++it) {
+    if (bx == kNoKey) return 1;
+    if (steps > n) return 1;  // each step adds a column: cannot be reached
+    const int g = (int)(bx >> 16);
+    const uint2 dets = S.ld[bx & 0xffffu];
+    // ---- the pick joins and claims its detectors: one lane each ----
+    if (warp == 0) {
+      const uint32_t d = half4(dets, lane & 3);
+      const bool on = lane < 4 && d != kNone16;
+      const uint32_t y = on ? S.lab[d] : 0u;
+      const bool free = on && y == kFree;
+      const unsigned fb = __ballot_sync(kFull, free);
+      const int sl = free ? nsl + __popc(fb & ((1u << lane) - 1u)) : (int)(y & 0xffffu);
+      const uint32_t other = on && !free && (y >> 16) != r ? y >> 16 : kNone16;
+      if (free && sl < I::CAP) {
+        S.lab[d] = (r << 16) | (uint32_t)sl;
+        S.sdet()[sl] = (uint16_t)d;
+        S.slab()[sl] = (uint16_t)r;
+        S.flags()[sl] = 0;
+      }
+      if (other != kNone16) S.parent()[other] = (uint16_t)r;
+      if (lane < 4) {
+        reinterpret_cast<uint16_t*>(&sc.ssl)[lane] = on ? (uint16_t)sl : kNone16;
+        reinterpret_cast<uint16_t*>(&sc.mlab)[lane] = (uint16_t)other;
+      }
+      if (lane == 0) {
+        S.joined[g >> 5] |= 1u << (g & 31);
+        sc.fresh = fb;
+        sc.nsl = nsl + __popc(fb);
+        if (nsl + __popc(fb) > I::CAP) sc.ovf = 1;
+      }
+    }
+    // the faults next to those detectors, asked for now and used if the detector is new: thread
+    // (detector q, edge e) from warp 1 on (the last warps when there are not enough)
+    constexpr int kFrom = NT > 32 ? 32 : 0;
+    const int q0 = (tid - kFrom) / D;
+    int near = kNone16;
+    if (tid >= kFrom && q0 < 4) {
+      const uint32_t d = half4(dets, q0);
+      if (d != kNone16) near = G.chk_pad[(size_t)d * D + (tid - kFrom) % D];
+    }
+    __syncthreads();
+    if (sc.ovf) return 3;
+    const int nsl0 = nsl;
+    nsl = sc.nsl;
+    const uint2 sl = sc.ssl, ml = sc.mlab;
+    const unsigned fresh = sc.fresh;
+    if ((ml.x & ml.y) != kFull) {
+      // ---- absorbed clusters take the label r ----
+      const uint32_t m0 = ml.x & 0xffffu, m1 = ml.x >> 16, m2 = ml.y & 0xffffu, m3 = ml.y >> 16;
+      for (int i = tid; i < nsl0; i += NT) {
+        const uint32_t y = S.slab()[i];
+        if (y == m0 || y == m1 || y == m2 || y == m3) {
+          S.slab()[i] = (uint16_t)r;
+          S.lab[S.sdet()[i]] = (r << 16) | (uint32_t)i;
         }
       }
-      for (int k2 = 0; k2 < nt; ++k2)
-        if ((t >> k2) & 1) cost += wfix[(int)(S.npk()[sel[k2]] & 0xffffffffu)];
-      if (cost < bcost) {
-        bcost = cost;
-        bt = t;
+      __syncthreads();
+    }
+    bk = bx = kNoKey;
+    // ---- new candidates; a fault listed here is a candidate of the cluster ----
+    auto admit = [&](int f) {
+      unsigned key;
+      uint2 v;
+      const int x = list_candidate(G, S, llr, f, key, v);
+      const unsigned fx = ((unsigned)f << 16) | (unsigned)x;
+      if (x >= 0 && (key < bk || (key == bk && fx < bx))) {
+        bk = key;
+        bx = fx;
       }
+    };
+    if (near != kNone16 && ((fresh >> q0) & 1u)) admit(near);
+    for (int x = NT - kFrom + tid; x < 4 * D; x += NT)  // pairs beyond the CTA's threads
+      if ((fresh >> (x / D)) & 1u) {
+        const int f = G.chk_pad[(size_t)half4(dets, x / D) * D + x % D];
+        if (f != kNone16) admit(f);
+      }
+    // ---- the column's image; meanwhile the search for the next pick ----
+    open_rows(S, nsl0, nsl, tid);
+    int pc = -1;
+    const uint32_t hit = column_image(G, S, sl, g, nsl, tid, pc);
+    if (pc >= 0) sc.piv[it % 3] = pc;
+    if (tid == 0) sc.piv[(it + 1) % 3] = -1;
+    scan();
+    publish();
+    __syncthreads();
+    if (sc.ovf) return 3;
+    const int p = sc.piv[it % 3];
+    nf = sc.nf;
+    fetch();
+    if (p < 0) keep_dependent(S, np, g, hit, tid);
+    else pivot_update(S, p, g, hit, nsl, tid);
+    bool bad = false;
+    for (int i = tid; i < nsl; i += NT) bad |= (S.flags()[i] & 3) == 1;
+    ++steps;
+    if (!__syncthreads_or(bad)) break;
+  }
+  if (tid == 0) sc.np = np;
+  __syncthreads();
+  return I::MU && sc.ovf ? 3 : 0;
+}
+
+// ---- LSD-mu reprocessing, one warp per cluster ----
+
+// Order key of the dependent column of index u.
+template <class I>
+__device__ __forceinline__ unsigned long long dep_key(const Shot<I>& S, int u) {
+  return ((unsigned long long)S.dpk()[u] << 32) | S.dpf()[u];
+}
+
+// The first `want` dependent columns of cluster r in key order; lane j returns the j-th (or
+// -1), count = how many there are.
+template <class I>
+__device__ int first_dependent(const Shot<I>& S, int r, int np, int want, int lane, int& count) {
+  int mine = -1;
+  unsigned long long last = 0;
+  int nt = 0;
+  for (int it = 0; it < want; ++it) {
+    unsigned long long bk = ~0ull;
+    int bi = -1;
+    for (int u = lane; u < np; u += 32) {
+      if (S.dpr()[u] != r) continue;
+      const unsigned long long ku = dep_key(S, u);
+      if ((it > 0 && ku <= last) || ku >= bk) continue;
+      bk = ku;
+      bi = u;
     }
     for (int off = 16; off > 0; off >>= 1) {
-      const long long oc = __shfl_xor_sync(kFull, bcost, off);
-      const int ot = __shfl_xor_sync(kFull, bt, off);
-      if (oc < bcost || (oc == bcost && ot < bt)) {
-        bcost = oc;
-        bt = ot;
+      const unsigned long long ok = __shfl_xor_sync(kFull, bk, off);
+      const int oi = __shfl_xor_sync(kFull, bi, off);
+      if (ok < bk) {
+        bk = ok;
+        bi = oi;
       }
     }
-    for (int w = lane; w < W; w += 32) {
-      uint32_t delta = 0;
-      for (int k2 = 0; k2 < nt; ++k2)
-        if ((bt >> k2) & 1) delta ^= S.npN()[sel[k2] * W + w];
-      S.xsol()[w] ^= delta;
+    if (bi < 0) break;
+    if (lane == nt) mine = bi;
+    ++nt;
+    last = bk;
+  }
+  count = nt;
+  return mine;
+}
+
+// Words of the local solution of every row (bit = the row's pivot column is in it).
+template <class I>
+__device__ void solution_words(const Shot<I>& S, uint32_t* xw, int nsl, int lane) {
+  for (int c = 0; 32 * c < nsl; ++c) {
+    const int i = 32 * c + lane;
+    const unsigned b = __ballot_sync(kFull, i < nsl && (S.flags()[i] & 3) == 3);
+    if (lane == 0) xw[c] = b;
+  }
+  __syncwarp();
+}
+
+// Exhaustive OSD over the first min(mu, #dependent) dependent columns of cluster r (App. D);
+// cost = sum of 2^-32 fixed-point channel weights, ties to the smaller pattern.  Rows that no
+// selected column touches cost every pattern the same and are left out.
+template <class I>
+__device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl, uint32_t* xw,
+                      uint32_t* uw, int lane) {
+  const long long* wfix = a.g.wfix;
+  const int wc = (nsl + 31) >> 5;
+  int nt;
+  const int mine = first_dependent(S, r, np, a.order, lane, nt);
+  if (nt == 0) return;
+  solution_words(S, xw, nsl, lane);
+  for (int w0 = 0; w0 < wc; w0 += 32) {  // rows that some selected column touches
+    const int w = w0 + lane;
+    uint32_t rows = 0;
+    for (int j = 0; j < nt; ++j) {
+      const int u = __shfl_sync(kFull, mine, j);
+      if (w < wc) rows |= S.npN()[(size_t)u * I::W + w];
     }
-    if (lane == 0) {
-      int ne = S.scal()[S_EXT];
-      for (int k2 = 0; k2 < nt; ++k2)
-        if ((bt >> k2) & 1) S.ext()[ne++] = (int)(S.npk()[sel[k2]] & 0xffffffffu);
-      S.scal()[S_EXT] = ne;
+    if (w < wc) uw[w] = rows;
+  }
+  __syncwarp();
+  const long long wmine = lane < nt ? wfix[S.dpf()[mine]] : 0;
+  long long bcost = LLONG_MAX;
+  int bt = 0;
+  for (int t0 = 0; t0 < (1 << nt); t0 += 32) {
+    const int t = t0 + lane;
+    long long cost = 0;
+    for (int w = 0; w < wc; ++w) {
+      uint32_t rows = uw[w];
+      if (rows == 0) continue;
+      const uint32_t nw = lane < nt ? S.npN()[(size_t)mine * I::W + w] : 0u;
+      const uint32_t x = xw[w];
+      while (rows) {
+        const int b = __ffs(rows) - 1;
+        rows &= rows - 1;
+        const unsigned pm = __ballot_sync(kFull, (nw >> b) & 1u);
+        if (((x >> b) ^ __popc(pm & (unsigned)t)) & 1u) cost += wfix[S.pcol()[32 * w + b]];
+      }
     }
-    __syncwarp();
+    for (int j = 0; j < nt; ++j) {
+      const long long wj = __shfl_sync(kFull, wmine, j);
+      if ((t >> j) & 1) cost += wj;
+    }
+    if (t < (1 << nt) && cost < bcost) {
+      bcost = cost;
+      bt = t;
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    const long long oc = __shfl_xor_sync(kFull, bcost, off);
+    const int ot = __shfl_xor_sync(kFull, bt, off);
+    if (oc < bcost || (oc == bcost && ot < bt)) {
+      bcost = oc;
+      bt = ot;
+    }
+  }
+  for (int j = 0; j < nt; ++j) {
+    if (!((bt >> j) & 1)) continue;
+    const int u = __shfl_sync(kFull, mine, j);
+    for (int w = 0; w < wc; ++w)
+      if ((S.npN()[(size_t)u * I::W + w] >> lane) & 1u) S.flags()[32 * w + lane] ^= 1;
+    if (lane == 0) S.ext()[atomicAdd(&S.sc->ext, 1)] = S.dpf()[u];
   }
 }
 
-// Cost of cluster r's local solution (xsol masked by cm) with the dependent columns of slots
-// u1 and u2 flipped (-1 = none).
-template <class L>
-__device__ __forceinline__ long long sparse_pattern_cost(const LSDArgs& a, const SShot<L>& S,
-                                                         int u1, int u2) {
-  constexpr int W = L::W;
+// Cost of the cluster's solution with dependent columns u1 and u2 (-1 = none) flipped, less the
+// unflipped solution's.
+template <class I>
+__device__ __forceinline__ long long pattern_delta(const LSDArgs& a, const Shot<I>& S,
+                                                   const uint32_t* xw, int wc, int u1, int u2) {
   const long long* wfix = a.g.wfix;
-  long long cost = 0;
-  for (int w = 0; w < W; ++w) {
-    uint32_t mw = S.xsol()[w] & S.cm()[w];
-    if (u1 >= 0) mw ^= S.npN()[u1 * W + w];
-    if (u2 >= 0) mw ^= S.npN()[u2 * W + w];
-    while (mw) {
-      const int b = __ffs(mw) - 1;
-      mw &= mw - 1;
-      cost += wfix[S.pcol()[w * 32 + b]];
+  long long cost = wfix[S.dpf()[u1]];
+  if (u2 >= 0) cost += wfix[S.dpf()[u2]];
+  for (int w = 0; w < wc; ++w) {
+    uint32_t rows = S.npN()[(size_t)u1 * I::W + w];
+    if (u2 >= 0) rows ^= S.npN()[(size_t)u2 * I::W + w];
+    const uint32_t x = xw[w];
+    while (rows) {
+      const int b = __ffs(rows) - 1;
+      rows &= rows - 1;
+      const long long c = wfix[S.pcol()[32 * w + b]];
+      cost += (x >> b) & 1u ? -c : c;
     }
   }
-  if (u1 >= 0) cost += wfix[(int)(S.npk()[u1] & 0xffffffffu)];
-  if (u2 >= 0) cost += wfix[(int)(S.npk()[u2] & 0xffffffffu)];
   return cost;
 }
 
-// OSD-CS-w reprocessing of every cluster (App. D), as osd_cs in lsd.cu: no flip, every
-// single dependent column, every pair among the first w in key order; ranked by
-// (cost, class, key) with class 0 = no flip, 1 = single (key = the column's 64-bit order
-// key), 2 = pair (key = i * 16 + j).
-template <class L>
-__device__ void sparse_osd_cs(const LSDArgs& a, const SShot<L>& S, int lane) {
-  constexpr int W = L::W;
-  const int nroots = collect_all(S, lane);
-  const int n_np = S.scal()[S_NP];
-  const int nsl = S.scal()[S_SLOTS];
-  const int w_cs = a.osd_cs;
-  for (int ci = 0; ci < nroots; ++ci) {
-    const int r = S.inv()[ci];
-    for (int c = 0; c < W; ++c) {
-      const int sl = c * 32 + lane;
-      const bool in = sl < nsl && S.dlab[S.dslot()[sl]] == r;
-      const unsigned bal = __ballot_sync(kFull, in);
-      if (lane == 0) S.cm()[c] = bal;
+// Combination sweep OSD-CS-w of cluster r (App. D), as osd_cs in lsd.cu: no flip, every single
+// dependent column, every pair among the first w in key order; ranked by (cost, class, key)
+// with class 0 = no flip, 1 = single (key = the column's order key), 2 = pair (key = 16 i + j).
+template <class I>
+__device__ void osd_cs(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl, uint32_t* xw,
+                       int lane) {
+  const int wc = (nsl + 31) >> 5;
+  int nt;
+  const int sel = first_dependent(S, r, np, a.osd_cs, lane, nt);
+  solution_words(S, xw, nsl, lane);
+  long long bc = LLONG_MAX;
+  int bcls = 3, b1 = -1, b2 = -1;
+  unsigned long long bkey = 0;
+  auto consider = [&](long long c, int cls, unsigned long long key, int u1, int u2) {
+    if (c < bc || (c == bc && (cls < bcls || (cls == bcls && key < bkey)))) {
+      bc = c;
+      bcls = cls;
+      bkey = key;
+      b1 = u1;
+      b2 = u2;
     }
-    __syncwarp();
-    int sel[kMaxCsOrder];
-    int nt = 0;
-    unsigned long long last = 0;
-    for (int it = 0; it < w_cs; ++it) {
-      unsigned long long bk = kNoKey;
-      int bi = -1;
-      for (int u = lane; u < n_np; u += 32) {
-        const unsigned long long ku = S.npk()[u];
-        if (it > 0 && ku <= last) continue;
-        if (S.parent()[S.fst[(int)(ku & 0xffffffffu)]] != r) continue;
-        if (ku < bk) {
-          bk = ku;
-          bi = u;
-        }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long ok = __shfl_xor_sync(kFull, bk, off);
-        const int oi = __shfl_xor_sync(kFull, bi, off);
-        if (ok < bk) {
-          bk = ok;
-          bi = oi;
-        }
-      }
-      if (bk == kNoKey) break;
-      sel[nt++] = bi;
-      last = bk;
+  };
+  if (lane == 0) consider(0, 0, 0, -1, -1);
+  for (int u = lane; u < np; u += 32) {
+    if (S.dpr()[u] != r) continue;
+    consider(pattern_delta(a, S, xw, wc, u, -1), 1, dep_key(S, u), u, -1);
+  }
+  const int npairs = nt * (nt - 1) / 2;
+  for (int t0 = 0; t0 < npairs; t0 += 32) {
+    const int t = t0 + lane;
+    int i = 0, rem = t < npairs ? t : 0;
+    while (rem >= nt - 1 - i) {
+      rem -= nt - 1 - i;
+      ++i;
     }
-    long long bc = LLONG_MAX;
-    int bcls = 3, b1 = -1, b2 = -1;
-    unsigned long long bkey = 0;
-    auto consider = [&](long long c, int cls, unsigned long long key, int u1, int u2) {
-      if (c < bc || (c == bc && (cls < bcls || (cls == bcls && key < bkey)))) {
-        bc = c;
-        bcls = cls;
-        bkey = key;
-        b1 = u1;
-        b2 = u2;
-      }
-    };
-    if (lane == 0) consider(sparse_pattern_cost(a, S, -1, -1), 0, 0, -1, -1);
-    for (int u = lane; u < n_np; u += 32) {
-      const unsigned long long ku = S.npk()[u];
-      if (S.parent()[S.fst[(int)(ku & 0xffffffffu)]] != r) continue;
-      consider(sparse_pattern_cost(a, S, u, -1), 1, ku, u, -1);
-    }
-    const int npairs = nt * (nt - 1) / 2;
-    for (int t = lane; t < npairs; t += 32) {
-      int i = 0, rem = t;
-      while (rem >= nt - 1 - i) {
-        rem -= nt - 1 - i;
-        ++i;
-      }
-      const int j = i + 1 + rem;
-      consider(sparse_pattern_cost(a, S, sel[i], sel[j]), 2, (unsigned long long)(i * 16 + j),
-               sel[i], sel[j]);
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      const long long oc = __shfl_xor_sync(kFull, bc, off);
-      const int ocls = __shfl_xor_sync(kFull, bcls, off);
-      const unsigned long long okey = __shfl_xor_sync(kFull, bkey, off);
-      const int o1 = __shfl_xor_sync(kFull, b1, off);
-      const int o2 = __shfl_xor_sync(kFull, b2, off);
-      consider(oc, ocls, okey, o1, o2);
-    }
-    if (b1 < 0) continue;  // no flip: OSD-0's local solution stands
-    for (int w = lane; w < W; w += 32) {
-      uint32_t delta = S.npN()[b1 * W + w];
-      if (b2 >= 0) delta ^= S.npN()[b2 * W + w];
-      S.xsol()[w] ^= delta;
-    }
-    if (lane == 0) {
-      int ne = S.scal()[S_EXT];
-      S.ext()[ne++] = (int)(S.npk()[b1] & 0xffffffffu);
-      if (b2 >= 0) S.ext()[ne++] = (int)(S.npk()[b2] & 0xffffffffu);
-      S.scal()[S_EXT] = ne;
-    }
-    __syncwarp();
+    const int j = i + 1 + rem;
+    const int u1 = __shfl_sync(kFull, sel, i), u2 = __shfl_sync(kFull, sel, j);
+    if (t < npairs)
+      consider(pattern_delta(a, S, xw, wc, u1, u2), 2, (unsigned long long)(i * 16 + j), u1, u2);
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    const long long oc = __shfl_xor_sync(kFull, bc, off);
+    const int ocls = __shfl_xor_sync(kFull, bcls, off);
+    const unsigned long long okey = __shfl_xor_sync(kFull, bkey, off);
+    const int o1 = __shfl_xor_sync(kFull, b1, off);
+    const int o2 = __shfl_xor_sync(kFull, b2, off);
+    consider(oc, ocls, okey, o1, o2);
+  }
+  if (b1 < 0) return;  // no flip: OSD-0's local solution stands
+  for (int w = 0; w < wc; ++w) {
+    uint32_t delta = S.npN()[(size_t)b1 * I::W + w];
+    if (b2 >= 0) delta ^= S.npN()[(size_t)b2 * I::W + w];
+    if ((delta >> lane) & 1u) S.flags()[32 * w + lane] ^= 1;
+  }
+  if (lane == 0) {
+    S.ext()[atomicAdd(&S.sc->ext, 1)] = S.dpf()[b1];
+    if (b2 >= 0) S.ext()[atomicAdd(&S.sc->ext, 1)] = S.dpf()[b2];
   }
 }
 
-// Work items come from a.queue / a.count as in lsd.cu.  Shots that overflow the capacity are
-// appended to spill[] (spill_count) when spill != nullptr, else reported unsolvable.
-template <int CAP, int SC, bool MU, bool GLOBAL_RT>
-__global__ void __launch_bounds__(128, 1) lsd_sparse_kernel(LSDArgs a, int* scratch, size_t stride,
-                                                         int* spill, unsigned long long* spill_count,
-                                                         const int* items, const unsigned long long* item_count) {
-  using L = SLay<CAP, SC, MU>;
-  constexpr int W = L::W;
+// Work items come from a.queue / a.count as in lsd.cu.  Shots that outgrow the instance are
+// appended to spill[] (counted in ctr->spill_count) when spill != nullptr, else reported
+// unsolvable.  The large instance (items != nullptr) takes those.
+template <class I>
+__global__ void __launch_bounds__(I::NT, I::BIG ? 1 : 2)
+lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, const int* items) {
+  constexpr int NT = I::NT;
   extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = blockIdx.x * (blockDim.x >> 5) + warp;
+  __shared__ Scal sc;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m = a.g.m, n = a.g.n;
-  // the spill instance keeps all of its state in its global scratch (no shared memory), so
-  // that many of its warps can be resident per SM
-  const size_t per_sm = GLOBAL_RT ? 0 : L::sm_total + L::rt_total;
-  SShot<L> S;
-  S.sm = smem + (size_t)warp * per_sm;
-  int* ws = scratch + (size_t)gw * stride;
-  S.dlab = ws;
-  S.slot = ws + m;
-  S.fst = ws + 2 * m;
-  S.front = ws + 2 * m + n;
-  S.rt = GLOBAL_RT ? reinterpret_cast<unsigned char*>(ws + 2 * m + 2 * n) : S.sm + L::sm_total;
-  if (GLOBAL_RT) S.sm = S.rt + L::rt_total;
-  // the spill instance also keeps one candidate mask per seed (up to kMaskSeeds) after its
-  // other state
-  const int wn_masks = GLOBAL_RT ? (n + 31) / 32 : 0;
-  S.wn = 0;
-  S.cmask = GLOBAL_RT ? reinterpret_cast<uint32_t*>(S.sm + L::sm_total) : nullptr;
-  SGraph G{a.g.chk_ptr, a.g.chk_var, a.g.var_ptr, a.g.var_chk, a.g.max_col_deg};
-
-  long long count;
-  if (items) count = (long long)*item_count;
-  else count = a.count_from_ctr ? (long long)a.ctr->lsd_count : a.count;
+  const int wn = (n + 31) / 32;
+  Shot<I> S;
+  S.sc = &sc;
+  S.sm = smem;
+  {
+    unsigned char* sp = smem + I::fixed;
+    unsigned char* gp = scratch + (size_t)blockIdx.x * stride;
+    auto take = [](unsigned char*& p, size_t bytes) {
+      unsigned char* q = p;
+      p += al16(bytes);
+      return q;
+    };
+    S.cand = reinterpret_cast<uint32_t*>(take(sp, (size_t)wn * 4));
+    S.joined = reinterpret_cast<uint32_t*>(take(sp, (size_t)wn * 4));
+    if constexpr (I::LG) S.lab = reinterpret_cast<uint32_t*>(take(gp, (size_t)m * 4));
+    else S.lab = reinterpret_cast<uint32_t*>(take(sp, (size_t)m * 4));
+    S.li = I::BIG ? take(gp, I::lists) : take(sp, I::lists);
+    S.lcap = I::lcap(n);
+    auto list = [&](unsigned char*& p) {
+      S.ld = reinterpret_cast<uint2*>(take(p, (size_t)S.lcap * 8));
+      S.lk = reinterpret_cast<uint32_t*>(take(p, (size_t)S.lcap * 4));
+      S.lf = reinterpret_cast<uint16_t*>(take(p, (size_t)S.lcap * 2));
+    };
+    if constexpr (I::BIG && I::LG) list(gp);
+    else list(sp);
+  }
+  const SGraph G{a.g.chk_ptr, a.g.var_ptr, a.g.var_chk, a.g.chk_pad,
+                 reinterpret_cast<const uint2*>(a.g.var_pad), a.g.max_col_deg, a.g.max_row_deg};
+  unsigned long long* const next = I::BIG ? &a.ctr->spill_next : &a.ctr->lsd_next;
+  const unsigned count = (unsigned)(items               ? a.ctr->spill_count
+                                    : a.count_from_ctr ? a.ctr->lsd_count
+                                                       : (unsigned long long)a.count);
   unsigned long long steps_acc = 0, unsolv = 0;
   int kappa_max = 0, nu_max = 0;
-  for (;;) {
-    unsigned long long item = 0;
-    if (lane == 0) item = atomicAdd(&a.ctr->lsd_next, 1ULL);
-    item = __shfl_sync(kFull, item, 0);
-    if (item >= (unsigned long long)count) break;
+  // the first item of a CTA is its block index, the others come from the counter
+  for (unsigned item = blockIdx.x; item < count;) {
     const long long qi = items ? (long long)items[item] : (long long)item;
     const long long shot = a.queue ? (long long)a.queue[qi] : qi;
     const float* llr = a.llr + (a.llr_by_item ? qi : shot) * n;
-    // the shot's correction: bytes, or packed words (set bits with atomicOr: lanes share words)
+    // the shot's correction: bytes, or packed words (set bits with atomicOr: threads share words)
     uint8_t* co = a.packed ? nullptr : a.corrections + shot * n;
     uint32_t* cw = a.packed ? reinterpret_cast<uint32_t*>(a.corrections) + shot * packed_words(n)
                             : nullptr;
 
-    // ---- init ----
-    for (int d = lane; d < m; d += 32) {
-      S.dlab[d] = -1;
-      S.slot[d] = -1;
+    // ---- init: one cluster per flipped detector ----
+    for (int d = tid; d < (m + 3) / 4; d += NT)
+      reinterpret_cast<uint4*>(S.lab)[d] = make_uint4(kFree, kFree, kFree, kFree);
+    for (int w = tid; w < wn; w += NT) S.cand[w] = S.joined[w] = 0u;
+    for (int w = tid; w < I::SC / 32; w += NT) S.growb()[w] = 0u;
+    if (tid == 0) {
+      sc.ns = sc.nf = sc.n_new = sc.merged = sc.ng = sc.np = sc.ovf = sc.ext = 0;
+      sc.item = gridDim.x + (unsigned)atomicAdd(next, 1ULL);
     }
-    for (int j = lane; j < n; j += 32) S.fst[j] = -2;
-    for (int sl = lane; sl < CAP; sl += 32) S.pcol()[sl] = -1;
-    for (int w = lane; w < W; w += 32) {
-      S.syn()[w] = 0;
-      S.xsol()[w] = 0;
-    }
-    if (lane < 16) S.scal()[lane] = 0;
-    __syncwarp();
-    int ns = 0;
-    for (int b0 = 0; b0 < m; b0 += 32) {
-      const int d = b0 + lane;
-      const bool f = d < m && syn_bit(a.syndromes, a.packed, shot, m, d) != 0;
-      const unsigned bal = __ballot_sync(kFull, f);
-      if (f) {
-        const int k = ns + __popc(bal & ((1u << lane) - 1u));
-        if (k < SC && k < CAP) {
-          S.seed()[k] = d;
-          S.parent()[k] = k;
-          S.mark()[k] = 0u;
-          S.gflag()[k] = 0;
-          S.dlab[d] = k;
-          S.slot[d] = k;
-          S.dslot()[k] = d;
-          atomicOr(&S.syn()[k >> 5], 1u << (k & 31));
-        }
+    __syncthreads();
+    const unsigned next_item = sc.item;
+    auto seed = [&](int d) {
+      const int k = atomicAdd(&sc.ns, 1);
+      if (k < I::SC && k < I::CAP) {
+        S.lab[d] = ((uint32_t)k << 16) | (uint32_t)k;
+        S.sdet()[k] = (uint16_t)d;
+        S.slab()[k] = (uint16_t)k;
+        S.parent()[k] = (uint16_t)k;
+        S.flags()[k] = 1;
+        S.inv()[k] = (uint16_t)k;
+        atomicOr(&S.growb()[k >> 5], 1u << (k & 31));
       }
-      ns += __popc(bal);
+    };
+    const uint8_t* sp = a.syndromes + shot * m;
+    if (!a.packed && (m & 3) == 0 && (reinterpret_cast<uintptr_t>(sp) & 3) == 0) {
+      for (int q = tid; q < m / 4; q += NT) {  // four detectors a load
+        const uint32_t v = reinterpret_cast<const uint32_t*>(sp)[q];
+        if (v == 0) continue;
+        for (int b = 0; b < 4; ++b)
+          if ((v >> (8 * b)) & 0xffu) seed(4 * q + b);
+      }
+    } else {
+      for (int d = tid; d < m; d += NT)
+        if (syn_bit(a.syndromes, a.packed, shot, m, d)) seed(d);
     }
+    __syncthreads();
+    const int ns = sc.ns;
     int status = LSD_SHOT_OK_LSD, steps = 0;
-    if (ns > SC || ns > CAP) status = kSpill;
-    S.wn = ns <= kMaskSeeds ? wn_masks : 0;
-    if (lane == 0) {
-      S.scal()[S_NSEED] = min(ns, SC);
-      S.scal()[S_SLOTS] = min(ns, CAP);
+    if (ns > I::SC || ns > I::CAP) {
+      status = kSpill;
+    } else {
+      if (tid == 0) sc.nsl = ns;
+      open_slots(G, S, llr, 0, ns, tid);
+      __syncthreads();
+      if (sc.ovf) status = kSpill;
     }
-    __syncwarp();
-    for (int w = lane; w < W; w += 32) S.sred()[w] = S.syn()[w];
-    // candidates next to the seeds (and each seed's candidate mask)
-    if (status == LSD_SHOT_OK_LSD) {
-      if (S.wn > 0) {
-        for (size_t w = lane; w < (size_t)ns * S.wn; w += 32) S.cmask[w] = 0u;
-        __syncwarp();
-      }
-      for (int k = lane; k < ns; k += 32) {
-        const int d = S.seed()[k];
-        uint32_t* cm = S.wn > 0 ? S.cmask + (size_t)k * S.wn : nullptr;
-        for (int e = G.chk_ptr[d]; e < G.chk_ptr[d + 1]; ++e) {
-          const int f = G.chk_var[e];
-          if (atomicCAS(&S.fst[f], -2, -1) == -2) {
-            const int q = atomicAdd(&S.scal()[S_NFRONT], 1);
-            S.front[q] = f;
-          }
-          if (cm) atomicOr(&cm[f >> 5], 1u << (f & 31));
-        }
-      }
-    }
-    __syncwarp();
-    int k = status == LSD_SHOT_OK_LSD ? ns : 0;
-    if (status == LSD_SHOT_OK_LSD && lane == 0)
-      for (int t = 0; t < ns; ++t) S.inv()[t] = t;
-    __syncwarp();
 
-    // ---- LSD-0 ----
+    // ---- LSD-0: grow every invalid cluster until all are valid ----
+    int k = status == LSD_SHOT_OK_LSD ? ns : 0;
     while (k > 0) {
-      if (steps > n) {
+      if (steps > n) {  // each step adds a column: cannot be reached
         status = LSD_SHOT_UNSOLVABLE;
         break;
       }
-      const int rc = sparse_step<L, MU, CAP>(G, S, llr, k, true, lane);
-      if (rc == 1) {
-        status = LSD_SHOT_UNSOLVABLE;
+      const bool single = k == 1 && G.max_col_deg <= 4;
+      const int rc = single ? grow_single(G, S, llr, S.inv()[0], n, steps, tid)
+                            : sparse_step(G, S, llr, k, true, tid);
+      if (rc) {
+        status = rc == 1 ? LSD_SHOT_UNSOLVABLE : kSpill;
         break;
       }
-      if (rc == 3) {
-        status = kSpill;
-        break;
-      }
+      if (single) break;
       ++steps;
-      k = collect_invalid(S, lane);
+      k = collect(S, sc.nsl, true, tid);
     }
-    // ---- LSD-mu ----
-    if constexpr (MU) {
-      if (status == LSD_SHOT_OK_LSD) {
-        for (int e = 0; e < a.order; ++e) {
-          k = collect_all(S, lane);
-          const int rc = sparse_step<L, MU, CAP>(G, S, llr, k, false, lane);
-          if (rc == 3) {
-            status = kSpill;
-            break;
-          }
-          if (rc == 2) break;
+    // ---- LSD-mu: mu more steps for every cluster, then the local reprocessing ----
+    if constexpr (I::MU) {
+      for (int e = 0; e < a.order && status == LSD_SHOT_OK_LSD; ++e) {
+        k = collect(S, sc.nsl, false, tid);
+        if (k == 0) break;
+        const int rc = sparse_step(G, S, llr, k, false, tid);
+        if (rc == 3) status = kSpill;
+        if (rc == 2) break;
+      }
+      __syncthreads();
+      const int np = sc.np;
+      if (status == LSD_SHOT_OK_LSD)
+        for (int u = tid; u < np; u += NT) {
+          const int f = S.dpf()[u];
+          S.dpr()[u] = (uint16_t)(S.lab[half4(G.var_pad[f], 0)] >> 16);
+          S.dpk()[u] = llr_bits(llr[f]);
         }
-        if (status == LSD_SHOT_OK_LSD) {
-          if (a.osd_cs >= 0)
-            sparse_osd_cs(a, S, lane);
-          else
-            sparse_osd_e(a, S, lane);
+      __syncthreads();
+      if (status == LSD_SHOT_OK_LSD && np > 0) {
+        uint32_t* xw = S.template s<uint32_t>(I::osd) + (size_t)warp * 2 * I::W;
+        const int nsl = sc.nsl;
+        for (int r = warp; r < ns; r += NT / 32) {
+          if (S.parent()[r] != r) continue;
+          if (a.osd_cs >= 0) osd_cs(a, S, r, np, nsl, xw, lane);
+          else osd_e(a, S, r, np, nsl, xw, xw + I::W, lane);
+          __syncwarp();
         }
+      }
+    }
+    __syncthreads();
+
+    // ---- the correction row, cleared; a shot without room goes to the large instance ----
+    if (status != kSpill || !spill) {
+      if (cw) {
+        for (int w = tid; w < packed_words(n); w += NT) cw[w] = 0u;
+      } else if ((n & 3) == 0 && (reinterpret_cast<uintptr_t>(co) & 3) == 0) {
+        for (int j = tid; j < n / 4; j += NT) reinterpret_cast<uint32_t*>(co)[j] = 0u;
+      } else {
+        for (int j = tid; j < n; j += NT) co[j] = 0;
       }
     }
     if (status == kSpill) {
-      if (lane == 0) {
-        if (spill) {
-          const unsigned long long q = atomicAdd(spill_count, 1ULL);
-          spill[q] = (int)qi;
-        } else {
-          if (a.status) a.status[shot] = LSD_SHOT_UNSOLVABLE;
-        }
+      if (tid == 0) {
+        if (spill) spill[atomicAdd(&a.ctr->spill_count, 1ULL)] = (int)qi;
+        else if (a.status) a.status[shot] = LSD_SHOT_UNSOLVABLE;
       }
-      if (!spill) {
-        if (cw)
-          for (int w = lane; w < packed_words(n); w += 32) cw[w] = 0u;
-        else
-          for (int j = lane; j < n; j += 32) co[j] = 0;
-        unsolv += 1;
-      }
-      __syncwarp();
+      if (!spill) unsolv += 1;
+      __syncthreads();
+      item = next_item;
       continue;
     }
-
-    // ---- statistics ----
-    const int nseed = S.scal()[S_NSEED];
-    for (int x = lane; x < nseed; x += 32) S.mark()[x] = 0u;
-    __syncwarp();
-    // every fault in a cluster was a candidate first: count them from the candidate history
-    // is not kept, so count over all faults of the claimed detectors' rows
-    {
-      const int nsl = S.scal()[S_SLOTS];
-      for (int sl = lane; sl < nsl; sl += 32) {
-        const int d = S.dslot()[sl];
-        for (int e = G.chk_ptr[d]; e < G.chk_ptr[d + 1]; ++e) {
-          const int f = G.chk_var[e];
-          const int lab = S.fst[f];
-          // count each clustered fault once: at its lowest claimed detector
-          if (lab >= 0) {
-            int lowest = INT_MAX;
-            for (int q = G.var_ptr[f]; q < G.var_ptr[f + 1]; ++q) lowest = min(lowest, (int)G.var_chk[q]);
-            if (lowest == d) atomicAdd(&S.mark()[S.parent()[lab]], 1u);
-          }
-        }
-      }
+    // ---- statistics: nu clusters, kappa = largest cluster in columns ----
+    for (int r = tid; r < ns; r += NT) S.best()[r] = 0u;
+    if (tid == 0) sc.red[0][0] = sc.red[1][0] = 0u;
+    __syncthreads();
+    const int nf = sc.nf, nsl = sc.nsl;
+    for (int x = tid; x < nf; x += NT) {
+      const int f = S.lf[x];
+      if ((S.joined[f >> 5] >> (f & 31)) & 1u)
+        atomicAdd(&S.best()[S.lab[half4(S.ld[x], 0)] >> 16], 1u);
     }
-    __syncwarp();
-    int nu = 0, kappa = 0;
-    for (int x = lane; x < nseed; x += 32) {
-      if (S.parent()[x] == x) {
-        ++nu;
-        kappa = max(kappa, (int)S.mark()[x]);
-      }
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      nu += __shfl_xor_sync(kFull, nu, off);
-      kappa = max(kappa, __shfl_xor_sync(kFull, kappa, off));
-    }
-    for (int x = lane; x < nseed; x += 32) S.mark()[x] = 0u;
-
-    // ---- corrections ----
-    if (cw)
-      for (int w = lane; w < packed_words(n); w += 32) cw[w] = 0u;
-    else
-      for (int j = lane; j < n; j += 32) co[j] = 0;
-    __syncwarp();
+    // ---- global decoding: union of the local solutions (Eq. 2) ----
     if (status == LSD_SHOT_OK_LSD) {
       auto set = [&](int j) {
-        if (cw)
-          atomicOr(cw + (j >> 5), 1u << (j & 31));
-        else
-          co[j] = 1;
+        if (cw) atomicOr(cw + (j >> 5), 1u << (j & 31));
+        else co[j] = 1;
       };
-      const int nsl = S.scal()[S_SLOTS];
-      for (int sl = lane; sl < nsl; sl += 32)
-        if (bit_of(S.xsol(), sl)) set(S.pcol()[sl]);
-      if constexpr (MU) {
-        const int ne = S.scal()[S_EXT];
-        for (int t = lane; t < ne; t += 32) set(S.ext()[t]);
+      for (int i = tid; i < nsl; i += NT)
+        if ((S.flags()[i] & 3) == 3) set(S.pcol()[i]);
+      if constexpr (I::MU) {
+        const int ne = sc.ext;
+        for (int t = tid; t < ne; t += NT) set(S.ext()[t]);
       }
     }
-    __syncwarp();
+    __syncthreads();
+    unsigned nu = 0, kappa = 0;
+    for (int r = tid; r < ns; r += NT)
+      if (S.parent()[r] == r) {
+        ++nu;
+        kappa = max(kappa, S.best()[r]);
+      }
+    nu = __reduce_add_sync(kFull, nu);
+    kappa = __reduce_max_sync(kFull, kappa);
     if (lane == 0) {
+      atomicAdd(&sc.red[0][0], nu);
+      atomicMax(&sc.red[1][0], kappa);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      nu = sc.red[0][0];
+      kappa = sc.red[1][0];
       if (a.status) a.status[shot] = (uint8_t)status;
       if (a.shot_info) {
-        a.shot_info[3 * shot] = nu;
-        a.shot_info[3 * shot + 1] = kappa;
+        a.shot_info[3 * shot] = (int)nu;
+        a.shot_info[3 * shot + 1] = (int)kappa;
         a.shot_info[3 * shot + 2] = steps;
       }
+      steps_acc += steps;
+      unsolv += status == LSD_SHOT_UNSOLVABLE ? 1 : 0;
+      kappa_max = max(kappa_max, (int)kappa);
+      nu_max = max(nu_max, (int)nu);
     }
-    steps_acc += steps;
-    unsolv += status == LSD_SHOT_UNSOLVABLE ? 1 : 0;
-    kappa_max = max(kappa_max, kappa);
-    nu_max = max(nu_max, nu);
-    __syncwarp();
+    item = next_item;
   }
-  if (lane == 0) {
+  if (tid == 0) {
     if (steps_acc) atomicAdd(&a.ctr->lsd_steps, steps_acc);
     if (unsolv) atomicAdd(&a.ctr->unsolvable, unsolv);
-    atomicMax(&a.ctr->kappa_max, kappa_max);
-    atomicMax(&a.ctr->nu_max, nu_max);
+    if (kappa_max) atomicMax(&a.ctr->kappa_max, kappa_max);
+    if (nu_max) atomicMax(&a.ctr->nu_max, nu_max);
   }
 }
 
-constexpr int kSmallCap = 256, kSmallSeeds = 256, kBigCap = 4096, kBigSeeds = 4096;
-constexpr int kSparseWarps = 4;
+template <bool MU, bool LG>
+using Small = Inst<512, 512, 512, MU, false, LG>;
+template <bool MU, bool LG>
+using Big = Inst<1024, 4096, 4096, MU, true, LG>;
 
-template <bool MU>
-size_t small_smem() {
-  return (size_t)kSparseWarps * (SLay<kSmallCap, kSmallSeeds, MU>::sm_total +
-                                 SLay<kSmallCap, kSmallSeeds, MU>::rt_total);
+// Calls fn with the instance for an m x n matrix.
+template <template <bool, bool> class T, bool MU, class F>
+auto pick_instance(int m, int n, F&& fn) {
+  if (smem_bytes<T<MU, false>>(m, n) > kSmemLimit) return fn(T<MU, true>());
+  return fn(T<MU, false>());
 }
-constexpr int kBigWarpsPerSm = 4;  // spill-instance warps (one per CTA) per SM
+template <class F>
+auto with_instance(bool big, bool mu, int m, int n, F&& fn) {
+  if (big) return mu ? pick_instance<Big, true>(m, n, fn) : pick_instance<Big, false>(m, n, fn);
+  return mu ? pick_instance<Small, true>(m, n, fn) : pick_instance<Small, false>(m, n, fn);
+}
 
 }  // namespace
 
-// Scratch ints per warp: dlab, slot (m each), fst, front (n each); the big instance adds the
-// elimination arrays.
-size_t sparse_scratch_ints(int m, int n, bool big, bool mu) {
-  size_t s = (size_t)2 * m + (size_t)2 * n;
-  if (big)
-    s += (mu ? SLay<kBigCap, kBigSeeds, true>::rt_total + SLay<kBigCap, kBigSeeds, true>::sm_total
-             : SLay<kBigCap, kBigSeeds, false>::rt_total + SLay<kBigCap, kBigSeeds, false>::sm_total) / 4 +
-         (size_t)kMaskSeeds * ((n + 31) / 32);  // candidate masks
-  return (s + 3) & ~(size_t)3;
+// Global scratch bytes per CTA.
+size_t sparse_scratch_bytes(int m, int n, bool big, bool mu) {
+  return with_instance(big, mu, m, n, [&](auto inst) { return scratch_bytes<decltype(inst)>(m, n); });
 }
 
 cudaError_t sparse_config(const DevGraph& g, int order, int* grid_small, int* grid_big) {
@@ -994,45 +1261,31 @@ cudaError_t sparse_config(const DevGraph& g, int order, int* grid_small, int* gr
   if (err != cudaSuccess) return err;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const bool mu = order > 0;
-  const void* fs = mu ? (const void*)lsd_sparse_kernel<kSmallCap, kSmallSeeds, true, false>
-                      : (const void*)lsd_sparse_kernel<kSmallCap, kSmallSeeds, false, false>;
-  const size_t ss = mu ? small_smem<true>() : small_smem<false>();
-  if (ss > (size_t)max_smem) return cudaErrorInvalidValue;
-  err = allow_max_dynamic_smem(fs, max_smem);
-  if (err != cudaSuccess) return err;
-  int per_sm = 0;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fs, kSparseWarps * 32, ss);
-  if (err != cudaSuccess) return err;
-  if (per_sm < 1) return cudaErrorInvalidValue;
-  *grid_small = per_sm * sms;
-  *grid_big = sms * kBigWarpsPerSm;  // each spill warp holds megabytes of global scratch
+  for (const bool big : {false, true}) {
+    err = with_instance(big, order > 0, g.m, g.n, [&](auto inst) {
+      using I = decltype(inst);
+      const void* fn = (const void*)lsd_sparse_kernel<I>;
+      cudaError_t e = allow_max_dynamic_smem(fn, max_smem);
+      if (e != cudaSuccess) return e;
+      int per_sm = 0;
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, I::NT, smem_bytes<I>(g.m, g.n));
+      if (e != cudaSuccess) return e;
+      if (per_sm < 1) return cudaErrorInvalidValue;
+      *(big ? grid_big : grid_small) = per_sm * sms;
+      return cudaSuccess;
+    });
+    if (err != cudaSuccess) return err;
+  }
   return cudaSuccess;
 }
 
-int sparse_warps_small() { return kSparseWarps; }
-
-cudaError_t launch_sparse(const LSDArgs& a, bool big, int grid, int* scratch, size_t stride,
-                          int* spill, unsigned long long* spill_count, const int* items,
-                          const unsigned long long* item_count, cudaStream_t st) {
-  const bool mu = a.order > 0;
-  if (!big) {
-    const size_t smem = mu ? small_smem<true>() : small_smem<false>();
-    if (mu)
-      lsd_sparse_kernel<kSmallCap, kSmallSeeds, true, false><<<grid, kSparseWarps * 32, smem, st>>>(
-          a, scratch, stride, spill, spill_count, items, item_count);
-    else
-      lsd_sparse_kernel<kSmallCap, kSmallSeeds, false, false><<<grid, kSparseWarps * 32, smem, st>>>(
-          a, scratch, stride, spill, spill_count, items, item_count);
-  } else {
-    if (mu)
-      lsd_sparse_kernel<kBigCap, kBigSeeds, true, true><<<grid, 32, 0, st>>>(
-          a, scratch, stride, nullptr, nullptr, items, item_count);
-    else
-      lsd_sparse_kernel<kBigCap, kBigSeeds, false, true><<<grid, 32, 0, st>>>(
-          a, scratch, stride, nullptr, nullptr, items, item_count);
-  }
-  return cudaGetLastError();
+cudaError_t launch_sparse(const LSDArgs& a, bool big, int grid, unsigned char* scratch, size_t stride,
+                          int* spill, const int* items, cudaStream_t st) {
+  return with_instance(big, a.order > 0, a.g.m, a.g.n, [&](auto inst) {
+    using I = decltype(inst);
+    lsd_sparse_kernel<I><<<grid, I::NT, smem_bytes<I>(a.g.m, a.g.n), st>>>(a, scratch, stride, spill, items);
+    return cudaGetLastError();
+  });
 }
 
 }  // namespace lsdgb
