@@ -18,6 +18,7 @@
 //              cluster adds its free faults; a merge ORs the masks; a fault joining a
 //              cluster is cleared.  (When the masks do not fit, a scan over the free faults
 //              with a 32-bit atomicMin per neighbouring cluster replaces them.)
+//   elimination: registers for at most 160 detectors (Elim below), else
 //   R[m][W], T[m][W], pcol[m]: the elimination state of every cluster at once.  A pivot
 //              column is stored at its pivot row d: R[d] is the reduced column (bit d set,
 //              zero at every other pivot row), T[d] the set of pivot rows whose original
@@ -27,12 +28,21 @@
 //   sred[W]    s reduced by the pivots; xsol[W] the pivot rows whose columns XOR to s - sred.
 //              A cluster is valid (Def. 4.2) iff sred has no bit on its rows.
 //
+// What bounds the small classes is instruction fetch (warps at different places of a shot):
+// the elimination in registers, the ranking by a register sort and the loop for the last
+// growing cluster take 10.4 k instructions a BB144 shot instead of 17.5 k, but the launch only
+// gained when the loops over a few items were no longer unrolled (119 -> 59 KB of code; stall
+// for want of instructions 4.0 per issue before).  LSD of 10^6 BB144 shots at p = 0.05 2.58 ->
+// 1.80 ms, of 10^5 with mu = 14 and OSD-CS-4 at p = 0.06 1.42 -> 0.84, OSD-E-6 1.32 -> 0.71,
+// of 10^5 BB288 shots 1.49 -> 0.89, of 10^5 BB72 0.179 -> 0.121 (64 registers: 1.85, 0.90, 0.120).
+//
 // A growth step: every growing cluster takes its lowest-rank candidate, all picks are applied
 // together, clusters that now share a detector (or a fault) are merged, then the new columns
 // are eliminated one by one in rank order: b' = b + sum of R[d] over pivot rows d in supp(b)
 // (one W-word XOR per nonzero of the sparse column), a new pivot at the lowest set bit of
 // b', and back-elimination of that row from the other pivots.  Validity is re-read from sred.
 #include <climits>
+#include <cmath>
 
 #include "lsd_internal.cuh"
 
@@ -67,13 +77,14 @@ struct Lay {
   static constexpr int Wn = (NN + 31) / 32;
   static constexpr int N2 = pow2_at_least(NN);
   static constexpr bool kMasks = (size_t)MM * Wn * 4 <= kMaskBudget;
-  // small classes rank the keys with shuffles and need no sort buffer
-  static constexpr bool kShuffleRank = NN <= 192;
+  // small classes keep the elimination in registers (Elim) and rank the keys by a sort in
+  // registers; they need no R, T and no sort buffer
+  static constexpr bool kReg = W <= 5;
   static constexpr size_t U = 0;
-  static constexpr size_t R = al16(max_sz(kShuffleRank ? 0 : (size_t)N2 * 8,
+  static constexpr size_t R = al16(max_sz(kReg ? (size_t)NN * 4 : (size_t)N2 * 8,
                                           max_sz(kMasks ? (size_t)MM * Wn * 4 : 0, (size_t)NN)));
-  static constexpr size_t T = R + (size_t)MM * W * 4;
-  static constexpr size_t flab = T + (size_t)MM * W * 4;
+  static constexpr size_t T = R + (kReg ? 0 : (size_t)MM * W * 4);
+  static constexpr size_t flab = T + (kReg ? 0 : (size_t)MM * W * 4);
   static constexpr size_t dlab = flab + (size_t)NN * 4;
   static constexpr size_t parent = dlab + (size_t)MM * 4;
   static constexpr size_t best = parent + (size_t)MM * 4;
@@ -108,8 +119,6 @@ struct Graph {
   // the same over (new detector, edge slot) pairs with the largest row degree: lane =
   // dl * D + de, dpass detectors per pass, edges de, de + estep, ... of each
   int dl, de, dpass, estep;
-  // log2 of the column degree rounded up to a power of two (column gathers of add_column)
-  int gshift;
 };
 
 __device__ __forceinline__ void set_lanes(Graph& G, int lane) {
@@ -125,8 +134,6 @@ __device__ __forceinline__ void set_lanes(Graph& G, int lane) {
     G.ppass = 1;
     G.dslots = D;
   }
-  G.gshift = 0;
-  while ((1 << G.gshift) < D) ++G.gshift;
   const int Dr = max(G.max_row_deg, 1);
   if (Dr <= 32) {
     G.dl = lane / Dr;
@@ -204,6 +211,7 @@ template <class L>
 __device__ __forceinline__ void uf_unite(const Shot<L>& S, int a, int b) {
   int* parent = S.parent();
   const volatile int* vp = parent;
+#pragma unroll 1
   for (;;) {
     a = uf_find(vp, a);
     b = uf_find(vp, b);
@@ -250,21 +258,92 @@ __device__ void warp_sort(unsigned long long* keys, int lane) {
   }
 }
 
+// The elimination of every cluster at once, in registers (classes of at most 160 detectors;
+// the larger ones keep R and T in shared memory).  Lane l holds rows l, l + 32, ... of M, the
+// product of the row operations done so far: M h has its only bit at the pivot row for a
+// column h already added.  So M is half of what R and T hold (their bits at rows without and
+// with a pivot), a column's image is one parity per row, and no row is searched for.
+//   s    M times the syndrome; a cluster is valid iff s has no bit on its rows without pivot,
+//        and the columns of the pivot rows with a bit are its solution (piv: rows with pivot)
+template <class L>
+struct Elim {
+  static constexpr int W = L::W;
+  uint32_t row[W][W], s[W], piv[W];
+  __device__ __forceinline__ void init(const Shot<L>& S, int lane) {
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+#pragma unroll
+      for (int w = 0; w < W; ++w) row[j][w] = j == w ? 1u << lane : 0u;
+      s[j] = S.syn()[j];
+      piv[j] = 0u;
+    }
+  }
+  __device__ __forceinline__ bool invalid() const {
+    uint32_t b = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) b |= s[w] & ~piv[w];
+    return b != 0;
+  }
+  // Adds the column with detector words h; its image M h in b.  Returns its pivot row, or -1:
+  // the column depends on the pivot columns of the rows in b.
+  __device__ __forceinline__ int add(const uint32_t (&h)[W], uint32_t (&b)[W], int lane) {
+    bool hit[W];
+    int p = -1;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      uint32_t x = 0;
+#pragma unroll
+      for (int w = 0; w < W; ++w) x ^= row[j][w] & h[w];
+      hit[j] = __popc(x) & 1;
+      b[j] = __ballot_sync(kFull, hit[j]);
+    }
+#pragma unroll
+    for (int j = W - 1; j >= 0; --j)
+      if (b[j] & ~piv[j]) p = 32 * j + __ffs(b[j] & ~piv[j]) - 1;
+    if (p < 0) return p;
+    const int pl = p & 31;
+    bool sp = false;
+    uint32_t pr[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      uint32_t v = row[0][w];
+#pragma unroll
+      for (int j = 1; j < W; ++j)
+        if (j == (p >> 5)) v = row[j][w];
+      pr[w] = __shfl_sync(kFull, v, pl);
+    }
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      const uint32_t pb = j == (p >> 5) ? 1u << pl : 0u;
+      sp = sp || (s[j] & pb) != 0;
+      piv[j] |= pb;
+      if ((pb >> lane) & 1u) hit[j] = false;
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if (hit[j]) row[j][w] ^= pr[w];
+    }
+    if (sp) {
+#pragma unroll
+      for (int j = 0; j < W; ++j) s[j] ^= b[j] & ~(j == (p >> 5) ? 1u << pl : 0u);
+    }
+    return p;
+  }
+};
 // Roots of all clusters, or of the invalid ones, into inv[].  A cluster is invalid iff the
 // reduced syndrome has a bit on one of its rows (labels are flattened, so dlab of a row is
 // its cluster's root); each such root is listed once, in no particular order (growth is
 // synchronous, so the order of the list does not matter).
 template <class L>
-__device__ int collect_roots(const LSDArgs& a, const Shot<L>& S, int m, bool only_invalid,
-                             int lane) {
-  if (only_invalid && L::W <= 4) {
+__device__ __forceinline__ int collect_roots(const LSDArgs& a, const Shot<L>& S, const Elim<L>& E,
+                                             int m, bool only_invalid, int lane) {
+  if (only_invalid && L::kReg) {
     // each invalid row marks its root in a bitmask over labels (cm, free until reprocessing);
     // the roots are then listed in ascending order by ballots, and the mask is cleared
     uint32_t* msk = S.cm();
 #pragma unroll
     for (int i = 0; i < L::W; ++i) {
       const int d = lane + 32 * i;
-      if ((S.sred()[i] >> lane) & 1u) {
+      if (((E.s[i] & ~E.piv[i]) >> lane) & 1u) {
         const int root = S.dlab()[d];
         if (root >= 0) atomicOr(&msk[root >> 5], 1u << (root & 31));
       }
@@ -301,11 +380,13 @@ __device__ int collect_roots(const LSDArgs& a, const Shot<L>& S, int m, bool onl
     }
     __syncwarp();
     const int count = S.scal()[5];
+#pragma unroll 1
     for (int t = lane; t < count; t += 32) S.mark()[S.inv()[t]] = 0u;
     __syncwarp();
     return count;
   }
   int count = 0;
+#pragma unroll 1
   for (int base = 0; base < m; base += 32) {
     const int d = base + lane;
     const bool seed = d < m && (a.single_cluster ? d == 0 : bit_of(S.syn(), d));
@@ -324,29 +405,8 @@ __device__ void add_column(const Graph& G, const Shot<L>& S, int m, int rk, int 
                            int q1, int lane) {
   constexpr int W = L::W;
   uint32_t bw = 0, tw = 0;
-  if ((W << G.gshift) <= 32) {
-    // lane (word wd, detector slot sl) reads one detector's contribution to one word; the
-    // 2^gshift slots of a word are XOR-reduced with shuffles and word w lands on lane w
-    const int wd = lane >> G.gshift, sl = lane & ((1 << G.gshift) - 1);
-    if (wd < W) {
-      const int q = q0 + sl;
-      if (q < q1) {
-        const int d = G.var_chk[q];
-        if ((d >> 5) == wd) bw = 1u << (d & 31);
-        if (S.pcol()[d] >= 0) {
-          bw ^= S.R()[d * W + wd];
-          tw = S.T()[d * W + wd];
-        }
-      }
-    }
-    for (int off = 1; off < (1 << G.gshift); off <<= 1) {
-      bw ^= __shfl_xor_sync(kFull, bw, off);
-      tw ^= __shfl_xor_sync(kFull, tw, off);
-    }
-    bw = __shfl_sync(kFull, bw, (lane << G.gshift) & 31);
-    tw = __shfl_sync(kFull, tw, (lane << G.gshift) & 31);
-    if (lane >= W) bw = tw = 0;
-  } else if (lane < W) {
+  if (lane < W) {
+#pragma unroll 1
     for (int q = q0; q < q1; ++q) {
       const int d = G.var_chk[q];
       if ((d >> 5) == lane) bw ^= 1u << (d & 31);
@@ -384,41 +444,14 @@ __device__ void add_column(const Graph& G, const Shot<L>& S, int m, int rk, int 
   }
   if (lane == 0) S.pcol()[p] = (int16_t)gcol;
   __syncwarp();
-  if constexpr (W <= 4) {
-    // back-elimination with the new pivot's words taken from the lanes that hold them and
-    // every row's test issued before the row updates
-    uint32_t rp[W], tp[W];
+#pragma unroll 1
+  for (int d = lane; d < m; d += 32) {
+    if (d == p || S.pcol()[d] < 0) continue;
+    if (S.R()[d * W + pw] & pb) {
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
-      rp[w] = __shfl_sync(kFull, bw, w);
-      tp[w] = __shfl_sync(kFull, tw, w);
-    }
-    bool hit[W];
-#pragma unroll
-    for (int i = 0; i < W; ++i) {
-      const int d = lane + 32 * i;
-      hit[i] = d < m && d != p && S.pcol()[d] >= 0 && (S.R()[d * W + pw] & pb) != 0;
-    }
-#pragma unroll
-    for (int i = 0; i < W; ++i) {
-      if (hit[i]) {
-        const int d = lane + 32 * i;
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-          S.R()[d * W + w] ^= rp[w];
-          S.T()[d * W + w] ^= tp[w];
-        }
-      }
-    }
-  } else {
-    for (int d = lane; d < m; d += 32) {
-      if (d == p || S.pcol()[d] < 0) continue;
-      if (S.R()[d * W + pw] & pb) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-          S.R()[d * W + w] ^= S.R()[p * W + w];
-          S.T()[d * W + w] ^= S.T()[p * W + w];
-        }
+      for (int w = 0; w < W; ++w) {
+        S.R()[d * W + w] ^= S.R()[p * W + w];
+        S.T()[d * W + w] ^= S.T()[p * W + w];
       }
     }
   }
@@ -429,21 +462,60 @@ __device__ void add_column(const Graph& G, const Shot<L>& S, int m, int rk, int 
   __syncwarp();
 }
 
-// add_column for the fault of rank rk (its column and CSC range read from shared memory).
+// Adds the column of fault g (rank rk, detector words h) to the elimination in registers.
 template <class L, bool MU>
-__device__ __forceinline__ void add_column(const Graph& G, const Shot<L>& S, int m, int rk,
-                                           int lane) {
-  const int gcol = S.fat()[rk];
-  add_column<L, MU>(G, S, m, rk, gcol, G.var_ptr[gcol], G.var_ptr[gcol + 1], lane);
+__device__ __forceinline__ void add_to_elim(const Shot<L>& S, Elim<L>& E, const uint32_t (&h)[L::W],
+                                            int g, int rk, int lane) {
+  uint32_t b[L::W];
+  const int p = E.add(h, b, lane);
+  if (p >= 0) {
+    if (lane == 0) S.pcol()[p] = (int16_t)g;
+  } else if constexpr (MU) {
+    // dependent column: remember its representation for LSD-mu's reprocessing
+    const int slot = __shfl_sync(kFull, S.scal()[1], 0);
+    if (lane == 0) {
+#pragma unroll
+      for (int w = 0; w < L::W; ++w) S.npN()[slot * L::W + w] = b[w];
+      S.npr()[slot] = (uint32_t)rk;
+      S.scal()[1] = slot + 1;
+    }
+    __syncwarp();
+  }
 }
 
-// The growth step of lsd_step when the clusters' candidate masks are kept and at most 32
+// Adds the n_new columns whose ranks are listed in srt[], in that order.
+template <class L, bool MU>
+__device__ __forceinline__ void add_columns(const Graph& G, const Shot<L>& S, Elim<L>& E, int m,
+                                            int n_new, int lane) {
+#pragma unroll 1
+  for (int t = 0; t < n_new; ++t) {
+    const int rk = S.srt()[t];
+    const int g = S.fat()[rk];
+    const int q0 = G.var_ptr[g], q1 = G.var_ptr[g + 1];
+    if constexpr (L::kReg) {
+      uint32_t h[L::W];
+#pragma unroll
+      for (int w = 0; w < L::W; ++w) h[w] = 0u;
+#pragma unroll 1
+      for (int q = q0; q < q1; ++q) {
+        const int d = G.var_chk[q];
+#pragma unroll
+        for (int w = 0; w < L::W; ++w) h[w] |= w == (d >> 5) ? 1u << (d & 31) : 0u;
+      }
+      add_to_elim<L, MU>(S, E, h, g, rk, lane);
+    } else {
+      add_column<L, MU>(G, S, m, rk, g, q0, q1, lane);
+    }
+  }
+}
+
+// The same when the clusters' candidate masks are kept and at most 32
 // clusters grow: lane t carries cluster inv[t]'s pick (rank, fault, CSC range) from the
 // search through the union to the column order, instead of passing it through shared memory.
 // Same result as the general step: the merges, claims and mask updates commute.
-template <class L, bool MU>
-__device__ int lsd_step_small(const Graph& G, const Shot<L>& S, int m, int k, bool strict,
-                              int lane) {
+template <class L>
+__device__ __forceinline__ int lsd_step_small(const Graph& G, const Shot<L>& S, int m, int k,
+                                              bool strict, int lane, int& n_new) {
   constexpr int Wn = L::Wn;
   // ---- find_candidate: the lowest set bit of the cluster's mask ----
   int r = 0;
@@ -459,6 +531,7 @@ __device__ int lsd_step_small(const Graph& G, const Shot<L>& S, int m, int k, bo
       for (int w = Wn - 1; w >= 0; --w)
         if (v[w]) pick = (unsigned)(w * 32 + __ffs(v[w]) - 1);
     } else {
+#pragma unroll 1
       for (int w = 0; w < Wn; ++w) {
         const uint32_t v = c[w];
         if (v) {
@@ -488,13 +561,15 @@ __device__ int lsd_step_small(const Graph& G, const Shot<L>& S, int m, int k, bo
     q1 = G.var_ptr[gcol + 1];
   }
   const unsigned bf = __ballot_sync(kFull, fresh);
-  const int n_new = __popc(bf);
+  n_new = __popc(bf);
   int n_det = 0;
+#pragma unroll 1
   for (int tb = 0; tb < k; tb += G.ppass) {
     const int src = tb + G.pl;
     const int rs = __shfl_sync(kFull, r, src & 31);
     const int qs0 = __shfl_sync(kFull, q0, src & 31);
     const int qs1 = __shfl_sync(kFull, q1, src & 31);
+#pragma unroll 1
     for (int so = 0; so < G.dslots; so += 32) {
       const int q = qs0 + G.ps + so;
       int d = 0;
@@ -514,6 +589,7 @@ __device__ int lsd_step_small(const Graph& G, const Shot<L>& S, int m, int k, bo
   // ---- flatten labels to roots; only after a merge ----
   const int merged = S.scal()[3];
   if (merged) {
+#pragma unroll 1
     for (int x = lane; x < m; x += 32) {
       const int root = uf_find(S.parent(), x);
       S.parent()[x] = root;
@@ -523,17 +599,20 @@ __device__ int lsd_step_small(const Graph& G, const Shot<L>& S, int m, int k, bo
     __syncwarp();
   }
   // ---- masks: fold merged labels into their roots, add the new detectors' free faults ----
+#pragma unroll 1
   for (int idx = lane; idx < merged * Wn; idx += 32) {
     const int x = S.mlist()[idx / Wn], w = idx % Wn;
     const uint32_t v = S.cand()[(size_t)x * Wn + w];
     if (v) atomicOr(&S.cand()[(size_t)S.parent()[x] * Wn + w], v);
   }
+#pragma unroll 1
   for (int tb = 0; tb < n_det; tb += G.dpass) {
     const int t = tb + G.dl;
     if (G.dl < G.dpass && t < n_det) {
       const int d = S.dnew()[t];
       uint32_t* c = S.cand() + (size_t)S.dlab()[d] * Wn;
       const int c1 = G.chk_ptr[d + 1];
+#pragma unroll 1
       for (int e = G.chk_ptr[d] + G.de; e < c1; e += G.estep) {
         const int f = G.chk_var[e];
         if (S.flab()[f] < 0) {
@@ -552,30 +631,30 @@ __device__ int lsd_step_small(const Graph& G, const Shot<L>& S, int m, int k, bo
   __syncwarp();
   // ---- the new columns in rank order: the warp minimum of the fresh picks, n_new times ----
   unsigned kt = fresh ? pick : kNone;
+#pragma unroll 1
   for (int t = 0; t < n_new; ++t) {
     const unsigned v = __reduce_min_sync(kFull, kt);
-    const int src = __ffs(__ballot_sync(kFull, kt == v)) - 1;
     if (kt == v) kt = kNone;
-    add_column<L, MU>(G, S, m, (int)v, __shfl_sync(kFull, gcol, src),
-                      __shfl_sync(kFull, q0, src), __shfl_sync(kFull, q1, src), lane);
+    if (lane == 0) S.srt()[t] = (uint16_t)v;
   }
+  __syncwarp();
   return 0;
 }
 
-// One synchronous growth step of the k clusters listed in inv[].
-// Returns 0 if clusters grew, 1 if strict and a cluster had no candidate, 2 if none grew.
-template <class L, bool MU>
-__device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, bool strict,
-                        int lane) {
+// Picks, merges and masks of a growth step of any number of clusters; the ranks of the new
+// columns go to srt[] in ascending order.
+template <class L>
+__device__ __noinline__ int lsd_step_many(const Graph& G, const Shot<L>& S, int m, int n, int k,
+                                          bool strict, int lane, int* n_new_out) {
   constexpr int Wn = L::Wn;
-  if constexpr (L::kMasks)
-    if (k <= 32) return lsd_step_small<L, MU>(G, S, m, k, strict, lane);
   // ---- find_candidate: the lowest-rank candidate of every growing cluster ----
   if constexpr (L::kMasks) {
+#pragma unroll 1
     for (int t = lane; t < k; t += 32) {
       const int r = S.inv()[t];
       const uint32_t* c = S.cand() + (size_t)r * Wn;
       unsigned pick = kNone;
+#pragma unroll 1
       for (int w = 0; w < Wn; ++w) {
         const uint32_t v = c[w];
         if (v) {
@@ -587,25 +666,30 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
     }
     __syncwarp();
   } else {
+#pragma unroll 1
     for (int t = lane; t < k; t += 32) {
       const int r = S.inv()[t];
       S.best()[r] = kNone;
       S.rflag()[r] = 1;
     }
     __syncwarp();
+#pragma unroll 1
     for (int j = lane; j < n; j += 32) {
       if (S.flab()[j] >= 0) continue;
       const unsigned rk = S.rank()[j];
       const int v1 = G.var_ptr[j + 1];
+#pragma unroll 1
       for (int q = G.var_ptr[j]; q < v1; ++q) {
         const int lab = S.dlab()[G.var_chk[q]];
         if (lab >= 0 && S.rflag()[lab]) atomicMin(&S.best()[lab], rk);
       }
     }
     __syncwarp();
+#pragma unroll 1
     for (int t = lane; t < k; t += 32) S.rflag()[S.inv()[t]] = 0;
   }
   bool none = false, some = false;
+#pragma unroll 1
   for (int t = lane; t < k; t += 32) {
     if (S.best()[S.inv()[t]] == kNone) none = true;
     else some = true;
@@ -622,6 +706,7 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
   // (the lists of new faults and newly claimed detectors are filled by ballots)
   const unsigned below = (1u << lane) - 1u;
   int n_new = 0, n_det = 0;
+#pragma unroll 1
   for (int base = 0; base < k; base += 32) {
     const int t = base + lane;
     const int r = t < k ? S.inv()[t] : 0;
@@ -643,11 +728,13 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
     // the picks' detectors: lane (pick pl, slot ps) claims detector ps of pick tb + pl, so a
     // pass covers ppass picks (the pick's owner lane passes its cluster and column range)
     const int cnt = min(32, k - base);
+#pragma unroll 1
     for (int tb = 0; tb < cnt; tb += G.ppass) {
       const int src = tb + G.pl;
       const int rs = __shfl_sync(kFull, r, src & 31);
       const int qs0 = __shfl_sync(kFull, q0, src & 31);
       const int qs1 = __shfl_sync(kFull, q1, src & 31);
+#pragma unroll 1
       for (int so = 0; so < G.dslots; so += 32) {
         const int q = qs0 + G.ps + so;
         int d = 0;
@@ -668,6 +755,7 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
   // ---- flatten labels to roots (later finds take one step); only after a merge ----
   const int merged = S.scal()[3];
   if (merged) {
+#pragma unroll 1
     for (int x = lane; x < m; x += 32) {
       const int root = uf_find(S.parent(), x);
       S.parent()[x] = root;
@@ -680,18 +768,21 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
     // fold the masks of merged labels into their roots; add the free faults next to the
     // newly claimed detectors
     const int nm = merged, nd = n_det;
+#pragma unroll 1
     for (int idx = lane; idx < nm * Wn; idx += 32) {
       const int x = S.mlist()[idx / Wn], w = idx % Wn;
       const uint32_t v = S.cand()[(size_t)x * Wn + w];
       if (v) atomicOr(&S.cand()[(size_t)S.parent()[x] * Wn + w], v);
     }
     // lanes over (new detector, edge slot) pairs
+#pragma unroll 1
     for (int tb = 0; tb < nd; tb += G.dpass) {
       const int t = tb + G.dl;
       if (G.dl < G.dpass && t < nd) {
         const int d = S.dnew()[t];
         uint32_t* c = S.cand() + (size_t)S.dlab()[d] * Wn;
         const int c1 = G.chk_ptr[d + 1];
+#pragma unroll 1
         for (int e = G.chk_ptr[d] + G.de; e < c1; e += G.estep) {
           const int f = G.chk_var[e];
           if (S.flab()[f] < 0) {
@@ -704,6 +795,7 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
     __syncwarp();
     // the step's new faults are no longer candidates
     const int nn = n_new;
+#pragma unroll 1
     for (int t = lane; t < nn; t += 32) {
       const unsigned rk = S.newr()[t];
       const int root = S.parent()[S.flab()[S.fat()[rk]]];
@@ -712,24 +804,109 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
     __syncwarp();
   }
   // ---- the step's new columns in reliability (rank) order ----
-  if (n_new <= 32) {  // lane t holds new column t; the warp minimum is taken n_new times
-    unsigned kt = lane < n_new ? (unsigned)S.newr()[lane] : kNone;
-    for (int t = 0; t < n_new; ++t) {
-      const unsigned v = __reduce_min_sync(kFull, kt);
-      if (kt == v) kt = kNone;
-      add_column<L, MU>(G, S, m, (int)v, lane);
-    }
-    return 0;
-  }
+#pragma unroll 1
   for (int t = lane; t < n_new; t += 32) {
     const unsigned kt = S.newr()[t];
     int pos = 0;
+#pragma unroll 1
     for (int u = 0; u < n_new; ++u) pos += (S.newr()[u] < kt) ? 1 : 0;
     S.srt()[pos] = (uint16_t)kt;
   }
   __syncwarp();
-  for (int t = 0; t < n_new; ++t) add_column<L, MU>(G, S, m, (int)S.srt()[t], lane);
+  *n_new_out = n_new;
   return 0;
+}
+
+// One synchronous growth step of the k clusters listed in inv[].
+// Returns 0 if clusters grew, 1 if strict and a cluster had no candidate, 2 if none grew.
+template <class L, bool MU>
+__device__ __forceinline__ int lsd_step(const Graph& G, const Shot<L>& S, Elim<L>& E, int m, int n,
+                                        int k, bool strict, int lane) {
+  int n_new = 0, rc;
+  if (L::kMasks && k <= 32) rc = lsd_step_small<L>(G, S, m, k, strict, lane, n_new);
+  else rc = lsd_step_many<L>(G, S, m, n, k, strict, lane, &n_new);
+  if (rc == 0) add_columns<L, MU>(G, S, E, m, n_new, lane);
+  return rc;
+}
+
+// Growth of the only invalid cluster (root r) until it is valid, the bulk of the steps (17 of
+// 19 on BB144 at p = 0.05): lsd_step without lists.  No other cluster grows, so the clusters it
+// meets are absorbed at once and r stays the root, and the whole elimination's validity is the
+// cluster's.  Returns false if the shot is unsolvable.
+template <class L, bool MU>
+__device__ __forceinline__ bool grow_single(const Graph& G, const Shot<L>& S, Elim<L>& E, int m,
+                                            int n, int r, int& steps, int lane) {
+  constexpr int W = L::W, Wn = L::Wn;
+  uint32_t* const c = S.cand() + (size_t)r * Wn;
+#pragma unroll 1
+  do {
+    if (steps > n) return false;  // each step adds a column: cannot be reached
+    const uint32_t v = lane < Wn ? c[lane] : 0u;
+    const unsigned nz = __ballot_sync(kFull, v != 0);
+    if (nz == 0) return false;
+    const int w0 = __ffs(nz) - 1;
+    const uint32_t word = __shfl_sync(kFull, v, w0);
+    const int rk = 32 * w0 + __ffs(word) - 1;
+    const int g = S.fat()[rk];
+    const int q0 = G.var_ptr[g], q1 = G.var_ptr[g + 1];
+    uint32_t h[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) h[w] = 0u;
+    if (lane == 0) S.flab()[g] = r;
+#pragma unroll 1
+    for (int qb = q0; qb < q1; qb += 32) {
+      const bool on = qb + lane < q1;
+      const int d = on ? G.var_chk[qb + lane] : 0;
+      const int lab = on ? S.dlab()[d] : r;
+      const bool free = lab < 0;
+      const unsigned fb = __ballot_sync(kFull, free);
+      unsigned ob = __ballot_sync(kFull, !free && lab != r);
+      if (free) S.dlab()[d] = r;
+#pragma unroll
+      for (int w = 0; w < W; ++w) h[w] |= __reduce_or_sync(kFull, on && (d >> 5) == w ? 1u << (d & 31) : 0u);
+      __syncwarp();
+      while (ob) {  // an absorbed cluster's labels and candidates
+        const int l = __shfl_sync(kFull, lab, __ffs(ob) - 1);
+        ob &= ~__ballot_sync(kFull, lab == l);
+#pragma unroll
+        for (int x0 = 0; x0 < W; ++x0) {
+          const int x = 32 * x0 + lane;
+          if (x < m) {
+            if (S.dlab()[x] == l) S.dlab()[x] = r;
+            if (S.parent()[x] == l) S.parent()[x] = r;
+          }
+        }
+        if (lane < Wn) c[lane] |= S.cand()[(size_t)l * Wn + lane];
+        __syncwarp();
+      }
+      // the free faults next to the newly claimed detectors: lanes over (detector, edge slot)
+      if (fb) {
+        const int nq = min(32, q1 - qb);
+#pragma unroll 1
+        for (int tb = 0; tb < nq; tb += G.dpass) {
+          const int q = tb + G.dl;
+          const int dq = __shfl_sync(kFull, d, q & 31);
+          if (G.dl < G.dpass && q < nq && ((fb >> q) & 1u)) {
+            const int c1 = G.chk_ptr[dq + 1];
+#pragma unroll 1
+            for (int e = G.chk_ptr[dq] + G.de; e < c1; e += G.estep) {
+              const int f = G.chk_var[e];
+              if (S.flab()[f] < 0) {
+                const unsigned fr = S.rank()[f];
+                atomicOr(&c[fr >> 5], 1u << (fr & 31));
+              }
+            }
+          }
+        }
+      }
+    }
+    add_to_elim<L, MU>(S, E, h, g, rk, lane);
+    ++steps;
+    __syncwarp();
+    // the pick is no longer a candidate (it may also have been one of an absorbed cluster)
+    if (lane == w0) c[w0] &= ~(1u << (rk & 31));
+  } while (E.invalid());
+  return true;
 }
 
 // LSD-mu reprocessing (App. D): exhaustive OSD over the first min(mu, #dependent) dependent
@@ -737,12 +914,13 @@ __device__ int lsd_step(const Graph& G, const Shot<L>& S, int m, int n, int k, b
 // weights; ties go to the smaller pattern.  Updates xsol and appends the chosen dependent
 // columns to ext[].
 template <class L>
-__device__ void osd_e(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
+__device__ void osd_e(const LSDArgs& a, const Shot<L>& S, const Elim<L>& E, int m, int lane) {
   constexpr int W = L::W;
   const long long* wfix = a.g.wfix;
   const int order = a.order;
-  const int nroots = collect_roots(a, S, m, false, lane);
+  const int nroots = collect_roots(a, S, E, m, false, lane);
   const int n_np = S.scal()[1];
+#pragma unroll 1
   for (int ci = 0; ci < nroots; ++ci) {
     const int r = S.inv()[ci];
 #pragma unroll
@@ -756,9 +934,11 @@ __device__ void osd_e(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
     int sel[kMaxOrder];
     int nt = 0;
     unsigned last = 0;
+#pragma unroll 1
     for (int it = 0; it < order; ++it) {
       unsigned bk = kNone;
       int bi = -1;
+#pragma unroll 1
       for (int u = lane; u < n_np; u += 32) {
         const unsigned ku = S.npr()[u];
         if (it > 0 && ku <= last) continue;
@@ -768,6 +948,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
           bi = u;
         }
       }
+#pragma unroll 1
       for (int off = 16; off > 0; off >>= 1) {
         const unsigned ok = __shfl_xor_sync(kFull, bk, off);
         const int oi = __shfl_xor_sync(kFull, bi, off);
@@ -783,11 +964,13 @@ __device__ void osd_e(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
     if (nt == 0) continue;
     long long bcost = LLONG_MAX;
     int bt = 0;
+#pragma unroll 1
     for (int t = lane; t < (1 << nt); t += 32) {
       long long cost = 0;
 #pragma unroll
       for (int w = 0; w < W; ++w) {
         uint32_t mw = S.xsol()[w] & S.cm()[w];
+#pragma unroll 1
         for (int k2 = 0; k2 < nt; ++k2)
           if ((t >> k2) & 1) mw ^= S.npN()[sel[k2] * W + w];
         while (mw) {
@@ -796,6 +979,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
           cost += wfix[S.pcol()[w * 32 + b]];
         }
       }
+#pragma unroll 1
       for (int k2 = 0; k2 < nt; ++k2)
         if ((t >> k2) & 1) cost += wfix[S.fat()[S.npr()[sel[k2]]]];
       if (cost < bcost) {
@@ -803,6 +987,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
         bt = t;
       }
     }
+#pragma unroll 1
     for (int off = 16; off > 0; off >>= 1) {
       const long long oc = __shfl_xor_sync(kFull, bcost, off);
       const int ot = __shfl_xor_sync(kFull, bt, off);
@@ -813,12 +998,14 @@ __device__ void osd_e(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
     }
     if (lane < W) {
       uint32_t delta = 0;
+#pragma unroll 1
       for (int k2 = 0; k2 < nt; ++k2)
         if ((bt >> k2) & 1) delta ^= S.npN()[sel[k2] * W + lane];
       S.xsol()[lane] ^= delta;
     }
     if (lane == 0) {
       int ne = S.scal()[2];
+#pragma unroll 1
       for (int k2 = 0; k2 < nt; ++k2)
         if ((bt >> k2) & 1) S.ext()[ne++] = S.fat()[S.npr()[sel[k2]]];
       S.scal()[2] = ne;
@@ -857,11 +1044,12 @@ __device__ __forceinline__ long long pattern_cost(const LSDArgs& a, const Shot<L
 // earlier pattern in that order.  A pattern is ranked by (cost, class, key): class 0 = no
 // flip, 1 = single (key = the column's rank), 2 = pair (key = i * 16 + j).
 template <class L>
-__device__ void osd_cs(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
+__device__ void osd_cs(const LSDArgs& a, const Shot<L>& S, const Elim<L>& E, int m, int lane) {
   constexpr int W = L::W;
-  const int nroots = collect_roots(a, S, m, false, lane);
+  const int nroots = collect_roots(a, S, E, m, false, lane);
   const int n_np = S.scal()[1];
   const int w_cs = a.osd_cs;
+#pragma unroll 1
   for (int ci = 0; ci < nroots; ++ci) {
     const int r = S.inv()[ci];
 #pragma unroll
@@ -876,9 +1064,11 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
     int sel[kMaxCsOrder];
     int nt = 0;
     unsigned last = 0;
+#pragma unroll 1
     for (int it = 0; it < w_cs; ++it) {
       unsigned bk = kNone;
       int bi = -1;
+#pragma unroll 1
       for (int u = lane; u < n_np; u += 32) {
         const unsigned ku = S.npr()[u];
         if (it > 0 && ku <= last) continue;
@@ -888,6 +1078,7 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
           bi = u;
         }
       }
+#pragma unroll 1
       for (int off = 16; off > 0; off >>= 1) {
         const unsigned ok = __shfl_xor_sync(kFull, bk, off);
         const int oi = __shfl_xor_sync(kFull, bi, off);
@@ -912,12 +1103,14 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
       }
     };
     if (lane == 0) consider(pattern_cost(a, S, -1, -1), 0, 0, -1, -1);
+#pragma unroll 1
     for (int u = lane; u < n_np; u += 32) {
       const unsigned ku = S.npr()[u];
       if (S.parent()[S.flab()[S.fat()[ku]]] != r) continue;
       consider(pattern_cost(a, S, u, -1), 1, (int)ku, u, -1);
     }
     const int npairs = nt * (nt - 1) / 2;
+#pragma unroll 1
     for (int t = lane; t < npairs; t += 32) {
       int i = 0, rem = t;
       while (rem >= nt - 1 - i) {
@@ -927,6 +1120,7 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<L>& S, int m, int lane) {
       const int j = i + 1 + rem;
       consider(pattern_cost(a, S, sel[i], sel[j]), 2, i * 16 + j, sel[i], sel[j]);
     }
+#pragma unroll 1
     for (int off = 16; off > 0; off >>= 1) {
       const long long oc = __shfl_xor_sync(kFull, bc, off);
       const int ocls = __shfl_xor_sync(kFull, bcls, off);
@@ -966,6 +1160,146 @@ __device__ __forceinline__ void lsd_flush(const LSDArgs& a, const LsdAcc& acc, i
   }
 }
 
+// The solution of the elimination in registers into xsol, for the reprocessing and the output.
+template <class L>
+__device__ __forceinline__ void store_solution(const Shot<L>& S, const Elim<L>& E, int lane) {
+  if (lane == 0) {
+#pragma unroll
+    for (int w = 0; w < L::W; ++w) S.xsol()[w] = E.s[w] & E.piv[w];
+  }
+  __syncwarp();
+}
+
+// Exact order by counting, for the keys that rank_by_sort's 32 bits do not tell apart.
+template <class L>
+__device__ __noinline__ void rank_by_counting(const Shot<L>& S, const uint32_t* bits, int n, int lane) {
+#pragma unroll 1
+  for (int j = lane; j < n; j += 32) {
+    const uint32_t mine = bits[j];
+    int rk = 0;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) rk += bits[i] < mine || (bits[i] == mine && i < j) ? 1 : 0;
+    S.rank()[j] = (uint16_t)rk;
+    S.fat()[rk] = (uint16_t)j;
+  }
+}
+
+// rank[] and fat[] of the shot's LLRs: a bitonic sort in registers (position = lane KP + t, so
+// that the small strides stay in a lane) of 32-bit words holding the LLR's place between the
+// shot's least and greatest (a monotone map: equal places only for neighbours) and the fault
+// index.  The order is then checked against the exact keys (LLR bits, index); neighbours that
+// share a place in the wrong order send the shot to the exact count.  About 650 instructions
+// for BB144 against 1800 for counting with shuffles; for BB288 it replaces a 64-bit sort in
+// shared memory, a quarter of its launch.
+template <class L>
+__device__ __forceinline__ void rank_by_sort(const Shot<L>& S, const float* lsrc, int n, int lane) {
+  constexpr int NN = 32 * L::Wn;
+  constexpr int KP = NN <= 128 ? 4 : NN <= 256 ? 8 : 16;
+  constexpr int IB = NN <= 256 ? 8 : 9;  // index bits
+  static_assert(NN <= 32 * KP && NN <= (1 << IB), "every fault has a place");
+  uint32_t* const bits = S.template at<uint32_t>(L::U);
+  float x[KP];
+  float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+  for (int t = 0; t < KP; ++t) {
+    const int j = lane + 32 * t;
+    x[t] = 0.f;
+    if (32 * t < NN && j < n) {
+      x[t] = lsrc[j];
+      bits[j] = llr_bits(x[t]);
+      lo = fminf(lo, x[t]);
+      hi = fmaxf(hi, x[t]);
+    }
+  }
+#pragma unroll 1
+  for (int off = 16; off > 0; off >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(kFull, lo, off));
+    hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, off));
+  }
+  constexpr float kPlaces = (float)((1u << (32 - IB)) - 8);
+  const float scale = kPlaces / fmaxf(hi - lo, 1e-30f);
+  uint32_t v[KP];
+#pragma unroll
+  for (int t = 0; t < KP; ++t) {
+    const int j = lane + 32 * t;
+    const uint32_t place = min((uint32_t)fmaxf((x[t] - lo) * scale, 0.f), (1u << (32 - IB)) - 2);
+    v[t] = 32 * t < NN && j < n ? place << IB | (uint32_t)j : 0xffffffffu;
+  }
+  // runs within a lane, in alternating directions (flip: descending as ascending complements)
+  auto in_lane = [&](int s) {
+#pragma unroll
+    for (int t = 0; t < KP; ++t) {
+      if (t & s) continue;
+      const uint32_t lo_v = min(v[t], v[t + s]);
+      v[t + s] = max(v[t], v[t + s]);
+      v[t] = lo_v;
+    }
+  };
+  auto flip = [&](int k) {  // positions whose run of k descends
+#pragma unroll
+    for (int t = 0; t < KP; ++t)
+      if (k < KP ? (t & k) != 0 : (lane & (k / KP)) != 0) v[t] = ~v[t];
+  };
+#pragma unroll
+  for (int k = 2; k <= KP; k <<= 1) {
+    flip(k);
+#pragma unroll
+    for (int s = k >> 1; s > 0; s >>= 1) in_lane(s);
+    flip(k);
+  }
+  // longer runs: strides across lanes, then within; rolled, since the launch is short of
+  // instruction fetch, not of issue slots
+#pragma unroll 1
+  for (int kl = 2; kl <= 32; kl <<= 1) {
+    const uint32_t fm = kl < 32 && (lane & kl) ? 0xffffffffu : 0u;
+#pragma unroll
+    for (int t = 0; t < KP; ++t) v[t] ^= fm;
+#pragma unroll 1
+    for (int sl = kl >> 1; sl > 0; sl >>= 1) {
+      const bool low = (lane & sl) == 0;
+#pragma unroll
+      for (int t = 0; t < KP; ++t) {
+        const uint32_t o = __shfl_xor_sync(kFull, v[t], sl);
+        v[t] = low ? min(v[t], o) : max(v[t], o);
+      }
+    }
+#pragma unroll
+    for (int s = KP >> 1; s > 0; s >>= 1) in_lane(s);
+#pragma unroll
+    for (int t = 0; t < KP; ++t) v[t] ^= fm;
+  }
+  __syncwarp();
+  // neighbours in place: exact keys ascending?
+  bool bad = false;
+  uint32_t kb[KP];
+#pragma unroll
+  for (int t = 0; t < KP; ++t) {
+    const int r = lane * KP + t;
+    kb[t] = r < n ? bits[v[t] & ((1u << IB) - 1)] : 0xffffffffu;
+  }
+  const uint32_t nk = __shfl_down_sync(kFull, kb[0], 1), nv = __shfl_down_sync(kFull, v[0], 1);
+#pragma unroll
+  for (int t = 0; t < KP; ++t) {
+    const uint32_t k1 = t + 1 < KP ? kb[t + 1 < KP ? t + 1 : t] : nk;
+    const uint32_t v1 = t + 1 < KP ? v[t + 1 < KP ? t + 1 : t] : nv;
+    const uint32_t j0 = v[t] & ((1u << IB) - 1), j1 = v1 & ((1u << IB) - 1);
+    if (lane * KP + t + 1 < n) bad |= kb[t] > k1 || (kb[t] == k1 && j0 > j1);
+  }
+  if (__any_sync(kFull, bad)) {
+    rank_by_counting<L>(S, bits, n, lane);
+    return;
+  }
+#pragma unroll
+  for (int t = 0; t < KP; ++t) {
+    const int r = lane * KP + t;
+    if (r < n) {
+      const uint32_t j = v[t] & ((1u << IB) - 1);
+      S.fat()[r] = (uint16_t)j;
+      S.rank()[j] = (uint16_t)r;
+    }
+  }
+}
+
 // LSD (Alg. 1, LSD-mu of App. D) of one shot by one warp: lsrc = the shot's soft
 // information (global or shared memory), ssrc = its syndrome; writes its correction and
 // status.
@@ -978,42 +1312,8 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
   constexpr int W = L::W, Wn = L::Wn, N2 = L::N2;
   const int m = a.g.m, n = a.g.n;
   // ---- the shot's reliability order ----
-  if constexpr (L::kShuffleRank) {
-    // rank of fault j = number of keys (bits', j') before (bits, j), counted with shuffles
-    // of the 32-bit LLR bits; the index tie-break is known from the positions: fault
-    // j' = src + 32 t2 precedes j = lane + 32 t on equal bits iff t2 < t, or t2 == t and
-    // src < lane.  Padding entries (j >= n) carry the largest bits and the largest index.
-    constexpr int KPL = (NN + 31) / 32;
-    unsigned myk[KPL];
-    int rk[KPL];
-#pragma unroll
-    for (int t = 0; t < KPL; ++t) {
-      const int j = lane + 32 * t;
-      myk[t] = j < n ? llr_bits(lsrc[j]) : 0xffffffffu;
-      rk[t] = 0;
-    }
-#pragma unroll 1
-    for (int src = 0; src < 32; ++src) {
-      const bool before = src < lane;
-#pragma unroll
-      for (int t2 = 0; t2 < KPL; ++t2) {
-        const unsigned other = __shfl_sync(kFull, myk[t2], src);
-#pragma unroll
-        for (int t = 0; t < KPL; ++t) {
-          if (t2 < t) rk[t] += (other <= myk[t]) ? 1 : 0;
-          else if (t2 > t) rk[t] += (other < myk[t]) ? 1 : 0;
-          else rk[t] += (other < myk[t] || (before && other == myk[t])) ? 1 : 0;
-        }
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < KPL; ++t) {
-      const int j = lane + 32 * t;
-      if (j < n) {
-        S.rank()[j] = (uint16_t)rk[t];
-        S.fat()[rk[t]] = (uint16_t)j;
-      }
-    }
+  if constexpr (L::kReg) {
+    rank_by_sort<L>(S, lsrc, n, lane);
   } else {
 #pragma unroll
     for (int j0 = 0; j0 < N2; j0 += 32) {
@@ -1022,6 +1322,7 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
     }
     __syncwarp();
     warp_sort<N2>(S.keys(), lane);
+#pragma unroll 1
     for (int r = lane; r < n; r += 32) {
       const int j = (int)(S.keys()[r] & 0xffffffffu);
       S.fat()[r] = (uint16_t)j;
@@ -1035,7 +1336,9 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
   // clears its mask below; the single cluster's mask is cleared here)
   if constexpr (L::kMasks)
     if (a.single_cluster && lane < Wn) S.cand()[lane] = 0;
+#pragma unroll 1
   for (int j = lane; j < n; j += 32) S.flab()[j] = -1;
+#pragma unroll 1
   for (int d = lane; d < m; d += 32) {
     S.dlab()[d] = -1;
     S.parent()[d] = d;
@@ -1065,8 +1368,10 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
   __syncwarp();
   int k = 0;
   if (a.single_cluster) {
+#pragma unroll 1
     for (int d = lane; d < m; d += 32) S.dlab()[d] = 0;
     if constexpr (L::kMasks) {
+#pragma unroll 1
       for (int r = lane; r < n; r += 32) {
         const int j = S.fat()[r];
         if (G.var_ptr[j + 1] > G.var_ptr[j]) atomicOr(&S.cand()[r >> 5], 1u << (r & 31));
@@ -1078,6 +1383,7 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
     k = anys ? 1 : 0;
     if (lane == 0) S.inv()[0] = 0;
   } else {
+#pragma unroll 1
     for (int b0 = 0; b0 < m; b0 += 32) {
       const int d = b0 + lane;
       const bool f = d < m && bit_of(S.syn(), d);
@@ -1090,6 +1396,7 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
 #pragma unroll
           for (int w = 0; w < Wn; ++w) c[w] = 0;
           const int c1 = G.chk_ptr[d + 1];
+#pragma unroll 1
           for (int e = G.chk_ptr[d]; e < c1; ++e) {
             const unsigned rk = S.rank()[G.chk_var[e]];
             c[rk >> 5] |= 1u << (rk & 31);
@@ -1101,6 +1408,8 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
   }
   __syncwarp();
 
+  Elim<L> E;
+  if constexpr (L::kReg) E.init(S, lane);
   // ---- LSD-0: grow every invalid cluster until all are valid ----
   int status = LSD_SHOT_OK_LSD, steps = 0;
   while (k > 0) {
@@ -1108,36 +1417,48 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
       status = LSD_SHOT_UNSOLVABLE;
       break;
     }
-    if (lsd_step<L, MU>(G, S, m, n, k, true, lane) == 1) {
+    if constexpr (L::kReg && L::kMasks) {
+      if (k == 1) {
+        if (!grow_single<L, MU>(G, S, E, m, n, S.inv()[0], steps, lane)) status = LSD_SHOT_UNSOLVABLE;
+        break;
+      }
+    }
+    if (lsd_step<L, MU>(G, S, E, m, n, k, true, lane) == 1) {
       status = LSD_SHOT_UNSOLVABLE;
       break;
     }
     ++steps;
-    k = collect_roots(a, S, m, true, lane);
+    k = collect_roots(a, S, E, m, true, lane);
   }
   // ---- LSD-mu: mu more steps for every cluster, then local OSD-E ----
   if constexpr (MU) {
     if (status == LSD_SHOT_OK_LSD) {
+#pragma unroll 1
       for (int e = 0; e < a.order; ++e) {
-        k = collect_roots(a, S, m, false, lane);
-        if (lsd_step<L, MU>(G, S, m, n, k, false, lane) == 2) break;
+        k = collect_roots(a, S, E, m, false, lane);
+        if (lsd_step<L, MU>(G, S, E, m, n, k, false, lane) == 2) break;
       }
+      if constexpr (L::kReg) store_solution(S, E, lane);
       if (a.osd_cs >= 0)
-        osd_cs(a, S, m, lane);
+        osd_cs(a, S, E, m, lane);
       else
-        osd_e(a, S, m, lane);
+        osd_e(a, S, E, m, lane);
     }
   }
 
+  if constexpr (L::kReg && !MU) store_solution(S, E, lane);
   // ---- statistics: nu clusters, kappa = largest cluster in columns ----
+#pragma unroll 1
   for (int d = lane; d < m; d += 32) S.best()[d] = 0;
   __syncwarp();
+#pragma unroll 1
   for (int j = lane; j < n; j += 32) {
     const int lab = S.flab()[j];
     if (lab >= 0) atomicAdd(&S.best()[S.parent()[lab]], 1u);
   }
   __syncwarp();
   int nu = 0, kappa = 0;
+#pragma unroll 1
   for (int d = lane; d < m; d += 32) {
     const bool seed = a.single_cluster ? d == 0 : bit_of(S.syn(), d);
     if (seed && S.parent()[d] == d) {
@@ -1145,6 +1466,7 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
       kappa = max(kappa, (int)S.best()[d]);
     }
   }
+#pragma unroll 1
   for (int off = 16; off > 0; off >>= 1) {
     nu += __shfl_xor_sync(kFull, nu, off);
     kappa = max(kappa, __shfl_xor_sync(kFull, kappa, off));
@@ -1152,19 +1474,23 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
 
   // ---- global decoding: union of the local solutions (Eq. 2) ----
   uint8_t* cs = S.cs();  // the masks are no longer needed
+#pragma unroll 1
   for (int j = lane; j < n; j += 32) cs[j] = 0;
   __syncwarp();
   if (status == LSD_SHOT_OK_LSD) {
+#pragma unroll 1
     for (int d = lane; d < m; d += 32)
       if (bit_of(S.xsol(), d)) cs[S.pcol()[d]] = 1;
     if constexpr (MU) {
       const int ne = S.scal()[2];
+#pragma unroll 1
       for (int t = lane; t < ne; t += 32) cs[S.ext()[t]] = 1;
     }
   }
   __syncwarp();
   if constexpr (PK) {
     uint32_t* co = reinterpret_cast<uint32_t*>(a.corrections) + shot * packed_words(n);
+#pragma unroll 1
     for (int base = 0; base < n; base += 32) {  // one ballot per word
       const int j = base + lane;
       const unsigned b = __ballot_sync(kFull, j < n && cs[j] != 0);
@@ -1172,6 +1498,7 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
     }
   } else {
     uint8_t* co = a.corrections + shot * n;
+#pragma unroll 1
     for (int j = lane; j < n; j += 32) co[j] = cs[j];
   }
   if (lane == 0) {
@@ -1190,7 +1517,8 @@ __device__ __forceinline__ void lsd_shot(const LSDArgs& a, const Graph& G,
 }
 
 template <int MM, int NN, bool MU, bool PK>
-__global__ void __launch_bounds__(256, MU ? 3 : 4) lsd_kernel(LSDArgs a, int graph_smem) {
+__global__ void __launch_bounds__(256, MU && MM > 96 && MM <= 160 ? 2 : 3)
+lsd_kernel(LSDArgs a, int graph_smem) {
   using L = Lay<MM, NN, MU>;
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1202,8 +1530,11 @@ __global__ void __launch_bounds__(256, MU ? 3 : 4) lsd_kernel(LSDArgs a, int gra
     int32_t* vp = cp + (m + 1);
     uint16_t* cv = reinterpret_cast<uint16_t*>(vp + (n + 1));
     uint16_t* vc = cv + E;
+#pragma unroll 1
     for (int i = threadIdx.x; i <= m; i += blockDim.x) cp[i] = a.g.chk_ptr[i];
+#pragma unroll 1
     for (int j = threadIdx.x; j <= n; j += blockDim.x) vp[j] = a.g.var_ptr[j];
+#pragma unroll 1
     for (int e = threadIdx.x; e < E; e += blockDim.x) {
       cv[e] = a.g.chk_var[e];
       vc[e] = a.g.var_chk[e];
@@ -1231,6 +1562,7 @@ __global__ void __launch_bounds__(256, MU ? 3 : 4) lsd_kernel(LSDArgs a, int gra
   // atomic's result only after the shot), hiding the atomic's round trip
   unsigned long long pending = 0;
   if (lane == 0) pending = atomicAdd(&a.ctr->lsd_next, 1ULL);
+#pragma unroll 1
   for (;;) {
     const unsigned long long item = __shfl_sync(kFull, pending, 0);
     if (item >= (unsigned long long)count) break;
@@ -1256,6 +1588,7 @@ constexpr SizeClass kClasses[] = {{40, 80}, {72, 144}, {96, 192}, {144, 288}, {2
 constexpr int kNumClasses = sizeof(kClasses) / sizeof(kClasses[0]);
 
 int size_class(int m, int n) {
+#pragma unroll 1
   for (int c = 0; c < kNumClasses; ++c)
     if (m <= kClasses[c].mm && n <= kClasses[c].nn) return c;
   return -1;

@@ -195,6 +195,7 @@ __device__ __forceinline__ int uf_find(const volatile uint16_t* parent, int x) {
 template <class I>
 __device__ __forceinline__ void uf_unite(const Shot<I>& S, int a, int b) {
   const volatile uint16_t* vp = S.parent();
+#pragma unroll 1
   for (;;) {
     a = uf_find(vp, a);
     b = uf_find(vp, b);
@@ -246,6 +247,7 @@ __device__ __forceinline__ void each_det(const SGraph& G, uint2 v, int f, F&& fn
   }
   if (G.max_col_deg > 4) {
     const int v1 = G.var_ptr[f + 1];
+#pragma unroll 1
     for (int q = G.var_ptr[f] + 4; q < v1; ++q) fn((int)G.var_chk[q]);
   }
 }
@@ -255,7 +257,9 @@ __device__ __forceinline__ void each_det(const SGraph& G, uint2 v, int f, F&& fn
 template <class I>
 __device__ __forceinline__ void open_rows(const Shot<I>& S, int from, int to, int tid) {
   const int w0 = (from + 31) >> 5, w1 = (to + 31) >> 5;
+#pragma unroll 1
   for (int i = tid; i < to; i += I::NT)
+#pragma unroll 1
     for (int w = i < from ? w0 : 0; w < w1; ++w)
       S.M()[(size_t)w * I::CAP + i] = (i >> 5) == w && i >= from ? 1u << (i & 31) : 0u;
 }
@@ -286,6 +290,7 @@ __device__ __forceinline__ void open_slots(const SGraph& G, const Shot<I>& S, co
                                            int from, int to, int tid) {
   open_rows(S, from, to, tid);
   const int D = G.max_row_deg;
+#pragma unroll 1
   for (int x = tid; x < (to - from) * D; x += I::NT) {
     const int f = G.chk_pad[(size_t)S.sdet()[from + x / D] * D + x % D];
     unsigned k;
@@ -316,12 +321,15 @@ __device__ __forceinline__ uint32_t column_image(const SGraph& G, const Shot<I>&
   }
   if (G.max_col_deg > 4) {
     const int v1 = G.var_ptr[g + 1];
+#pragma unroll 1
     for (int q = G.var_ptr[g] + 4; q < v1; ++q) {
       const uint32_t s = S.lab[G.var_chk[q]] & 0xffffu;
+#pragma unroll 1
       for (int j = 0; tid + NT * j < nsl; ++j)
         hit ^= ((S.M()[(size_t)(s >> 5) * CAP + tid + NT * j] >> (s & 31)) & 1u) << j;
     }
   }
+#pragma unroll 1
   for (uint32_t h = hit; h; h &= h - 1) {
     const int i = tid + NT * (__ffs(h) - 1);
     if (!(S.flags()[i] & 2)) pc = i;
@@ -343,6 +351,7 @@ __device__ __forceinline__ void pivot_update(const Shot<I>& S, int p, int g, uin
   }
   const bool sp = S.flags()[p] & 1;
   if (!__any_sync(kFull, hit != 0)) return;
+#pragma unroll 1
   for (int c0 = 0; c0 < wc; c0 += 32) {
     const uint32_t v = c0 + lane < wc ? S.M()[(size_t)(c0 + lane) * CAP + p] : 0u;
     unsigned nz = __ballot_sync(kFull, v != 0);
@@ -357,6 +366,7 @@ __device__ __forceinline__ void pivot_update(const Shot<I>& S, int p, int g, uin
     }
   }
   if (sp)
+#pragma unroll 1
     for (uint32_t h = hit; h; h &= h - 1) S.flags()[tid + NT * (__ffs(h) - 1)] ^= 1;
 }
 
@@ -387,9 +397,11 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
   const int ncr = S.sc->ncr, wc = (nsl + 31) >> 5;
   uint16_t* const rows = S.template s<uint16_t>(I::rows) + warp * 32;
   uint32_t* const M = S.M();
+#pragma unroll 1
   for (int c = warp; c < ncr; c += I::NW) {
     const int r = S.inv()[c];
     int cnt = 0;
+#pragma unroll 1
     for (int b0 = 0; b0 < nsl; b0 += 32) {
       const bool in = b0 + lane < nsl && S.slab()[b0 + lane] == r;
       const unsigned b = __ballot_sync(kFull, in);
@@ -401,6 +413,7 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
     __syncwarp();
     const bool mine = lane < cnt;
     const int i = mine ? rows[lane] : 0;
+#pragma unroll 1
     for (int t0 = 0; t0 < n_new; t0 += 32) {
       unsigned todo = __ballot_sync(kFull, t0 + lane < n_new && S.sroot()[t0 + lane] == r);
       while (todo) {
@@ -426,6 +439,7 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
               continue;
             }
             uint32_t* const row = S.npN() + (size_t)k * I::W;
+#pragma unroll 1
             for (int w = lane; w < I::W; w += 32) row[w] = 0u;
             __syncwarp();
             if (hit) atomicOr(row + (i >> 5), 1u << (i & 31));
@@ -443,6 +457,7 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
           S.pcol()[p] = (uint16_t)g;
         }
         if (__any_sync(kFull, hit)) {
+#pragma unroll 1
           for (int c0 = 0; c0 < wc; c0 += 32) {
             const uint32_t v = c0 + lane < wc ? M[(size_t)(c0 + lane) * CAP + p] : 0u;
             unsigned nz = __ballot_sync(kFull, v != 0);
@@ -473,6 +488,7 @@ __device__ __forceinline__ void add_columns(const SGraph& G, const Shot<I>& S, i
     __syncthreads();
   }
   int np = S.sc->np, done = 0;
+#pragma unroll 1
   for (int t = 0; t < n_new; ++t) {
     if (by_warp) {
       const int r = S.sroot()[t];
@@ -492,6 +508,7 @@ __device__ __forceinline__ void add_columns(const SGraph& G, const Shot<I>& S, i
   }
   __syncthreads();
   if (by_warp)
+#pragma unroll 1
     for (int c = tid; c < S.sc->ncr; c += I::NT) {
       const int r = S.inv()[c];
       atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
@@ -504,6 +521,7 @@ __device__ __forceinline__ void add_columns(const SGraph& G, const Shot<I>& S, i
 template <class I>
 __device__ __forceinline__ int collect(const Shot<I>& S, int nsl, bool only_invalid, int tid) {
   if (only_invalid) {
+#pragma unroll 1
     for (int i = tid; i < nsl; i += I::NT) {
       if ((S.flags()[i] & 3) != 1) continue;
       const int r = S.slab()[i];
@@ -512,6 +530,7 @@ __device__ __forceinline__ int collect(const Shot<I>& S, int nsl, bool only_inva
     }
   } else {
     const int ns = S.sc->ns;
+#pragma unroll 1
     for (int r = tid; r < ns; r += I::NT) {
       if (S.parent()[r] != r) continue;
       atomicOr(&S.growb()[r >> 5], 1u << (r & 31));
@@ -532,13 +551,16 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
   const int nf = sc.nf, nsl0 = sc.nsl;
   // ---- find_candidate: the least LLR bits of every growing cluster, then the least fault
   // that has them ----
+#pragma unroll 1
   for (int t = tid; t < k; t += NT) {
     const int r = S.inv()[t];
     S.best()[r] = kNoKey;
     S.bidx()[r] = kNoKey;
   }
   __syncthreads();
+#pragma unroll 1
   for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
     for (int x = tid; x < nf; x += NT) {
       const int f = S.lf[x];
       if ((S.joined[f >> 5] >> (f & 31)) & 1u) continue;
@@ -558,6 +580,7 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
     __syncthreads();
   }
   bool some = false, none = false;
+#pragma unroll 1
   for (int t = tid; t < k; t += NT) {
     const bool has = S.bidx()[S.inv()[t]] != kNoKey;
     some |= has;
@@ -567,6 +590,7 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
   some = __syncthreads_or(some);
   const bool stop = (strict && none) || !some;
   // ---- every pick joins its cluster and claims its detectors; clusters that meet merge ----
+#pragma unroll 1
   for (int t = tid; t < k; t += NT) {
     const int r = S.inv()[t];
     atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
@@ -589,8 +613,10 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
   // ---- labels to roots after a merge ----
   if (sc.merged) {
     const int ns = sc.ns;
+#pragma unroll 1
     for (int x = tid; x < ns; x += NT) S.parent()[x] = (uint16_t)uf_find(S.parent(), x);
     __syncthreads();
+#pragma unroll 1
     for (int i = tid; i < nsl; i += NT) {
       const int r = S.parent()[S.slab()[i]];
       S.slab()[i] = (uint16_t)r;
@@ -600,9 +626,11 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
   }
   open_slots(G, S, llr, nsl0, nsl, tid);
   // ---- the new columns in key order, with their clusters and the slots of their detectors ----
+#pragma unroll 1
   for (int t = tid; t < n_new; t += NT) {
     const unsigned long long kt = S.newk()[t];
     int pos = 0;
+#pragma unroll 1
     for (int u = 0; u < n_new; ++u) pos += S.newk()[u] < kt ? 1 : 0;
     const int g = (int)(kt & 0xffffffffu);
     S.sg()[pos] = (uint16_t)g;
@@ -627,6 +655,7 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
   add_columns(G, S, n_new, nsl, tid);
   if (I::MU && sc.ovf) return 3;
   if (n_new > 1 && G.max_col_deg > 4) {  // (the marks of the clusters with columns, unused there)
+#pragma unroll 1
     for (int c = tid; c < sc.ncr; c += NT) {
       const int r = S.inv()[c];
       atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
@@ -651,6 +680,7 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
   const int D = G.max_row_deg;
   unsigned bk, bx;  // the thread's best entry: LLR bits, then fault << 16 | entry
   auto scan = [&] {
+#pragma unroll 1
     for (int x = tid; x < nf; x += NT) {
       const unsigned key = S.lk[x];
       if (key > bk) continue;
@@ -696,6 +726,7 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
   }
   __syncthreads();
   fetch();
+#pragma unroll 1
   for (int it = 0;; ++it) {
     if (bx == kNoKey) return 1;
     if (steps > n) return 1;  // each step adds a column: cannot be reached
@@ -746,6 +777,7 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
     if ((ml.x & ml.y) != kFull) {
       // ---- absorbed clusters take the label r ----
       const uint32_t m0 = ml.x & 0xffffu, m1 = ml.x >> 16, m2 = ml.y & 0xffffu, m3 = ml.y >> 16;
+#pragma unroll 1
       for (int i = tid; i < nsl0; i += NT) {
         const uint32_t y = S.slab()[i];
         if (y == m0 || y == m1 || y == m2 || y == m3) {
@@ -768,6 +800,7 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
       }
     };
     if (near != kNone16 && ((fresh >> q0) & 1u)) admit(near);
+#pragma unroll 1
     for (int x = NT - kFrom + tid; x < 4 * D; x += NT)  // pairs beyond the CTA's threads
       if ((fresh >> (x / D)) & 1u) {
         const int f = G.chk_pad[(size_t)half4(dets, x / D) * D + x % D];
@@ -789,6 +822,7 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
     if (p < 0) keep_dependent(S, np, g, hit, tid);
     else pivot_update(S, p, g, hit, nsl, tid);
     bool bad = false;
+#pragma unroll 1
     for (int i = tid; i < nsl; i += NT) bad |= (S.flags()[i] & 3) == 1;
     ++steps;
     if (!__syncthreads_or(bad)) break;
@@ -813,9 +847,11 @@ __device__ int first_dependent(const Shot<I>& S, int r, int np, int want, int la
   int mine = -1;
   unsigned long long last = 0;
   int nt = 0;
+#pragma unroll 1
   for (int it = 0; it < want; ++it) {
     unsigned long long bk = ~0ull;
     int bi = -1;
+#pragma unroll 1
     for (int u = lane; u < np; u += 32) {
       if (S.dpr()[u] != r) continue;
       const unsigned long long ku = dep_key(S, u);
@@ -823,6 +859,7 @@ __device__ int first_dependent(const Shot<I>& S, int r, int np, int want, int la
       bk = ku;
       bi = u;
     }
+#pragma unroll 1
     for (int off = 16; off > 0; off >>= 1) {
       const unsigned long long ok = __shfl_xor_sync(kFull, bk, off);
       const int oi = __shfl_xor_sync(kFull, bi, off);
@@ -843,6 +880,7 @@ __device__ int first_dependent(const Shot<I>& S, int r, int np, int want, int la
 // Words of the local solution of every row (bit = the row's pivot column is in it).
 template <class I>
 __device__ void solution_words(const Shot<I>& S, uint32_t* xw, int nsl, int lane) {
+#pragma unroll 1
   for (int c = 0; 32 * c < nsl; ++c) {
     const int i = 32 * c + lane;
     const unsigned b = __ballot_sync(kFull, i < nsl && (S.flags()[i] & 3) == 3);
@@ -863,9 +901,11 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
   const int mine = first_dependent(S, r, np, a.order, lane, nt);
   if (nt == 0) return;
   solution_words(S, xw, nsl, lane);
+#pragma unroll 1
   for (int w0 = 0; w0 < wc; w0 += 32) {  // rows that some selected column touches
     const int w = w0 + lane;
     uint32_t rows = 0;
+#pragma unroll 1
     for (int j = 0; j < nt; ++j) {
       const int u = __shfl_sync(kFull, mine, j);
       if (w < wc) rows |= S.npN()[(size_t)u * I::W + w];
@@ -876,9 +916,11 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
   const long long wmine = lane < nt ? wfix[S.dpf()[mine]] : 0;
   long long bcost = LLONG_MAX;
   int bt = 0;
+#pragma unroll 1
   for (int t0 = 0; t0 < (1 << nt); t0 += 32) {
     const int t = t0 + lane;
     long long cost = 0;
+#pragma unroll 1
     for (int w = 0; w < wc; ++w) {
       uint32_t rows = uw[w];
       if (rows == 0) continue;
@@ -891,6 +933,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
         if (((x >> b) ^ __popc(pm & (unsigned)t)) & 1u) cost += wfix[S.pcol()[32 * w + b]];
       }
     }
+#pragma unroll 1
     for (int j = 0; j < nt; ++j) {
       const long long wj = __shfl_sync(kFull, wmine, j);
       if ((t >> j) & 1) cost += wj;
@@ -900,6 +943,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
       bt = t;
     }
   }
+#pragma unroll 1
   for (int off = 16; off > 0; off >>= 1) {
     const long long oc = __shfl_xor_sync(kFull, bcost, off);
     const int ot = __shfl_xor_sync(kFull, bt, off);
@@ -908,9 +952,11 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
       bt = ot;
     }
   }
+#pragma unroll 1
   for (int j = 0; j < nt; ++j) {
     if (!((bt >> j) & 1)) continue;
     const int u = __shfl_sync(kFull, mine, j);
+#pragma unroll 1
     for (int w = 0; w < wc; ++w)
       if ((S.npN()[(size_t)u * I::W + w] >> lane) & 1u) S.flags()[32 * w + lane] ^= 1;
     if (lane == 0) S.ext()[atomicAdd(&S.sc->ext, 1)] = S.dpf()[u];
@@ -925,6 +971,7 @@ __device__ __forceinline__ long long pattern_delta(const LSDArgs& a, const Shot<
   const long long* wfix = a.g.wfix;
   long long cost = wfix[S.dpf()[u1]];
   if (u2 >= 0) cost += wfix[S.dpf()[u2]];
+#pragma unroll 1
   for (int w = 0; w < wc; ++w) {
     uint32_t rows = S.npN()[(size_t)u1 * I::W + w];
     if (u2 >= 0) rows ^= S.npN()[(size_t)u2 * I::W + w];
@@ -962,11 +1009,13 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<I>& S, int r, int np, int ns
     }
   };
   if (lane == 0) consider(0, 0, 0, -1, -1);
+#pragma unroll 1
   for (int u = lane; u < np; u += 32) {
     if (S.dpr()[u] != r) continue;
     consider(pattern_delta(a, S, xw, wc, u, -1), 1, dep_key(S, u), u, -1);
   }
   const int npairs = nt * (nt - 1) / 2;
+#pragma unroll 1
   for (int t0 = 0; t0 < npairs; t0 += 32) {
     const int t = t0 + lane;
     int i = 0, rem = t < npairs ? t : 0;
@@ -979,6 +1028,7 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<I>& S, int r, int np, int ns
     if (t < npairs)
       consider(pattern_delta(a, S, xw, wc, u1, u2), 2, (unsigned long long)(i * 16 + j), u1, u2);
   }
+#pragma unroll 1
   for (int off = 16; off > 0; off >>= 1) {
     const long long oc = __shfl_xor_sync(kFull, bc, off);
     const int ocls = __shfl_xor_sync(kFull, bcls, off);
@@ -988,6 +1038,7 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<I>& S, int r, int np, int ns
     consider(oc, ocls, okey, o1, o2);
   }
   if (b1 < 0) return;  // no flip: OSD-0's local solution stands
+#pragma unroll 1
   for (int w = 0; w < wc; ++w) {
     uint32_t delta = S.npN()[(size_t)b1 * I::W + w];
     if (b2 >= 0) delta ^= S.npN()[(size_t)b2 * I::W + w];
@@ -1045,6 +1096,7 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
   unsigned long long steps_acc = 0, unsolv = 0;
   int kappa_max = 0, nu_max = 0;
   // the first item of a CTA is its block index, the others come from the counter
+#pragma unroll 1
   for (unsigned item = blockIdx.x; item < count;) {
     const long long qi = items ? (long long)items[item] : (long long)item;
     const long long shot = a.queue ? (long long)a.queue[qi] : qi;
@@ -1055,9 +1107,12 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
                             : nullptr;
 
     // ---- init: one cluster per flipped detector ----
+#pragma unroll 1
     for (int d = tid; d < (m + 3) / 4; d += NT)
       reinterpret_cast<uint4*>(S.lab)[d] = make_uint4(kFree, kFree, kFree, kFree);
+#pragma unroll 1
     for (int w = tid; w < wn; w += NT) S.cand[w] = S.joined[w] = 0u;
+#pragma unroll 1
     for (int w = tid; w < I::SC / 32; w += NT) S.growb()[w] = 0u;
     if (tid == 0) {
       sc.ns = sc.nf = sc.n_new = sc.merged = sc.ng = sc.np = sc.ovf = sc.ext = 0;
@@ -1079,13 +1134,16 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
     };
     const uint8_t* sp = a.syndromes + shot * m;
     if (!a.packed && (m & 3) == 0 && (reinterpret_cast<uintptr_t>(sp) & 3) == 0) {
+#pragma unroll 1
       for (int q = tid; q < m / 4; q += NT) {  // four detectors a load
         const uint32_t v = reinterpret_cast<const uint32_t*>(sp)[q];
         if (v == 0) continue;
+#pragma unroll 1
         for (int b = 0; b < 4; ++b)
           if ((v >> (8 * b)) & 0xffu) seed(4 * q + b);
       }
     } else {
+#pragma unroll 1
       for (int d = tid; d < m; d += NT)
         if (syn_bit(a.syndromes, a.packed, shot, m, d)) seed(d);
     }
@@ -1121,6 +1179,7 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
     }
     // ---- LSD-mu: mu more steps for every cluster, then the local reprocessing ----
     if constexpr (I::MU) {
+#pragma unroll 1
       for (int e = 0; e < a.order && status == LSD_SHOT_OK_LSD; ++e) {
         k = collect(S, sc.nsl, false, tid);
         if (k == 0) break;
@@ -1131,6 +1190,7 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
       __syncthreads();
       const int np = sc.np;
       if (status == LSD_SHOT_OK_LSD)
+#pragma unroll 1
         for (int u = tid; u < np; u += NT) {
           const int f = S.dpf()[u];
           S.dpr()[u] = (uint16_t)(S.lab[half4(G.var_pad[f], 0)] >> 16);
@@ -1140,6 +1200,7 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
       if (status == LSD_SHOT_OK_LSD && np > 0) {
         uint32_t* xw = S.template s<uint32_t>(I::osd) + (size_t)warp * 2 * I::W;
         const int nsl = sc.nsl;
+#pragma unroll 1
         for (int r = warp; r < ns; r += NT / 32) {
           if (S.parent()[r] != r) continue;
           if (a.osd_cs >= 0) osd_cs(a, S, r, np, nsl, xw, lane);
@@ -1153,10 +1214,13 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
     // ---- the correction row, cleared; a shot without room goes to the large instance ----
     if (status != kSpill || !spill) {
       if (cw) {
+#pragma unroll 1
         for (int w = tid; w < packed_words(n); w += NT) cw[w] = 0u;
       } else if ((n & 3) == 0 && (reinterpret_cast<uintptr_t>(co) & 3) == 0) {
+#pragma unroll 1
         for (int j = tid; j < n / 4; j += NT) reinterpret_cast<uint32_t*>(co)[j] = 0u;
       } else {
+#pragma unroll 1
         for (int j = tid; j < n; j += NT) co[j] = 0;
       }
     }
@@ -1171,10 +1235,12 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
       continue;
     }
     // ---- statistics: nu clusters, kappa = largest cluster in columns ----
+#pragma unroll 1
     for (int r = tid; r < ns; r += NT) S.best()[r] = 0u;
     if (tid == 0) sc.red[0][0] = sc.red[1][0] = 0u;
     __syncthreads();
     const int nf = sc.nf, nsl = sc.nsl;
+#pragma unroll 1
     for (int x = tid; x < nf; x += NT) {
       const int f = S.lf[x];
       if ((S.joined[f >> 5] >> (f & 31)) & 1u)
@@ -1186,15 +1252,18 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
         if (cw) atomicOr(cw + (j >> 5), 1u << (j & 31));
         else co[j] = 1;
       };
+#pragma unroll 1
       for (int i = tid; i < nsl; i += NT)
         if ((S.flags()[i] & 3) == 3) set(S.pcol()[i]);
       if constexpr (I::MU) {
         const int ne = sc.ext;
+#pragma unroll 1
         for (int t = tid; t < ne; t += NT) set(S.ext()[t]);
       }
     }
     __syncthreads();
     unsigned nu = 0, kappa = 0;
+#pragma unroll 1
     for (int r = tid; r < ns; r += NT)
       if (S.parent()[r] == r) {
         ++nu;
@@ -1261,6 +1330,7 @@ cudaError_t sparse_config(const DevGraph& g, int order, int* grid_small, int* gr
   if (err != cudaSuccess) return err;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+#pragma unroll 1
   for (const bool big : {false, true}) {
     err = with_instance(big, order > 0, g.m, g.n, [&](auto inst) {
       using I = decltype(inst);

@@ -50,6 +50,27 @@ def test_equals_dense_kernel(L, name, order, cs, ties):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("name", ["bb72", "bb144", "bb288", "ldpc_96x192", "irreg_37x61"])
+@pytest.mark.parametrize("kind", ["close", "infinite", "constant"])
+def test_order_of_close_llrs(L, name, kind):
+    """LLRs that a coarse key cannot tell apart (an outlier stretches their range, neighbours
+    differ in the last bits, in falling order), infinities, and all equal."""
+    h = code(name)
+    n, shots = h.shape[1], 200
+    probs = np.full(n, 0.06, np.float32)
+    s = torch.from_numpy(I.syndromes(h, I.sample_errors(12, shots, probs.astype(np.float64)))).cuda()
+    x = np.ones((shots, n), np.float32)
+    if kind != "constant":
+        steps = np.random.default_rng(6).integers(0, 40, (shots, n)) + 40 * (n - np.arange(n))
+        x += (steps * 2.0 ** -23).astype(np.float32)
+        x[:, 3] = 1e9 if kind == "close" else np.inf
+        x[::2, 5] = -1e9 if kind == "close" else -np.inf
+    llr = torch.from_numpy(x).cuda()
+    got, want = (L.Decoder(h, probs, 5, 2, lsd_kernel=k).postprocess(llr, s) for k in (1, 2))
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+
+
 def test_syndromes_outside_the_image(L):
     """Unsolvable shots among solvable ones: the same statuses as the dense kernel."""
     h = code("rep_boundary")[1:]           # a chain without boundary and an isolated row
