@@ -39,6 +39,7 @@
 #include <utility>
 #include <vector>
 
+#include "bp_shot.cuh"
 #include "lsd_internal.cuh"
 
 using namespace lsdgb;
@@ -157,14 +158,15 @@ __global__ void __launch_bounds__(256) gbp_init(GD g) {
 }
 
 // Iteration t (t >= 1): q = Lam - r on every edge of a check, then the scaled min-sum
-// message.  For t >= 2 it also tests the hard decision [Lam < 0] of iteration t-1 against s
-// (Sec. 4.3's early exit; sign bits stand for "< 0": no Lam is -0), accumulating into
-// bp_unsat[t & 1]; gbp_var(t) stops the shot, keeping Lam of iteration t-1, when it passed.
+// message.  For t >= 2 its return value (a check is unsatisfied) also tests the hard decision
+// [Lam < 0] of iteration t-1 against s (Sec. 4.3's early exit; sign bits stand for "< 0": no
+// Lam is -0): ored into bp_unsat[t & 1], once per block; the variable half of iteration t
+// stops the shot, keeping Lam of iteration t-1, when it passed.
 // A warp reads 32 consecutive checks' k-th edges: the column indices and messages are
 // contiguous, Lam is gathered.
 template <int DCMAX>
-__device__ __forceinline__ void check_phase(const GD& g, const uint8_t* __restrict__ s,
-                                            float alpha, int t) {
+__device__ __forceinline__ bool check_phase(const GD& g, const uint8_t* __restrict__ s,
+                                            float alpha) {
   bool bad = false;
   for (long long i = gtid(); i < g.m; i += gstride()) {
     unsigned hp = s[i] ? 0x80000000u : 0u;  // bit 31: syndrome ^ signs of Lam
@@ -203,15 +205,15 @@ __device__ __forceinline__ void check_phase(const GD& g, const uint8_t* __restri
           __uint_as_float(__float_as_uint(mag) | ((par ^ qb[k]) & 0x80000000u));
     }
   }
-  if (t >= 2 && __any_sync(kFullMask, bad) && (threadIdx.x & 31) == 0)
-    atomicOr(&g.ctr->bp_unsat[t & 1], 1);
+  return bad;
 }
 
 template <int DCMAX>
 __global__ void __launch_bounds__(256) gbp_check(GD g, const uint8_t* __restrict__ s,
                                                   float alpha, int t) {
   if (*(volatile int*)&g.ctr->bp_stop) return;
-  check_phase<DCMAX>(g, s, alpha, t);
+  const bool bad = check_phase<DCMAX>(g, s, alpha);
+  if (__syncthreads_or(t >= 2 && bad) && threadIdx.x == 0) atomicOr(&g.ctr->bp_unsat[t & 1], 1);
 }
 
 // Lam of iteration t: prior plus the incoming messages in ascending check order.
@@ -228,9 +230,10 @@ __device__ __forceinline__ void var_phase(const GD& g) {
 }
 
 // Iteration t's decision before its variable half: stop (true) when iteration t-1
-// satisfied the syndrome, keeping its posteriors; else clear the next test's slot.
-__device__ __forceinline__ bool bp_converged_before(const GD& g, int t) {
-  if (t >= 2 && *(volatile int*)&g.ctr->bp_unsat[t & 1] == 0) {
+// satisfied the syndrome (unsat: its test's result), keeping its posteriors; else clear the
+// next test's slot.
+__device__ __forceinline__ bool bp_converged_before(const GD& g, int t, int unsat) {
+  if (t >= 2 && unsat == 0) {
     if (gtid() == 0) {
       g.ctr->bp_conv = 1;
       g.ctr->bp_iters = t - 1;
@@ -247,12 +250,12 @@ __device__ __forceinline__ bool bp_converged_before(const GD& g, int t) {
 
 __global__ void __launch_bounds__(256) gbp_var(GD g, int t) {
   if (*(volatile int*)&g.ctr->bp_stop) return;
-  if (bp_converged_before(g, t)) return;
+  if (bp_converged_before(g, t, *(volatile int*)&g.ctr->bp_unsat[t & 1])) return;
   var_phase(g);
 }
 
 // The test after the last iteration T (slot (T+1) & 1, cleared by iteration T).
-__device__ __forceinline__ void syn_phase(const GD& g, const uint8_t* __restrict__ s, int slot) {
+__device__ __forceinline__ bool syn_phase(const GD& g, const uint8_t* __restrict__ s) {
   bool bad = false;
   for (long long i = gtid(); i < g.m; i += gstride()) {
     unsigned hp = s[i] ? 0x80000000u : 0u;
@@ -263,71 +266,192 @@ __device__ __forceinline__ void syn_phase(const GD& g, const uint8_t* __restrict
     }
     bad |= (hp >> 31) != 0u;
   }
-  if (__any_sync(kFullMask, bad) && (threadIdx.x & 31) == 0) atomicOr(&g.ctr->bp_unsat[slot], 1);
+  return bad;
 }
 
 __global__ void __launch_bounds__(256) gbp_syn(GD g, const uint8_t* __restrict__ s, int slot) {
   if (*(volatile int*)&g.ctr->bp_stop) return;
-  syn_phase(g, s, slot);
+  const bool bad = syn_phase(g, s);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&g.ctr->bp_unsat[slot], 1);
 }
 
-// Grid-wide barrier of the persistent launch (all blocks co-resident: cooperative launch).
-// The arrival counter only grows; barrier b waits for b * gridDim.x arrivals.  The wait is
-// bounded by limit_ns of the global timer: past it the block flags bp_fail and every block
-// leaves at its next barrier, the host reporting LSD_ERR_TIMEOUT.  `arrive` false (the
-// timeout test only) withholds this block's arrival.
+// Grid-wide barrier of the persistent launches (all blocks co-resident: cooperative launch).
+// The arrival counter only grows; barrier b waits for b * gridDim.x arrivals.  Before arriving
+// the block ors `bad` over its threads into *flag; the return value is *flag after the barrier,
+// or -1: the wait is bounded by limit_ns of the global timer, past it the block flags bp_fail
+// and every block leaves at its next barrier, the host reporting LSD_ERR_TIMEOUT.  Only one
+// thread of a block reads the flags.  `arrive` false (the timeout test only) withholds this
+// block's arrival.
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
 
-__device__ __forceinline__ bool grid_barrier(const GD& g, unsigned target, long long limit_ns,
-                                             bool arrive = true) {
-  __syncthreads();
+__device__ __forceinline__ int grid_barrier(const GD& g, unsigned target, long long limit_ns,
+                                            int* flag, bool bad, bool arrive = true) {
+  __shared__ int s_flag;
+  const int any = __syncthreads_or(bad);
   if (threadIdx.x == 0) {
+    if (any) atomicOr(flag, 1);
     __threadfence();
     if (arrive) atomicAdd(&g.ctr->bar_arrive, 1u);
-    const unsigned long long t0 = global_ns();
-    while (*(volatile unsigned*)&g.ctr->bar_arrive < target &&
-           !*(volatile int*)&g.ctr->bp_fail) {
-      if ((long long)(global_ns() - t0) > limit_ns) {
-        atomicOr(&g.ctr->bp_fail, 1);
+    bool ok = true;
+    unsigned long long t0 = 0;
+    for (unsigned spin = 1; *(volatile unsigned*)&g.ctr->bar_arrive < target; ++spin) {
+      if (spin & 63u) continue;  // the clock and the failure flag are looked at now and then
+      const unsigned long long now = global_ns();
+      if (t0 == 0) t0 = now;
+      if ((long long)(now - t0) > limit_ns) atomicOr(&g.ctr->bp_fail, 1);
+      if (*(volatile int*)&g.ctr->bp_fail) {
+        ok = false;
         break;
       }
-      __nanosleep(64);
     }
     __threadfence();
+    s_flag = ok ? *(volatile int*)flag : -1;
   }
   __syncthreads();
-  return *(volatile int*)&g.ctr->bp_fail == 0;
+  const int f = s_flag;
+  __syncthreads();
+  return f;
 }
 
-// All T iterations in one launch: check half, barrier, decision, variable half, barrier.
-// hold != 0 (the timeout test only): block 0 withholds its first arrival.
-template <int DCMAX>
-__global__ void __launch_bounds__(256) gbp_persistent(GD g, const uint8_t* __restrict__ s,
-                                                       float alpha, int T, long long limit_ns,
-                                                       int hold) {
+// Frame of the persistent launches: check half, barrier, decision, variable half, barrier, for
+// all T iterations, then the last test.  hold != 0 (the timeout test only): block 0 withholds
+// its first arrival.
+template <class Check, class Var, class Syn>
+__device__ __forceinline__ void bp_persistent(const GD& g, int T, long long limit_ns, int hold,
+                                              Check&& check, Var&& var, Syn&& syn) {
   unsigned target = 0;
   const unsigned nb = gridDim.x;
   for (int t = 1; t <= T; ++t) {
-    check_phase<DCMAX>(g, s, alpha, t);
+    const bool bad = check(t);
     target += nb;
-    if (!grid_barrier(g, target, limit_ns, !(hold && t == 1 && blockIdx.x == 0))) return;
-    if (bp_converged_before(g, t)) return;
-    var_phase(g);
+    const int unsat = grid_barrier(g, target, limit_ns, &g.ctr->bp_unsat[t & 1], t >= 2 && bad,
+                                   !(hold && t == 1 && blockIdx.x == 0));
+    if (unsat < 0) return;
+    if (bp_converged_before(g, t, unsat)) return;
+    var();
     target += nb;
-    if (!grid_barrier(g, target, limit_ns)) return;
+    if (grid_barrier(g, target, limit_ns, &g.ctr->bp_unsat[t & 1], false) < 0) return;
   }
-  const int slot = (T + 1) & 1;
-  syn_phase(g, s, slot);
+  const bool bad = syn();
   target += nb;
-  if (!grid_barrier(g, target, limit_ns)) return;
-  if (gtid() == 0) {
-    g.ctr->bp_conv = g.ctr->bp_unsat[slot] == 0;
+  const int unsat = grid_barrier(g, target, limit_ns, &g.ctr->bp_unsat[(T + 1) & 1], bad);
+  if (unsat >= 0 && gtid() == 0) {
+    g.ctr->bp_conv = unsat == 0;
     g.ctr->bp_stop = 1;
   }
+}
+
+// Any graph: tables and messages through L2.
+template <int DCMAX>
+__global__ void __launch_bounds__(256) gbp_persistent(GD g, const uint8_t* __restrict__ s,
+                                                       float alpha, int T, long long limit_ns,
+                                                       int hold, int, int) {
+  bp_persistent(
+      g, T, limit_ns, hold, [&](int) { return check_phase<DCMAX>(g, s, alpha); },
+      [&] { var_phase(g); }, [&] { return syn_phase(g, s); });
+}
+
+// Graphs whose tables fit the SMs' shared memory (640 000 faults, 307 200 detectors of column
+// weight 3 to 4: 217 KB of each): one block per SM, thread t owns the checks and variables
+// (c gridDim + block) blockDim + t; their tables, priors and messages stay on chip, so an
+// iteration moves the gathered posteriors and messages and the stored ones, half of what
+// gbp_persistent moves, and each half waits for one L2 access instead of two in a row.
+// Measured per iteration at 640 000 faults: gbp_persistent 24.6 us, this kernel 10.4 (15.0 with
+// the gathers past the L1: half of them are of single words, and 1024 consecutive checks or
+// variables share their sectors); 160 000 faults, 10.3 -> 4.5 us.  Of that, one arrival and one
+// flag update per block instead of 1216 blocks' and every warp's, and a poll without sleep.
+// The gathers are plain loads: the barrier's fences on both sides make other blocks' stores
+// visible to them (and drop stale L1 lines).
+// Same values as gbp_persistent (the check update is that of the batch kernels, bp_shot.cuh).
+constexpr int kResDc = 8, kResDv = 4, kResC = 2, kResV = 6;
+__global__ void __launch_bounds__(1024) gbp_resident(GD g, const uint8_t* __restrict__ s, float alpha,
+                                                      int T, long long limit_ns, int hold, int cpt,
+                                                      int vpt) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int NT = blockDim.x, tid = threadIdx.x;
+  int* const col = reinterpret_cast<int*>(smem);                  // [cpt][dc][NT], -1 past a row
+  float* const msg = reinterpret_cast<float*>(col + cpt * g.dc * NT);
+  int* const pos = reinterpret_cast<int*>(msg + cpt * g.dc * NT);  // [vpt][dv][NT], -1 past a column
+  float* const pri = reinterpret_cast<float*>(pos + vpt * g.dv * NT);
+  const int i0 = blockIdx.x * NT + tid, step = gridDim.x * NT;
+  unsigned sbits = 0;
+  for (int c = 0; c < cpt; ++c) {
+    const int i = i0 + c * step;
+    if (i < g.m && s[i]) sbits |= 1u << c;
+    for (int k = 0; k < g.dc; ++k) {
+      col[(c * g.dc + k) * NT + tid] = i < g.m ? g.ell_col[(long long)k * g.m + i] : -1;
+      msg[(c * g.dc + k) * NT + tid] = 0.f;
+    }
+  }
+  for (int v = 0; v < vpt; ++v) {
+    const int j = i0 + v * step;
+    for (int k = 0; k < g.dv; ++k)
+      pos[(v * g.dv + k) * NT + tid] = j < g.n ? g.ell_pos[(long long)k * g.n + j] : -1;
+    pri[v * NT + tid] = j < g.n ? g.prior[j] : 0.f;
+  }
+  const float kInf = __uint_as_float(0x7f800000u);
+  // the gathers of every check (variable) are asked for before any is used
+  auto check = [&](int t) {
+    const float* const lam = t == 1 ? g.prior : g.lam;
+    float q[kResC][kResDc];
+#pragma unroll
+    for (int c = 0; c < kResC; ++c)
+#pragma unroll
+      for (int k = 0; k < kResDc; ++k) {
+        const int j = c < cpt && k < g.dc ? col[(c * g.dc + k) * NT + tid] : -1;
+        q[c][k] = j >= 0 ? lam[j] : kInf;  // +inf changes no minimum, sign or parity
+      }
+    bool bad = false;
+#pragma unroll
+    for (int c = 0; c < kResC; ++c) {
+      const uint32_t sbit = (sbits >> c) << 31;
+      uint32_t hp = sbit;
+      float x[kResDc];
+#pragma unroll
+      for (int k = 0; k < kResDc; ++k) {
+        hp ^= __float_as_uint(q[c][k]);
+        if (c < cpt && k < g.dc) q[c][k] = __fsub_rn(q[c][k], msg[(c * g.dc + k) * NT + tid]);
+      }
+      bad |= (hp >> 31) != 0u;
+      excluded_min<kResDc>(q[c], x);
+      const float salpha = __uint_as_float(__float_as_uint(alpha) ^ sbit);
+      const int i = i0 + c * step;
+#pragma unroll
+      for (int k = 0; k < kResDc; ++k) {
+        if (c < cpt && k < g.dc && i < g.m) {
+          const float y = __fmul_rn(x[k], salpha);
+          msg[(c * g.dc + k) * NT + tid] = y;
+          g.r[(long long)k * g.m + i] = y;  // (a place past the row's end is read by nobody)
+        }
+      }
+    }
+    return bad;
+  };
+  auto var = [&] {
+    float in[kResV][kResDv];
+#pragma unroll
+    for (int v = 0; v < kResV; ++v)
+#pragma unroll
+      for (int k = 0; k < kResDv; ++k) {
+        const int p = v < vpt && k < g.dv ? pos[(v * g.dv + k) * NT + tid] : -1;
+        in[v][k] = p >= 0 ? g.r[p] : 0.f;  // + 0 leaves the sum as it is (never -0)
+      }
+#pragma unroll
+    for (int v = 0; v < kResV; ++v) {
+      const int j = i0 + v * step;
+      if (v < vpt && j < g.n) {
+        float L = pri[v * NT + tid];
+#pragma unroll
+        for (int k = 0; k < kResDv; ++k) L = __fadd_rn(L, in[v][k]);
+        g.lam[j] = L;
+      }
+    }
+  };
+  bp_persistent(g, T, limit_ns, hold, check, var, [&] { return syn_phase(g, s); });
 }
 
 __global__ void gbp_final(GD g, int slot) {
@@ -1008,6 +1132,9 @@ struct lsd_giant {
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   int64_t launches = 0;
   int coop_grid = 0;  // blocks of the persistent BP launch (0: launch per half-iteration)
+  const void* coop_fn = nullptr;
+  int coop_block = 256, coop_cpt = 0, coop_vpt = 0;  // cpt > 0: gbp_resident
+  size_t coop_smem = 0;
   long long bar_limit_ns = 1000000000LL;  // bound of a grid-barrier wait
   int hold_barrier = 0;                   // timeout test: block 0 withholds an arrival
 };
@@ -1325,6 +1452,31 @@ int lsd_giant_create(lsd_giant** out, int32_t m, int32_t n, int64_t nnz, const i
     if (err == cudaSuccess && coop && per_sm > 0) {
       const long long need = (std::max<long long>(m, n) + 255) / 256;
       G->coop_grid = (int)std::min<long long>(need, (long long)per_sm * G->sms);
+      G->coop_fn = fn;
+      // tables on chip when they fit: a block per SM, as many threads as give each about two
+      // variables (at most 1024)
+      int max_smem = 0;
+      err = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+      const int block = (int)std::min<long long>(1024, (n / (2LL * G->sms) + 128) / 128 * 128);
+      const long long cap = (long long)block * G->sms;
+      const long long cpt = (m + cap - 1) / cap, vpt = (n + cap - 1) / cap;
+      if (err == cudaSuccess && dc >= 1 && dc <= kResDc && dv <= kResDv && cpt <= kResC && vpt <= kResV) {
+        const size_t smem = (size_t)block * 4 * (2 * cpt * dc + vpt * (dv + 1));
+        int res_per_sm = 0;
+        const void* res = (const void*)gbp_resident;
+        if (smem + 1024 <= (size_t)max_smem &&
+            allow_max_dynamic_smem(res, max_smem) == cudaSuccess &&
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res_per_sm, res, block, smem) == cudaSuccess &&
+            res_per_sm > 0) {
+          G->coop_fn = res;
+          G->coop_grid = (int)std::min<long long>(G->sms, (std::max<long long>(m, n) + block - 1) / block);
+          G->coop_block = block;
+          G->coop_cpt = (int)((m + (long long)block * G->coop_grid - 1) / ((long long)block * G->coop_grid));
+          G->coop_vpt = (int)((n + (long long)block * G->coop_grid - 1) / ((long long)block * G->coop_grid));
+          G->coop_smem = smem;
+        }
+        cudaGetLastError();
+      }
     }
     if (err != cudaSuccess) rc = gfail(err);
   }
@@ -1372,8 +1524,10 @@ int lsd_giant_decode(lsd_giant* G, const uint8_t* syndrome, uint8_t* correction,
   cudaEventRecord(G->ev[0], G->st);
   cudaError_t e = cudaMemsetAsync(g.ctr, 0, sizeof(GCtr), G->st);
   if (e != cudaSuccess) return gfail(e);
-  gbp_init<<<grid, 256, 0, G->st>>>(g);
-  if ((rc = check_launch(G))) return rc;
+  if (G->coop_cpt == 0 || G->bp_iters == 0) {  // (gbp_resident starts from the priors itself)
+    gbp_init<<<grid, 256, 0, G->st>>>(g);
+    if ((rc = check_launch(G))) return rc;
+  }
   // iterations in chunks of 2, 4, 8, ... with a look at the stop flag after each, so that a
   // shot that converges early is not followed by the remaining iterations' launches
   bool stopped = false;
@@ -1384,11 +1538,9 @@ int lsd_giant_decode(lsd_giant* G, const uint8_t* syndrome, uint8_t* correction,
     int T = G->bp_iters;
     long long limit = G->bar_limit_ns;
     int hold = G->hold_barrier;
-    void* args[] = {(void*)&g, (void*)&sp, (void*)&alpha, (void*)&T, (void*)&limit, (void*)&hold};
-    const void* fn = g.dc <= 8    ? (const void*)gbp_persistent<8>
-                     : g.dc <= 16 ? (const void*)gbp_persistent<16>
-                                  : (const void*)gbp_persistent<32>;
-    e = cudaLaunchCooperativeKernel(fn, G->coop_grid, 256, args, 0, G->st);
+    void* args[] = {(void*)&g,     (void*)&sp,   (void*)&alpha,        (void*)&T,
+                    (void*)&limit, (void*)&hold, (void*)&G->coop_cpt, (void*)&G->coop_vpt};
+    e = cudaLaunchCooperativeKernel(G->coop_fn, G->coop_grid, G->coop_block, args, G->coop_smem, G->st);
     G->launches++;
     if (e != cudaSuccess) return gfail(e);
     stopped = true;
