@@ -60,7 +60,7 @@ struct lsd_decoder {
   float* d_probs = nullptr;  // channel probabilities (sampler)
   // sparse LSD (large matrices)
   bool sparse = false;
-  int sp_grid_small = 0, sp_grid_big = 0;
+  int sp_grid_small = 0, sp_grid_big = 0;  // (large: 0 when no shot can outgrow the small one)
   unsigned char* d_sp_small = nullptr;
   unsigned char* d_sp_big = nullptr;
   int* d_spill = nullptr;
@@ -250,7 +250,7 @@ int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
                         (size_t)d->sp_grid_big * d->sp_stride_big)))
       return rc;
   }
-  if ((size_t)max_items > d->spill_cap) {
+  if (d->sp_grid_big > 0 && (size_t)max_items > d->spill_cap) {
     cudaError_t e = cudaStreamSynchronize(d->st);
     if (e != cudaSuccess) return cuda_fail(e);
     dev_free(d, d->d_spill, d->spill_cap * sizeof(int));
@@ -263,6 +263,7 @@ int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
   cudaError_t e = launch_sparse(l, false, d->sp_grid_small, d->d_sp_small, d->sp_stride_small,
                                 d->d_spill, nullptr, d->st);
   d->launches++;
+  if (d->sp_grid_big == 0) return e == cudaSuccess ? LSD_OK : cuda_fail(e);
   if (e == cudaSuccess)
     e = launch_sparse(l, true, d->sp_grid_big, d->d_sp_big, d->sp_stride_big, nullptr, d->d_spill,
                       d->st);
@@ -1255,7 +1256,8 @@ int lsdgb::bp_batch_counted(lsd_decoder* d, int64_t max_shots, const long long* 
   if (!d || max_shots <= 0 || !shots_dev || !syndromes || !corrections) return LSD_ERR_INVALID_ARG;
   if (!d->lsd_ok) return LSD_ERR_UNSUPPORTED;
   if ((size_t)max_shots > d->cap_shots) return LSD_ERR_ADMISSION;
-  if (d->sparse && (!d->d_sp_big || (size_t)max_shots > d->spill_cap)) return LSD_ERR_ADMISSION;
+  if (d->sparse && (!d->d_sp_big || (d->sp_grid_big > 0 && (size_t)max_shots > d->spill_cap)))
+    return LSD_ERR_ADMISSION;
   int rc = reset_counters(d);
   if (rc) return rc;
   BPArgs a = bp_args(d, max_shots, syndromes);

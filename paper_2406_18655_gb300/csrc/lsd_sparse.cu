@@ -80,22 +80,31 @@ struct Inst {
   static constexpr size_t fixed = al16(osd + (MU ? (size_t)NW * 2 * W * 4 : 0));
   // lists
   static constexpr size_t newk = 0;                               // new columns of a step
-  static constexpr size_t M = newk + (size_t)SC * 8;
-  static constexpr size_t npN = M + (size_t)CAP * W * 4;          // dependent columns' images
-  static constexpr size_t ssl = npN + (MU ? (size_t)CAP * W * 4 : 0);  // slots of new columns
+  static constexpr size_t ssl = newk + (size_t)SC * 8;            // slots of new columns
   static constexpr size_t sg = ssl + (size_t)SC * 8;              // their faults, in key order
   static constexpr size_t sroot = sg + (size_t)SC * 2;            // their clusters
   static constexpr size_t dpf = sroot + (size_t)SC * 2;           // faults of dependent columns
   static constexpr size_t ext = dpf + (MU ? (size_t)CAP * 2 : 0);
   static constexpr size_t dpr = ext + (MU ? (size_t)CAP * 2 : 0);      // their clusters
   static constexpr size_t dpk = dpr + (MU ? (size_t)CAP * 2 : 0);      // their LLR bits
-  static constexpr size_t lists = al16(dpk + (MU ? (size_t)CAP * 4 : 0));
+  static constexpr size_t M = al16(dpk + (MU ? (size_t)CAP * 4 : 0));
+  // Rows of M and bits of the dependent columns' images (npN, after M): a shot has at most as
+  // many slots as the graph has detectors.
+  static __host__ __device__ int row_stride(int m) {
+    const int r = (m + 31) & ~31;
+    return BIG && r < CAP ? r : CAP;
+  }
+  static __host__ __device__ size_t list_bytes(int m) {
+    const size_t r = (size_t)row_stride(m);
+    return al16(M + r * (r / 32) * 4 + (MU ? (size_t)CAP * (r / 32) * 4 : 0));
+  }
   // Candidate list entries.  A shot that lists half of a large code's faults has percolated
   // and goes to the large instance.
   static __host__ __device__ int lcap(int n) {
     if (BIG) return n;
-    const int half = n / 2 > 1024 ? n / 2 : 1024;
-    return half < 2816 ? half : 2816;
+    const int half = n / 2 > 1536 ? n / 2 : 1536;
+    const int cap = half < 2816 ? half : 2816;
+    return cap < n ? cap : n;
   }
 };
 
@@ -104,15 +113,21 @@ __host__ __device__ inline size_t cand_bytes(size_t cap) {
   return al16(cap * 8) + al16(cap * 4) + al16(cap * 2);
 }
 
+// No shot can outgrow the small instance I: the large one is not launched.
+template <class I>
+bool always_fits(int m, int n) {
+  return m <= I::CAP && m <= I::SC && n <= I::lcap(n) && (!I::MU || n <= I::CAP);
+}
+
 template <class I>
 size_t smem_bytes(int m, int n) {
   return I::fixed + (I::LG ? 0 : al16((size_t)m * 4)) + 2 * al16((size_t)(n + 31) / 32 * 4) +
-         (I::BIG ? 0 : I::lists) + (I::BIG && I::LG ? 0 : cand_bytes((size_t)I::lcap(n)));
+         (I::BIG ? 0 : I::list_bytes(m)) + (I::BIG && I::LG ? 0 : cand_bytes((size_t)I::lcap(n)));
 }
 // Global scratch bytes of a CTA.
 template <class I>
 size_t scratch_bytes(int m, int n) {
-  return (I::LG ? al16((size_t)m * 4) : 0) + (I::BIG ? I::lists : 0) +
+  return (I::LG ? al16((size_t)m * 4) : 0) + (I::BIG ? I::list_bytes(m) : 0) +
          (I::BIG && I::LG ? cand_bytes((size_t)n) : 0);
 }
 
@@ -150,7 +165,10 @@ struct Shot {
   uint32_t* lk;
   uint16_t* lf;
   int lcap;
+  int rs;               // row stride of M (large instance; constant for the small one)
   Scal* sc;
+  __device__ __forceinline__ int stride() const { return I::BIG ? rs : I::CAP; }
+  __device__ __forceinline__ int words() const { return stride() >> 5; }
   template <class T>
   __device__ __forceinline__ T* s(size_t off) const { return reinterpret_cast<T*>(sm + off); }
   template <class T>
@@ -166,7 +184,7 @@ struct Shot {
   __device__ __forceinline__ unsigned char* flags() const { return s<unsigned char>(I::flags); }
   __device__ __forceinline__ unsigned long long* newk() const { return l<unsigned long long>(I::newk); }
   __device__ __forceinline__ uint32_t* M() const { return l<uint32_t>(I::M); }
-  __device__ __forceinline__ uint32_t* npN() const { return l<uint32_t>(I::npN); }
+  __device__ __forceinline__ uint32_t* npN() const { return M() + (size_t)stride() * words(); }
   __device__ __forceinline__ uint16_t* ssl() const { return l<uint16_t>(I::ssl); }
   __device__ __forceinline__ uint16_t* sg() const { return l<uint16_t>(I::sg); }
   __device__ __forceinline__ uint16_t* sroot() const { return l<uint16_t>(I::sroot); }
@@ -261,7 +279,7 @@ __device__ __forceinline__ void open_rows(const Shot<I>& S, int from, int to, in
   for (int i = tid; i < to; i += I::NT)
 #pragma unroll 1
     for (int w = i < from ? w0 : 0; w < w1; ++w)
-      S.M()[(size_t)w * I::CAP + i] = (i >> 5) == w && i >= from ? 1u << (i & 31) : 0u;
+      S.M()[(size_t)w * S.stride() + i] = (i >> 5) == w && i >= from ? 1u << (i & 31) : 0u;
 }
 
 // Fault f is next to a newly claimed detector: lists it if it is not listed; returns its entry
@@ -314,7 +332,7 @@ __device__ __forceinline__ uint32_t column_image(const SGraph& G, const Shot<I>&
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const uint32_t s = half4(sl, q);
-        if (s != kNone16) x ^= S.M()[(size_t)(s >> 5) * CAP + i] >> (s & 31);
+        if (s != kNone16) x ^= S.M()[(size_t)(s >> 5) * S.stride() + i] >> (s & 31);
       }
       hit |= (x & 1u) << j;
     }
@@ -326,7 +344,7 @@ __device__ __forceinline__ uint32_t column_image(const SGraph& G, const Shot<I>&
       const uint32_t s = S.lab[G.var_chk[q]] & 0xffffu;
 #pragma unroll 1
       for (int j = 0; tid + NT * j < nsl; ++j)
-        hit ^= ((S.M()[(size_t)(s >> 5) * CAP + tid + NT * j] >> (s & 31)) & 1u) << j;
+        hit ^= ((S.M()[(size_t)(s >> 5) * S.stride() + tid + NT * j] >> (s & 31)) & 1u) << j;
     }
   }
 #pragma unroll 1
@@ -353,13 +371,13 @@ __device__ __forceinline__ void pivot_update(const Shot<I>& S, int p, int g, uin
   if (!__any_sync(kFull, hit != 0)) return;
 #pragma unroll 1
   for (int c0 = 0; c0 < wc; c0 += 32) {
-    const uint32_t v = c0 + lane < wc ? S.M()[(size_t)(c0 + lane) * CAP + p] : 0u;
+    const uint32_t v = c0 + lane < wc ? S.M()[(size_t)(c0 + lane) * S.stride() + p] : 0u;
     unsigned nz = __ballot_sync(kFull, v != 0);
     while (nz) {
       const int w = __ffs(nz) - 1;
       nz &= nz - 1;
       const uint32_t pv = __shfl_sync(kFull, v, w);
-      uint32_t* const row = S.M() + (size_t)(c0 + w) * CAP + tid;
+      uint32_t* const row = S.M() + (size_t)(c0 + w) * S.stride() + tid;
 #pragma unroll
       for (int j = 0; j < I::RPT; ++j)
         if ((hit >> j) & 1u) row[NT * j] ^= pv;
@@ -381,7 +399,8 @@ __device__ __forceinline__ void keep_dependent(const Shot<I>& S, int& np, int g,
 #pragma unroll
     for (int j = 0; j < I::RPT; ++j) {
       const unsigned b = __ballot_sync(kFull, (hit >> j) & 1u);
-      if ((tid & 31) == 0) S.npN()[(size_t)np * I::W + I::NW * j + (tid >> 5)] = b;
+      const int w = I::NW * j + (tid >> 5);
+      if ((tid & 31) == 0 && w < S.words()) S.npN()[(size_t)np * S.words() + w] = b;
     }
     if (tid == 0) S.dpf()[np] = (uint16_t)g;
     ++np;
@@ -425,7 +444,7 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const uint32_t s = half4(sl, q);
-          if (mine && s != kNone16) x ^= M[(size_t)(s >> 5) * CAP + i] >> (s & 31);
+          if (mine && s != kNone16) x ^= M[(size_t)(s >> 5) * S.stride() + i] >> (s & 31);
         }
         bool hit = (x & 1u) != 0;
         const unsigned nb = __ballot_sync(kFull, hit && !(S.flags()[i] & 2));
@@ -438,9 +457,9 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
               S.sc->ovf = 1;
               continue;
             }
-            uint32_t* const row = S.npN() + (size_t)k * I::W;
+            uint32_t* const row = S.npN() + (size_t)k * S.words();
 #pragma unroll 1
-            for (int w = lane; w < I::W; w += 32) row[w] = 0u;
+            for (int w = lane; w < S.words(); w += 32) row[w] = 0u;
             __syncwarp();
             if (hit) atomicOr(row + (i >> 5), 1u << (i & 31));
             if (lane == 0) S.dpf()[k] = (uint16_t)g;
@@ -459,13 +478,13 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
         if (__any_sync(kFull, hit)) {
 #pragma unroll 1
           for (int c0 = 0; c0 < wc; c0 += 32) {
-            const uint32_t v = c0 + lane < wc ? M[(size_t)(c0 + lane) * CAP + p] : 0u;
+            const uint32_t v = c0 + lane < wc ? M[(size_t)(c0 + lane) * S.stride() + p] : 0u;
             unsigned nz = __ballot_sync(kFull, v != 0);
             while (nz) {
               const int w = __ffs(nz) - 1;
               nz &= nz - 1;
               const uint32_t pv = __shfl_sync(kFull, v, w);
-              if (hit) M[(size_t)(c0 + w) * CAP + i] ^= pv;
+              if (hit) M[(size_t)(c0 + w) * S.stride() + i] ^= pv;
             }
           }
           if (sp && hit) S.flags()[i] ^= 1;
@@ -908,7 +927,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
 #pragma unroll 1
     for (int j = 0; j < nt; ++j) {
       const int u = __shfl_sync(kFull, mine, j);
-      if (w < wc) rows |= S.npN()[(size_t)u * I::W + w];
+      if (w < wc) rows |= S.npN()[(size_t)u * S.words() + w];
     }
     if (w < wc) uw[w] = rows;
   }
@@ -924,7 +943,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
     for (int w = 0; w < wc; ++w) {
       uint32_t rows = uw[w];
       if (rows == 0) continue;
-      const uint32_t nw = lane < nt ? S.npN()[(size_t)mine * I::W + w] : 0u;
+      const uint32_t nw = lane < nt ? S.npN()[(size_t)mine * S.words() + w] : 0u;
       const uint32_t x = xw[w];
       while (rows) {
         const int b = __ffs(rows) - 1;
@@ -958,7 +977,7 @@ __device__ void osd_e(const LSDArgs& a, const Shot<I>& S, int r, int np, int nsl
     const int u = __shfl_sync(kFull, mine, j);
 #pragma unroll 1
     for (int w = 0; w < wc; ++w)
-      if ((S.npN()[(size_t)u * I::W + w] >> lane) & 1u) S.flags()[32 * w + lane] ^= 1;
+      if ((S.npN()[(size_t)u * S.words() + w] >> lane) & 1u) S.flags()[32 * w + lane] ^= 1;
     if (lane == 0) S.ext()[atomicAdd(&S.sc->ext, 1)] = S.dpf()[u];
   }
 }
@@ -973,8 +992,8 @@ __device__ __forceinline__ long long pattern_delta(const LSDArgs& a, const Shot<
   if (u2 >= 0) cost += wfix[S.dpf()[u2]];
 #pragma unroll 1
   for (int w = 0; w < wc; ++w) {
-    uint32_t rows = S.npN()[(size_t)u1 * I::W + w];
-    if (u2 >= 0) rows ^= S.npN()[(size_t)u2 * I::W + w];
+    uint32_t rows = S.npN()[(size_t)u1 * S.words() + w];
+    if (u2 >= 0) rows ^= S.npN()[(size_t)u2 * S.words() + w];
     const uint32_t x = xw[w];
     while (rows) {
       const int b = __ffs(rows) - 1;
@@ -1040,8 +1059,8 @@ __device__ void osd_cs(const LSDArgs& a, const Shot<I>& S, int r, int np, int ns
   if (b1 < 0) return;  // no flip: OSD-0's local solution stands
 #pragma unroll 1
   for (int w = 0; w < wc; ++w) {
-    uint32_t delta = S.npN()[(size_t)b1 * I::W + w];
-    if (b2 >= 0) delta ^= S.npN()[(size_t)b2 * I::W + w];
+    uint32_t delta = S.npN()[(size_t)b1 * S.words() + w];
+    if (b2 >= 0) delta ^= S.npN()[(size_t)b2 * S.words() + w];
     if ((delta >> lane) & 1u) S.flags()[32 * w + lane] ^= 1;
   }
   if (lane == 0) {
@@ -1077,7 +1096,8 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
     S.joined = reinterpret_cast<uint32_t*>(take(sp, (size_t)wn * 4));
     if constexpr (I::LG) S.lab = reinterpret_cast<uint32_t*>(take(gp, (size_t)m * 4));
     else S.lab = reinterpret_cast<uint32_t*>(take(sp, (size_t)m * 4));
-    S.li = I::BIG ? take(gp, I::lists) : take(sp, I::lists);
+    S.li = I::BIG ? take(gp, I::list_bytes(m)) : take(sp, I::list_bytes(m));
+    S.rs = I::row_stride(m);
     S.lcap = I::lcap(n);
     auto list = [&](unsigned char*& p) {
       S.ld = reinterpret_cast<uint2*>(take(p, (size_t)S.lcap * 8));
@@ -1331,7 +1351,11 @@ cudaError_t sparse_config(const DevGraph& g, int order, int* grid_small, int* gr
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
 #pragma unroll 1
+  *grid_big = 0;
   for (const bool big : {false, true}) {
+    if (big && with_instance(false, order > 0, g.m, g.n,
+                             [&](auto inst) { return always_fits<decltype(inst)>(g.m, g.n); }))
+      break;
     err = with_instance(big, order > 0, g.m, g.n, [&](auto inst) {
       using I = decltype(inst);
       const void* fn = (const void*)lsd_sparse_kernel<I>;
