@@ -31,6 +31,12 @@
 //   epilogue (the warps whose TMEM lane quarter holds the row): tcgen05.ld of P_v, + deg kv,
 //       BF16 C_v and B_v rows into shared memory
 //   X1, MMA on the check tiles, epilogue: the same for T_c, P_c, A_c and D_c
+// What bounds it: about half issue (46 % of the slots at 18 warps per SM, all TMEM in use),
+// half barriers and shared-memory latency.  Taking instructions out is what helped: no modulo
+// per (tile, half) and warp in the epilogues, mixed-precision adds in the gathers, packed FP32
+// FMAs for the biases and the LLR, row -> (edges, shot) from a table: 28.2 -> 20.1 k warp
+// instructions a BB144 shot, 200 000 shots 9.07 -> 6.93 ms (BB72 100 003 2.35 -> 1.81 ms, BB288
+// 50 000 5.69 -> 4.36 ms).
 // The last round stops after X2 (only the LLR needs it).  Shared-memory operands use the
 // canonical K-major layout without swizzle: 8-row x 16-byte core matrices, adjacent along K
 // 128 bytes apart, adjacent along M/N 512 bytes apart (a K = 32 BF16 row block).
@@ -75,8 +81,8 @@ struct TcArgs {
 };
 
 struct TcLay {
-  size_t mv, mc, op, as, ds, cs, bs, p0, pc0, kv, kc, u, y0, llr, degv, degc, sig, vptr, cptr,
-      vadj, cadj, misc, total;
+  size_t mv, mc, op, as, ds, cs, bs, p0, pc0, kv, kc, u, y0, llr, sig,
+      vadj, cadj, vinfo, cinfo, misc, total;
 };
 
 __host__ __device__ inline size_t al(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -103,13 +109,11 @@ __host__ __device__ inline TcLay tc_layout(int m, int n, int E, int vt, int ct, 
   L.u = o; o += 128;
   L.y0 = o; o += al((size_t)n * 4, 16);
   L.llr = o; o += al(N * 4, 16);
-  L.degv = o; o += al((size_t)n * 4, 16);
-  L.degc = o; o += al((size_t)m * 4, 16);
   L.sig = o; o += al(M * 4, 16);
-  L.vptr = o; o += al((size_t)(n + 1) * 4, 16);          // the graph: CSC / CSR row starts
-  L.cptr = o; o += al((size_t)(m + 1) * 4, 16);
   L.vadj = o; o += al((size_t)E * 4, 16);                // per edge: row * 64 | swizzle bits
   L.cadj = o; o += al((size_t)E * 4, 16);
+  L.vinfo = o; o += al(N * 8, 16);                       // per row: its edges, its shot's rows
+  L.cinfo = o; o += al(M * 8, 16);
   L.misc = o; o += 64;                                   // kappa, TMEM address, mbarrier, flags
   L.total = o;
   return L;
@@ -160,14 +164,16 @@ __device__ __forceinline__ unsigned long long global_ns() {
 __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity) {
   const uint32_t a = smem_u32(mbar);
   uint32_t done = 0;
-  const unsigned long long t0 = global_ns();
-  while (true) {
+  unsigned long long t0 = 0;
+  for (int spin = 0;; ++spin) {
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
         "selp.u32 %0, 1, 0, p;\n}"
         : "=r"(done) : "r"(a), "r"(parity) : "memory");
     if (done) return true;
-    if (global_ns() - t0 > 1000000000ull) return false;
+    if (spin < 32) continue;
+    if (t0 == 0) t0 = global_ns();
+    else if (global_ns() - t0 > 1000000000ull) return false;
   }
 }
 
@@ -221,21 +227,38 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 // acc (8 FP32 values as four f32x2 pairs) += relu(p + q) for 8 BF16 pairs: the sum and the
-// relu in one packed BF16 FMA (one rounding), the accumulation in FP32.
+// relu in one packed BF16 FMA (one rounding), the accumulation in FP32 by the mixed-precision
+// add, which takes a BF16 half as it is (unpacking both halves with two logic instructions and
+// adding the pair: 8.95 ms for 200 000 BB144 shots instead of 8.49).
 __device__ __forceinline__ void relu_acc8(const uint4 p, const uint4 q, unsigned long long acc[4]) {
   const uint32_t pw[4] = {p.x, p.y, p.z, p.w}, qw[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     uint32_t d;
     asm("fma.rn.relu.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(pw[i]), "r"(0x3F803F80u), "r"(qw[i]));
-    unsigned long long x;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(d << 16), "r"(d & 0xffff0000u));
-    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[i]) : "l"(x));
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i]));
+    asm("{.reg .b16 l, h;\nmov.b32 {l, h}, %2;\nadd.f32.bf16 %0, l, %0;\nadd.f32.bf16 %1, h, %1;}"
+        : "+f"(lo), "+f"(hi) : "r"(d));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(acc[i]) : "f"(lo), "f"(hi));
   }
 }
-__device__ __forceinline__ void unpack_acc8(const unsigned long long acc[4], float s[8]) {
+// The 8 sums as BF16 (one 16-byte operand chunk).
+__device__ __forceinline__ uint4 pack_acc8(const unsigned long long acc[4]) {
+  uint32_t w[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) asm("mov.b64 {%0, %1}, %2;" : "=f"(s[2 * i]), "=f"(s[2 * i + 1]) : "l"(acc[i]));
+  for (int i = 0; i < 4; ++i) {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i]));
+    w[i] = pack2(lo, hi);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
+                                                   unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
 }
 
 // BF16 node rows [rows][32]: the 16-byte chunk b of row r sits at chunk b ^ ((r >> 1) & 3),
@@ -263,7 +286,7 @@ __host__ __device__ __forceinline__ int p0_index(int v, int o) {
 // hi for hf = 1).
 __device__ __forceinline__ void tc_half(uint32_t taddr, int hf, int r, int l, int n, bool check,
                                         int mode, float nb, const float* p0, const float* pc0,
-                                        const float* k, const float* deg, const float* sig,
+                                        const float* k, const uint2* info, const float* sig,
                                         unsigned char* dst) {
   const bool ok = l >= 0;
   float f[32];
@@ -288,9 +311,19 @@ __device__ __forceinline__ void tc_half(uint32_t taddr, int hf, int r, int l, in
     tmem_st16(taddr + hf * 32 + 16, f + 16);
   } else {
     tmem_ld32(taddr + hf * 32, f);
-    const float dk = ok ? nb * deg[l] : 0.f;
+    const uint32_t e = ok ? info[r].x : 0u;
+    const float dk = nb * (float)((e >> 16) - (e & 0xffffu));
+    unsigned long long dk2;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(dk2) : "f"(dk));
+    const ulonglong2* k2 = reinterpret_cast<const ulonglong2*>(k + hf * 32);
 #pragma unroll
-    for (int i = 0; i < 32; ++i) f[i] = fmaf(dk, k[hf * 32 + i], f[i]);
+    for (int i = 0; i < 16; ++i) {
+      const ulonglong2 kk = k2[i >> 1];
+      unsigned long long x;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(f[2 * i]), "f"(f[2 * i + 1]));
+      x = fma2(dk2, i & 1 ? kk.y : kk.x, x);
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(f[2 * i]), "=f"(f[2 * i + 1]) : "l"(x));
+    }
   }
   if (ok) {
 #pragma unroll
@@ -321,13 +354,11 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32, 1) prior_tc_kernel(TcArgs a)
   float* u = reinterpret_cast<float*>(smem + L.u);
   float* y0 = reinterpret_cast<float*>(smem + L.y0);
   float* llr = reinterpret_cast<float*>(smem + L.llr);
-  float* degv = reinterpret_cast<float*>(smem + L.degv);
-  float* degc = reinterpret_cast<float*>(smem + L.degc);
   float* sig = reinterpret_cast<float*>(smem + L.sig);
-  int* vptr = reinterpret_cast<int*>(smem + L.vptr);
-  int* cptr = reinterpret_cast<int*>(smem + L.cptr);
   uint32_t* vadj = reinterpret_cast<uint32_t*>(smem + L.vadj);
   uint32_t* cadj = reinterpret_cast<uint32_t*>(smem + L.cadj);
+  uint2* vinfo = reinterpret_cast<uint2*>(smem + L.vinfo);
+  uint2* cinfo = reinterpret_cast<uint2*>(smem + L.cinfo);
   float* kappa = reinterpret_cast<float*>(smem + L.misc);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L.misc + 8);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + L.misc + 16);
@@ -407,15 +438,21 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32, 1) prior_tc_kernel(TcArgs a)
 #pragma unroll 1
     for (int j = 0; j < HD; ++j) acc = fmaf(__ldg(P + POff::wo + j), h0[v * HD + j], acc);
     y0[v] = acc;
-    degv[v] = (float)(__ldg(a.var_ptr + v + 1) - __ldg(a.var_ptr + v));
   }
-  for (int c = tid; c < m; c += T) degc[c] = (float)(__ldg(a.chk_ptr + c + 1) - __ldg(a.chk_ptr + c));
-  for (int v = tid; v <= n; v += T) vptr[v] = __ldg(a.var_ptr + v);
-  for (int c = tid; c <= m; c += T) cptr[c] = __ldg(a.chk_ptr + c);
   for (int e = tid; e < a.E; e += T) {
     const uint32_t c = __ldg(a.var_chk + e), v = __ldg(a.chk_var + e);
     vadj[e] = (c << 6) | ((c >> 1) & 3u);
     cadj[e] = (v << 6) | ((v >> 1) & 3u);
+  }
+  // group row -> its edges (first | end << 16; none for a padding row) and the byte offset of
+  // its shot's rows of the other kind
+  for (int r = tid; r < NR; r += T) {
+    const int s = (int)__umulhi((uint32_t)r, a.inv_n8), v = r - s * n8;
+    vinfo[r] = make_uint2(v < n ? __ldg(a.var_ptr + v) | __ldg(a.var_ptr + v + 1) << 16 : 0, (s * m8) << 6);
+  }
+  for (int r = tid; r < MR; r += T) {
+    const int s = (int)__umulhi((uint32_t)r, a.inv_m8), c = r - s * m8;
+    cinfo[r] = make_uint2(c < m ? __ldg(a.chk_ptr + c) | __ldg(a.chk_ptr + c + 1) << 16 : 0, (s * n8) << 6);
   }
   __syncthreads();
   {  // the staging is done: operand rows past the last node stay zero (finite)
@@ -449,8 +486,11 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32, 1) prior_tc_kernel(TcArgs a)
                     unsigned char* lo, unsigned char* hi) {
     const int rows = check ? MR : NR, r8 = check ? m8 : n8, nn = check ? m : n;
     const uint32_t inv = check ? a.inv_m8 : a.inv_n8;
-    for (int i = 0; i < tiles; ++i) {
-      if (i * 128 + q * 32 >= rows) continue;
+    int k = wslot - rot;
+    if (k < 0) k += nq;
+    for (; k < 2 * tiles; k += nq) {
+      const int i = k >> 1, hf = k & 1;
+      if (i * 128 + q * 32 >= rows) break;
       const uint32_t taddr = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(col0 + 64 * i);
       const int r = i * 128 + q * 32 + lane;
       int l = -1;
@@ -458,15 +498,13 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32, 1) prior_tc_kernel(TcArgs a)
         l = r - (int)__umulhi((uint32_t)r, inv) * r8;
         if (l >= nn) l = -1;
       }
-      for (int hf = 0; hf < 2; ++hf) {
-        if ((2 * i + hf + rot) % nq != wslot) continue;
-        tc_half(taddr, hf, r, l, n, check, mode, nb, p0, pc0, check ? kc : kv,
-                check ? degc : degv, sig, hf ? hi : lo);
-      }
+      tc_half(taddr, hf, r, l, n, check, mode, nb, p0, pc0, check ? kc : kv, check ? cinfo : vinfo,
+              sig, hf ? hi : lo);
     }
   };
   // the MMA of `tiles` tiles: accumulators at column col0 + 64 i, operand tile i, weights w.
-  // The issuing thread alone waits for completion; the others wait at the barrier.
+  // The issuing thread alone waits for completion; the others wait at the barrier (all warps
+  // polling an mbarrier per tile, without that barrier, was slower: 9.08 -> 9.6 ms).
   auto mma_tiles = [&](int tiles, int col0, const unsigned char* w) -> bool {
     int ok = 1;
     if (tid == 0) {
@@ -512,35 +550,35 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32, 1) prior_tc_kernel(TcArgs a)
       // LLR update ----
       for (int base = warp * 32; base < 2 * NR; base += T) {
         const int task = base + lane, r = task >> 1, h = task & 1;
-        const int sh = (int)__umulhi((uint32_t)r, a.inv_n8), v = r - sh * n8;
-        const bool live = task < 2 * NR && v < n;
-        float s[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) s[k] = 0.f;
-        if (live) {
+        const uint2 info = task < 2 * NR ? vinfo[r] : make_uint2(0u, 0u);
+        const int e0 = (int)(info.x & 0xffffu), e1 = (int)(info.x >> 16);
+        unsigned long long acc0[4] = {0ull, 0ull, 0ull, 0ull}, acc1[4] = {0ull, 0ull, 0ull, 0ull};
+        if (e0 < e1) {
           const uint4 q0 = *row_chunk(bs, r, 2 * h), q1 = *row_chunk(bs, r, 2 * h + 1);
-          unsigned long long acc0[4] = {0ull, 0ull, 0ull, 0ull}, acc1[4] = {0ull, 0ull, 0ull, 0ull};
-          const uint32_t xo = (uint32_t)(sh * m8) << 6;  // the shot's check rows
-          const int e1 = vptr[v + 1];
-          for (int e = vptr[v]; e < e1; ++e) {
-            const uint32_t x = vadj[e] + xo;
-            relu_acc8(edge_chunk(as, x, 2 * h), q0, acc0);
-            relu_acc8(edge_chunk(as, x, 2 * h + 1), q1, acc1);
+          for (int e = e0; e < e1; ++e) {
+            const uint32_t x = vadj[e] + info.y;
+            const uint32_t o = (x & ~63u) + (((2 * h ^ x) & 3u) << 4);  // edge_chunk 2 h
+            relu_acc8(*reinterpret_cast<const uint4*>(as + o), q0, acc0);
+            relu_acc8(*reinterpret_cast<const uint4*>(as + (o ^ 16u)), q1, acc1);
           }
-          unpack_acc8(acc0, s);
-          unpack_acc8(acc1, s + 8);
         }
         if (!last && task < 2 * NR) {  // padding rows of the operand are zero
-          *reinterpret_cast<uint4*>(op + koff(r, 16 * h)) =
-              make_uint4(pack2(s[0], s[1]), pack2(s[2], s[3]), pack2(s[4], s[5]), pack2(s[6], s[7]));
-          *reinterpret_cast<uint4*>(op + koff(r, 16 * h + 8)) =
-              make_uint4(pack2(s[8], s[9]), pack2(s[10], s[11]), pack2(s[12], s[13]), pack2(s[14], s[15]));
+          *reinterpret_cast<uint4*>(op + koff(r, 16 * h)) = pack_acc8(acc0);
+          *reinterpret_cast<uint4*>(op + koff(r, 16 * h + 8)) = pack_acc8(acc1);
         }
-        float dot = 0.f;
+        const ulonglong2* u2 = reinterpret_cast<const ulonglong2*>(u + 16 * h);
+        unsigned long long d2 = 0ull;
 #pragma unroll
-        for (int k = 0; k < 16; ++k) dot = fmaf(u[16 * h + k], s[k], dot);
+        for (int k = 0; k < 4; ++k) {
+          const ulonglong2 uu = u2[k];
+          d2 = fma2(uu.x, k < 2 ? acc0[2 * k & 3] : acc1[2 * k & 3], d2);
+          d2 = fma2(uu.y, k < 2 ? acc0[(2 * k + 1) & 3] : acc1[(2 * k + 1) & 3], d2);
+        }
+        float dot, doth;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(dot), "=f"(doth) : "l"(d2));
+        dot += doth;
         dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-        if (live && h == 0) llr[r] += dot + degv[v] * kap;
+        if (task < 2 * NR && h == 0) llr[r] += dot + (float)(e1 - e0) * kap;
       }
       if (last) break;
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -555,18 +593,14 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32, 1) prior_tc_kernel(TcArgs a)
       // ---- X1: T_c = sum_v relu(C_v + D_c) ----
       for (int task = tid; task < 4 * MR; task += T) {
         const int r = task >> 2, b = task & 3;
-        const int sh = (int)__umulhi((uint32_t)r, a.inv_m8), c = r - sh * m8;
-        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (c < m) {
+        unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+        const uint2 info = cinfo[r];
+        const int e0 = (int)(info.x & 0xffffu), e1 = (int)(info.x >> 16);
+        if (e0 < e1) {
           const uint4 qd = *row_chunk(ds, r, b);
-          unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
-          const uint32_t xo = (uint32_t)(sh * n8) << 6;  // the shot's variable rows
-          const int e1 = cptr[c + 1];
-          for (int e = cptr[c]; e < e1; ++e) relu_acc8(edge_chunk(cs, cadj[e] + xo, b), qd, acc);
-          unpack_acc8(acc, s);
+          for (int e = e0; e < e1; ++e) relu_acc8(edge_chunk(cs, cadj[e] + info.y, b), qd, acc);
         }
-        *reinterpret_cast<uint4*>(op + koff(r, 8 * b)) =
-            make_uint4(pack2(s[0], s[1]), pack2(s[2], s[3]), pack2(s[4], s[5]), pack2(s[6], s[7]));
+        *reinterpret_cast<uint4*>(op + koff(r, 8 * b)) = pack_acc8(acc);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncthreads();
@@ -595,8 +629,8 @@ __global__ void __launch_bounds__(kTcMaxWarps * 32, 1) prior_tc_kernel(TcArgs a)
       if (s >= ns || c >= m) continue;
       unsigned par = sig[rr] < 0.f ? 1u : 0u;
       const float* ls = llr + s * n8;
-      const int e1 = cptr[c + 1];
-      for (int e = cptr[c]; e < e1; ++e) par ^= ls[cadj[e] >> 6] < 0.f;
+      const uint32_t ee = cinfo[rr].x;
+      for (uint32_t e = ee & 0xffffu; e < ee >> 16; ++e) par ^= ls[cadj[e] >> 6] < 0.f;
       if (par) s_bad[s] = 1;
     }
     __syncthreads();
