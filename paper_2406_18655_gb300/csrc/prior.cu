@@ -131,7 +131,7 @@ __global__ void sample_kernel(unsigned long long seed, long long first, long lon
 // One CTA owns one shot at a time; all node arrays live in shared memory.
 // ======================================================================================
 
-constexpr int kFwdWarps = 8;    // training kernel (warps 0-5 own the weight gradients)
+constexpr int kTrainWarps = 16;  // training kernel (warps 0-11 own the weight gradients, two each)
 constexpr int kInfWarps = 9;    // inference kernel: 9 warps give BB144's 9 variable tiles one each
 
 struct FwdArgs {
@@ -200,19 +200,27 @@ __device__ __forceinline__ int bsw(int r, int col) {
   return (r << 5) + ((((col >> 3) ^ ((r >> 1) & 3)) << 3) | (col & 7));
 }
 
+// Operand fragments by ldmatrix: four 8 x 8 blocks a load instead of four 32-bit loads (the
+// 8 rows of a block lie in different banks).
+__device__ __forceinline__ void ldm4(uint32_t r[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ void ldm4t(uint32_t r[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+// A operand: rows r0 .. r0+15, columns k0 .. k0+15.
 __device__ __forceinline__ void fa_sw(uint32_t a[4], const __nv_bfloat16* base, int r0, int k0,
                                       int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  a[0] = ld32(base + bsw(r0 + g, k0 + 2 * t));
-  a[1] = ld32(base + bsw(r0 + g + 8, k0 + 2 * t));
-  a[2] = ld32(base + bsw(r0 + g, k0 + 2 * t + 8));
-  a[3] = ld32(base + bsw(r0 + g + 8, k0 + 2 * t + 8));
+  ldm4(a, base + bsw(r0 + (lane & 15), k0 + 8 * (lane >> 4)));
 }
-__device__ __forceinline__ void fb_sw(uint32_t b[2], const __nv_bfloat16* base, int n0, int k0,
-                                      int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  b[0] = ld32(base + bsw(n0 + g, k0 + 2 * t));
-  b[1] = ld32(base + bsw(n0 + g, k0 + 2 * t + 8));
+// B operand: rows n0 .. n0+7 (output columns), all 32 columns: b[0..1] the first K = 16 step,
+// b[2..3] the second.
+__device__ __forceinline__ void fb_sw(uint32_t b[4], const __nv_bfloat16* base, int n0, int lane) {
+  ldm4(b, base + bsw(n0 + (lane & 7), 8 * (lane >> 3)));
 }
 
 struct FwdSmem {
@@ -290,12 +298,10 @@ __device__ __forceinline__ void g_step(const FwdSmem& S, int rows, int r0, bool 
     __syncwarp();  // the aggregate rows are overwritten by this warp's projections below
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        uint32_t bf[2];
-        fb_sw(bf, W2, nt * 8, j * 16, lane);
-        mma16816(c[nt], af[j], bf);
-      }
+      uint32_t bf[4];
+      fb_sw(bf, W2, nt * 8, lane);
+      mma16816(c[nt], af[0], bf);
+      mma16816(c[nt], af[1], bf + 2);
       const int col = nt * 8 + 2 * t;
       if (ra < rows) *reinterpret_cast<float2*>(h + fsw(ra, col)) = make_float2(c[nt][0], c[nt][1]);
       if (rb < rows) *reinterpret_cast<float2*>(h + fsw(rb, col)) = make_float2(c[nt][2], c[nt][3]);
@@ -349,12 +355,10 @@ __device__ __forceinline__ void g_step(const FwdSmem& S, int rows, int r0, bool 
       u[2] = fmaf(sb, ws[col], b1[col]);
       u[3] = fmaf(sb, ws[col + 1], b1[col + 1]);
     }
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      uint32_t bf[2];
-      fb_sw(bf, Wp, nt * 8, j * 16, lane);
-      mma16816(u, ah[j], bf);
-    }
+    uint32_t bf[4];
+    fb_sw(bf, Wp, nt * 8, lane);
+    mma16816(u, ah[0], bf);
+    mma16816(u, ah[1], bf + 2);
     __nv_bfloat16* P = nt < 4 ? (CHECK ? S.ac : S.cv) : (CHECK ? S.dc : S.bv);
     if (ra < rows) *reinterpret_cast<uint32_t*>(P + bsw(ra, col)) = pack2(u[0], u[1]);
     if (rb < rows) *reinterpret_cast<uint32_t*>(P + bsw(rb, col)) = pack2(u[2], u[3]);
@@ -370,9 +374,10 @@ __device__ __forceinline__ void unpack8(const uint4 v, float f[8]) {
   }
 }
 
-// The gather step for the 16 destination rows r0..r0+15 of one warp (4 lanes per row).
-__device__ __forceinline__ void x_tile(int count, int r0, const int32_t* __restrict__ ptr,
-                                       const uint16_t* __restrict__ adj,
+// The gather step for the 16 destination rows r0..r0+15 of one warp (4 lanes per row).  ptr and
+// adj may lie in shared memory (plain loads).
+__device__ __forceinline__ void x_tile(int count, int r0, const int32_t* ptr,
+                                       const uint16_t* adj,
                                        const __nv_bfloat16* src, __nv_bfloat16* dst, int lane) {
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
@@ -383,10 +388,10 @@ __device__ __forceinline__ void x_tile(int count, int r0, const int32_t* __restr
     unpack8(*dp, q);
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = 0.f;
-    const int e1 = __ldg(ptr + d + 1);
-    for (int e = __ldg(ptr + d); e < e1; ++e) {
+    const int e1 = ptr[d + 1];
+    for (int e = ptr[d]; e < e1; ++e) {
       float p[8];
-      unpack8(*reinterpret_cast<const uint4*>(src + bsw(__ldg(adj + e), 8 * b)), p);
+      unpack8(*reinterpret_cast<const uint4*>(src + bsw(adj[e], 8 * b)), p);
 #pragma unroll
       for (int k = 0; k < 8; ++k) acc[k] += fmaxf(p[k] + q[k], 0.f);
     }
@@ -553,7 +558,13 @@ struct TrainArgs {
   float* grads;
   double* loss;
   float inv_norm;
+  int E, graph_smem;       // graph_smem: the graph is staged behind the layout
 };
+
+// Shared memory of the staged graph.
+__host__ __device__ inline size_t train_graph_bytes(int m, int n, int E) {
+  return a16((size_t)(n + 1) * 4) + a16((size_t)(m + 1) * 4) + 2 * a16((size_t)E * 2);
+}
 
 struct TLay {
   int npad, mpad;
@@ -612,13 +623,12 @@ __device__ __forceinline__ void tile_mm(float acc[NT][4], const __nv_bfloat16* A
   fa_sw(af[0], A, r0, 0, lane);
   fa_sw(af[1], A, r0, 16, lane);
 #pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      uint32_t bf[2];
-      fb_sw(bf, Wt, w0 + nt * 8, j * 16, lane);
-      mma16816(acc[nt], af[j], bf);
-    }
+  for (int nt = 0; nt < NT; ++nt) {
+    uint32_t bf[4];
+    fb_sw(bf, Wt, w0 + nt * 8, lane);
+    mma16816(acc[nt], af[0], bf);
+    mma16816(acc[nt], af[1], bf + 2);
+  }
 }
 
 template <int NT>
@@ -662,39 +672,29 @@ __device__ __forceinline__ void tile_update_f32(float* h, const __nv_bfloat16* A
 __device__ __forceinline__ float bf_at(const __nv_bfloat16* base, int r, int c) {
   return __bfloat162float(base[bsw(r, c)]);
 }
-__device__ __forceinline__ uint32_t bf_pair(const __nv_bfloat16* base, int r0, int r1, int c) {
-  return pack_bf(base[bsw(r0, c)], base[bsw(r1, c)]);
-}
-
-// acc (32 x 32, j x k) += sum over rows of G[row][j] H[row][k]  (rows 0..K, K % 16 == 0; the
-// padding rows of G and H are zero)
-__device__ __forceinline__ void wgrad_mm(float acc[2][4][4], const __nv_bfloat16* G,
-                                         const __nv_bfloat16* H, int K, int lane) {
-  const int g = lane >> 2, t = lane & 3;
+// acc (rows j = 16 mt .. 16 mt + 15 of the 32 x 32 gradient, j x k) += sum over rows of
+// G[row][j] H[row][k]  (rows 0..K, K % 16 == 0; the padding rows of G and H are zero).  Two
+// warps share a gradient, 16 of its rows each: split over the summed rows instead, the sums
+// would be taken in another order.
+__device__ __forceinline__ void wgrad_mm(float acc[4][4], const __nv_bfloat16* G,
+                                         const __nv_bfloat16* H, int K, int mt, int lane) {
+  // transposed loads: blocks (k0, j), (k0, j + 8), (k0 + 8, j), (k0 + 8, j + 8) of G, and
+  // (k0, k), (k0 + 8, k), (k0, k + 8), (k0 + 8, k + 8) of H
+  const int l8 = lane & 7, b0 = (lane >> 3) & 1, b1 = lane >> 4;
+#pragma unroll 1
   for (int k0 = 0; k0 < K; k0 += 16) {
-    const int ka = k0 + 2 * t, kb = ka + 8;
-    uint32_t af[2][4];
+    uint32_t af[4], bf[2][4];
+    ldm4t(af, G + bsw(k0 + 8 * b1 + l8, 16 * mt + 8 * b0));
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      const int j = mt * 16 + g;
-      af[mt][0] = bf_pair(G, ka, ka + 1, j);
-      af[mt][1] = bf_pair(G, ka, ka + 1, j + 8);
-      af[mt][2] = bf_pair(G, kb, kb + 1, j);
-      af[mt][3] = bf_pair(G, kb, kb + 1, j + 8);
-    }
+    for (int np = 0; np < 2; ++np) ldm4t(bf[np], H + bsw(k0 + 8 * b0 + l8, 16 * np + 8 * b1));
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      uint32_t bf[2];
-      const int kk = nt * 8 + g;
-      bf[0] = bf_pair(H, ka, ka + 1, kk);
-      bf[1] = bf_pair(H, kb, kb + 1, kk);
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) mma16816(acc[mt][nt], af[mt], bf);
+    for (int np = 0; np < 2; ++np) {
+      mma16816(acc[2 * np], af, bf[np]);
+      mma16816(acc[2 * np + 1], af, bf[np] + 2);
     }
   }
 }
 
-// Copy `rows` rows of 32 BF16 values (row-major, global) into a swizzled shared array.
 __device__ __forceinline__ void load_rows(__nv_bfloat16* dst, const __nv_bfloat16* src, int rows) {
   for (int i = threadIdx.x; i < rows * 4; i += blockDim.x) {
     const int r = i >> 2, b = i & 3;
@@ -703,7 +703,12 @@ __device__ __forceinline__ void load_rows(__nv_bfloat16* dst, const __nv_bfloat1
   }
 }
 
-__global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArgs a) {
+// Training, one CTA per SM and shot.  Bound by latency between its barriers (issue 43 %); at 16
+// warps a shot's 14 row tiles are one pass, a weight gradient is shared by two warps, the row
+// sums run beside them, and the graph is read from shared memory.  4096 BB144 pairs, 4 rounds:
+// 1.81 ms with 8 warps and 32-bit (weight gradients: 16-bit) fragment loads, now 1.39; BB72
+// 1.06 -> 0.96.
+__global__ void __launch_bounds__(kTrainWarps * 32, 1) prior_train_kernel(TrainArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int m = a.m, n = a.n, R = a.rounds;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -734,6 +739,25 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
   float* gv = S.hv;  // after the forward pass: dL/dh_v, dL/dh_c
   float* gc = S.hc;
 
+  const int32_t *var_ptr = a.var_ptr, *chk_ptr = a.chk_ptr;
+  const uint16_t *var_chk = a.var_chk, *chk_var = a.chk_var;
+  if (a.graph_smem) {
+    unsigned char* q = smem + L.total;
+    int32_t* vp = reinterpret_cast<int32_t*>(q);
+    int32_t* cp = reinterpret_cast<int32_t*>(q += a16((size_t)(n + 1) * 4));
+    uint16_t* vc = reinterpret_cast<uint16_t*>(q += a16((size_t)(m + 1) * 4));
+    uint16_t* cv = reinterpret_cast<uint16_t*>(q += a16((size_t)a.E * 2));
+    for (int j = threadIdx.x; j <= n; j += blockDim.x) vp[j] = a.var_ptr[j];
+    for (int i = threadIdx.x; i <= m; i += blockDim.x) cp[i] = a.chk_ptr[i];
+    for (int e = threadIdx.x; e < a.E; e += blockDim.x) {
+      vc[e] = a.var_chk[e];
+      cv[e] = a.chk_var[e];
+    }
+    var_ptr = vp;
+    chk_ptr = cp;
+    var_chk = vc;
+    chk_var = cv;
+  }
   // ---- parameters, graph degrees, zero padding ----
   const float* P = a.params;
   for (int i = threadIdx.x; i < HD * HD; i += blockDim.x) {
@@ -790,34 +814,32 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
   auto save_hv = [&](int t) { return save + (size_t)t * n * HD; };
   auto save_hc = [&](int t) { return save + (size_t)(R + 1) * n * HD + (size_t)t * m * HD; };
 
-  float wacc[2][4][4];  // warps 0-5: one weight gradient (32 x 32)
+  float wacc[4][4];  // warps 0-11: 16 rows of a weight gradient (32 x 32), warp % 6 which
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) wacc[i][j][q] = 0.f;
+    for (int q = 0; q < 4; ++q) wacc[j][q] = 0.f;
   double loss_acc = 0.0;
 
   for (long long shot = blockIdx.x; shot < a.shots; shot += gridDim.x) {
     const uint8_t* sp = a.syndromes + shot * m;
     const uint8_t* ep = a.errors + shot * n;
     // ================= forward (prior_fwd_kernel, saving every state) =================
-    for (int tile = warp; tile < vt + ct; tile += kFwdWarps) {
+    for (int tile = warp; tile < vt + ct; tile += kTrainWarps) {
       if (tile < vt) g_step<false>(S, n, tile * 16, false, true, nullptr, lane, sp, save_hv(0));
       else g_step<true>(S, m, (tile - vt) * 16, false, true, nullptr, lane, sp, save_hc(0));
     }
     __syncthreads();
     for (int r = 0; r < R; ++r) {
       const bool last = r == R - 1;
-      for (int tile = warp; tile < vt; tile += kFwdWarps) {
-        x_tile(n, tile * 16, a.var_ptr, a.var_chk, S.ac, S.bv, lane);
+      for (int tile = warp; tile < vt; tile += kTrainWarps) {
+        x_tile(n, tile * 16, var_ptr, var_chk, S.ac, S.bv, lane);
         g_step<false>(S, n, tile * 16, true, !last, S.llr, lane, nullptr, save_hv(r + 1));
       }
       __syncthreads();
       if (last) break;
-      for (int tile = warp; tile < ct; tile += kFwdWarps) {
-        x_tile(m, tile * 16, a.chk_ptr, a.chk_var, S.cv, S.dc, lane);
+      for (int tile = warp; tile < ct; tile += kTrainWarps) {
+        x_tile(m, tile * 16, chk_ptr, chk_var, S.cv, S.dc, lane);
         g_step<true>(S, m, tile * 16, true, true, nullptr, lane, nullptr, save_hc(r + 1));
       }
       __syncthreads();
@@ -833,7 +855,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
     __syncthreads();
     {
       float dwo = 0.f, dbo = 0.f;
-      for (int v = warp; v < n; v += kFwdWarps) {
+      for (int v = warp; v < n; v += kTrainWarps) {
         dwo = fmaf(S.llr[v], S.hv[fsw(v, lane)], dwo);
         dbo += S.llr[v];
       }
@@ -860,7 +882,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
       }
       __syncthreads();
       // projections A, D (checks), B, C (variables); gT = W2vc^T g_hc'
-      for (int tile = warp; tile < vt + ct; tile += kFwdWarps) {
+      for (int tile = warp; tile < vt + ct; tile += kTrainWarps) {
         const int g = lane >> 2, t = lane & 3;
         if (tile < vt) {
           const int r0 = tile * 16;
@@ -903,8 +925,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
           float bvv[8];
           unpack8(*reinterpret_cast<const uint4*>(S.cv + bsw(v, 8 * b)), x0);
           unpack8(*reinterpret_cast<const uint4*>(S.bv + bsw(v, 8 * b)), bvv);
-          for (int e = a.var_ptr[v]; e < a.var_ptr[v + 1]; ++e) {
-            const int c = a.var_chk[e];
+          for (int e = var_ptr[v], e1 = var_ptr[v + 1]; e < e1; ++e) {
+            const int c = var_chk[e];
             float av[8], dv[8], tv[8];
             unpack8(*reinterpret_cast<const uint4*>(S.ac + bsw(c, 8 * b)), av);
             unpack8(*reinterpret_cast<const uint4*>(S.dc + bsw(c, 8 * b)), dv);
@@ -926,8 +948,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
           float tv[8];
           unpack8(*reinterpret_cast<const uint4*>(S.dc + bsw(c, 8 * b)), x0);
           unpack8(*reinterpret_cast<const uint4*>(gT + bsw(c, 8 * b)), tv);
-          for (int e = a.chk_ptr[c]; e < a.chk_ptr[c + 1]; ++e) {
-            const int v = a.chk_var[e];
+          for (int e = chk_ptr[c], e1 = chk_ptr[c + 1]; e < e1; ++e) {
+            const int v = chk_var[e];
             float cvv[8];
             unpack8(*reinterpret_cast<const uint4*>(S.cv + bsw(v, 8 * b)), cvv);
 #pragma unroll
@@ -949,13 +971,13 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
       }
       __syncthreads();
       // g_hv' += Uvc^T gC (and its BF16 copy);  g_hc = g_hc' + Vvc^T gD
-      for (int tile = warp; tile < vt + ct; tile += kFwdWarps) {
+      for (int tile = warp; tile < vt + ct; tile += kTrainWarps) {
         if (tile < vt) tile_update_f32(gv, gC, tile * 16, n, WT + 2 * HD * HD, ghv, lane);
         else tile_update_f32(gc, gD, (tile - vt) * 16, m, WT + 1 * HD * HD, nullptr, lane);
       }
       __syncthreads();
       // gS = W2cv^T g_hv'
-      for (int tile = warp; tile < vt; tile += kFwdWarps) {
+      for (int tile = warp; tile < vt; tile += kTrainWarps) {
         float acc[4][4] = {};
         tile_mm<4>(acc, ghv, tile * 16, WT + 3 * HD * HD, 0, lane);
         tile_store_bf16<4>(gS, tile * 16, n, acc, lane);
@@ -972,9 +994,9 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
           float sv[8];
           unpack8(*reinterpret_cast<const uint4*>(S.bv + bsw(v, 8 * b)), x0);
           unpack8(*reinterpret_cast<const uint4*>(gS + bsw(v, 8 * b)), sv);
-          for (int e = a.var_ptr[v]; e < a.var_ptr[v + 1]; ++e) {
+          for (int e = var_ptr[v], e1 = var_ptr[v + 1]; e < e1; ++e) {
             float av[8];
-            unpack8(*reinterpret_cast<const uint4*>(S.ac + bsw(a.var_chk[e], 8 * b)), av);
+            unpack8(*reinterpret_cast<const uint4*>(S.ac + bsw(var_chk[e], 8 * b)), av);
 #pragma unroll
             for (int k = 0; k < 8; ++k) acc[k] += (av[k] + x0[k] > 0.f) ? 1.f : 0.f;
           }
@@ -986,8 +1008,8 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
         } else {  // check c: gA_c = sum_v gS_v [A_c + B_v > 0]
           const int c = (i >> 2) - n;
           unpack8(*reinterpret_cast<const uint4*>(S.ac + bsw(c, 8 * b)), x0);
-          for (int e = a.chk_ptr[c]; e < a.chk_ptr[c + 1]; ++e) {
-            const int v = a.chk_var[e];
+          for (int e = chk_ptr[c], e1 = chk_ptr[c + 1]; e < e1; ++e) {
+            const int v = chk_var[e];
             float bvv[8], sv[8];
             unpack8(*reinterpret_cast<const uint4*>(S.bv + bsw(v, 8 * b)), bvv);
             unpack8(*reinterpret_cast<const uint4*>(gS + bsw(v, 8 * b)), sv);
@@ -1001,91 +1023,76 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 1) prior_train_kernel(TrainArg
       }
       __syncthreads();
       // g_hc += Ucv^T gA;  g_hv = g_hv' + Vcv^T gB;  then the parameter gradients of the round
-      for (int tile = warp; tile < vt + ct; tile += kFwdWarps) {
+      for (int tile = warp; tile < vt + ct; tile += kTrainWarps) {
         if (tile < vt) tile_update_f32(gv, gB, tile * 16, n, WT + 5 * HD * HD, nullptr, lane);
         else tile_update_f32(gc, gA, (tile - vt) * 16, m, WT + 4 * HD * HD, nullptr, lane);
       }
-      switch (warp) {
-        case 0: wgrad_mm(wacc, ghc, Tc, L.mpad, lane); break;   // dW2vc
-        case 1: wgrad_mm(wacc, gD, hcA, L.mpad, lane); break;   // dVvc
-        case 2: wgrad_mm(wacc, gC, hvB, L.npad, lane); break;   // dUvc
-        case 3: wgrad_mm(wacc, ghv, Sv, L.npad, lane); break;   // dW2cv
-        case 4: wgrad_mm(wacc, gA, hcA, L.mpad, lane); break;   // dUcv
-        case 5: wgrad_mm(wacc, gB, hvA, L.npad, lane); break;   // dVcv
-        case 6: {
-          float b2 = 0.f, ws = 0.f, b1 = 0.f;
-          for (int c = 0; c < m; ++c) {
-            const float gd = bf_at(gD, c, lane);
-            b2 = fmaf(S.degc[c], bf_at(ghc, c, lane), b2);
-            ws = fmaf(S.sig[c], gd, ws);
-            b1 += gd;
-          }
-          vg[VG_b2vc * HD + lane] += b2;
-          vg[VG_wsvc * HD + lane] += ws;
-          vg[VG_b1vc * HD + lane] += b1;
-          break;
+      // weighted and plain sums over the rows of G, lane = feature
+      auto sums = [&](const __nv_bfloat16* G, int rows, const float* wt, int slot_w, int slot_1) {
+        float sw = 0.f, s1 = 0.f;
+        for (int i = 0; i < rows; ++i) {
+          const float x = bf_at(G, i, lane);
+          sw = fmaf(wt[i], x, sw);
+          s1 += x;
         }
-        default: {
-          float b2 = 0.f, ws = 0.f, b1 = 0.f;
-          for (int v = 0; v < n; ++v) b2 = fmaf(S.degv[v], bf_at(ghv, v, lane), b2);
-          for (int c = 0; c < m; ++c) {
-            const float ga = bf_at(gA, c, lane);
-            ws = fmaf(S.sig[c], ga, ws);
-            b1 += ga;
-          }
-          vg[VG_b2cv * HD + lane] += b2;
-          vg[VG_wscv * HD + lane] += ws;
-          vg[VG_b1cv * HD + lane] += b1;
-          break;
-        }
+        vg[slot_w * HD + lane] += sw;
+        if (slot_1 >= 0) vg[slot_1 * HD + lane] += s1;
+      };
+      switch (warp < 12 ? warp % 6 : warp) {
+        case 0: wgrad_mm(wacc, ghc, Tc, L.mpad, warp / 6, lane); break;   // dW2vc
+        case 1: wgrad_mm(wacc, gD, hcA, L.mpad, warp / 6, lane); break;   // dVvc
+        case 2: wgrad_mm(wacc, gC, hvB, L.npad, warp / 6, lane); break;   // dUvc
+        case 3: wgrad_mm(wacc, ghv, Sv, L.npad, warp / 6, lane); break;   // dW2cv
+        case 4: wgrad_mm(wacc, gA, hcA, L.mpad, warp / 6, lane); break;   // dUcv
+        case 5: wgrad_mm(wacc, gB, hvA, L.npad, warp / 6, lane); break;   // dVcv
+        case 12: sums(gD, m, S.sig, VG_wsvc, VG_b1vc); break;
+        case 13: sums(ghc, m, S.degc, VG_b2vc, -1); break;
+        case 14: sums(ghv, n, S.degv, VG_b2cv, -1); break;
+        default: sums(gA, m, S.sig, VG_wscv, VG_b1cv); break;
       }
       __syncthreads();
     }
     // ================= the initial states =================
-    if (warp == 0) {
-      float d0 = 0.f, d1 = 0.f;
-      for (int v = 0; v < n; ++v) {
+    {
+      float d0 = 0.f, d1 = 0.f, e0 = 0.f, e1 = 0.f;
+      for (int v = warp; v < n; v += kTrainWarps) {
         const float z = fmaf(S.lam[v], S.vec[F_a0 * HD + lane], S.vec[F_a1 * HD + lane]);
         const float gz = z > 0.f ? gv[fsw(v, lane)] : 0.f;
         d0 = fmaf(gz, S.lam[v], d0);
         d1 += gz;
       }
-      vg[VG_a0 * HD + lane] += d0;
-      vg[VG_a1 * HD + lane] += d1;
-    } else if (warp == 1) {
-      float d0 = 0.f, d1 = 0.f;
-      for (int c = 0; c < m; ++c) {
+      for (int c = warp; c < m; c += kTrainWarps) {
         const float gcv = gc[fsw(c, lane)];
-        d0 = fmaf(S.sig[c], gcv, d0);
-        d1 += gcv;
+        e0 = fmaf(S.sig[c], gcv, e0);
+        e1 += gcv;
       }
-      vg[VG_u0 * HD + lane] += d0;
-      vg[VG_u1 * HD + lane] += d1;
+      atomicAdd(&vg[VG_a0 * HD + lane], d0);
+      atomicAdd(&vg[VG_a1 * HD + lane], d1);
+      atomicAdd(&vg[VG_u0 * HD + lane], e0);
+      atomicAdd(&vg[VG_u1 * HD + lane], e1);
     }
     __syncthreads();
   }
   // ---- flush the CTA's gradients ----
   float* G = a.grads;
-  if (warp < 6) {
+  if (warp < 12) {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
+    for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-      for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int j = mt * 16 + g + (q >> 1) * 8, k = nt * 8 + 2 * t + (q & 1);
-          int idx;
-          switch (warp) {
-            case 0: idx = POff::W2vc + j * HD + k; break;
-            case 1: idx = POff::W1vc + j * DIN + HD + k; break;
-            case 2: idx = POff::W1vc + j * DIN + k; break;
-            case 3: idx = POff::W2cv + j * HD + k; break;
-            case 4: idx = POff::W1cv + j * DIN + k; break;
-            default: idx = POff::W1cv + j * DIN + HD + k; break;
-          }
-          atomicAdd(&G[idx], wacc[mt][nt][q]);
+      for (int q = 0; q < 4; ++q) {
+        const int j = (warp / 6) * 16 + g + (q >> 1) * 8, k = nt * 8 + 2 * t + (q & 1);
+        int idx;
+        switch (warp % 6) {
+          case 0: idx = POff::W2vc + j * HD + k; break;
+          case 1: idx = POff::W1vc + j * DIN + HD + k; break;
+          case 2: idx = POff::W1vc + j * DIN + k; break;
+          case 3: idx = POff::W2cv + j * HD + k; break;
+          case 4: idx = POff::W1cv + j * DIN + k; break;
+          default: idx = POff::W1cv + j * DIN + HD + k; break;
         }
+        atomicAdd(&G[idx], wacc[nt][q]);
+      }
   }
   __syncthreads();
   for (int k = threadIdx.x; k < HD; k += blockDim.x) {
@@ -1130,7 +1137,7 @@ cudaError_t prior_config(int m, int n, int E, bool train, int* grid) {
   const size_t smem = prior_smem(m, n, E, train);
   if (smem > (size_t)max_smem) return cudaErrorInvalidValue;
   const void* fn = train ? (const void*)prior_train_kernel : (const void*)prior_fwd_kernel;
-  const int threads = (train ? kFwdWarps : kInfWarps) * 32;
+  const int threads = (train ? kTrainWarps : kInfWarps) * 32;
   err = allow_max_dynamic_smem(fn, max_smem);
   if (err != cudaSuccess) return err;
   int per_sm = 0;
@@ -1199,7 +1206,16 @@ cudaError_t launch_prior(bool train, int grid, const DevGraph& g, int rounds, co
   (void)llr_out;
   const long long blocks = shots < grid ? shots : grid;
   if (blocks <= 0) return cudaSuccess;
-  prior_train_kernel<<<(int)blocks, kFwdWarps * 32, train_layout(g.m, g.n).total, st>>>(a);
+  // the graph in shared memory when it fits behind the rest
+  int dev = 0, max_smem = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess)
+    err = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (err != cudaSuccess) return err;
+  const size_t base = train_layout(g.m, g.n).total, gb = train_graph_bytes(g.m, g.n, g.E);
+  a.E = g.E;
+  a.graph_smem = base + gb <= (size_t)max_smem ? 1 : 0;
+  prior_train_kernel<<<(int)blocks, kTrainWarps * 32, base + (a.graph_smem ? gb : 0), st>>>(a);
   return cudaGetLastError();
 }
 
