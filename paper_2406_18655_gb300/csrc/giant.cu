@@ -20,19 +20,18 @@
 // are copied into the root's (new) block at an offset, rows shifted by that many bits: the
 // row supports are disjoint, so the merged rows stay reduced.
 //
-// Per growth step (one host round trip):
+// All in one cooperative launch, a grid barrier after each phase.  Per growth step:
 //   find      every candidate fault offers its key to the growing clusters next to it
 //   union     each invalid cluster takes its best candidate; collisions unite clusters
-//   flatten   union-find paths compressed to one hop
-//   plan      slot offsets of absorbed clusters and of newly claimed detectors, per root
+//   plan      union-find paths compressed to one hop; slot offsets of absorbed clusters and of
+//             newly claimed detectors, per root
 //   relocate  a root that merged or outgrew its block moves to a new, larger block
-//   absorb    absorbed blocks copied (shifted) into their root's block
-//   claim     new detectors get slots; faults next to them become candidates
-//   add       each changed root adds its new columns in key order (on-the-fly elimination)
-//   collect   the invalid roots of the next step
+//   absorb    absorbed blocks copied (shifted) into their root's block; new detectors get slots,
+//             and faults next to them become candidates
+//   add       each changed root adds its new columns in key order (on-the-fly elimination);
+//             the invalid ones are the next step's
 #include <algorithm>
 #include <climits>
-#include <cstddef>
 #include <cstdint>
 #include <cstring>
 #include <new>
@@ -50,6 +49,10 @@ constexpr unsigned kFullMask = 0xffffffffu;
 constexpr unsigned long long kNoKey = ~0ull;
 constexpr int kWcMax = 8;                     // reduction words per lane
 constexpr int kMaxSlots = 32 * 32 * kWcMax;   // 8192 detectors per cluster
+constexpr int kLsdBlock = 1024;               // threads of a block of the persistent P-LSD
+constexpr int kTailClusters = 64;             // invalid clusters that one block goes on with
+// bound of its barrier waits: a step may hold thousands of eliminations in one large cluster
+constexpr long long kLsdLimitNs = 30000000000LL;
 constexpr int kUfLimit = 1 << 20;             // bound on union-find retries and path length
 // a minimum over an empty set (a check of degree 1): 2^100, as in the batch kernels
 constexpr float kEmptyMinF = 1267650600228229401496703205376.0f;
@@ -59,7 +62,7 @@ struct GCtr {
   int ns, nfront, unsolvable, overflow, uf_fail, too_big, ndep, dep_top;
   int bp_stop, bp_unsat[2], bp_iters, bp_conv, bp_fail;
   unsigned bar_arrive;  // grid barrier of the persistent BP launch
-  int nu, kappa;
+  int nu, kappa, steps, stuck;
   int ninv[2];
   // reset every step
   int nmerged, nchg, nnew, nclaim, bucket_top, pad;
@@ -79,7 +82,7 @@ struct GD {
   // per detector / per fault
   int *dlab, *lslot, *fst, *front;
   // per seed ordinal (at most m)
-  int *parent, *inv0, *inv1, *mlist, *chg, *cap, *nsl, *ncol, *valid, *grow, *mark, *extra,
+  int *parent, *inv0, *inv1, *mlist, *chg, *cap, *nsl, *ncol, *grow, *mark, *extra,
       *newslots, *aoff, *newcnt, *boff;
   unsigned long long *best, *blk;
   // per step lists (at most m entries each)
@@ -130,6 +133,15 @@ __device__ long long arena_alloc(const GD& g, size_t words) {
     return -1;
   }
   return (long long)off;
+}
+
+// Next place of a counter for each of the warp's active lanes, one atomic for all of them.
+__device__ __forceinline__ int take_place(int* ctr) {
+  const unsigned act = __activemask();
+  const int lane = threadIdx.x & 31, lead = __ffs(act) - 1;
+  int base = 0;
+  if (lane == lead) base = atomicAdd(ctr, __popc(act));
+  return __shfl_sync(act, base, lead) + __popc(act & ((1u << lane) - 1u));
 }
 
 __device__ __forceinline__ unsigned long long llr_key(float x, int j) {
@@ -468,6 +480,12 @@ __global__ void __launch_bounds__(256) gcopy_hard(GD g, uint8_t* __restrict__ co
 // P-LSD
 // ---------------------------------------------------------------------------------------
 
+// The threads that share a phase: the grid's, or one block's.
+struct Span {
+  long long tid, n;
+};
+__device__ __forceinline__ Span grid_span() { return {gtid(), gstride()}; }
+
 __device__ int gfind(const GD& g, int x) {
   const volatile int* par = g.parent;
   for (int it = 0; it < kUfLimit; ++it) {
@@ -499,58 +517,81 @@ __device__ void gunite(const GD& g, int a, int b) {
   atomicOr(&g.ctr->uf_fail, 1);
 }
 
-__device__ __forceinline__ void add_candidates(const GD& g, int d) {
-  for (int e = g.chk_ptr[d]; e < g.chk_ptr[d + 1]; ++e) {
-    const int f = g.chk_var[e];
-    if (atomicCAS(&g.fst[f], -2, -1) == -2) g.front[atomicAdd(&g.ctr->nfront, 1)] = f;
-  }
+__device__ __forceinline__ void add_candidate(const GD& g, int f) {
+  if (atomicCAS(&g.fst[f], -2, -1) == -2) g.front[take_place(&g.ctr->nfront)] = f;
 }
 
-__global__ void __launch_bounds__(256) glsd_reset(GD g) {
-  for (long long d = gtid(); d < g.m; d += gstride()) g.dlab[d] = -1;
-  for (long long j = gtid(); j < g.n; j += gstride()) g.fst[j] = -2;
+__device__ __forceinline__ void glsd_reset(const GD& g, const Span& S, uint8_t* corr) {
+  for (long long d = S.tid; d < g.m; d += S.n) g.dlab[d] = -1;
+  for (long long j = S.tid; j < g.n; j += S.n) g.fst[j] = -2;
+  for (long long j = S.tid; j < g.n; j += S.n) corr[j] = 0;
 }
 
 // One cluster per flipped detector (Alg. 2's initialization), each in a 32-slot block.
-__global__ void __launch_bounds__(256) glsd_seed(GD g, const uint8_t* __restrict__ s) {
+__device__ __forceinline__ void glsd_seed(const GD& g, const Span& S, const uint8_t* __restrict__ s) {
   constexpr int C = 32;
-  const size_t words = blk_words(C);
-  for (long long d = gtid(); d < g.m; d += gstride()) {
-    if (!s[d]) continue;
-    const int ord = atomicAdd(&g.ctr->ns, 1);
-    g.dlab[d] = ord;
-    g.lslot[d] = 0;
-    g.parent[ord] = ord;
-    g.inv0[ord] = ord;
-    const long long off = arena_alloc(g, words);
-    if (off < 0) continue;
-    g.blk[ord] = (unsigned long long)off;
-    g.cap[ord] = C;
-    g.nsl[ord] = 1;
-    g.ncol[ord] = 0;
-    g.valid[ord] = 0;
-    g.grow[ord] = 1;
-    g.best[ord] = kNoKey;
-    g.mark[ord] = 0;
-    g.extra[ord] = 0;
-    g.newslots[ord] = 0;
-    g.newcnt[ord] = 0;
-    g.depcnt[ord] = 0;
-    const Blk B = blk_at(g, (unsigned long long)off, C);
-    for (size_t w = 0; w < words; ++w) B.b[w] = 0u;
-    for (int p = 0; p < C; ++p) B.pcol()[p] = -1;
-    B.det()[0] = (int)d;
-    B.sred()[0] = 1u;
-    add_candidates(g, (int)d);
+  constexpr int words = 2 * C + 2 * C + 2;  // blk_words(C)
+  const int lane = threadIdx.x & 31;
+  for (long long d0 = (S.tid >> 5) * 32; d0 < g.m; d0 += S.n) {
+    const long long d = d0 + lane;
+    const bool seed = d < g.m && s[d] != 0;
+    const unsigned sb = __ballot_sync(kFullMask, seed);
+    if (sb == 0) continue;
+    // the warp's seeds take consecutive ordinals and blocks, and it clears the blocks together
+    const int cnt = __popc(sb), rank = __popc(sb & ((1u << lane) - 1u));
+    int ord0 = 0;
+    long long off0 = 0;
+    if (lane == 0) {
+      ord0 = atomicAdd(&g.ctr->ns, cnt);
+      atomicAdd(&g.ctr->ninv[0], cnt);
+      off0 = arena_alloc(g, (size_t)words * cnt);
+    }
+    ord0 = __shfl_sync(kFullMask, ord0, 0);
+    off0 = __shfl_sync(kFullMask, off0, 0);
+    const int ord = ord0 + rank;
+    if (seed) {
+      g.dlab[d] = ord;
+      g.lslot[d] = 0;
+      g.parent[ord] = ord;
+      g.inv0[ord] = ord;
+    }
+    if (off0 < 0) continue;  // (the whole warp)
+    for (int w = lane; w < words * cnt; w += 32)
+      g.arena[off0 + w] = (unsigned)(w % words - 2 * C) < (unsigned)C ? 0xffffffffu : 0u;  // pcol = -1
+    __syncwarp();
+    if (seed) {
+      const unsigned long long off = (unsigned long long)off0 + (unsigned long long)rank * words;
+      g.blk[ord] = off;
+      g.cap[ord] = C;
+      g.nsl[ord] = 1;
+      g.ncol[ord] = 0;
+      g.grow[ord] = 1;
+      g.best[ord] = kNoKey;
+      g.mark[ord] = 0;
+      g.extra[ord] = 0;
+      g.newslots[ord] = 0;
+      g.newcnt[ord] = 0;
+      g.depcnt[ord] = 0;
+      const Blk B = blk_at(g, off, C);
+      B.det()[0] = (int)d;
+      B.sred()[0] = 1u;
+    }
+    for (unsigned left = sb; left; left &= left - 1) {
+      const long long ds = d0 + __ffs(left) - 1;
+      for (int e = g.chk_ptr[ds] + lane; e < g.chk_ptr[ds + 1]; e += 32) add_candidate(g, g.chk_var[e]);
+    }
   }
 }
 
-__global__ void glsd_seed_count(GD g) { g.ctr->ninv[0] = g.ctr->ns; }
-
-// find_candidate: every live candidate offers its key to the growing roots next to it.
-__global__ void __launch_bounds__(256) glsd_find(GD g, const float* __restrict__ llr) {
+// find_candidate: every live candidate offers its key to the growing roots next to it.  The
+// step's counters are cleared here (nothing in this phase reads them).
+__device__ __forceinline__ void glsd_find(const GD& g, const Span& S, const float* __restrict__ llr, int par) {
+  if (S.tid == 0) {
+    g.ctr->nmerged = g.ctr->nchg = g.ctr->nnew = g.ctr->nclaim = g.ctr->bucket_top = 0;
+    g.ctr->ninv[par ^ 1] = 0;
+  }
   const int nf = g.ctr->nfront;
-  for (long long i = gtid(); i < nf; i += gstride()) {
+  for (long long i = S.tid; i < nf; i += S.n) {
     const int f = g.front[i];
     if (g.fst[f] != -1) continue;
     const unsigned long long key = llr_key(llr[f], f);
@@ -563,80 +604,114 @@ __global__ void __launch_bounds__(256) glsd_find(GD g, const float* __restrict__
   }
 }
 
-// parallel_union: each invalid cluster takes its pick; collisions unite.
-__global__ void __launch_bounds__(256) glsd_union(GD g, int par, int strict) {
+// The same from the side of a few growing roots: warps share the 32-slot chunks of each.
+__device__ __forceinline__ void glsd_find_roots(const GD& g, const Span& S,
+                                                const float* __restrict__ llr, int par) {
+  if (S.tid == 0) {
+    g.ctr->nmerged = g.ctr->nchg = g.ctr->nnew = g.ctr->nclaim = g.ctr->bucket_top = 0;
+    g.ctr->ninv[par ^ 1] = 0;
+  }
   const int cnt = g.ctr->ninv[par];
   const int* inv = par ? g.inv1 : g.inv0;
-  for (long long t = gtid(); t < cnt; t += gstride()) {
-    const int r = inv[t];
-    const unsigned long long key = g.best[r];
-    if (key == kNoKey) {
-      if (strict) atomicOr(&g.ctr->unsolvable, 1);  // LSD-mu: a full cluster just stops
-      continue;
-    }
-    const int f = (int)(key & 0xffffffffu);
-    const int old = atomicCAS(&g.fst[f], -1, r);
-    if (old == -1) {
-      const int k = atomicAdd(&g.ctr->nnew, 1);
-      g.nc_g[k] = f;
-      g.nc_r[k] = r;
-      g.nc_key[k] = key;
-    } else {
-      gunite(g, r, old);
-    }
-    for (int q = g.var_ptr[f]; q < g.var_ptr[f + 1]; ++q) {
-      const int d = g.var_chk[q];
-      const int o = atomicCAS(&g.dlab[d], -1, r);
-      if (o == -1) {
-        const int k = atomicAdd(&g.ctr->nclaim, 1);
-        g.cl_d[k] = d;
-        g.cl_r[k] = r;
-      } else if (o != r) {
-        gunite(g, r, o);
+  const int lane = threadIdx.x & 31;
+  const long long warp = S.tid >> 5, warps = S.n >> 5;
+  for (int t0 = 0; t0 < cnt; t0 += 32) {
+    const int mine = t0 + lane < cnt ? inv[t0 + lane] : 0;
+    const int nmine = t0 + lane < cnt ? g.nsl[mine] : 0;
+    for (int i = 0; i < min(32, cnt - t0); ++i) {
+      const int n = __shfl_sync(kFullMask, nmine, i);
+      const long long c0 = (warp + warps - i % warps) % warps;
+      if (c0 * 32 >= n) continue;
+      const int r = __shfl_sync(kFullMask, mine, i);
+      const Blk D = blk_of(g, r);
+      unsigned long long best = kNoKey;
+      for (long long c = c0; c * 32 < n; c += warps) {
+        const long long sl = c * 32 + lane;
+        if (sl >= n) continue;
+        const int d = D.det()[sl];
+        for (int e = g.chk_ptr[d]; e < g.chk_ptr[d + 1]; ++e) {
+          const int f = g.chk_var[e];
+          if (g.fst[f] == -1) best = min(best, llr_key(llr[f], f));
+        }
       }
+      for (int off = 16; off > 0; off >>= 1)
+        best = min(best, __shfl_xor_sync(kFullMask, best, off));
+      if (lane == 0 && best != kNoKey) atomicMin(&g.best[r], best);
     }
   }
 }
 
-__global__ void __launch_bounds__(256) glsd_flatten(GD g) {
-  const int ns = g.ctr->ns;
-  for (long long x = gtid(); x < ns; x += gstride()) g.parent[x] = gfind(g, (int)x);
+// parallel_union: each invalid cluster takes its pick; collisions unite.
+__device__ __forceinline__ void glsd_union(const GD& g, const Span& S, int par, int strict) {
+  const int cnt = g.ctr->ninv[par];
+  const int* inv = par ? g.inv1 : g.inv0;
+  const int per = 1 + g.dv;  // a thread per pick and per detector next to it
+  for (long long t = S.tid; t < (long long)cnt * per; t += S.n) {
+    const int r = inv[t / per], i = (int)(t % per);
+    const unsigned long long key = g.best[r];
+    if (key == kNoKey) {
+      if (strict && i == 0) atomicOr(&g.ctr->unsolvable, 1);  // LSD-mu: a full cluster just stops
+      continue;
+    }
+    const int f = (int)(key & 0xffffffffu);
+    if (i == 0) {
+      const int old = atomicCAS(&g.fst[f], -1, r);
+      if (old == -1) {
+        const int k = take_place(&g.ctr->nnew);
+        g.nc_g[k] = f;
+        g.nc_r[k] = r;
+        g.nc_key[k] = key;
+      } else {
+        gunite(g, r, old);
+      }
+      continue;
+    }
+    const int q = g.var_ptr[f] + i - 1;
+    if (q >= g.var_ptr[f + 1]) continue;
+    const int d = g.var_chk[q];
+    const int o = atomicCAS(&g.dlab[d], -1, r);
+    if (o == -1) {
+      const int k = take_place(&g.ctr->nclaim);
+      g.cl_d[k] = d;
+      g.cl_r[k] = r;
+    } else if (o != r) {
+      gunite(g, r, o);
+    }
+  }
 }
 
 __device__ __forceinline__ void mark_changed(const GD& g, int R) {
-  if (atomicCAS(&g.mark[R], 0, 1) == 0) g.chg[atomicAdd(&g.ctr->nchg, 1)] = R;
+  if (atomicCAS(&g.mark[R], 0, 1) == 0) g.chg[take_place(&g.ctr->nchg)] = R;
 }
 
 // Offsets inside each root's grown block: absorbed clusters, then new detectors; ranks of
-// the new columns.
-__global__ void __launch_bounds__(256) glsd_plan(GD g) {
+// the new columns.  The labels used below are left one hop from their root, with `flat` all
+// labels (a step without a union leaves them so).
+__device__ __forceinline__ void glsd_plan(const GD& g, const Span& S, bool flat) {
   const int nm = g.ctr->nmerged, nc = g.ctr->nclaim, nn = g.ctr->nnew;
-  for (long long t = gtid(); t < (long long)nm + nc + nn; t += gstride()) {
-    if (t < nm) {
-      const int A = g.mlist[t];
-      const int R = g.parent[A];
+  const int ns = flat && nm > 0 ? g.ctr->ns : 0;
+  for (long long x = S.tid; x < ns; x += S.n) g.parent[x] = gfind(g, (int)x);
+  for (long long t = S.tid; t < (long long)nm + nc + nn; t += S.n) {
+    const int k = (int)(t < nm ? t : t < nm + nc ? t - nm : t - nm - nc);
+    const int A = t < nm ? g.mlist[k] : t < nm + nc ? g.cl_r[k] : g.nc_r[k];
+    const int R = gfind(g, A);
+    g.parent[A] = R;
+    if (t < nm)
       g.aoff[A] = atomicAdd(&g.extra[R], g.nsl[A]);
-      mark_changed(g, R);
-    } else if (t < nm + nc) {
-      const int k = (int)(t - nm);
-      const int R = g.parent[g.cl_r[k]];
+    else if (t < nm + nc)
       g.cl_rel[k] = atomicAdd(&g.newslots[R], 1);
-      mark_changed(g, R);
-    } else {
-      const int k = (int)(t - nm - nc);
-      const int R = g.parent[g.nc_r[k]];
+    else
       g.nc_rank[k] = atomicAdd(&g.newcnt[R], 1);
-      mark_changed(g, R);
-    }
+    mark_changed(g, R);
   }
 }
 
 // A root that merged or outgrew its block moves to a new zeroed block (its own slots copied
 // at the same positions); every changed root reserves room for its new columns' list.
-__global__ void __launch_bounds__(256) glsd_relocate(GD g) {
+__device__ __forceinline__ void glsd_relocate(const GD& g, const Span& S) {
   const int lane = threadIdx.x & 31;
   const int nchg = g.ctr->nchg;
-  for (long long t = gwarp(); t < nchg; t += gwarps()) {
+  for (long long t = (S.tid >> 5); t < nchg; t += (S.n >> 5)) {
     const int R = g.chg[t];
     const int base = g.nsl[R];
     const int need = base + g.extra[R] + g.newslots[R];
@@ -691,10 +766,10 @@ __device__ __forceinline__ unsigned shifted_word(const unsigned* src, int sw, in
 }
 
 // Absorbed clusters copied into their root's block at their offset (rows shifted).
-__global__ void __launch_bounds__(256) glsd_absorb(GD g) {
+__device__ __forceinline__ void glsd_absorb(const GD& g, const Span& S) {
   const int lane = threadIdx.x & 31;
   const int nm = g.ctr->nmerged;
-  for (long long t = gwarp(); t < nm; t += gwarps()) {
+  for (long long t = (S.tid >> 5); t < nm; t += (S.n >> 5)) {
     const int A = g.mlist[t];
     const int R = g.parent[A];
     if (g.ctr->too_big || g.ctr->overflow) continue;
@@ -727,38 +802,43 @@ __global__ void __launch_bounds__(256) glsd_absorb(GD g) {
 
 // New detectors take their slots; faults next to them become candidates (Def. 4.3); the new
 // columns are placed in their root's list.
-__global__ void __launch_bounds__(256) glsd_claim(GD g) {
+__device__ __forceinline__ void glsd_claim(const GD& g, const Span& S) {
   const int nc = g.ctr->nclaim, nn = g.ctr->nnew;
   if (g.ctr->too_big || g.ctr->overflow) return;
-  for (long long t = gtid(); t < (long long)nc + nn; t += gstride()) {
-    if (t < nc) {
-      const int k = (int)t;
+  const int dc = g.dc;  // a thread per new detector and edge
+  for (long long t = S.tid; t < (long long)nc * dc + nn; t += S.n) {
+    if (t < (long long)nc * dc) {
+      const int k = (int)(t / dc), i = (int)(t % dc);
       const int d = g.cl_d[k];
-      const int R = g.parent[g.cl_r[k]];
-      const int slot = g.nsl[R] + g.extra[R] + g.cl_rel[k];
-      const Blk D = blk_of(g, R);
-      D.det()[slot] = d;
-      g.lslot[d] = slot;
-      add_candidates(g, d);
+      if (i == 0) {
+        const int R = g.parent[g.cl_r[k]];
+        const int slot = g.nsl[R] + g.extra[R] + g.cl_rel[k];
+        blk_of(g, R).det()[slot] = d;
+        g.lslot[d] = slot;
+      }
+      const int e = g.chk_ptr[d] + i;
+      if (e < g.chk_ptr[d + 1]) add_candidate(g, g.chk_var[e]);
     } else {
-      const int k = (int)(t - nc);
+      const int k = (int)(t - (long long)nc * dc);
       const int R = g.parent[g.nc_r[k]];
       g.bucket[g.boff[R] + g.nc_rank[k]] = k;
     }
   }
 }
 
-// Adds fault f to the elimination of block D (nslots slots in use), as the batch kernels do.
-__device__ void gadd_column(const GD& g, const Blk& D, int nslots, int f, int lane) {
+// Adds fault f to the elimination of block D (nslots slots in use), as the batch kernels do; WC: words
+// per lane (one holds 1024 slots, which few clusters outgrow).
+template <int WC>
+__device__ __forceinline__ void gadd_column(const GD& g, const Blk& D, int nslots, int f, int lane) {
   const int wc = (nslots + 31) >> 5;
-  unsigned bw[kWcMax], tw[kWcMax];
+  unsigned bw[WC], tw[WC];
 #pragma unroll
-  for (int c = 0; c < kWcMax; ++c) bw[c] = tw[c] = 0u;
+  for (int c = 0; c < WC; ++c) bw[c] = tw[c] = 0u;
   for (int q = g.var_ptr[f]; q < g.var_ptr[f + 1]; ++q) {
     const int sl = g.lslot[g.var_chk[q]];
     const bool piv = D.pcol()[sl] >= 0;
 #pragma unroll
-    for (int c = 0; c < kWcMax; ++c) {
+    for (int c = 0; c < WC; ++c) {
       const int w = c * 32 + lane;
       if (w < wc) {
         if ((sl >> 5) == w) bw[c] ^= 1u << (sl & 31);
@@ -771,7 +851,7 @@ __device__ void gadd_column(const GD& g, const Blk& D, int nslots, int f, int la
   }
   int p = -1;
 #pragma unroll
-  for (int c = 0; c < kWcMax; ++c) {
+  for (int c = 0; c < WC; ++c) {
     const unsigned nz = __ballot_sync(kFullMask, bw[c] != 0u);
     if (p < 0 && nz) {
       const int wl = __ffs(nz) - 1;
@@ -786,12 +866,12 @@ __device__ void gadd_column(const GD& g, const Blk& D, int nslots, int f, int la
   const int pw = p >> 5;
   const unsigned pb = 1u << (p & 31);
 #pragma unroll
-  for (int c = 0; c < kWcMax; ++c)
+  for (int c = 0; c < WC; ++c)
     if (c * 32 + lane == pw) tw[c] ^= pb;
   const bool sflag = (D.sred()[pw] & pb) != 0u;
   __syncwarp();
 #pragma unroll
-  for (int c = 0; c < kWcMax; ++c) {
+  for (int c = 0; c < WC; ++c) {
     const int w = c * 32 + lane;
     if (w < wc) {
       D.R(p)[w] = bw[c];
@@ -808,7 +888,7 @@ __device__ void gadd_column(const GD& g, const Blk& D, int nslots, int f, int la
       const int dd = d0 + __ffs(bal) - 1;
       bal &= bal - 1;
 #pragma unroll
-      for (int c = 0; c < kWcMax; ++c) {
+      for (int c = 0; c < WC; ++c) {
         const int w = c * 32 + lane;
         if (w < wc) {
           D.R(dd)[w] ^= bw[c];
@@ -820,7 +900,7 @@ __device__ void gadd_column(const GD& g, const Blk& D, int nslots, int f, int la
   }
   if (sflag) {
 #pragma unroll
-    for (int c = 0; c < kWcMax; ++c) {
+    for (int c = 0; c < WC; ++c) {
       const int w = c * 32 + lane;
       if (w < wc) {
         D.sred()[w] ^= bw[c];
@@ -831,65 +911,133 @@ __device__ void gadd_column(const GD& g, const Blk& D, int nslots, int f, int la
   __syncwarp();
 }
 
-// on_the_fly_elimination of every changed root: its new columns in key order, then its
-// validity.
-__global__ void __launch_bounds__(256) glsd_add(GD g) {
-  const int lane = threadIdx.x & 31;
-  const int nchg = g.ctr->nchg;
-  if (g.ctr->too_big || g.ctr->overflow) return;
-  for (long long t = gwarp(); t < nchg; t += gwarps()) {
-    const int R = g.chg[t];
-    const int nslots = g.nsl[R] + g.extra[R] + g.newslots[R];
-    const Blk D = blk_of(g, R);
-    const int cnt = g.newcnt[R];
-    const int* bk = g.bucket + g.boff[R];
-    unsigned long long last = 0;
-    for (int it = 0; it < cnt; ++it) {
-      unsigned long long best = kNoKey;
-      int bi = -1;
-      for (int u = lane; u < cnt; u += 32) {
-        const int k = bk[u];
-        const unsigned long long key = g.nc_key[k];
-        if ((it == 0 || key > last) && key < best) {
-          best = key;
-          bi = k;
-        }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(kFullMask, best, off);
-        const int oi = __shfl_xor_sync(kFullMask, bi, off);
-        if (ob < best) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      last = best;
-      gadd_column(g, D, nslots, g.nc_g[bi], lane);
+// The same by one thread, for a cluster of at most 32 slots: a row is one word.
+__device__ __forceinline__ void gadd_column_small(const GD& g, const Blk& D, int nslots, int f) {
+  unsigned bw = 0u, tw = 0u;
+  for (int q = g.var_ptr[f]; q < g.var_ptr[f + 1]; ++q) {
+    const int sl = g.lslot[g.var_chk[q]];
+    bw ^= 1u << sl;
+    if (D.pcol()[sl] >= 0) {
+      bw ^= D.R(sl)[0];
+      tw ^= D.T(sl)[0];
     }
-    bool any = false;
-    for (int w = lane; w < ((nslots + 31) >> 5); w += 32) any |= D.sred()[w] != 0u;
-    any = __any_sync(kFullMask, any);
-    if (lane == 0) {
-      g.valid[R] = any ? 0 : 1;
-      g.ncol[R] += cnt;
-      g.nsl[R] = nslots;
-      g.extra[R] = 0;
-      g.newslots[R] = 0;
-      g.newcnt[R] = 0;
-      g.mark[R] = 0;
+  }
+  if (bw == 0u) {
+    if (g.order > 0) g.dep_f[atomicAdd(&g.ctr->ndep, 1)] = f;
+    return;
+  }
+  const int p = __ffs(bw) - 1;
+  const unsigned pb = 1u << p;
+  tw ^= pb;
+  D.R(p)[0] = bw;
+  D.T(p)[0] = tw;
+  D.pcol()[p] = f;
+  for (int d = 0; d < nslots; ++d) {
+    if (d == p || D.pcol()[d] < 0) continue;
+    const unsigned r = D.R(d)[0];
+    if (r & pb) {
+      D.R(d)[0] = r ^ bw;
+      D.T(d)[0] ^= tw;
     }
+  }
+  if (D.sred()[0] & pb) {
+    D.sred()[0] ^= bw;
+    D.xsol()[0] ^= tw;
   }
 }
 
-__global__ void __launch_bounds__(256) glsd_collect(GD g, int par_next) {
-  const int ns = g.ctr->ns;
-  int* inv = par_next ? g.inv1 : g.inv0;
-  for (long long x = gtid(); x < ns; x += gstride()) {
-    const bool invalid = g.parent[x] == x && !g.valid[x];
-    g.grow[x] = invalid ? 1 : 0;
-    if (invalid) {
-      g.best[x] = kNoKey;
-      inv[atomicAdd(&g.ctr->ninv[par_next], 1)] = (int)x;
+// After the columns of root R: its sizes, and (collect) whether it grows in the next step.
+__device__ __forceinline__ void added(const GD& g, int R, int nslots, int cnt, bool invalid,
+                                      int par_next, bool collect) {
+  g.ncol[R] += cnt;
+  g.nsl[R] = nslots;
+  g.extra[R] = 0;
+  g.newslots[R] = 0;
+  g.newcnt[R] = 0;
+  g.mark[R] = 0;
+  if (!collect) return;
+  g.grow[R] = invalid ? 1 : 0;
+  if (invalid) {
+    g.best[R] = kNoKey;
+    (par_next ? g.inv1 : g.inv0)[atomicAdd(&g.ctr->ninv[par_next], 1)] = R;
+  }
+}
+
+// on_the_fly_elimination of every changed root: its new columns in key order, then its
+// validity; collect: the invalid ones are the next step's (an invalid root always changes: it
+// takes a fault, or unites with the cluster that took it, or the shot is unsolvable).  A warp
+// per root; where there are more roots than warps (the first steps: clusters of a few slots) a
+// warp takes `per` of them, a lane each, and works on the larger ones together.
+__device__ __forceinline__ void glsd_add(const GD& g, const Span& S, int par_next, bool collect) {
+  const int lane = threadIdx.x & 31;
+  const int nchg = g.ctr->nchg;
+  if (g.ctr->too_big || g.ctr->overflow) return;
+  const long long warps = S.n >> 5;
+  const int per = (int)min(32LL, (nchg + warps - 1) / warps);
+  for (long long t0 = (S.tid >> 5) * per; t0 < nchg; t0 += warps * per) {
+    const bool have = lane < per && t0 + lane < nchg;
+    const int mine = have ? g.chg[t0 + lane] : 0;
+    const int mslots = have ? g.nsl[mine] + g.extra[mine] + g.newslots[mine] : 0;
+    const bool small = have && per > 1 && mslots <= 32;
+    if (small) {
+      const Blk D = blk_of(g, mine);
+      const int cnt = g.newcnt[mine];
+      const int* bk = g.bucket + g.boff[mine];
+      unsigned long long last = 0;
+      for (int it = 0; it < cnt; ++it) {
+        unsigned long long best = kNoKey;
+        int bi = -1;
+        for (int u = 0; u < cnt; ++u) {
+          const int k = bk[u];
+          const unsigned long long key = g.nc_key[k];
+          if ((it == 0 || key > last) && key < best) {
+            best = key;
+            bi = k;
+          }
+        }
+        last = best;
+        gadd_column_small(g, D, mslots, g.nc_g[bi]);
+      }
+      added(g, mine, mslots, cnt, D.sred()[0] != 0u, par_next, collect);
+    }
+    __syncwarp();
+    for (unsigned left = __ballot_sync(kFullMask, have && !small); left; left &= left - 1) {
+      const int R = __shfl_sync(kFullMask, mine, __ffs(left) - 1);
+      const int nslots = __shfl_sync(kFullMask, mslots, __ffs(left) - 1);
+      const Blk D = blk_of(g, R);
+      const int cnt = g.newcnt[R];
+      const int* bk = g.bucket + g.boff[R];
+      unsigned long long last = 0;
+      for (int it = 0; it < cnt; ++it) {
+        unsigned long long best = kNoKey;
+        int bi = -1;
+        for (int u = lane; u < cnt; u += 32) {
+          const int k = bk[u];
+          const unsigned long long key = g.nc_key[k];
+          if ((it == 0 || key > last) && key < best) {
+            best = key;
+            bi = k;
+          }
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+          const unsigned long long ob = __shfl_xor_sync(kFullMask, best, off);
+          const int oi = __shfl_xor_sync(kFullMask, bi, off);
+          if (ob < best) {
+            best = ob;
+            bi = oi;
+          }
+        }
+        last = best;
+        if (nslots <= 1024)
+          gadd_column<1>(g, D, nslots, g.nc_g[bi], lane);
+        else
+          gadd_column<kWcMax>(g, D, nslots, g.nc_g[bi], lane);
+      }
+      bool any = false;
+      for (int w = lane; w < ((nslots + 31) >> 5); w += 32) any |= D.sred()[w] != 0u;
+      any = __any_sync(kFullMask, any);
+      if (lane == 0) added(g, R, nslots, cnt, any, par_next, collect);
+      __syncwarp();
     }
   }
 }
@@ -1093,16 +1241,22 @@ __global__ void __launch_bounds__(256) glsd_reprocess(GD g, const float* __restr
 }
 
 // Local solutions (Eq. 2): the pivot columns in each root's xsol; nu and kappa.
-__global__ void __launch_bounds__(256) glsd_solve(GD g, uint8_t* __restrict__ corr, int write) {
+__device__ __forceinline__ void glsd_solve(const GD& g, const Span& S, uint8_t* __restrict__ corr, bool write) {
   const int lane = threadIdx.x & 31;
   const int ns = g.ctr->ns;
-  for (long long x = gwarp(); x < ns; x += gwarps()) {
-    if (g.parent[x] != x) continue;
-    if (lane == 0) {
-      atomicAdd(&g.ctr->nu, 1);
-      atomicMax(&g.ctr->kappa, g.ncol[x]);
+  for (long long x0 = (S.tid >> 5) * 32; x0 < ns; x0 += S.n) {
+    const long long x = x0 + lane;
+    const bool root = x < ns && g.parent[x] == x;
+    const int nu = __popc(__ballot_sync(kFullMask, root));
+    const int kappa = __reduce_max_sync(kFullMask, root ? g.ncol[x] : 0);
+    if (lane == 0 && nu) {
+      atomicAdd(&g.ctr->nu, nu);
+      atomicMax(&g.ctr->kappa, kappa);
     }
-    if (!write) continue;
+  }
+  if (!write) return;
+  for (long long x = (S.tid >> 5); x < ns; x += (S.n >> 5)) {
+    if (g.parent[x] != x) continue;
     const Blk D = blk_of(g, (int)x);
     const int nx = g.nsl[x];
     for (int p = lane; p < nx; p += 32) {
@@ -1112,8 +1266,94 @@ __global__ void __launch_bounds__(256) glsd_solve(GD g, uint8_t* __restrict__ co
   }
 }
 
-__global__ void __launch_bounds__(256) gzero(uint8_t* __restrict__ p, long long nbytes) {
-  for (long long i = gtid(); i < nbytes; i += gstride()) p[i] = 0;
+// One phase per launch: LSD-mu's growth steps (every cluster grows, none is collected).
+enum Phase { kFind, kUnion, kPlan, kRelocate, kAbsorb, kAdd, kSolve };
+struct PhaseArgs {
+  const float* llr;
+  const uint8_t* s;
+  uint8_t* corr;
+};
+
+template <int P>
+__global__ void __launch_bounds__(256) glsd_phase(GD g, PhaseArgs a) {
+  const Span S = grid_span();
+  if constexpr (P == kFind) glsd_find(g, S, a.llr, 0);
+  if constexpr (P == kUnion) glsd_union(g, S, 0, 0);
+  if constexpr (P == kPlan) glsd_plan(g, S, true);
+  if constexpr (P == kRelocate) glsd_relocate(g, S);
+  if constexpr (P == kAbsorb) {
+    glsd_absorb(g, S);
+    glsd_claim(g, S);
+  }
+  if constexpr (P == kAdd) glsd_add(g, S, 1, false);
+  if constexpr (P == kSolve) glsd_solve(g, S, a.corr, true);
+}
+
+// P-LSD in one cooperative launch, a grid barrier between the phases: every block reads the
+// step's verdict from counters that do not change before the next barrier, so all leave the
+// loop together.  Bound by the latency of dependent loads and atomics: a thread or a warp per
+// item of a phase, and a barrier of about 2.5 us.  Most steps are the growth of a last few
+// clusters: from kTailClusters invalid ones on (their number never grows) block 0 goes on alone,
+// with barriers of its own and its L1 kept from phase to phase, and looks for candidates from the
+// clusters' side; the others wait at the last grid barrier.  640 000 faults at p = 0.03: 22 steps
+// 2.02 -> 0.71 ms, 3 steps 0.56 -> 0.36 (before: nine launches and a look by the host per step,
+// 79 us; all steps on the grid: 1.25 ms and 0.39).  kTailClusters 16: the same; 256: 0.78 and 0.43.
+__global__ void __launch_bounds__(kLsdBlock) glsd_persistent(GD g, PhaseArgs a, long long limit_ns) {
+  unsigned target = 0;
+  bool alone = false;
+  Span S = grid_span();
+  auto grid_sync = [&] {
+    target += gridDim.x;
+    return grid_barrier(g, target, limit_ns, &g.ctr->unsolvable, false) >= 0;
+  };
+  auto sync = [&] {
+    if (!alone) return grid_sync();
+    __syncthreads();
+    return true;
+  };
+  glsd_reset(g, S, a.corr);
+  if (!sync()) return;
+  glsd_seed(g, S, a.s);
+  if (!sync()) return;
+  int par = 0, steps = 0;
+  const auto failed = [&] { return (g.ctr->overflow | g.ctr->uf_fail | g.ctr->too_big) != 0; };
+  while (!failed() && !g.ctr->unsolvable && g.ctr->ninv[par] != 0 && steps <= g.n) {
+    if (!alone && g.ctr->ninv[par] <= kTailClusters) {
+      alone = true;
+      if (blockIdx.x != 0) break;
+      S = {(long long)threadIdx.x, (long long)blockDim.x};
+    }
+    if (alone)
+      glsd_find_roots(g, S, a.llr, par);
+    else
+      glsd_find(g, S, a.llr, par);
+    if (!sync()) return;
+    glsd_union(g, S, par, 1);
+    if (!sync()) return;
+    glsd_plan(g, S, !alone);
+    if (!sync()) return;
+    glsd_relocate(g, S);
+    if (!sync()) return;
+    glsd_absorb(g, S);
+    glsd_claim(g, S);
+    if (!sync()) return;
+    glsd_add(g, S, par ^ 1, true);
+    if (!sync()) return;
+    // a step in which some invalid cluster found no candidate does not count (Alg. 1)
+    if (g.ctr->unsolvable) break;
+    ++steps;
+    par ^= 1;
+  }
+  if (gtid() == 0) {
+    g.ctr->steps = steps;
+    g.ctr->stuck = g.ctr->unsolvable || (!failed() && g.ctr->ninv[par] != 0);
+  }
+  if (!grid_sync()) return;
+  S = grid_span();
+  const bool stuck = g.ctr->stuck != 0;
+  if (stuck || (g.order == 0 && !failed())) glsd_solve(g, S, a.corr, !stuck);
+  if (g.order > 0)  // LSD-mu's steps look labels up in one hop
+    for (long long x = S.tid; x < g.ctr->ns; x += S.n) g.parent[x] = gfind(g, (int)x);
 }
 
 }  // namespace
@@ -1135,6 +1375,7 @@ struct lsd_giant {
   const void* coop_fn = nullptr;
   int coop_block = 256, coop_cpt = 0, coop_vpt = 0;  // cpt > 0: gbp_resident
   size_t coop_smem = 0;
+  int lsd_grid = 1;  // blocks of glsd_persistent (1: no cooperative launch needed)
   long long bar_limit_ns = 1000000000LL;  // bound of a grid-barrier wait
   int hold_barrier = 0;                   // timeout test: block 0 withholds an arrival
 };
@@ -1174,103 +1415,52 @@ int check_launch(lsd_giant* G) {
   return e == cudaSuccess ? LSD_OK : gfail(e);
 }
 
+template <int P>
+int run_phase(lsd_giant* G, const PhaseArgs& a) {
+  glsd_phase<P><<<grid_threads(G), 256, 0, G->st>>>(G->g, a);
+  return check_launch(G);
+}
+
+int step_error(const GCtr& h) {
+  if (h.overflow) return LSD_ERR_ADMISSION;
+  if (h.uf_fail) return LSD_ERR_TIMEOUT;
+  if (h.too_big) return LSD_ERR_UNSUPPORTED;
+  return LSD_OK;
+}
+
 // P-LSD of the shot; writes corr (zero unless solved) and the info fields.
 int run_plsd(lsd_giant* G, const float* llr, const uint8_t* s, uint8_t* corr,
              lsd_giant_info* info) {
   const GD& g = G->g;
   const int grid = grid_threads(G);
+  const GCtr& h = *G->h_ctr;
+  PhaseArgs a{llr, s, corr};
   int rc;
-  // counters of the whole call (BP fields are kept)
-  {
-    cudaError_t e = cudaMemsetAsync(g.ctr, 0, offsetof(GCtr, bp_stop), G->st);
-    if (e == cudaSuccess)
-      e = cudaMemsetAsync(&g.ctr->nu, 0, sizeof(GCtr) - offsetof(GCtr, nu), G->st);
-    if (e != cudaSuccess) return gfail(e);
-  }
-  glsd_reset<<<grid, 256, 0, G->st>>>(g);
-  if ((rc = check_launch(G))) return rc;
-  glsd_seed<<<grid, 256, 0, G->st>>>(g, s);
-  if ((rc = check_launch(G))) return rc;
-  glsd_seed_count<<<1, 1, 0, G->st>>>(g);
-  if ((rc = check_launch(G))) return rc;
-  gzero<<<grid, 256, 0, G->st>>>(corr, G->n);
-  if ((rc = check_launch(G))) return rc;
-  int status = LSD_SHOT_OK_LSD, steps = 0, par = 0;
+  cudaError_t e = cudaMemsetAsync(g.ctr, 0, sizeof(GCtr), G->st);
+  if (e != cudaSuccess) return gfail(e);
+  long long limit = kLsdLimitNs;
+  void* args[] = {(void*)&g, (void*)&a, (void*)&limit};
+  const void* fn = (const void*)glsd_persistent;
+  e = G->lsd_grid > 1 ? cudaLaunchCooperativeKernel(fn, G->lsd_grid, kLsdBlock, args, 0, G->st)
+                      : cudaLaunchKernel(fn, 1, kLsdBlock, args, 0, G->st);
+  G->launches++;
+  if (e != cudaSuccess) return gfail(e);
   if ((rc = read_ctr(G))) return rc;
-  for (;;) {
-    const GCtr& h = *G->h_ctr;
-    if (h.overflow) return LSD_ERR_ADMISSION;
-    if (h.uf_fail) return LSD_ERR_TIMEOUT;
-    if (h.too_big) return LSD_ERR_UNSUPPORTED;
-    if (h.unsolvable) {
-      status = LSD_SHOT_UNSOLVABLE;
-      break;
-    }
-    if (h.ninv[par] == 0) break;
-    if (steps > G->n) {
-      status = LSD_SHOT_UNSOLVABLE;
-      break;
-    }
-    const int nxt = par ^ 1;
-    cudaError_t e = cudaMemsetAsync(&g.ctr->nmerged, 0, 6 * sizeof(int), G->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&g.ctr->ninv[nxt], 0, sizeof(int), G->st);
-    if (e != cudaSuccess) return gfail(e);
-    glsd_find<<<grid, 256, 0, G->st>>>(g, llr);
-    if ((rc = check_launch(G))) return rc;
-    glsd_union<<<grid, 256, 0, G->st>>>(g, par, 1);
-    if ((rc = check_launch(G))) return rc;
-    glsd_flatten<<<grid, 256, 0, G->st>>>(g);
-    if ((rc = check_launch(G))) return rc;
-    glsd_plan<<<grid, 256, 0, G->st>>>(g);
-    if ((rc = check_launch(G))) return rc;
-    glsd_relocate<<<grid, 256, 0, G->st>>>(g);
-    if ((rc = check_launch(G))) return rc;
-    glsd_absorb<<<grid, 256, 0, G->st>>>(g);
-    if ((rc = check_launch(G))) return rc;
-    glsd_claim<<<grid, 256, 0, G->st>>>(g);
-    if ((rc = check_launch(G))) return rc;
-    glsd_add<<<grid, 256, 0, G->st>>>(g);
-    if ((rc = check_launch(G))) return rc;
-    glsd_collect<<<grid, 256, 0, G->st>>>(g, nxt);
-    if ((rc = check_launch(G))) return rc;
-    // a step in which some invalid cluster found no candidate does not count (Alg. 1)
-    if ((rc = read_ctr(G))) return rc;
-    if (G->h_ctr->unsolvable) {
-      status = LSD_SHOT_UNSOLVABLE;
-      break;
-    }
-    ++steps;
-    par = nxt;
-  }
+  if (h.bp_fail) return LSD_ERR_TIMEOUT;
+  const bool unsolvable = h.stuck != 0;
+  if (!unsolvable && (rc = step_error(h))) return rc;
   // ---- LSD-mu: mu more steps in which every cluster grows, then local reprocessing ----
-  if (status == LSD_SHOT_OK_LSD && g.order > 0) {
-    for (int e = 0; e < g.order; ++e) {
-      cudaError_t err = cudaMemsetAsync(&g.ctr->nmerged, 0, 6 * sizeof(int), G->st);
-      if (err == cudaSuccess) err = cudaMemsetAsync(&g.ctr->ninv[par], 0, sizeof(int), G->st);
-      if (err != cudaSuccess) return gfail(err);
-      glsd_collect_all<<<grid, 256, 0, G->st>>>(g, par);
+  if (!unsolvable && g.order > 0) {
+    for (int k = 0; k < g.order; ++k) {
+      e = cudaMemsetAsync(g.ctr->ninv, 0, sizeof(g.ctr->ninv), G->st);
+      if (e != cudaSuccess) return gfail(e);
+      glsd_collect_all<<<grid, 256, 0, G->st>>>(g, 0);
       if ((rc = check_launch(G))) return rc;
-      glsd_find<<<grid, 256, 0, G->st>>>(g, llr);
-      if ((rc = check_launch(G))) return rc;
-      glsd_union<<<grid, 256, 0, G->st>>>(g, par, 0);
-      if ((rc = check_launch(G))) return rc;
-      glsd_flatten<<<grid, 256, 0, G->st>>>(g);
-      if ((rc = check_launch(G))) return rc;
-      glsd_plan<<<grid, 256, 0, G->st>>>(g);
-      if ((rc = check_launch(G))) return rc;
-      glsd_relocate<<<grid, 256, 0, G->st>>>(g);
-      if ((rc = check_launch(G))) return rc;
-      glsd_absorb<<<grid, 256, 0, G->st>>>(g);
-      if ((rc = check_launch(G))) return rc;
-      glsd_claim<<<grid, 256, 0, G->st>>>(g);
-      if ((rc = check_launch(G))) return rc;
-      glsd_add<<<grid, 256, 0, G->st>>>(g);
-      if ((rc = check_launch(G))) return rc;
-      if ((rc = read_ctr(G))) return rc;
-      const GCtr& h = *G->h_ctr;
-      if (h.overflow) return LSD_ERR_ADMISSION;
-      if (h.uf_fail) return LSD_ERR_TIMEOUT;
-      if (h.too_big) return LSD_ERR_UNSUPPORTED;
+      if ((rc = run_phase<kFind>(G, a)) || (rc = run_phase<kUnion>(G, a)) ||
+          (rc = run_phase<kPlan>(G, a)) || (rc = run_phase<kRelocate>(G, a)) ||
+          (rc = run_phase<kAbsorb>(G, a)) || (rc = run_phase<kAdd>(G, a)) ||
+          (rc = read_ctr(G)) || (rc = step_error(h)))
+        return rc;
       if (h.nnew == 0 && h.nclaim == 0 && h.nmerged == 0) break;  // nothing could grow
     }
     glsd_dep_rank<<<grid, 256, 0, G->st>>>(g);
@@ -1280,18 +1470,15 @@ int run_plsd(lsd_giant* G, const float* llr, const uint8_t* s, uint8_t* corr,
     glsd_dep_place<<<grid, 256, 0, G->st>>>(g);
     if ((rc = check_launch(G))) return rc;
     glsd_reprocess<<<grid, 256, 0, G->st>>>(g, llr, corr);
-    if ((rc = check_launch(G))) return rc;
+    if ((rc = check_launch(G)) || (rc = run_phase<kSolve>(G, a)) || (rc = read_ctr(G))) return rc;
   }
-  glsd_solve<<<grid, 256, 0, G->st>>>(g, corr, status == LSD_SHOT_OK_LSD ? 1 : 0);
-  if ((rc = check_launch(G))) return rc;
-  if ((rc = read_ctr(G))) return rc;
-  if (G->h_ctr->overflow) return LSD_ERR_ADMISSION;
+  if (h.overflow) return LSD_ERR_ADMISSION;
   if (info) {
-    info->status = status;
-    info->nu = G->h_ctr->nu;
-    info->kappa = G->h_ctr->kappa;
-    info->steps = steps;
-    info->arena_bytes_used = (int64_t)G->h_ctr->arena_top * 4;
+    info->status = unsolvable ? LSD_SHOT_UNSOLVABLE : LSD_SHOT_OK_LSD;
+    info->nu = h.nu;
+    info->kappa = h.kappa;
+    info->steps = h.steps;
+    info->arena_bytes_used = (int64_t)h.arena_top * 4;
   }
   return LSD_OK;
 }
@@ -1391,7 +1578,7 @@ int lsd_giant_create(lsd_giant** out, int32_t m, int32_t n, int64_t nnz, const i
   A(&g.fst, n);
   A(&g.front, n);
   for (int** p : {&g.parent, &g.inv0, &g.inv1, &g.mlist, &g.chg, &g.cap, &g.nsl, &g.ncol,
-                  &g.valid, &g.grow, &g.mark, &g.extra, &g.newslots, &g.aoff, &g.newcnt,
+                  &g.grow, &g.mark, &g.extra, &g.newslots, &g.aoff, &g.newcnt,
                   &g.boff, &g.nc_g, &g.nc_r, &g.nc_rank, &g.bucket, &g.cl_d, &g.cl_r,
                   &g.cl_rel})
     A(p, m);
@@ -1478,6 +1665,12 @@ int lsd_giant_create(lsd_giant** out, int32_t m, int32_t n, int64_t nnz, const i
         cudaGetLastError();
       }
     }
+    // persistent P-LSD: a block per SM, and no more than give every cluster there can be a warp
+    if (err == cudaSuccess && coop)
+      err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)glsd_persistent,
+                                                          kLsdBlock, 0);
+    if (err == cudaSuccess && coop && per_sm > 0)
+      G->lsd_grid = std::min(G->sms, (m + kLsdBlock / 32 - 1) / (kLsdBlock / 32));
     if (err != cudaSuccess) rc = gfail(err);
   }
   g.dc = dc;
