@@ -572,7 +572,7 @@ def giant_leg(args, stream):
         bd.close()
     return {"points": out, "hgp_3072x6400_one_shot": cmp,
             "note": "latency = host wall time of one synchronous decode (BP up to 100 "
-                    "iterations, then P-LSD with one host round trip per growth step)"}
+                    "iterations, then P-LSD in one launch with grid barriers)"}
 
 
 def hooks_leg(args, hx, hz, stream, flush, barrier, checker):

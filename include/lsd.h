@@ -88,9 +88,11 @@ typedef struct lsd_options {
                              padded), 3 = latency: of the CTA-per-shot register shapes that
                              fit, the one with the most threads (at least one fault per
                              thread), for small batches such as the server's; else as 0 */
-  int32_t lsd_kernel;     /* LSD kernel: 0 = auto, 1 = dense (state indexed by detector and
-                             fault, m <= 512, n <= 2048), 2 = sparse (state sized by what a shot
-                             touches; any m, n < 65536; no single_cluster) */
+  int32_t lsd_kernel;     /* LSD kernel: 0 = auto (dense up to 144 detectors and 288 faults and
+                             for single_cluster, else sparse), 1 = dense (a warp per shot, state
+                             indexed by detector and fault, m <= 512, n <= 2048), 2 = sparse (a
+                             CTA per shot, state sized by what a shot touches; any m,
+                             n < 65536; no single_cluster) */
   int32_t osd_method;     /* local reprocessing of LSD-mu (lsd_order > 0, App. D): 0 = exhaustive
                              OSD-E over the first mu dependent columns of each cluster
                              (lsd_order <= 12; default); 1 = combination sweep OSD-CS-w: no
@@ -238,9 +240,9 @@ int lsd_get_stats(lsd_decoder* dec, lsd_stats* stats);
  *   syndromes    device [shots][m] bytes.  corrections device [shots][n] bytes.
  *   status       device [shots] bytes, nullable.
  * Behaviour:
- *   - Decoders whose LSD runs in the sparse kernel (more than 512 detectors or 2048 faults:
- *     the large HGP and space-time matrices) are refused with LSD_ERR_UNSUPPORTED, since
- *     that kernel's per-warp scratch is not part of the array; so is a decoder without LSD.
+ *   - LSD runs in the dense kernel.  Decoders beyond it (more than 512 detectors or 2048
+ *     faults: the large HGP and space-time matrices) are refused with LSD_ERR_UNSUPPORTED,
+ *     since the sparse kernel's scratch is not part of the array; so is a decoder without LSD.
  *   - The first call on a device looks up the array's device address on that device (the
  *     current one); make that first call before any stream capture.  Later calls reuse it.
  *     A lookup that fails returns LSD_ERR_CUDA and is retried by the next call.
@@ -478,10 +480,9 @@ int lsd_giant_create(lsd_giant** out, int32_t m, int32_t n, int64_t nnz, const i
 
 /*
  * lsd_giant_decode -- BP (min-sum, flooding, early exit on H e_hat = s, Sec. 4.3), then
- * P-LSD on the posteriors when BP does not converge.  Synchronous (one host round trip per
- * growth step).  BP runs as one cooperative launch whose blocks meet at grid barriers; a
- * barrier that waits past its bound (about a second) makes the call return
- * LSD_ERR_TIMEOUT.
+ * P-LSD on the posteriors when BP does not converge.  Synchronous.  BP and P-LSD run as one
+ * cooperative launch each, whose blocks meet at grid barriers; a barrier that waits past its
+ * bound (about a second in BP, 30 seconds in P-LSD) makes the call return LSD_ERR_TIMEOUT.
  *   syndrome     device [m] bytes.   correction  device [n] bytes (written).
  *   posteriors   device [n] float32, nullable: the BP posteriors.
  *   info         host, nullable.
