@@ -509,7 +509,7 @@ __device__ void gunite(const GD& g, int a, int b) {
       b = t;
     }
     if (atomicCAS(g.parent + a, a, b) == a) {
-      const int k = atomicAdd(&g.ctr->nmerged, 1);
+      const int k = take_place(&g.ctr->nmerged);
       g.mlist[k] = a;
       return;
     }
@@ -527,59 +527,91 @@ __device__ __forceinline__ void glsd_reset(const GD& g, const Span& S, uint8_t* 
   for (long long j = S.tid; j < g.n; j += S.n) corr[j] = 0;
 }
 
-// One cluster per flipped detector (Alg. 2's initialization), each in a 32-slot block.
+// One cluster per flipped detector (Alg. 2's initialization), each in a 32-slot block: seed `ord`
+// takes the ord-th block of the arena.  The seeds' candidates are dealt to the lanes by (seed,
+// edge) and collected per block: an atomic on one counter per warp took as long as the rest.
 __device__ __forceinline__ void glsd_seed(const GD& g, const Span& S, const uint8_t* __restrict__ s) {
   constexpr int C = 32;
   constexpr int words = 2 * C + 2 * C + 2;  // blk_words(C)
-  const int lane = threadIdx.x & 31;
-  for (long long d0 = (S.tid >> 5) * 32; d0 < g.m; d0 += S.n) {
-    const long long d = d0 + lane;
+  constexpr int kFound = 2048;
+  __shared__ int s_found[kFound], s_det[32][32], s_cnt[32], s_nfound, s_base;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int dc = g.dc;
+  for (long long b0 = S.tid - threadIdx.x; b0 < g.m; b0 += S.n) {
+    const long long d = b0 + threadIdx.x;
     const bool seed = d < g.m && s[d] != 0;
     const unsigned sb = __ballot_sync(kFullMask, seed);
-    if (sb == 0) continue;
-    // the warp's seeds take consecutive ordinals and blocks, and it clears the blocks together
     const int cnt = __popc(sb), rank = __popc(sb & ((1u << lane) - 1u));
-    int ord0 = 0;
-    long long off0 = 0;
-    if (lane == 0) {
-      ord0 = atomicAdd(&g.ctr->ns, cnt);
-      atomicAdd(&g.ctr->ninv[0], cnt);
-      off0 = arena_alloc(g, (size_t)words * cnt);
+    if (seed) s_det[warp][rank] = (int)d;
+    if (lane == 0) s_cnt[warp] = cnt;
+    if (threadIdx.x == 0) s_nfound = 0;
+    __syncthreads();
+    // ordinals: the warps' counts summed by warp 0, one atomic for the block
+    if (warp == 0) {
+      const int mine = lane < (int)(blockDim.x >> 5) ? s_cnt[lane] : 0;
+      int pre = mine;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFullMask, pre, o);
+        if (lane >= o) pre += v;
+      }
+      int base = 0;
+      if (lane == 31 && pre) {
+        base = atomicAdd(&g.ctr->ns, pre);
+        atomicAdd(&g.ctr->ninv[0], pre);
+        atomicAdd(&g.ctr->arena_top, (unsigned long long)words * pre);
+      }
+      base = __shfl_sync(kFullMask, base, 31);
+      s_cnt[lane] = base + pre - mine;
     }
-    ord0 = __shfl_sync(kFullMask, ord0, 0);
-    off0 = __shfl_sync(kFullMask, off0, 0);
-    const int ord = ord0 + rank;
+    __syncthreads();
+    const int ord0 = s_cnt[warp];
+    const unsigned long long off0 = (unsigned long long)ord0 * words;
+    const bool fits = off0 + (unsigned long long)words * cnt <= g.arena_words;
+    if (cnt && !fits && lane == 0) atomicOr(&g.ctr->overflow, 1);
     if (seed) {
+      const int ord = ord0 + rank;
       g.dlab[d] = ord;
       g.lslot[d] = 0;
       g.parent[ord] = ord;
       g.inv0[ord] = ord;
     }
-    if (off0 < 0) continue;  // (the whole warp)
-    for (int w = lane; w < words * cnt; w += 32)
-      g.arena[off0 + w] = (unsigned)(w % words - 2 * C) < (unsigned)C ? 0xffffffffu : 0u;  // pcol = -1
-    __syncwarp();
-    if (seed) {
-      const unsigned long long off = (unsigned long long)off0 + (unsigned long long)rank * words;
-      g.blk[ord] = off;
-      g.cap[ord] = C;
-      g.nsl[ord] = 1;
-      g.ncol[ord] = 0;
-      g.grow[ord] = 1;
-      g.best[ord] = kNoKey;
-      g.mark[ord] = 0;
-      g.extra[ord] = 0;
-      g.newslots[ord] = 0;
-      g.newcnt[ord] = 0;
-      g.depcnt[ord] = 0;
-      const Blk B = blk_at(g, off, C);
-      B.det()[0] = (int)d;
-      B.sred()[0] = 1u;
+    if (fits) {
+      for (int w = lane; w < words * cnt; w += 32) {
+        const int q = w % words;  // pcol = -1, det[0] the seed, sred[0] = 1
+        g.arena[off0 + w] = (unsigned)(q - 2 * C) < (unsigned)C ? 0xffffffffu
+                            : q == 3 * C ? (unsigned)s_det[warp][w / words] : q == 4 * C ? 1u : 0u;
+      }
+      if (seed) {
+        const int ord = ord0 + rank;
+        g.blk[ord] = off0 + (unsigned long long)rank * words;
+        g.cap[ord] = C;
+        g.nsl[ord] = 1;
+        g.ncol[ord] = 0;
+        g.grow[ord] = 1;
+        g.best[ord] = kNoKey;
+        g.mark[ord] = 0;
+        g.extra[ord] = 0;
+        g.newslots[ord] = 0;
+        g.newcnt[ord] = 0;
+        g.depcnt[ord] = 0;
+      }
+      for (int i = lane; i < cnt * dc; i += 32) {
+        const int ds = s_det[warp][i / dc];
+        const int e = g.chk_ptr[ds] + i % dc;
+        if (e >= g.chk_ptr[ds + 1]) continue;
+        const int f = g.chk_var[e];
+        if (atomicCAS(&g.fst[f], -2, -1) != -2) continue;
+        const int k = atomicAdd(&s_nfound, 1);
+        if (k < kFound) s_found[k] = f;
+        else g.front[atomicAdd(&g.ctr->nfront, 1)] = f;
+      }
     }
-    for (unsigned left = sb; left; left &= left - 1) {
-      const long long ds = d0 + __ffs(left) - 1;
-      for (int e = g.chk_ptr[ds] + lane; e < g.chk_ptr[ds + 1]; e += 32) add_candidate(g, g.chk_var[e]);
-    }
+    __syncthreads();
+    const int nf = min(s_nfound, kFound);
+    if (threadIdx.x == 0 && nf) s_base = atomicAdd(&g.ctr->nfront, nf);
+    __syncthreads();
+    for (int k = threadIdx.x; k < nf; k += blockDim.x) g.front[s_base + k] = s_found[k];
+    __syncthreads();
   }
 }
 
@@ -765,38 +797,75 @@ __device__ __forceinline__ unsigned shifted_word(const unsigned* src, int sw, in
   return v;
 }
 
-// Absorbed clusters copied into their root's block at their offset (rows shifted).
+// The same for a cluster of at most 32 slots by one thread (into a fresh block: zero words are
+// left out).
+__device__ __forceinline__ void or_shifted(unsigned* dst, unsigned v, int o) {
+  const int q = o >> 5, b = o & 31;
+  if (v << b) atomicOr(&dst[q], v << b);
+  if (b && (v >> (32 - b))) atomicOr(&dst[q + 1], v >> (32 - b));
+}
+__device__ __forceinline__ void absorb_small(const GD& g, const Blk& A, const Blk& D, int o, int nA) {
+  or_shifted(D.sred(), A.sred()[0], o);
+  or_shifted(D.xsol(), A.xsol()[0], o);
+  for (int p = 0; p < nA; ++p) {
+    const int c = A.pcol()[p], d = A.det()[p];
+    D.pcol()[o + p] = c;
+    D.det()[o + p] = d;
+    g.lslot[d] = o + p;
+    if (c < 0) continue;
+    or_shifted(D.R(o + p), A.R(p)[0], o);
+    or_shifted(D.T(o + p), A.T(p)[0], o);
+  }
+}
+
+// Absorbed clusters copied into their root's block at their offset (rows shifted): a warp per
+// cluster; where there are more of them than warps (the first step: single seeds) a warp takes
+// `per`, a lane each, and the ones of more than 8 slots together.
 __device__ __forceinline__ void glsd_absorb(const GD& g, const Span& S) {
   const int lane = threadIdx.x & 31;
   const int nm = g.ctr->nmerged;
-  for (long long t = (S.tid >> 5); t < nm; t += (S.n >> 5)) {
-    const int A = g.mlist[t];
-    const int R = g.parent[A];
-    if (g.ctr->too_big || g.ctr->overflow) continue;
-    const Blk S = blk_of(g, A), D = blk_of(g, R);
-    const int o = g.nsl[R] + g.aoff[A];
-    const int nA = g.nsl[A];
-    for (int p = lane; p < nA; p += 32) {
-      D.pcol()[o + p] = S.pcol()[p];
-      const int d = S.det()[p];
-      D.det()[o + p] = d;
-      g.lslot[d] = o + p;
+  if (g.ctr->too_big || g.ctr->overflow) return;
+  const long long warps = S.n >> 5;
+  const int per = (int)min(32LL, (nm + warps - 1) / warps);
+  for (long long t0 = (S.tid >> 5) * per; t0 < nm; t0 += warps * per) {
+    const bool have = lane < per && t0 + lane < nm;
+    const int mine = have ? g.mlist[t0 + lane] : 0;
+    const int mroot = have ? g.parent[mine] : 0;
+    const int mn = have ? g.nsl[mine] : 0;
+    const int mo = have ? g.nsl[mroot] + g.aoff[mine] : 0;
+    const bool small = have && per > 1 && mn <= 8;
+    if (small) absorb_small(g, blk_of(g, mine), blk_of(g, mroot), mo, mn);
+    if (have) {
+      const int nc = g.ncol[mine];
+      if (nc) atomicAdd(&g.ncol[mroot], nc);
     }
-    const int w0 = o >> 5, w1 = min(D.W, ((o + nA + 31) >> 5) + 1);
-    for (int w = w0 + lane; w < w1; w += 32) {
-      const unsigned a = shifted_word(S.sred(), S.W, o, w);
-      const unsigned b = shifted_word(S.xsol(), S.W, o, w);
-      if (a) atomicOr(&D.sred()[w], a);
-      if (b) atomicOr(&D.xsol()[w], b);
-    }
-    for (int p = 0; p < nA; ++p) {
-      if (S.pcol()[p] < 0) continue;
+    __syncwarp();
+    for (unsigned left = __ballot_sync(kFullMask, have && !small); left; left &= left - 1) {
+      const int src = __ffs(left) - 1;
+      const Blk A = blk_of(g, __shfl_sync(kFullMask, mine, src));
+      const Blk D = blk_of(g, __shfl_sync(kFullMask, mroot, src));
+      const int o = __shfl_sync(kFullMask, mo, src), nA = __shfl_sync(kFullMask, mn, src);
+      for (int p = lane; p < nA; p += 32) {
+        D.pcol()[o + p] = A.pcol()[p];
+        const int d = A.det()[p];
+        D.det()[o + p] = d;
+        g.lslot[d] = o + p;
+      }
+      const int w0 = o >> 5, w1 = min(D.W, ((o + nA + 31) >> 5) + 1);
       for (int w = w0 + lane; w < w1; w += 32) {
-        D.R(o + p)[w] = shifted_word(S.R(p), S.W, o, w);
-        D.T(o + p)[w] = shifted_word(S.T(p), S.W, o, w);
+        const unsigned a = shifted_word(A.sred(), A.W, o, w);
+        const unsigned b = shifted_word(A.xsol(), A.W, o, w);
+        if (a) atomicOr(&D.sred()[w], a);
+        if (b) atomicOr(&D.xsol()[w], b);
+      }
+      for (int p = 0; p < nA; ++p) {
+        if (A.pcol()[p] < 0) continue;
+        for (int w = w0 + lane; w < w1; w += 32) {
+          D.R(o + p)[w] = shifted_word(A.R(p), A.W, o, w);
+          D.T(o + p)[w] = shifted_word(A.T(p), A.W, o, w);
+        }
       }
     }
-    if (lane == 0) atomicAdd(&g.ncol[R], g.ncol[A]);
   }
 }
 
@@ -1296,8 +1365,9 @@ __global__ void __launch_bounds__(256) glsd_phase(GD g, PhaseArgs a) {
 // clusters: from kTailClusters invalid ones on (their number never grows) block 0 goes on alone,
 // with barriers of its own and its L1 kept from phase to phase, and looks for candidates from the
 // clusters' side; the others wait at the last grid barrier.  640 000 faults at p = 0.03: 22 steps
-// 2.02 -> 0.71 ms, 3 steps 0.56 -> 0.36 (before: nine launches and a look by the host per step,
-// 79 us; all steps on the grid: 1.25 ms and 0.39).  kTailClusters 16: the same; 256: 0.78 and 0.43.
+// 2.02 -> 0.65 ms, 3 steps 0.56 -> 0.29 (before: nine launches and a look by the host per step,
+// 79 us; all steps on the grid: 1.25 ms and 0.39; seeds counted by warp and single seeds absorbed
+// by a warp each: 0.71 and 0.36).  kTailClusters 16: the same; 256: 0.07 ms longer.
 __global__ void __launch_bounds__(kLsdBlock) glsd_persistent(GD g, PhaseArgs a, long long limit_ns) {
   unsigned target = 0;
   bool alone = false;

@@ -21,7 +21,7 @@ def L():
 
 
 @pytest.mark.parametrize("name,p,copies,order", [
-    ("bb72", 0.08, 3000, 0), ("bb72", 0.08, 20, 0), ("bb72", 0.08, 2, 0), ("bb72", 0.06, 900, 3),
+    ("bb72", 0.08, 12000, 0), ("bb72", 0.08, 3000, 0), ("bb72", 0.08, 20, 0), ("bb72", 0.08, 2, 0), ("bb72", 0.06, 900, 3),
     ("irreg_37x61", 0.1, 2500, 0), ("ldpc_96x192", 0.06, 400, 0)])
 def test_direct_sum(L, name, p, copies, order):
     """A direct sum of blocks with a shot of the batch in each: clusters never leave their block,
