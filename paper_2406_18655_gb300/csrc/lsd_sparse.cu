@@ -388,22 +388,20 @@ __device__ __forceinline__ void pivot_update(const Shot<I>& S, int p, int g, uin
     for (uint32_t h = hit; h; h &= h - 1) S.flags()[tid + NT * (__ffs(h) - 1)] ^= 1;
 }
 
-// Keeps a dependent column for LSD-mu: its image is its combination of pivot rows.
+// Keeps a dependent column for LSD-mu: its image is its combination of pivot rows.  np counts
+// the ones without room too (the same in every thread; the caller compares it with CAP).
 template <class I>
 __device__ __forceinline__ void keep_dependent(const Shot<I>& S, int& np, int g, uint32_t hit, int tid) {
   if constexpr (I::MU) {
-    if (np >= I::CAP) {
-      S.sc->ovf = 1;
-      return;
-    }
+    if (np++ >= I::CAP) return;
+    const int at = np - 1;
 #pragma unroll
     for (int j = 0; j < I::RPT; ++j) {
       const unsigned b = __ballot_sync(kFull, (hit >> j) & 1u);
       const int w = I::NW * j + (tid >> 5);
-      if ((tid & 31) == 0 && w < S.words()) S.npN()[(size_t)np * S.words() + w] = b;
+      if ((tid & 31) == 0 && w < S.words()) S.npN()[(size_t)at * S.words() + w] = b;
     }
-    if (tid == 0) S.dpf()[np] = (uint16_t)g;
-    ++np;
+    if (tid == 0) S.dpf()[at] = (uint16_t)g;
   }
 }
 
@@ -532,7 +530,10 @@ __device__ __forceinline__ void add_columns(const SGraph& G, const Shot<I>& S, i
       const int r = S.inv()[c];
       atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
     }
-  if (tid == 0) S.sc->np = np;
+  if (tid == 0) {
+    S.sc->np = np;
+    if (np > I::CAP) S.sc->ovf = 1;
+  }
   __syncthreads();
 }
 
@@ -689,6 +690,10 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
 // searched, so the next pick is known when the validity is.  No other cluster grows, so the
 // absorbed clusters are relabelled at once and r stays the root.  Steps taken are added to
 // `steps`; returns as sparse_step (0: valid).  Needs columns of at most four detectors.
+// Every thread has to leave at the same barrier, so room is judged by counters that nobody
+// writes between the barrier after which they are read and the next one (nsl, nf), or that
+// every thread counts for itself (np): not by a flag, which a fast warp may set before a slow
+// one has read it.
 template <class I>
 __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, uint32_t r, int n,
                            int& steps, int tid) {
@@ -775,7 +780,6 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
         S.joined[g >> 5] |= 1u << (g & 31);
         sc.fresh = fb;
         sc.nsl = nsl + __popc(fb);
-        if (nsl + __popc(fb) > I::CAP) sc.ovf = 1;
       }
     }
     // the faults next to those detectors, asked for now and used if the detector is new: thread
@@ -788,9 +792,9 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
       if (d != kNone16) near = G.chk_pad[(size_t)d * D + (tid - kFrom) % D];
     }
     __syncthreads();
-    if (sc.ovf) return 3;
     const int nsl0 = nsl;
     nsl = sc.nsl;
+    if (nsl > I::CAP) return 3;
     const uint2 sl = sc.ssl, ml = sc.mlab;
     const unsigned fresh = sc.fresh;
     if ((ml.x & ml.y) != kFull) {
@@ -834,12 +838,13 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
     scan();
     publish();
     __syncthreads();
-    if (sc.ovf) return 3;
     const int p = sc.piv[it % 3];
     nf = sc.nf;
+    if (nf > S.lcap) return 3;
     fetch();
     if (p < 0) keep_dependent(S, np, g, hit, tid);
     else pivot_update(S, p, g, hit, nsl, tid);
+    if (I::MU && np > I::CAP) return 3;
     bool bad = false;
 #pragma unroll 1
     for (int i = tid; i < nsl; i += NT) bad |= (S.flags()[i] & 3) == 1;
@@ -848,7 +853,7 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
   }
   if (tid == 0) sc.np = np;
   __syncthreads();
-  return I::MU && sc.ovf ? 3 : 0;
+  return 0;
 }
 
 // ---- LSD-mu reprocessing, one warp per cluster ----

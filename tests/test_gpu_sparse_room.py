@@ -1,0 +1,63 @@
+"""Shots that outgrow the small instance of the CTA-per-shot LSD kernel, thousands at a time so
+that every CTA meets them one after another: all its threads have to see the want of room at the
+same barrier, or the CTA's later shots are decoded wrongly.  Every output is compared with the
+dense kernel's (itself pinned to the oracle elsewhere)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2406_18655_gb300 import inputs as I  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_2406_18655_gb300 import build, lsd
+    build.build()
+    lsd.lib()
+    return lsd
+
+
+def _columns(m, n, weight, seed):
+    """n columns of the given weight, spread evenly over the rows (no row beyond 32 edges)."""
+    rng = np.random.default_rng(seed)
+    while True:
+        h = np.zeros((m, n), np.uint8)
+        for j in range(n):
+            p = 1.0 / (1.0 + h.sum(1)) ** 4
+            h[rng.choice(m, weight, replace=False, p=p / p.sum()), j] = 1
+        if h.sum(1).max() <= 32:
+            return h
+
+
+def _compare(L, h, s, order, cs, seed):
+    n, shots = h.shape[1], s.shape[0]
+    llr = np.random.default_rng(seed).normal(1.5, 2.0, (shots, n)).astype(np.float32)
+    probs = np.full(n, 0.05, np.float32)
+    args = torch.from_numpy(llr).cuda(), torch.from_numpy(s).cuda()
+    got, want = (L.Decoder(h, probs, 5, order, osd_cs=cs, lsd_kernel=k).postprocess(*args)
+                 for k in (2, 1))
+    for a, b in zip(got[:2], want[:2]):
+        assert torch.equal(a, b)
+    ok = (want[1] == 2).cpu()  # (an unsolvable shot's statistics depend on where it stopped)
+    assert torch.equal(got[2].cpu()[ok], want[2].cpu()[ok])
+    return want[1].cpu().numpy()
+
+
+@pytest.mark.parametrize("order,cs", [(0, None), (3, 2)])
+def test_list_of_a_single_cluster(L, order, cs):
+    """One seed, columns of weight 3: its cluster lists more than 1536 faults before it is
+    valid."""
+    h = _columns(512, 2048, 3, 1)
+    s = np.zeros((4000, 512), np.uint8)
+    s[np.arange(4000), np.random.default_rng(2).integers(0, 512, 4000)] = 1
+    assert 2 in _compare(L, h, s, order, cs, 3)
+
+
+def test_dependent_columns_of_a_single_cluster(L):
+    """One seed and columns of even weight: no solution, and 1201 dependent columns on the way."""
+    h = _columns(300, 1500, 4, 4)
+    s = np.zeros((2000, 300), np.uint8)
+    s[np.arange(2000), np.random.default_rng(5).integers(0, 300, 2000)] = 1
+    assert set(_compare(L, h, s, 2, None, 6)) == {3}
