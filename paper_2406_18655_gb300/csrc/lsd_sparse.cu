@@ -140,12 +140,14 @@ struct SGraph {
   int max_col_deg, max_row_deg;
 };
 
-struct Scal {        // shared scalars
+// Shared scalars.  nsl, nf and np go on counting past the arrays' ends: a shot has outgrown the
+// instance when one of them has, which is looked at after a barrier that no writer of that
+// counter passes before the next one, so that all threads see the same.
+struct Scal {
   int ns, nsl, nf;   // seeds, slots, candidates so far
   int n_new, merged; // columns and merges of the step
   int ng, ncr;       // growing clusters; clusters with new columns
-  int np, ext;       // dependent columns kept for LSD-mu; those in the solution
-  int ovf;
+  int np, ext;       // dependent columns for LSD-mu; those in the solution
   int piv[3];
   unsigned item;
   uint2 ssl;         // the single cluster's new column: slots of its detectors,
@@ -237,10 +239,7 @@ __device__ __forceinline__ void claim(const Shot<I>& S, int d, int r) {
   const uint32_t o = atomicCAS(&S.lab[d], kFree, ((uint32_t)r << 16) | 0xffffu);
   if (o == kFree) {
     const int sl = atomicAdd(&S.sc->nsl, 1);
-    if (sl >= I::CAP) {
-      S.sc->ovf = 1;
-      return;
-    }
+    if (sl >= I::CAP) return;
     S.lab[d] = ((uint32_t)r << 16) | (uint32_t)sl;
     S.sdet()[sl] = (uint16_t)d;
     S.slab()[sl] = (uint16_t)r;
@@ -290,10 +289,7 @@ __device__ __forceinline__ int list_candidate(const SGraph& G, const Shot<I>& S,
   const uint32_t b = 1u << (f & 31);
   if ((atomicOr(&S.cand[f >> 5], b) & b) != 0) return -1;
   const int q = atomicAdd(&S.sc->nf, 1);
-  if (q >= S.lcap) {
-    S.sc->ovf = 1;
-    return -1;
-  }
+  if (q >= S.lcap) return -1;
   v = G.var_pad[f];
   k = llr_bits(llr[f]);
   S.lf[q] = (uint16_t)f;
@@ -451,10 +447,7 @@ __device__ void add_columns_by_warp(const Shot<I>& S, int n_new, int nsl, int ti
             int k = 0;
             if (lane == 0) k = atomicAdd(&S.sc->np, 1);
             k = __shfl_sync(kFull, k, 0);
-            if (k >= CAP) {
-              S.sc->ovf = 1;
-              continue;
-            }
+            if (k >= CAP) continue;
             uint32_t* const row = S.npN() + (size_t)k * S.words();
 #pragma unroll 1
             for (int w = lane; w < S.words(); w += 32) row[w] = 0u;
@@ -530,10 +523,7 @@ __device__ __forceinline__ void add_columns(const SGraph& G, const Shot<I>& S, i
       const int r = S.inv()[c];
       atomicAnd(&S.growb()[r >> 5], ~(1u << (r & 31)));
     }
-  if (tid == 0) {
-    S.sc->np = np;
-    if (np > I::CAP) S.sc->ovf = 1;
-  }
+  if (tid == 0) S.sc->np = np;
   __syncthreads();
 }
 
@@ -628,8 +618,8 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
   }
   __syncthreads();
   if (stop) return strict && none ? 1 : 2;
-  if (sc.ovf) return 3;
   const int nsl = sc.nsl, n_new = sc.n_new;
+  if (nsl > I::CAP) return 3;
   // ---- labels to roots after a merge ----
   if (sc.merged) {
     const int ns = sc.ns;
@@ -670,10 +660,10 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
     }
   }
   __syncthreads();
-  if (sc.ovf) return 3;
+  if (sc.nf > S.lcap) return 3;
   if (tid == 0) sc.n_new = sc.merged = 0;
   add_columns(G, S, n_new, nsl, tid);
-  if (I::MU && sc.ovf) return 3;
+  if (I::MU && sc.np > I::CAP) return 3;
   if (n_new > 1 && G.max_col_deg > 4) {  // (the marks of the clusters with columns, unused there)
 #pragma unroll 1
     for (int c = tid; c < sc.ncr; c += NT) {
@@ -692,8 +682,7 @@ __device__ int sparse_step(const SGraph& G, const Shot<I>& S, const float* llr, 
 // `steps`; returns as sparse_step (0: valid).  Needs columns of at most four detectors.
 // Every thread has to leave at the same barrier, so room is judged by counters that nobody
 // writes between the barrier after which they are read and the next one (nsl, nf), or that
-// every thread counts for itself (np): not by a flag, which a fast warp may set before a slow
-// one has read it.
+// every thread counts for itself (np).
 template <class I>
 __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, uint32_t r, int n,
                            int& steps, int tid) {
@@ -1140,7 +1129,7 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
 #pragma unroll 1
     for (int w = tid; w < I::SC / 32; w += NT) S.growb()[w] = 0u;
     if (tid == 0) {
-      sc.ns = sc.nf = sc.n_new = sc.merged = sc.ng = sc.np = sc.ovf = sc.ext = 0;
+      sc.ns = sc.nf = sc.n_new = sc.merged = sc.ng = sc.np = sc.ext = 0;
       sc.item = gridDim.x + (unsigned)atomicAdd(next, 1ULL);
     }
     __syncthreads();
@@ -1181,7 +1170,7 @@ lsd_sparse_kernel(LSDArgs a, unsigned char* scratch, size_t stride, int* spill, 
       if (tid == 0) sc.nsl = ns;
       open_slots(G, S, llr, 0, ns, tid);
       __syncthreads();
-      if (sc.ovf) status = kSpill;
+      if (sc.nf > S.lcap) status = kSpill;
     }
 
     // ---- LSD-0: grow every invalid cluster until all are valid ----

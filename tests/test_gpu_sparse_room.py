@@ -61,3 +61,27 @@ def test_dependent_columns_of_a_single_cluster(L):
     s = np.zeros((2000, 300), np.uint8)
     s[np.arange(2000), np.random.default_rng(5).integers(0, 300, 2000)] = 1
     assert set(_compare(L, h, s, 2, None, 6)) == {3}
+
+
+@pytest.mark.parametrize("order,cs", [(0, None), (3, 2)])
+def test_list_of_many_clusters(L, order, cs):
+    """30 seeds list some 350 faults, and more than 1536 after four steps of all of them."""
+    h = _columns(512, 2048, 3, 1)
+    rng = np.random.default_rng(7)
+    s = np.zeros((4000, 512), np.uint8)
+    for row in s:
+        row[rng.choice(512, 30, replace=False)] = 1
+    assert 2 in _compare(L, h, s, order, cs, 8)
+
+
+@pytest.mark.parametrize("rows", [8, 33])
+def test_dependent_columns_of_many_clusters(L, rows):
+    """A direct sum of blocks with a seed in each, grown until all its columns are in: 960 (of
+    clusters that a warp takes) or 924 dependent columns (of clusters that the CTA takes)."""
+    b = _columns(rows, 3 * rows, 3, 9)
+    blocks = 480 // rows
+    h = np.kron(np.eye(blocks, dtype=np.uint8), b)
+    s = np.zeros((1000, h.shape[0]), np.uint8)
+    for k in range(blocks):
+        s[np.arange(1000), k * rows + np.random.default_rng(k).integers(0, rows, 1000)] = 1
+    assert 2 in _compare(L, h, s, 3 * rows, 4, 10)
