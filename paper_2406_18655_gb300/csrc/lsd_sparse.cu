@@ -731,14 +731,13 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
   bk = bx = kNoKey;
   scan();
   publish();
-  if (tid == 0) {
-    S.growb()[r >> 5] = 0u;
-    sc.ng = 0;
-    sc.merged = 0;
-    sc.piv[0] = -1;
-  }
+  if (tid == 0) sc.piv[0] = -1;
   __syncthreads();
   fetch();
+  if (tid == 0) {  // (after the barrier: the caller's threads read ng after the one before it)
+    S.growb()[r >> 5] = 0u;
+    sc.ng = sc.merged = 0;
+  }
 #pragma unroll 1
   for (int it = 0;; ++it) {
     if (bx == kNoKey) return 1;

@@ -1,12 +1,14 @@
-"""Shots that outgrow the small instance of the CTA-per-shot LSD kernel, thousands at a time so
-that every CTA meets them one after another: all its threads have to see the want of room at the
-same barrier, or the CTA's later shots are decoded wrongly.  Every output is compared with the
+"""Shots that outgrow the small instance of the CTA-per-shot LSD kernel, or change from many
+growing clusters to one, thousands at a time so that every CTA meets them one after another: all
+its threads have to take each turn at the same barrier, or the CTA's later shots are decoded
+wrongly.  Every output is compared with the
 dense kernel's (itself pinned to the oracle elsewhere)."""
 import numpy as np
 import pytest
 import torch
 
-from paper_2406_18655_gb300 import inputs as I  # noqa: F401
+from paper_2406_18655_gb300 import inputs as I
+from tests.gpu_cases import code
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +87,13 @@ def test_dependent_columns_of_many_clusters(L, rows):
     for k in range(blocks):
         s[np.arange(1000), k * rows + np.random.default_rng(k).integers(0, rows, 1000)] = 1
     assert 2 in _compare(L, h, s, 3 * rows, 4, 10)
+
+
+@pytest.mark.parametrize("order,cs", [(0, None), (2, None)])
+@pytest.mark.parametrize("name,p", [("bb72", 0.04), ("bb144", 0.04), ("rep_boundary", 0.15)])
+def test_several_clusters_then_one(L, name, p, order, cs):
+    """Small shots that go on with their last invalid cluster alone: the count of growing
+    clusters is read by every thread before it is cleared."""
+    h = code(name)
+    e = I.sample_errors(13, 60000, np.full(h.shape[1], p))
+    assert 2 in _compare(L, h, I.syndromes(h, e), order, cs, 14)
