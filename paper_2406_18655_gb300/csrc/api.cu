@@ -242,14 +242,13 @@ int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
     return e == cudaSuccess ? LSD_OK : cuda_fail(e);
   }
   int rc;
-  if (!d->d_sp_big) {
-    if ((rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_small),
-                        (size_t)d->sp_grid_small * d->sp_stride_small)))
-      return rc;
-    if ((rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_big),
-                        (size_t)d->sp_grid_big * d->sp_stride_big)))
-      return rc;
-  }
+  // (each by its own pointer: a call after one that found no room for the second keeps the first)
+  if (!d->d_sp_small && (rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_small),
+                                        (size_t)d->sp_grid_small * d->sp_stride_small)))
+    return rc;
+  if (!d->d_sp_big && (rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_big),
+                                      (size_t)d->sp_grid_big * d->sp_stride_big)))
+    return rc;
   if (d->sp_grid_big > 0 && (size_t)max_items > d->spill_cap) {
     cudaError_t e = cudaStreamSynchronize(d->st);
     if (e != cudaSuccess) return cuda_fail(e);
