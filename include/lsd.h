@@ -89,7 +89,9 @@ typedef struct lsd_options {
                              fit, the one with the most threads (at least one fault per
                              thread), for small batches such as the server's; else as 0 */
   int32_t lsd_kernel;     /* LSD kernel: 0 = auto (dense up to 144 detectors and 288 faults and
-                             for single_cluster, else sparse), 1 = dense (a warp per shot, state
+                             for single_cluster, else sparse; dense as well where it takes the
+                             matrix and mem_budget or the device has no room for the sparse
+                             one's tables and scratch), 1 = dense (a warp per shot, state
                              indexed by detector and fault, m <= 512, n <= 2048), 2 = sparse (a
                              CTA per shot, state sized by what a shot touches; any m,
                              n < 65536; no single_cluster) */

@@ -60,10 +60,12 @@ struct lsd_decoder {
   float* d_probs = nullptr;  // channel probabilities (sampler)
   // sparse LSD (large matrices)
   bool sparse = false;
+  int sparse_rc = 0;         // its tables found no room: every LSD call returns this
   int sp_grid_small = 0, sp_grid_big = 0;  // (large: 0 when no shot can outgrow the small one)
   unsigned char* d_sp_small = nullptr;
   unsigned char* d_sp_big = nullptr;
   int* d_spill = nullptr;
+  size_t sp_tables = 0;      // bytes of g.chk_pad and g.var_pad together
   size_t sp_stride_small = 0, sp_stride_big = 0, spill_cap = 0;
 };
 
@@ -99,8 +101,9 @@ bool prior_uses_tc(const lsd_prior* p) {
 }
 
 // Device allocation charged to the decoder (and to its memory budget).
-int dev_alloc(lsd_decoder* d, void** p, size_t bytes) {
-  if (bytes == 0) bytes = 16;
+constexpr size_t alloc_size(size_t bytes) { return bytes ? bytes : 16; }
+int try_alloc(lsd_decoder* d, void** p, size_t bytes) {
+  bytes = alloc_size(bytes);
   if (d->opt.mem_budget && d->bytes + bytes > d->opt.mem_budget) return LSD_ERR_ADMISSION;
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
@@ -118,6 +121,31 @@ void dev_free(lsd_decoder* d, void* p, size_t bytes) {
   if (it != d->allocs.end()) d->allocs.erase(it);
   cudaFree(p);
   d->bytes -= bytes;
+}
+
+bool no_room(int rc) { return rc == LSD_ERR_ADMISSION || rc == LSD_ERR_OOM; }
+
+// A matrix that both LSD kernels take goes over to the dense one, which holds no scratch (the
+// same results): whatever a budget has room for with that kernel, it has room for.  False when
+// the sparse kernel is not in use or is the only one.
+bool drop_sparse(lsd_decoder* d) {
+  if (!d->sparse || !d->dense) return false;
+  cudaStreamSynchronize(d->st);  // (an error of earlier work is reported by the next call)
+  dev_free(d, d->d_sp_small, alloc_size((size_t)d->sp_grid_small * d->sp_stride_small));
+  dev_free(d, d->d_sp_big, alloc_size((size_t)d->sp_grid_big * d->sp_stride_big));
+  dev_free(d, d->d_spill, d->spill_cap * sizeof(int));
+  dev_free(d, const_cast<uint16_t*>(d->g.chk_pad), d->sp_tables);
+  d->g.chk_pad = d->g.var_pad = nullptr;
+  d->d_sp_small = d->d_sp_big = nullptr;
+  d->d_spill = nullptr;
+  d->spill_cap = 0;
+  d->sparse = false;
+  return true;
+}
+
+int dev_alloc(lsd_decoder* d, void** p, size_t bytes) {
+  const int rc = try_alloc(d, p, bytes);
+  return no_room(rc) && drop_sparse(d) ? try_alloc(d, p, bytes) : rc;
 }
 
 template <typename T>
@@ -233,20 +261,15 @@ int decode_chunk(lsd_decoder* d, int64_t shots, const uint8_t* syn, uint8_t* cor
   return e == cudaSuccess ? LSD_OK : cuda_fail(e);
 }
 
-// LSD launch on the decoder's queue or batch: the dense kernel, or for large matrices the
-// sparse kernel followed by its global-memory instance for the shots that spilled.
-int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
-  if (!d->sparse) {
-    cudaError_t e = launch_lsd(l, d->lsd_warps, d->lsd_grid, d->lsd_smem, d->st);
-    d->launches++;
-    return e == cudaSuccess ? LSD_OK : cuda_fail(e);
-  }
+// Scratch of the sparse LSD for a launch of up to max_items shots.
+int ensure_sparse(lsd_decoder* d, int64_t max_items) {
+  if (d->sparse_rc) return d->sparse_rc;
   int rc;
   // (each by its own pointer: a call after one that found no room for the second keeps the first)
-  if (!d->d_sp_small && (rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_small),
+  if (!d->d_sp_small && (rc = try_alloc(d, reinterpret_cast<void**>(&d->d_sp_small),
                                         (size_t)d->sp_grid_small * d->sp_stride_small)))
     return rc;
-  if (!d->d_sp_big && (rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_sp_big),
+  if (!d->d_sp_big && (rc = try_alloc(d, reinterpret_cast<void**>(&d->d_sp_big),
                                       (size_t)d->sp_grid_big * d->sp_stride_big)))
     return rc;
   if (d->sp_grid_big > 0 && (size_t)max_items > d->spill_cap) {
@@ -255,12 +278,28 @@ int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
     dev_free(d, d->d_spill, d->spill_cap * sizeof(int));
     d->d_spill = nullptr;
     d->spill_cap = 0;
-    if ((rc = dev_alloc(d, reinterpret_cast<void**>(&d->d_spill), (size_t)max_items * sizeof(int))))
+    if ((rc = try_alloc(d, reinterpret_cast<void**>(&d->d_spill), (size_t)max_items * sizeof(int))))
       return rc;
     d->spill_cap = (size_t)max_items;
   }
-  cudaError_t e = launch_sparse(l, false, d->sp_grid_small, d->d_sp_small, d->sp_stride_small,
-                                d->d_spill, nullptr, d->st);
+  return LSD_OK;
+}
+
+// LSD launch on the decoder's queue or batch: the dense kernel, or the sparse kernel followed by
+// its large instance for the shots that outgrew the small one.
+int run_lsd(lsd_decoder* d, const LSDArgs& l, int64_t max_items) {
+  if (d->sparse) {
+    const int rc = ensure_sparse(d, max_items);
+    if (rc && !(no_room(rc) && drop_sparse(d))) return rc;
+  }
+  cudaError_t e;
+  if (!d->sparse) {
+    e = launch_lsd(l, d->lsd_warps, d->lsd_grid, d->lsd_smem, d->st);
+    d->launches++;
+    return e == cudaSuccess ? LSD_OK : cuda_fail(e);
+  }
+  e = launch_sparse(l, false, d->sp_grid_small, d->d_sp_small, d->sp_stride_small, d->d_spill,
+                    nullptr, d->st);
   d->launches++;
   if (d->sp_grid_big == 0) return e == cudaSuccess ? LSD_OK : cuda_fail(e);
   if (e == cudaSuccess)
@@ -448,32 +487,41 @@ int lsd_create(lsd_decoder** out, int32_t m, int32_t n, int64_t nnz, const int32
   else
     cudaGetLastError();
   // The sparse LSD takes the matrices that the dense kernel does not, and those whose dense
-  // ranking is a sort in shared memory (more than 144 detectors or 288 faults).  Not for the
-  // single-cluster mode, whose one cluster holds every detector from the start.
+  // ranking is a sort in shared memory (more than 144 detectors or 288 faults), where it is the
+  // faster one also when every shot of a batch reaches LSD: dense / sparse of 16 to 50 000 shots
+  // 3.1-7.6 for LSD-0 of a 144 x 324 space-time matrix (7.41 / 0.97 ms for 50 000), 1.7-4.5 for
+  // its LSD-6 and LSD-14 with OSD-CS-4; 1.4-5.5 and 1.8-4.2 for (3,6)-regular 150 x 300 and 240 x
+  // 480 at p = 0.01 to 0.08 (percolating at the last: 21.4 / 15.0 ms); 11-45 beyond 256 detectors
+  // or 768 faults.  Not for the single-cluster mode, whose one cluster holds every detector from
+  // the start.
   const bool prefer_sparse = !d->dense || (o.lsd_kernel == 0 && (m > 144 || n > 288));
   if (prefer_sparse && o.lsd_kernel != 1 && !o.single_cluster) {
-    const int D = std::max(max_row, 1);
-    std::vector<uint16_t> chk_pad((size_t)m * D, 0xffff), var_pad((size_t)n * 4, 0xffff);
-    for (int i = 0; i < m; ++i)
-      for (int q = chk_ptr[i]; q < chk_ptr[i + 1]; ++q) chk_pad[(size_t)i * D + q - chk_ptr[i]] = chk_var[q];
-    for (int j = 0; j < n; ++j)
-      for (int q = var_ptr[j]; q < std::min(var_ptr[j + 1], var_ptr[j] + 4); ++q)
-        var_pad[(size_t)j * 4 + q - var_ptr[j]] = var_chk[q];
-    uint16_t *d_chk_pad = nullptr, *d_var_pad = nullptr;
-    if ((rc = upload(d, &d_chk_pad, chk_pad)) || (rc = upload(d, &d_var_pad, var_pad))) {
-      lsd_destroy(d);
-      return rc;
-    }
-    ce = cudaStreamSynchronize(d->st);
-    if (ce != cudaSuccess) {
-      lsd_destroy(d);
-      return cuda_fail(ce);
-    }
-    g.chk_pad = d_chk_pad;
-    g.var_pad = d_var_pad;
     if (sparse_config(g, lsd_order, &d->sp_grid_small, &d->sp_grid_big) == cudaSuccess) {
-      d->sparse = true;
+      // one allocation: the rows' columns padded to the largest row, the columns' first four rows
+      const int D = std::max(max_row, 1);
+      const size_t rows_at = ((size_t)m * D + 3) & ~(size_t)3;  // (read eight bytes at a time)
+      std::vector<uint16_t> pad(rows_at + (size_t)n * 4, 0xffff);
+      for (int i = 0; i < m; ++i)
+        for (int q = chk_ptr[i]; q < chk_ptr[i + 1]; ++q) pad[(size_t)i * D + q - chk_ptr[i]] = chk_var[q];
+      for (int j = 0; j < n; ++j)
+        for (int q = var_ptr[j]; q < std::min(var_ptr[j + 1], var_ptr[j] + 4); ++q)
+          pad[rows_at + (size_t)j * 4 + q - var_ptr[j]] = var_chk[q];
+      uint16_t* d_pad = nullptr;
+      rc = upload(d, &d_pad, pad);
+      if (rc == LSD_OK && (ce = cudaStreamSynchronize(d->st)) != cudaSuccess) rc = cuda_fail(ce);
+      if (rc != LSD_OK && !no_room(rc)) {
+        lsd_destroy(d);
+        return rc;
+      }
+      // no room for the tables: the dense kernel if it takes the matrix, else BP alone
+      d->sparse = rc == LSD_OK || !d->dense;
+      d->sparse_rc = d->sparse ? rc : LSD_OK;
       d->lsd_ok = true;
+      if (rc == LSD_OK) {
+        g.chk_pad = d_pad;
+        g.var_pad = d_pad + rows_at;
+        d->sp_tables = pad.size() * sizeof(uint16_t);
+      }
       d->sp_stride_small = sparse_scratch_bytes(m, n, false, lsd_order > 0);
       d->sp_stride_big = sparse_scratch_bytes(m, n, true, lsd_order > 0);
     } else {
