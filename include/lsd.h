@@ -74,7 +74,8 @@ typedef struct lsd_options {
   int32_t no_early_exit;  /* 0 = a shot stops BP once H e_hat = s (default); 1 = run all iterations */
   int32_t single_cluster; /* 1 = LSD seeds one cluster holding every detector; it then equals OSD-0 */
   int32_t bp_lanes;       /* threads cooperating on one shot in BP: 0 = auto, else 8, 16 or 32 */
-  int32_t lsd_warps;      /* warps per CTA of the LSD kernel: 0 = auto, else 1..16 */
+  int32_t lsd_warps;      /* warps per CTA of the dense LSD kernel: 0 = auto, else 1..16 (the
+                             sparse kernel's CTAs have a fixed size) */
   int32_t bp_kernel;      /* BP kernel: 0 = auto (register tables when a shape fits and,
                              for the CTA-per-shot shapes, the graph has at least as many
                              checks as the shape has threads; else generic), 1 = generic
@@ -653,7 +654,9 @@ int lsd_server_destroy(lsd_server* s);
  * lsd_autotune -- time the decoder's launch variants on a sample batch and keep the fastest:
  * every BP kernel variant compatible with H and the BP method (register-resident shapes,
  * generic 8/16/32-lane groups, one CTA per shot), then the LSD kernel's warps per CTA
- * (2, 4, 8, 16 for the dense kernel).  Results of the decoder do not depend on the choice.
+ * (2, 4, 8, 16 for the dense kernel) and, for a matrix that both LSD kernels take and the
+ * default gives to the sparse one, the sparse kernel as well (reported as 0 warps).  Results of
+ * the decoder do not depend on the choice.
  *   syndromes   device [shots][m] bytes, a representative sample (e.g. 10^5 shots).
  *   report      host, nullable: the chosen variants and their times.
  * Allocates temporary device buffers and synchronizes.

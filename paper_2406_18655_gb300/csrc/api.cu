@@ -1244,23 +1244,30 @@ extern "C" int lsd_autotune(lsd_decoder* d, int64_t shots, const uint8_t* syndro
     rep.bp_variant = best_v;
     rep.ms_bp_best = best_ms;
   }
-  // ---- LSD warps per CTA (dense kernel) ----
-  if (!rc && d->lsd_ok && !d->sparse) {
-    const int w0 = d->lsd_warps;
-    int best_w = w0, best_g = d->lsd_grid;
+  // ---- LSD: warps per CTA of the dense kernel, and the sparse kernel (candidate 0) where it
+  // was chosen for a matrix that the dense one takes too ----
+  if (!rc && d->dense) {
+    const bool sparse0 = d->sparse;
+    const int w0 = sparse0 ? 0 : d->lsd_warps;
+    int best_w = d->lsd_warps, best_g = d->lsd_grid;
     size_t best_s = d->lsd_smem;
     float best_ms = 0.f;
-    const int cand[] = {2, 4, 8, 16};
+    bool best_sparse = sparse0;
+    const int cand[] = {0, 2, 4, 8, 16};
     for (int w : cand) {
+      if (w == 0 && !sparse0) continue;
       int ww = 0, grid = 0, words = 0;
       size_t smem = 0;
-      if (lsd_config(d->g, d->order, w, &ww, &grid, &smem, &words) != cudaSuccess || ww != w) {
+      d->sparse = w == 0;
+      if (w && (lsd_config(d->g, d->order, w, &ww, &grid, &smem, &words) != cudaSuccess || ww != w)) {
         cudaGetLastError();
         continue;
       }
-      d->lsd_warps = ww;
-      d->lsd_grid = grid;
-      d->lsd_smem = smem;
+      if (w) {
+        d->lsd_warps = ww;
+        d->lsd_grid = grid;
+        d->lsd_smem = smem;
+      }
       float ms = 0.f;
       rc = timed([&]() { return lsd_decode_batch(d, shots, syndromes, corr, st, nullptr, nullptr); },
                  &ms);
@@ -1273,15 +1280,21 @@ extern "C" int lsd_autotune(lsd_decoder* d, int64_t shots, const uint8_t* syndro
       if (w == w0) rep.ms_lsd_first = ms;
       if (best_ms == 0.f || ms < best_ms) {
         best_ms = ms;
-        best_w = ww;
-        best_g = grid;
-        best_s = smem;
+        best_sparse = d->sparse;
+        if (w) {
+          best_w = ww;
+          best_g = grid;
+          best_s = smem;
+        }
       }
     }
     d->lsd_warps = best_w;
     d->lsd_grid = best_g;
     d->lsd_smem = best_s;
-    rep.lsd_warps = best_w;
+    // (a decoder that found no room for the sparse kernel's scratch above has dropped its tables)
+    d->sparse = sparse0 && d->g.chk_pad;
+    if (!best_sparse) drop_sparse(d);
+    rep.lsd_warps = d->sparse ? 0 : best_w;
     rep.ms_lsd_best = best_ms;
   }
   if (t0) cudaEventDestroy(t0);

@@ -123,3 +123,20 @@ def test_large_graphs_against_oracle(L, base, p, order, cs, shots):
     got = info.cpu().numpy()
     for k, key in enumerate(("nu", "kappa", "steps")):
         assert np.array_equal(got[:, k], r[key])
+
+
+@pytest.mark.parametrize("order", [0, 6])
+def test_autotune_times_both_kernels(L, order):
+    """A matrix that both kernels take: the report has the dense kernel's shapes and the sparse
+    kernel, and the decoder's results stay, whichever it kept."""
+    h = code("st_bb72_d6")
+    probs = np.full(h.shape[1], 0.02, np.float32)
+    s = torch.from_numpy(I.syndromes(h, I.sample_errors(4, 3000, probs.astype(np.float64)))).cuda()
+    d = L.Decoder(h, probs, 10, order)
+    want = d.decode(s)
+    rep = d.autotune(s)
+    dense = L.Decoder(h, probs, 10, order, lsd_kernel=1).autotune(s)
+    assert rep["lsd_candidates"] == 1 + dense["lsd_candidates"]
+    assert 0 < rep["ms_lsd_best"] <= rep["ms_lsd_first"]
+    for a, b in zip(d.decode(s), want):
+        assert torch.equal(a, b)
