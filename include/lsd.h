@@ -485,7 +485,8 @@ int lsd_giant_create(lsd_giant** out, int32_t m, int32_t n, int64_t nnz, const i
  * lsd_giant_decode -- BP (min-sum, flooding, early exit on H e_hat = s, Sec. 4.3), then
  * P-LSD on the posteriors when BP does not converge.  Synchronous.  BP and P-LSD run as one
  * cooperative launch each, whose blocks meet at grid barriers; a barrier that waits past its
- * bound (about a second in BP, 30 seconds in P-LSD) makes the call return LSD_ERR_TIMEOUT.
+ * bound (about a second in BP, 30 seconds without progress in P-LSD, however long the whole
+ * takes) makes the call return LSD_ERR_TIMEOUT.
  *   syndrome     device [m] bytes.   correction  device [n] bytes (written).
  *   posteriors   device [n] float32, nullable: the BP posteriors.
  *   info         host, nullable.
@@ -505,6 +506,10 @@ int lsd_giant_postprocess(lsd_giant* dec, const float* llr, const uint8_t* syndr
  * operation and the one-second bound.  LSD_ERR_UNSUPPORTED when the device cannot run the
  * cooperative launch. */
 int lsd_giant_test_hold_barrier(lsd_giant* dec, int32_t hold, int64_t limit_ns);
+
+/* lsd_giant_test_lsd_bound -- the same for P-LSD's launch: its barrier waits are bounded by
+ * limit_ns (0 = the default of 30 seconds); with hold != 0, block 0 withholds its first arrival. */
+int lsd_giant_test_lsd_bound(lsd_giant* dec, int32_t hold, int64_t limit_ns);
 
 /* lsd_giant_kernel_launches -- kernels launched so far by the giant-shot decoder. */
 int lsd_giant_kernel_launches(const lsd_giant* dec, int64_t* count);

@@ -51,7 +51,8 @@ constexpr int kWcMax = 8;                     // reduction words per lane
 constexpr int kMaxSlots = 32 * 32 * kWcMax;   // 8192 detectors per cluster
 constexpr int kLsdBlock = 1024;               // threads of a block of the persistent P-LSD
 constexpr int kTailClusters = 64;             // invalid clusters that one block goes on with
-// bound of its barrier waits: a step may hold thousands of eliminations in one large cluster
+// bound of its barrier waits, from the last sign of progress on: a phase may hold thousands of
+// eliminations in one large cluster, and block 0 goes through the last steps alone
 constexpr long long kLsdLimitNs = 30000000000LL;
 constexpr int kUfLimit = 1 << 20;             // bound on union-find retries and path length
 // a minimum over an empty set (a check of degree 1): 2^100, as in the batch kernels
@@ -61,7 +62,8 @@ struct GCtr {
   // whole call
   int ns, nfront, unsolvable, overflow, uf_fail, too_big, ndep, dep_top;
   int bp_stop, bp_unsat[2], bp_iters, bp_conv, bp_fail;
-  unsigned bar_arrive;  // grid barrier of the persistent BP launch
+  unsigned bar_arrive;  // grid barrier of the persistent launches
+  int progress;         // P-LSD: changes while blocks that the others wait for get on
   int nu, kappa, steps, stuck;
   int ninv[2];
   // reset every step
@@ -290,9 +292,9 @@ __global__ void __launch_bounds__(256) gbp_syn(GD g, const uint8_t* __restrict__
 // Grid-wide barrier of the persistent launches (all blocks co-resident: cooperative launch).
 // The arrival counter only grows; barrier b waits for b * gridDim.x arrivals.  Before arriving
 // the block ors `bad` over its threads into *flag; the return value is *flag after the barrier,
-// or -1: the wait is bounded by limit_ns of the global timer, past it the block flags bp_fail
-// and every block leaves at its next barrier, the host reporting LSD_ERR_TIMEOUT.  Only one
-// thread of a block reads the flags.  `arrive` false (the timeout test only) withholds this
+// or -1: the wait is bounded by limit_ns of the global timer since its start or the last change
+// of `progress` that it saw, past it the block flags bp_fail and every block leaves at its next
+// barrier, the host reporting LSD_ERR_TIMEOUT.  Only one thread of a block reads the flags.  `arrive` false (the timeout test only) withholds this
 // block's arrival.
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
@@ -310,10 +312,13 @@ __device__ __forceinline__ int grid_barrier(const GD& g, unsigned target, long l
     if (arrive) atomicAdd(&g.ctr->bar_arrive, 1u);
     bool ok = true;
     unsigned long long t0 = 0;
+    int seen = 0;
     for (unsigned spin = 1; *(volatile unsigned*)&g.ctr->bar_arrive < target; ++spin) {
-      if (spin & 63u) continue;  // the clock and the failure flag are looked at now and then
+      if (spin & 63u) continue;  // the clock and the flags are looked at now and then
       const unsigned long long now = global_ns();
-      if (t0 == 0) t0 = now;
+      const int got_to = *(volatile int*)&g.ctr->progress;
+      if (t0 == 0 || got_to != seen) t0 = now;
+      seen = got_to;
       if ((long long)(now - t0) > limit_ns) atomicOr(&g.ctr->bp_fail, 1);
       if (*(volatile int*)&g.ctr->bp_fail) {
         ok = false;
@@ -1097,10 +1102,12 @@ __device__ __forceinline__ void glsd_add(const GD& g, const Span& S, int par_nex
           }
         }
         last = best;
-        if (nslots <= 1024)
+        if (nslots <= 1024) {
           gadd_column<1>(g, D, nslots, g.nc_g[bi], lane);
-        else
+        } else {  // (milliseconds each in the largest clusters)
+          if (lane == 0) atomicAdd(&g.ctr->progress, 1);
           gadd_column<kWcMax>(g, D, nslots, g.nc_g[bi], lane);
+        }
       }
       bool any = false;
       for (int w = lane; w < ((nslots + 31) >> 5); w += 32) any |= D.sred()[w] != 0u;
@@ -1364,17 +1371,20 @@ __global__ void __launch_bounds__(256) glsd_phase(GD g, PhaseArgs a) {
 // item of a phase, and a barrier of about 2.5 us.  Most steps are the growth of a last few
 // clusters: from kTailClusters invalid ones on (their number never grows) block 0 goes on alone,
 // with barriers of its own and its L1 kept from phase to phase, and looks for candidates from the
-// clusters' side; the others wait at the last grid barrier.  640 000 faults at p = 0.03: 22 steps
+// clusters' side; the others wait at the last grid barrier, whose bound starts again at every step
+// of block 0, which leaves in turn when they have given up.  640 000 faults at p = 0.03: 22 steps
 // 2.02 -> 0.65 ms, 3 steps 0.56 -> 0.29 (before: nine launches and a look by the host per step,
 // 79 us; all steps on the grid: 1.25 ms and 0.39; seeds counted by warp and single seeds absorbed
 // by a warp each: 0.71 and 0.36).  kTailClusters 16: the same; 256: 0.07 ms longer.
-__global__ void __launch_bounds__(kLsdBlock) glsd_persistent(GD g, PhaseArgs a, long long limit_ns) {
+__global__ void __launch_bounds__(kLsdBlock) glsd_persistent(GD g, PhaseArgs a, long long limit_ns, int hold) {
   unsigned target = 0;
   bool alone = false;
   Span S = grid_span();
   auto grid_sync = [&] {
     target += gridDim.x;
-    return grid_barrier(g, target, limit_ns, &g.ctr->unsolvable, false) >= 0;
+    // hold (the timeout test only): block 0 withholds its first arrival
+    const bool arrive = !(hold && target == gridDim.x && blockIdx.x == 0);
+    return grid_barrier(g, target, limit_ns, &g.ctr->unsolvable, false, arrive) >= 0;
   };
   auto sync = [&] {
     if (!alone) return grid_sync();
@@ -1407,8 +1417,13 @@ __global__ void __launch_bounds__(kLsdBlock) glsd_persistent(GD g, PhaseArgs a, 
     glsd_absorb(g, S);
     glsd_claim(g, S);
     if (!sync()) return;
+    int given_up = 0;  // (asked for before the phase, so that its reply does not add to the step)
+    if (alone && threadIdx.x == 0) {
+      atomicAdd(&g.ctr->progress, 1);
+      given_up = *(volatile int*)&g.ctr->bp_fail;
+    }
     glsd_add(g, S, par ^ 1, true);
-    if (!sync()) return;
+    if (alone ? __syncthreads_or(given_up) != 0 : !grid_sync()) return;
     // a step in which some invalid cluster found no candidate does not count (Alg. 1)
     if (g.ctr->unsolvable) break;
     ++steps;
@@ -1448,6 +1463,8 @@ struct lsd_giant {
   int lsd_grid = 1;  // blocks of glsd_persistent (1: no cooperative launch needed)
   long long bar_limit_ns = 1000000000LL;  // bound of a grid-barrier wait
   int hold_barrier = 0;                   // timeout test: block 0 withholds an arrival
+  long long lsd_limit_ns = kLsdLimitNs;   // the same of P-LSD's launch
+  int lsd_hold = 0;
 };
 
 namespace {
@@ -1508,8 +1525,7 @@ int run_plsd(lsd_giant* G, const float* llr, const uint8_t* s, uint8_t* corr,
   int rc;
   cudaError_t e = cudaMemsetAsync(g.ctr, 0, sizeof(GCtr), G->st);
   if (e != cudaSuccess) return gfail(e);
-  long long limit = kLsdLimitNs;
-  void* args[] = {(void*)&g, (void*)&a, (void*)&limit};
+  void* args[] = {(void*)&g, (void*)&a, (void*)&G->lsd_limit_ns, (void*)&G->lsd_hold};
   const void* fn = (const void*)glsd_persistent;
   e = G->lsd_grid > 1 ? cudaLaunchCooperativeKernel(fn, G->lsd_grid, kLsdBlock, args, 0, G->st)
                       : cudaLaunchKernel(fn, 1, kLsdBlock, args, 0, G->st);
@@ -1864,6 +1880,13 @@ int lsd_giant_test_hold_barrier(lsd_giant* G, int32_t hold, int64_t limit_ns) {
   if (!G->coop_grid) return LSD_ERR_UNSUPPORTED;
   G->hold_barrier = hold ? 1 : 0;
   G->bar_limit_ns = hold ? (long long)limit_ns : 1000000000LL;
+  return LSD_OK;
+}
+
+int lsd_giant_test_lsd_bound(lsd_giant* G, int32_t hold, int64_t limit_ns) {
+  if (!G || limit_ns < 0) return LSD_ERR_INVALID_ARG;
+  G->lsd_hold = hold ? 1 : 0;
+  G->lsd_limit_ns = limit_ns ? (long long)limit_ns : kLsdLimitNs;
   return LSD_OK;
 }
 

@@ -37,7 +37,7 @@ EXPORTS = ("lsd_create", "lsd_decode_batch", "lsd_decode_batch_host", "lsd_bp_ba
            "lsd_window_decode", "lsd_window_kernel_launches", "lsd_window_destroy",
            "lsd_window_stream_reset", "lsd_window_stream_push", "lsd_giant_create",
            "lsd_giant_decode", "lsd_giant_postprocess", "lsd_giant_kernel_launches",
-           "lsd_giant_destroy", "lsd_giant_test_hold_barrier", "lsd_bp_variant_name",
+           "lsd_giant_destroy", "lsd_giant_test_hold_barrier", "lsd_giant_test_lsd_bound", "lsd_bp_variant_name",
            "lsd_server_create_with_windows", "lsd_server_submit_round",
            "lsd_server_get_code_report", "lsd_prior_set_kernel", "lsd_prior_get_kernel",
            "lsd_decode_batch_packed", "lsd_decode_batch_host_packed")
@@ -145,6 +145,7 @@ def lib():
     L.lsd_giant_kernel_launches.argtypes = [P, C.POINTER(C.c_int64)]
     L.lsd_giant_destroy.argtypes = [P]
     L.lsd_giant_test_hold_barrier.argtypes = [P, C.c_int32, C.c_int64]
+    L.lsd_giant_test_lsd_bound.argtypes = [P, C.c_int32, C.c_int64]
     L.lsd_window_stream_reset.argtypes = [P, C.c_int64]
     L.lsd_window_stream_push.argtypes = [P, P, P, P, C.POINTER(C.c_int32),
                                          C.POINTER(C.c_int32)]
@@ -638,6 +639,11 @@ class GiantDecoder:
         """Timeout-path test facility (lsd_giant_test_hold_barrier)."""
         _check(lib().lsd_giant_test_hold_barrier(self._h, int(hold), limit_ns),
                "lsd_giant_test_hold_barrier")
+
+    def test_lsd_bound(self, hold: bool = False, limit_ns: int = 0):
+        """The same for P-LSD (lsd_giant_test_lsd_bound)."""
+        _check(lib().lsd_giant_test_lsd_bound(self._h, int(hold), limit_ns),
+               "lsd_giant_test_lsd_bound")
 
 
 class Prior:

@@ -62,3 +62,42 @@ def test_cluster_beyond_1024_detectors(L):
     assert info["status"] == r["status"][0] == 2
     assert np.array_equal(corr.cpu().numpy(), r["corrections"][0])
     assert (info["nu"], info["kappa"], info["steps"]) == (r["nu"][0], r["kappa"][0], r["steps"][0])
+
+
+def _chain(L, n, blocks):
+    """`blocks` chains of n faults, a seed at the end of the first: n growth steps of one cluster,
+    by one block while the others wait."""
+    i = np.arange(n * blocks)
+    j = i[i % n != n - 1]
+    rows, cols = np.concatenate([i, j + 1]), np.concatenate([i, j])
+    gd = L.GiantDecoder(n * blocks, n * blocks, rows, cols, np.full(n * blocks, 0.1, np.float32), 5)
+    s = torch.zeros(n * blocks, dtype=torch.uint8, device="cuda")
+    s[0] = 1
+    return gd, torch.ones(n * blocks, device="cuda"), s
+
+
+def test_bound_starts_again_with_every_step(L):
+    """The blocks that wait out the last clusters' steps wait for longer than their bound in all,
+    but not for any one step."""
+    gd, llr, s = _chain(L, 1400, 8)
+    gd.postprocess(llr, s)  # (the first call also loads the kernel)
+    want, info = gd.postprocess(llr, s)
+    assert info["status"] == 2 and info["steps"] == 1400 and int(want.sum()) == 1400
+    limit = int(info["ms_lsd"] * 1e6 / 4)   # a step takes 1/1400 of it
+    gd.test_lsd_bound(limit_ns=limit)
+    got, again = gd.postprocess(llr, s)
+    assert again["ms_lsd"] * 1e6 > 2 * limit
+    assert again["status"] == 2 and torch.equal(got, want)
+
+
+def test_lsd_timeout_leaves_the_device_usable(L):
+    """A P-LSD barrier whose wait runs out (block 0 withholds its first arrival) makes the call
+    return LSD_ERR_TIMEOUT; the next call, with the hold lifted, decodes."""
+    gd, llr, s = _chain(L, 40, 100)
+    gd.test_lsd_bound(True, limit_ns=20_000_000)
+    with pytest.raises(L.LsdError) as err:
+        gd.postprocess(llr, s)
+    assert err.value.code == L.LSD_ERR_TIMEOUT
+    gd.test_lsd_bound()
+    corr, info = gd.postprocess(llr, s)
+    assert info["status"] == 2 and int(corr.sum()) == 40
