@@ -820,6 +820,10 @@ __global__ void __launch_bounds__(kTrainWarps * 32, 1) prior_train_kernel(TrainA
 #pragma unroll
     for (int q = 0; q < 4; ++q) wacc[j][q] = 0.f;
   double loss_acc = 0.0;
+  // gradients of a0, a1, u0, u1 over the warp's nodes of all the CTA's shots: added up at the
+  // end in the warps' order, the same in every run (shared atomics in every shot: in the order they
+  // came, and 1.38 ms instead of 1.36 for 4096 BB144 pairs; one warp over all nodes: 1.52)
+  float ini[4] = {0.f, 0.f, 0.f, 0.f};
 
   for (long long shot = blockIdx.x; shot < a.shots; shot += gridDim.x) {
     const uint8_t* sp = a.syndromes + shot * m;
@@ -1053,24 +1057,24 @@ __global__ void __launch_bounds__(kTrainWarps * 32, 1) prior_train_kernel(TrainA
       __syncthreads();
     }
     // ================= the initial states =================
-    {
-      float d0 = 0.f, d1 = 0.f, e0 = 0.f, e1 = 0.f;
-      for (int v = warp; v < n; v += kTrainWarps) {
-        const float z = fmaf(S.lam[v], S.vec[F_a0 * HD + lane], S.vec[F_a1 * HD + lane]);
-        const float gz = z > 0.f ? gv[fsw(v, lane)] : 0.f;
-        d0 = fmaf(gz, S.lam[v], d0);
-        d1 += gz;
-      }
-      for (int c = warp; c < m; c += kTrainWarps) {
-        const float gcv = gc[fsw(c, lane)];
-        e0 = fmaf(S.sig[c], gcv, e0);
-        e1 += gcv;
-      }
-      atomicAdd(&vg[VG_a0 * HD + lane], d0);
-      atomicAdd(&vg[VG_a1 * HD + lane], d1);
-      atomicAdd(&vg[VG_u0 * HD + lane], e0);
-      atomicAdd(&vg[VG_u1 * HD + lane], e1);
+    for (int v = warp; v < n; v += kTrainWarps) {
+      const float z = fmaf(S.lam[v], S.vec[F_a0 * HD + lane], S.vec[F_a1 * HD + lane]);
+      const float gz = z > 0.f ? gv[fsw(v, lane)] : 0.f;
+      ini[0] = fmaf(gz, S.lam[v], ini[0]);
+      ini[1] += gz;
     }
+    for (int c = warp; c < m; c += kTrainWarps) {
+      const float gcv = gc[fsw(c, lane)];
+      ini[2] = fmaf(S.sig[c], gcv, ini[2]);
+      ini[3] += gcv;
+    }
+    __syncthreads();
+  }
+  // ---- the initial states' sums, warp by warp ----
+  for (int w = 0; w < kTrainWarps; ++w) {
+    if (warp == w)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) vg[(VG_a0 + q) * HD + lane] += ini[q];
     __syncthreads();
   }
   // ---- flush the CTA's gradients ----

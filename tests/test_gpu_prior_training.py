@@ -46,3 +46,15 @@ def test_gradient_shapes(L, name, rounds):  # noqa: F811
     assert abs(loss - ref_loss) <= 0.01 * abs(ref_loss)
     assert np.linalg.norm(g - ref_g) <= 1e-2 * np.linalg.norm(ref_g)
     assert g @ ref_g >= 0.9999 * np.linalg.norm(g) * np.linalg.norm(ref_g)
+
+
+def test_initial_state_gradients_in_one_order(L):  # noqa: F811
+    """One pair is one block: the gradients of the initial states (the first 128 values) are sums
+    in a fixed order, the same bits in every run."""
+    h = code("bb144")
+    probs = np.full(h.shape[1], 0.06, np.float32)
+    e = I.sample_errors(22, 1, probs.astype(np.float64))
+    s = torch.from_numpy(I.syndromes(h, e)).cuda()
+    pr = L.Prior(L.Decoder(h, probs, 10), rounds=3, params=params_case(6).astype(np.float32))
+    runs = {pr.gradient(s, torch.from_numpy(e).cuda())[1][:128].tobytes() for _ in range(200)}
+    assert len(runs) == 1
