@@ -460,7 +460,10 @@ __global__ void __launch_bounds__(512) bp_cta_kernel(BPArgs a) {
 //   PAD  rows may be shorter than DC (else chk_ptr[i] = i DC)
 //   MSG  the thread's messages stay in registers too (else they are read back from its words)
 //   PRI  the priors of its variables as well (else shared memory)
-template <int NT, int CPL, int DC, int VPL, int DV, bool PAD, int MINB, bool PK, bool MSG, bool PRI>
+//   ALL  every slot is computed; else those that no check or variable of this graph falls into
+//        are left out, by a branch that all threads take alike (see regcta_all)
+template <int NT, int CPL, int DC, int VPL, int DV, bool PAD, int MINB, bool PK, bool MSG, bool PRI,
+          bool ALL>
 __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_shot[2];
@@ -509,6 +512,7 @@ __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
     if constexpr (PRI) prior[v] = lam;
     else s_prior[j] = lam;
   }
+  const int cpl = ALL ? CPL : (m + NT - 1) / NT, vpl = ALL ? VPL : (n + NT - 1) / NT;  // slots in use
   auto word = [&](uint32_t pair, int half) { return w[half ? pair >> 16 : pair & 0xffffu]; };
   // the syndrome bits of a shot's checks of this thread
   auto load_syndrome = [&](long long shot) {
@@ -575,6 +579,7 @@ __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
         // ---- check phase: parities and q (in the messages' place), then the new messages ----
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
+          if (!ALL && c > 0 && c >= cpl) break;
           uint32_t hp = (sbits >> c) << 31;
 #pragma unroll
           for (int k = 0; k < DC; ++k) {
@@ -591,6 +596,7 @@ __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
         if (!msgs) break;
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
+          if (!ALL && c > 0 && c >= cpl) break;
           float x[DC];
           excluded_min<DC>(msg[c], x);
           const float salpha = __uint_as_float(__float_as_uint(a.alpha) ^ ((sbits >> c) << 31));
@@ -605,6 +611,7 @@ __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
         // ---- check phase (the update of bp_reg_kernel) ----
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
+          if (!ALL && c > 0 && c >= cpl) break;
           const uint32_t sbit = (sbits >> c) << 31;
           uint32_t hp = sbit;
           float q[DC], x[DC];
@@ -632,6 +639,7 @@ __global__ void __launch_bounds__(NT, MINB) bp_regcta_kernel(BPArgs a) {
       // ---- variable phase ----
 #pragma unroll
       for (int v = 0; v < VPL; ++v) {
+        if (!ALL && v > 0 && v >= vpl) break;
         float L = PRI ? prior[PRI ? v : 0] : s_prior[tid + NT * v];
 #pragma unroll
         for (int k = 0; k < DV; ++k) L = __fadd_rn(L, word(ve[v][k >> 1], k & 1));
@@ -762,13 +770,16 @@ const void* generic_fn(int v) {
 struct RegCtaShape {
   int nt, cpl, dc, vpl, dv;
   bool pad, pri;
-  const void* fn;
-  const void* fn_pk;
+  const void* fn[2][2];  // [all slots][packed]
   const char* name;
 };
-#define LSD_REGCTA_SHAPE(NT, C, DCx, V, DVx, P, MB, MS, PR)                                        \
-  {NT, C, DCx, V, DVx, P, PR, (const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, false, MS, PR>, \
-   (const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, true, MS, PR>,                          \
+#define LSD_REGCTA_FN(NT, C, DCx, V, DVx, P, MB, MS, PR, ALLx)                          \
+  {(const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, false, MS, PR, ALLx>,       \
+   (const void*)bp_regcta_kernel<NT, C, DCx, V, DVx, P, MB, true, MS, PR, ALLx>}
+#define LSD_REGCTA_SHAPE(NT, C, DCx, V, DVx, P, MB, MS, PR)                              \
+  {NT, C, DCx, V, DVx, P, PR,                                                           \
+   {LSD_REGCTA_FN(NT, C, DCx, V, DVx, P, MB, MS, PR, false),                            \
+    LSD_REGCTA_FN(NT, C, DCx, V, DVx, P, MB, MS, PR, true)},                            \
    "bp_regcta_kernel<" #NT "," #C "," #DCx "," #V "," #DVx "," #P "," #MB ">"}
 const RegCtaShape kRegCtaShapes[] = {
     LSD_REGCTA_SHAPE(512, 6, 7, 13, 4, false, 1, false, false),  // m <= 3072, n <= 6656 (HGP of a 48 x 64 (3,4) code)
@@ -792,6 +803,7 @@ const RegCtaShape kRegCtaShapes[] = {
     LSD_REGCTA_SHAPE(512, 1, 8, 2, 3, true, 1, true, true),   // m <= 512, n <= 1024 (BB72, d = 6)
 };
 #undef LSD_REGCTA_SHAPE
+#undef LSD_REGCTA_FN
 constexpr int kNumRegCtaShapes = sizeof(kRegCtaShapes) / sizeof(kRegCtaShapes[0]);
 
 size_t regcta_smem(const RegCtaShape& s, const DevGraph&) {
@@ -800,6 +812,16 @@ size_t regcta_smem(const RegCtaShape& s, const DevGraph&) {
 bool regcta_fits(const RegCtaShape& s, const DevGraph& g) {
   const bool rows = s.pad ? g.max_row_deg <= s.dc : (g.min_row_deg == s.dc && g.max_row_deg == s.dc);
   return rows && g.m <= s.nt * s.cpl && g.n <= s.nt * s.vpl && g.max_col_deg <= s.dv;
+}
+// Whether a graph takes the instance that computes every slot: when at most an eighth of the
+// slots of variables is idle, and none of checks.  The branches of the other one cost graphs that fill the shape 2-4 % (10 000
+// HGP 3072 x 6400 shots 1113 us with all slots, 1156 without the idle ones; 20 000 BB288 d = 18
+// 1232, 1256; one idle slot of nine, BB144 hooks d = 5: 538, 550), and save the others up
+// to half (HGP 768 x 1600: 757, 404; BB144 d = 4: 191, 142; (3,6)-regular 480 x 960: 337, 224; one
+// idle slot of variables of six, BB72 d = 5: 64.6, 62.8; two of eleven, BB144 d = 10: 269, 261).
+bool regcta_all(const RegCtaShape& s, const DevGraph& g) {
+  const auto slots = [&](int count) { return (count + s.nt - 1) / s.nt; };
+  return slots(g.m) == s.cpl && 8 * (s.vpl - slots(g.n)) <= s.vpl;
 }
 
 constexpr int kCtaBase = 6 + kNumRegShapes;     // + method: one CTA per shot
@@ -811,10 +833,14 @@ int lanes_of(int variant) {
   if (variant >= 6) return kRegShapes[variant - 6].G;
   return variant % 3 == 0 ? 8 : variant % 3 == 1 ? 16 : 32;
 }
-// The kernel of a variant; `packed`: the instance with bit-packed syndromes and corrections
-// (the generic and cache-read kernels take the layout from their arguments at run time).
-const void* variant_fn(int v, bool packed = false) {
-  if (is_regcta(v)) return packed ? kRegCtaShapes[v - kRegCtaBase].fn_pk : kRegCtaShapes[v - kRegCtaBase].fn;
+// The kernel of a variant for a graph; `packed`: the instance with bit-packed syndromes and
+// corrections (the generic and cache-read kernels take the layout from their arguments at run
+// time).
+const void* variant_fn(int v, const DevGraph& g, bool packed = false) {
+  if (is_regcta(v)) {
+    const RegCtaShape& s = kRegCtaShapes[v - kRegCtaBase];
+    return s.fn[regcta_all(s, g)][packed];
+  }
   if (is_cta(v)) return v == kCtaBase ? (const void*)bp_cta_kernel<0> : (const void*)bp_cta_kernel<1>;
   if (v >= 6) return packed ? kRegShapes[v - 6].fn_pk : kRegShapes[v - 6].fn;
   return generic_fn(v);
@@ -946,10 +972,10 @@ cudaError_t bp_config(const DevGraph& g, int lanes, int method, int kind, int* v
   }
   *block = b;
   *smem = gb + grp;
-  const void* fn = variant_fn(v);
+  const void* fn = variant_fn(v, g);
   err = allow_max_dynamic_smem(fn, max_smem);
-  if (err == cudaSuccess && variant_fn(v, true) != fn)
-    err = allow_max_dynamic_smem(variant_fn(v, true), max_smem);
+  if (err == cudaSuccess && variant_fn(v, g, true) != fn)
+    err = allow_max_dynamic_smem(variant_fn(v, g, true), max_smem);
   if (err != cudaSuccess) return err;
   int per_sm = 0;
   err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, b, *smem);
@@ -962,7 +988,7 @@ cudaError_t bp_config(const DevGraph& g, int lanes, int method, int kind, int* v
 
 cudaError_t launch_bp(const BPArgs& a, int variant, int grid, int block, size_t smem,
                       cudaStream_t st) {
-  const void* fn = variant_fn(variant, a.packed != 0);
+  const void* fn = variant_fn(variant, a.g, a.packed != 0);
   void* args[] = {const_cast<BPArgs*>(&a)};
   return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, st);
 }

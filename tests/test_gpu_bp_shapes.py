@@ -63,3 +63,24 @@ def test_messages_that_outgrow_the_empty_minimum(L, name, alpha, early):
     pass 2^100, where every minimum starts, and have to be clamped as by the generic kernel."""
     h = _matrix(name)
     _compare(L, h, 0.12, 60, 300, 2, seed=9, ms_scaling=alpha, no_early_exit=not early)
+
+
+@pytest.mark.parametrize("name", ["st_bb72_d3", "st_bb72_d8", "st_bb144_d2", "st_bb144_d10", "st_bb288_d15",
+                                  "hooks_bb72_d3", "hooks_bb144_d4", "ldpc_512", "ldpc_600", "ldpc_1100",
+                                  "hgp_24", "hgp_30"])
+@pytest.mark.parametrize("kernel", [2, 3])
+def test_graphs_that_leave_slots_idle(L, name, kernel):
+    """Graphs well below the bounds of their shape, whose idle slots are left out."""
+    if name.startswith("st_"):
+        _, c, d = name.split("_")
+        h = I.space_time(code(c), int(d[1:]))
+    elif name.startswith("hooks"):
+        _, c, d = name.split("_")
+        h = I.space_time_hooks(code(c), int(d[1:]), seed=6)[0]
+    elif name.startswith("ldpc"):
+        m = int(name[5:])
+        h = I.random_regular_ldpc(m, 2 * m, 3, 6, seed=3)
+    else:
+        b = int(name[4:])
+        h = I.hgp(I.random_regular_ldpc(b, b // 3 * 4, 3, 4, seed=7 + b))[0]
+    _compare(L, h, 0.01, 401, 12, kernel, seed=5)
