@@ -771,13 +771,13 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
       }
     }
     // the faults next to those detectors, asked for now and used if the detector is new: thread
-    // (detector q, edge e) from warp 1 on (the last warps when there are not enough)
-    constexpr int kFrom = NT > 32 ? 32 : 0;
-    const int q0 = (tid - kFrom) / D;
+    // (detector q, edge e) from warp 1 on
+    static_assert(NT - 32 >= 4 * kMaxRowDeg, "a thread for every edge of four detectors");
+    const int q0 = (tid - 32) / D;
     int near = kNone16;
-    if (tid >= kFrom && q0 < 4) {
+    if (tid >= 32 && q0 < 4) {
       const uint32_t d = half4(dets, q0);
-      if (d != kNone16) near = G.chk_pad[(size_t)d * D + (tid - kFrom) % D];
+      if (d != kNone16) near = G.chk_pad[(size_t)d * D + (tid - 32) % D];
     }
     __syncthreads();
     const int nsl0 = nsl;
@@ -811,12 +811,6 @@ __device__ int grow_single(const SGraph& G, const Shot<I>& S, const float* llr, 
       }
     };
     if (near != kNone16 && ((fresh >> q0) & 1u)) admit(near);
-#pragma unroll 1
-    for (int x = NT - kFrom + tid; x < 4 * D; x += NT)  // pairs beyond the CTA's threads
-      if ((fresh >> (x / D)) & 1u) {
-        const int f = G.chk_pad[(size_t)half4(dets, x / D) * D + x % D];
-        if (f != kNone16) admit(f);
-      }
     // ---- the column's image; meanwhile the search for the next pick ----
     open_rows(S, nsl0, nsl, tid);
     int pc = -1;
@@ -1343,7 +1337,6 @@ cudaError_t sparse_config(const DevGraph& g, int order, int* grid_small, int* gr
   if (err != cudaSuccess) return err;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-#pragma unroll 1
   *grid_big = 0;
   for (const bool big : {false, true}) {
     if (big && with_instance(false, order > 0, g.m, g.n,
