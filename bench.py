@@ -37,15 +37,14 @@ if ROOT not in sys.path:
 
 METRIC = "shots/s + p99 latency: BB[[144,12,12]] BP+LSD vs learned+LSD at equal LER"
 UNIT = "shots/s"
-# Algorithmic work of min-sum BP per edge per executed iteration: abs, two-minimum
-# tracking, sign parity, select, scaling multiply, sign apply, the variable-side add
-# and subtract, and the hard-decision parity (about ten integer / FP32 operations).
-OPS_PER_EDGE_ITER = 10
+# Shared-memory words of min-sum BP per edge per executed iteration, which bound its kernels: the
+# message stored by its check and gathered by its variable, the posterior gathered by the check.
+WORDS_PER_EDGE_ITER = 3
 L2_FLUSH_BYTES = 256 << 20
 # DRAM bytes (read + write) of one 10^6-shot BP launch on this workload (BB144, p = 0.05,
 # 50 iterations), per kernel variant, from a one-pass ncu capture of the full workload;
 # a variant without a capture reports traffic null.
-BP_TRAFFIC_BYTES = {"bp_reg_kernel<32,3,6,5,3>": 75725312 + 152473088}
+BP_TRAFFIC_BYTES = {"bp_reg_kernel<32,3,6,5,3>": 76231936 + 152832512}
 
 
 def parse():
@@ -606,20 +605,20 @@ def hooks_leg(args, hx, hz, stream, flush, barrier, checker):
 
 
 def _bp_onchip_roofline(E, n, m, shots, st):
-    """BP with its message state on chip (one CTA per HGP shot): algorithmic ops against the
-    ALU peak, and the launch's algorithmic DRAM I/O (syndromes in; corrections of converged
-    shots and LLR rows of queued ones out) as GB/s."""
-    peak, src = alu_peak()
+    """BP with its message state on chip (one CTA per HGP shot): its shared-memory words against
+    the SMs' shared-memory rate, and the launch's algorithmic DRAM I/O (syndromes in; corrections
+    of converged shots and LLR rows of queued ones out) as GB/s."""
+    peak, src = smem_peak()
     s_bp = st["ms_bp"] / 1e3
-    ops = OPS_PER_EDGE_ITER * E * st["bp_iterations"]
+    smem = 4.0 * WORDS_PER_EDGE_ITER * E * st["bp_iterations"]
     io = shots * m + st["bp_converged"] * n + st["lsd_shots"] * 4 * n
     # a design that streams the messages reads and writes every FP32 edge message once per
     # iteration (8 B per edge-iteration): the bytes it would move, against the measured HBM
     # copy bandwidth, in this launch's time
     stream_bytes = 8.0 * E * st["bp_iterations"]
     hbm, hbm_src = hbm_peak()
-    return {"bound": "alu", "achieved_tops": ops / s_bp / 1e12, "peak_tops": peak,
-            "frac": ops / s_bp / 1e12 / peak, "peak_source": src,
+    return {"bound": "shared memory", "achieved_tbps": smem / s_bp / 1e12, "peak_tbps": peak,
+            "frac": smem / s_bp / 1e12 / peak, "peak_source": src,
             "io_bytes": int(io), "io_gbps": io / s_bp / 1e9,
             "streaming_equivalent": {"bytes": stream_bytes, "gbps": stream_bytes / s_bp / 1e9,
                                      "peak_gbps": hbm, "frac": stream_bytes / s_bp / 1e9 / hbm,
@@ -638,8 +637,8 @@ def hbm_peak():
         return 6800.0, "fallback (6.8 TB/s)"
 
 
-def alu_peak():
-    """(Tops/s, description): FP32/INT32 lanes x the maximum SM clock of MEASURED_PEAKS.json."""
+def smem_peak():
+    """(TB/s, description): 128 bytes a cycle and SM at the maximum SM clock of MEASURED_PEAKS.json."""
     import torch
     peaks = {}
     try:
@@ -649,7 +648,7 @@ def alu_peak():
         pass
     mhz = float(peaks.get("sm_max_mhz", 2070.0))
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    return sms * 128 * mhz * 1e6 / 1e12, f"{sms} SMs x 128 lanes x {mhz:.0f} MHz (max SM clock)"
+    return sms * 128 * mhz * 1e6 / 1e12, f"{sms} SMs x 128 B x {mhz:.0f} MHz (max SM clock)"
 
 
 def hgp_leg(args, stream, flush, barrier):
@@ -969,14 +968,14 @@ def run_ours(args):
     E = int(hx.sum())
     bp_ms_avg = float(np.mean(bp_ms))
     iters_per_step = iters_sum / args.steps
-    peak, peak_src = alu_peak()
-    achieved = OPS_PER_EDGE_ITER * E * iters_per_step / (bp_ms_avg / 1000.0) / 1e12
+    peak, peak_src = smem_peak()
+    achieved = 4 * WORDS_PER_EDGE_ITER * E * iters_per_step / (bp_ms_avg / 1000.0) / 1e12
     bp_name = bp_variant_name(tune["bp_variant"]) if tune else None
-    roofline = {"bound": "alu", "kernel": bp_name or "bp (default variant)",
-                "achieved": achieved, "peak": peak, "unit": "Tops/s", "frac": achieved / peak,
+    roofline = {"bound": "shared memory", "kernel": bp_name or "bp (default variant)",
+                "achieved": achieved, "peak": peak, "unit": "TB/s", "frac": achieved / peak,
                 "traffic": BP_TRAFFIC_BYTES.get(bp_name),
                 "peak_source": peak_src,
-                "ops_per_unit": f"{OPS_PER_EDGE_ITER} x {E} edges x {iters_per_step:.0f} "
+                "bytes_per_unit": f"4 B x {WORDS_PER_EDGE_ITER} words x {E} edges x {iters_per_step:.0f} "
                                 "shot-iterations"}
     legs = {"lsd_clusters": clusters, "autotune": tune, "learned": learned,
             "p_sweep": p_sweep, "lsd_mu_cs4": lsd_mu, "windows": windows, "giant_shot": giant,

@@ -451,8 +451,9 @@ __global__ void __launch_bounds__(512) bp_cta_kernel(BPArgs a) {
 // minimum (they start at kBig) and no sign or parity, and the message written for it is read
 // by nobody but its own q: the update equals the unpadded one bit for bit, without a
 // predicate.  Same results as bp_kernel<G, 0>.
-// Bound by shared-memory wavefronts: with DC words per row the row stride of 8 words made
-// every store, reload and gather of a message an 8-way bank conflict.  BP of 100 003 shots of
+// Bound by shared-memory wavefronts (68 % of the cycles for BB144 d = 12, 78 % for HGP, at two
+// CTAs of 256 or one of 512 threads per SM) and their latency: with DC words per row the row stride
+// of 8 words made every store, reload and gather of a message an 8-way bank conflict.  BP of 100 003 shots of
 // the BB144 d = 12 space-time matrix 3.30 -> 1.21 ms, 20 000 of BB288 d = 18 2.62 -> 1.20 ms,
 // 99 991 of the BB144 d = 6 hooks matrix 3.19 -> 2.10 ms, 50 000 of HGP at p = 0.02 8.89 ->
 // 5.86 ms.  Testing the parities before the messages are computed (MSG) costs a barrier and
@@ -766,7 +767,9 @@ const void* generic_fn(int v) {
 // Shapes of bp_regcta_kernel: (NT, CPL, DC, VPL, DV, PAD, MINB), then MSG and PRI; rows of
 // degree exactly DC (PAD false) or at most DC (PAD true), columns of degree at most DV; MINB
 // CTAs per SM bound the registers a thread may take.  MSG and PRI are set where the bound
-// leaves room for them (spilled messages cost more than reading them back from shared memory).
+// leaves room for them (spilled messages cost more than reading them back from shared memory);
+// some instances still spill up to 80 bytes, the 1024-thread ones up to 124, parts of the index
+// tables that are read back once an iteration.
 struct RegCtaShape {
   int nt, cpl, dc, vpl, dv;
   bool pad, pri;

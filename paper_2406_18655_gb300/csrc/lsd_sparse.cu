@@ -4,17 +4,17 @@
 //
 // One CTA owns one shot.  A shot needs few growth steps on a handful of clusters, or a thousand
 // columns when its clusters percolate, and a batch has from one such shot to a few per cent of
-// it; so what bounds the kernel is the latency of its longest shot (the SMs are busy for a
-// tenth to a fifth of it), and a step is spread over the CTA with the state in shared memory
-// and few barriers.  One warp per shot with its state in global scratch took, for
-//   50 000 HGP shots, p = 0.02, LSD-0 / LSD-10   5.3 / 13.0 ms, now 0.82 / 2.3 ms
-//   5000 HGP shots, p = 0.05 (percolating)       80-84 ms, now 7.8 ms
-//   100 003 BB144 d = 12, 20 000 BB288 d = 18    1.0, 0.58 ms, now 0.16, 0.09 ms
-//   99 991 BB144 hooks d = 6                     2.8 ms, now 0.38 ms
-// and the dense kernel, which ranks every fault first, 1.9 ms for 100 003 BB72 hooks d = 6
-// (now 0.12) and 0.69 ms for 50 001 BB144 windows (now 0.12).  Threads per shot, small / large
-// instance: 128 / 256 1.46 and 17.5 ms (HGP p = 0.02, 0.05), 256 / 512 0.98 and 11.1, 512 /
-// 1024 0.82 and 7.8.
+// it; so what bounds the kernel is the latency of its longest shot (issue 21-24 %; the first stall
+// is the barrier, 5 per issue), and a step is spread over the CTA with the state in shared memory
+// and few barriers.  LSD of the same shots by one warp per shot with its state in global scratch,
+// and now:
+//   50 000 HGP shots, p = 0.02, LSD-0 / LSD-10   7.7 / 16.5 ms, now 1.18 / 3.1 ms
+//   5000 HGP shots, p = 0.05 (percolating)       33.6 ms, now 5.5 ms
+//   100 003 BB144 d = 12, 20 000 BB288 d = 18    1.15, 0.67 ms, now 0.135, 0.090 ms
+//   99 991 BB144 hooks d = 6                     1.09 ms, now 0.18 ms
+// and by the dense kernel, which ranks every fault first, 2.33 ms for 100 003 BB72 hooks d = 6
+// (now 0.12) and 0.64 ms for 50 001 BB144 windows (now 0.09).  256 / 512 threads per shot (small /
+// large instance) instead of 512 / 1024: 1.43, 3.6 and 6.7 ms for the HGP rows.
 //   lab[m]     of a claimed detector: label << 16 | slot, else kFree.  A label is the number
 //              of a seed (flipped detector), flattened to the cluster's root after a merge; a
 //              slot is the detector's elimination row, in the order of claiming.

@@ -703,11 +703,11 @@ __device__ __forceinline__ void load_rows(__nv_bfloat16* dst, const __nv_bfloat1
   }
 }
 
-// Training, one CTA per SM and shot.  Bound by latency between its barriers (issue 43 %); at 16
-// warps a shot's 14 row tiles are one pass, a weight gradient is shared by two warps, the row
-// sums run beside them, and the graph is read from shared memory.  4096 BB144 pairs, 4 rounds:
-// 1.81 ms with 8 warps and 32-bit (weight gradients: 16-bit) fragment loads, now 1.39; BB72
-// 1.06 -> 0.96.
+// Training, one CTA per SM and shot.  Bound by latency between its barriers (issue 43 %; two in a
+// forward round, seven in a backward one); at 16 warps a shot's 14 row tiles are one pass, a weight
+// gradient is shared by two warps, the row sums run beside them, and the graph is read from shared
+// memory.  4096 BB144 pairs, 4 rounds: 1.82 ms with 8 warps and 32-bit (weight gradients: 16-bit)
+// fragment loads, now 1.37; BB72 1.08 -> 0.96.
 __global__ void __launch_bounds__(kTrainWarps * 32, 1) prior_train_kernel(TrainArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int m = a.m, n = a.n, R = a.rounds;
